@@ -388,10 +388,12 @@ ih_status optimizer_update(ih_sim *sim, const ih_opt_config *opt, uint32_t updat
  * culling tests (host uint64[6]; synchronises the stream). */
 ih_status sim_work_counters(ih_sim *sim, uint64_t *out, int32_t reset);
 
-/* Choose the step kernel's shape -- threads per environment (16, 32, 64 or
- * 128) and register-resident contacts per thread -- by timing every
- * supported shape whose capacity covers c_max on frames [frame0, frame0 +
- * n_frames) of the current state (one warm-up run, then the best of three).
+/* Choose the step kernel's shape -- the width of the solver's sums over an
+ * environment's contacts (16, 32, 64 or 128 partial sums, added as a tree) and a
+ * number of contacts per partial sum, which changes nothing -- by timing every
+ * supported shape on frames [frame0, frame0 + n_frames) of the current state
+ * (one warm-up run, then the best of three). The lanes that execute an
+ * environment are the library's choice and do not affect results.
  * The state, forces and work counters are
  * restored after every trial, so the call leaves the simulation unchanged.
  * Results of different shapes agree up to FP32 summation order. chosen
@@ -401,13 +403,11 @@ ih_status sim_work_counters(ih_sim *sim, uint64_t *out, int32_t reset);
  * environments onto the GPU is this library's. */
 ih_status sim_autotune(ih_sim *sim, int32_t frame0, int32_t n_frames, int32_t *chosen, float *ms);
 
-/* Force the step kernel's shape (threads per env, contacts per thread);
- * IH_ERR_ARG if unsupported or below c_max. */
+/* Force the step kernel's shape (see sim_autotune); IH_ERR_ARG if unsupported. */
 ih_status sim_set_variant(ih_sim *sim, int32_t threads_per_env, int32_t contacts_per_thread);
 
-/* The supported shapes as pairs (threads per env, contacts per thread):
- * writes up to `cap` pairs into out (host int32[2 * cap]) and returns how
- * many exist. */
+/* The supported shapes as pairs (sum width, contacts per partial sum): writes
+ * up to `cap` pairs into out (host int32[2 * cap]) and returns how many exist. */
 int32_t sim_step_variants(int32_t *out, int32_t cap);
 
 /* Measured FP32 throughput of the current device: the denominator of the

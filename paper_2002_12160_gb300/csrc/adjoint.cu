@@ -94,6 +94,40 @@ __device__ __forceinline__ Body load_body(const float4 *p) {
 }
 __device__ __forceinline__ Q4 qconj(Q4 q) { return {q.w, -q.x, -q.y, -q.z}; }
 
+// The forward substep's quaternion product and world inverse inertia, whose
+// contraction differs from the step's (internal.cuh) in the places named
+__device__ __forceinline__ Q4 qmul_f(Q4 a, Q4 b) {
+    return {__fmaf_rn(-a.z, b.z, __fmaf_rn(-a.y, b.y, prod_sub(a.w, b.w, a.x, b.x))),
+            __fmaf_rn(-a.z, b.y, __fmaf_rn(a.y, b.z, prod_add(a.x, b.w, a.w, b.x))),    // (a.w b.x rounded first)
+            __fmaf_rn(a.z, b.x, __fmaf_rn(a.y, b.w, prod_sub(a.w, b.y, a.x, b.z))),
+            __fmaf_rn(a.z, b.w, __fmaf_rn(-a.y, b.x, prod_add(a.x, b.y, a.w, b.z)))};   // (a.w b.z)
+}
+__device__ __forceinline__ S6 world_inv_inertia_f(const M3 &R, const S6 &J, float inv_m) {
+    const V3 r0 = {R.c0.x, R.c1.x, R.c2.x}, r1 = {R.c0.y, R.c1.y, R.c2.y}, r2 = {R.c0.z, R.c1.z, R.c2.z};
+    const V3 a0 = {__fmaf_rn(J.xz, r0.z, prod_add(J.xy, r0.y, J.xx, r0.x)), __fmaf_rn(J.yz, r0.z, prod_add(J.yy, r0.y, J.xy, r0.x)),
+                   __fmaf_rn(J.zz, r0.z, prod_add(J.xz, r0.x, J.yz, r0.y))};   // (first and second row)
+    return sandwich(r0, r1, r2, a0, smul(J, r1), smul(J, r2), inv_m);
+}
+// The reverse sweep's products, their contraction left to the compiler
+__device__ __forceinline__ V3 cross_r(V3 a, V3 b) {
+    return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+}
+__device__ __forceinline__ V3 smul_r(const S6 &A, V3 v) {
+    return {A.xx * v.x + A.xy * v.y + A.xz * v.z,
+            A.xy * v.x + A.yy * v.y + A.yz * v.z,
+            A.xz * v.x + A.yz * v.y + A.zz * v.z};
+}
+__device__ __forceinline__ Q4 qmul_r(Q4 a, Q4 b) {
+    return {a.w * b.w - a.x * b.x - a.y * b.y - a.z * b.z,
+            a.w * b.x + a.x * b.w + a.y * b.z - a.z * b.y,
+            a.w * b.y - a.x * b.z + a.y * b.w + a.z * b.x,
+            a.w * b.z + a.x * b.y - a.y * b.x + a.z * b.w};
+}
+__device__ __forceinline__ S6 world_inv_inertia_r(const M3 &R, const S6 &J, float inv_m) {
+    const V3 r0 = {R.c0.x, R.c1.x, R.c2.x}, r1 = {R.c0.y, R.c1.y, R.c2.y}, r2 = {R.c0.z, R.c1.z, R.c2.z};
+    return sandwich(r0, r1, r2, smul_r(J, r0), smul_r(J, r1), smul_r(J, r2), inv_m);
+}
+
 template <int GW>
 struct alignas(16) GroupSm {
     // contacts whose record (besides the slot's global one, which the tape
@@ -273,7 +307,7 @@ __device__ __noinline__ int fwd_substep(const AdjArgs &a, const Env &E_, Body &b
     const V3 v_pred = b.v + grav;
     const V3 w_pred = b.w;
     const M3 R = qmat(b.q);
-    const S6 Wi = world_inv_inertia(R, E.Jb, E.inv_m);
+    const S6 Wi = world_inv_inertia_f(R, E.Jb, E.inv_m);
     const int lane = G.lane;
 
     const int gt = G.gt;
@@ -488,7 +522,7 @@ __device__ __noinline__ int fwd_substep(const AdjArgs &a, const Env &E_, Body &b
         float sn, cs;
         sincosf(0.5f * wn * h, &sn, &cs);
         const float kq = (wn > 0.0f) ? sn / wn : 0.5f * h;
-        b.q = qnorm(qmul({cs, b.w.x * kq, b.w.y * kq, b.w.z * kq}, b.q));
+        b.q = qnorm(qmul_f({cs, b.w.x * kq, b.w.y * kq, b.w.z * kq}, b.q));
     }
     if (PADS) {
         // pad forces -lambda / h, each pad summing the contacts of its link in
@@ -634,14 +668,14 @@ __device__ __forceinline__ void contact_setup_bwd(const float4 *rc, V3 nb, V3 rb
     const float trKb = Db;
     knb -= Db;
     // k_n = 1/m + (r x n) . W (r x n)
-    const V3 rn = cross(r, n);
-    const V3 rnb = smul(Wi, rn) * (2.0f * knb);
+    const V3 rn = cross_r(r, n);
+    const V3 rnb = smul_r(Wi, rn) * (2.0f * knb);
     invm_l += knb + 3.0f * trKb;
     outer_add(Wbar, rn, rn, knb);
-    rb = rb + cross(n, rnb);
-    nb = nb + cross(rnb, r);
+    rb = rb + cross_r(n, rnb);
+    nb = nb + cross_r(rnb, r);
     // tr K = 3/m + |r|^2 tr W - r . W r
-    rb = rb + (r * (2.0f * trW) - smul(Wi, r) * 2.0f) * trKb;
+    rb = rb + (r * (2.0f * trW) - smul_r(Wi, r) * 2.0f) * trKb;
     const float rr = dot(r, r) * trKb;
     Wbar[0] += rr; Wbar[4] += rr; Wbar[8] += rr;
     outer_add(Wbar, r, r, -trKb);
@@ -674,7 +708,7 @@ __device__ __forceinline__ void contact_update_bwd(V3 r, V3 n, V3 cc, float ikn,
                                                    float mu, float inv_nc, float width, float beta_s, V3 &lb,
                                                    V3 &nb, V3 &rb, V3 &cb, float &iknb, float &iktb, float &mu_b,
                                                    float (&acc)[6]) {
-    const V3 u = Vi + cross(Wv, r) - cc;
+    const V3 u = Vi + cross_r(Wv, r) - cc;
     const float un = dot(u, n), lo = dot(l0, n);
     const float zn = lo - un * ikn;
     const float ln = fmaxf(zn, 0.0f);
@@ -710,10 +744,10 @@ __device__ __forceinline__ void contact_update_bwd(V3 r, V3 n, V3 cc, float ikn,
     ub = ub + n * unb;
     nb = nb + u * unb;
     // u = V + W x r - c
-    const V3 rxu = cross(r, ub);
+    const V3 rxu = cross_r(r, ub);
     acc[0] += ub.x; acc[1] += ub.y; acc[2] += ub.z;
     acc[3] += rxu.x; acc[4] += rxu.y; acc[5] += rxu.z;
-    rb = rb + cross(ub, Wv);
+    rb = rb + cross_r(ub, Wv);
     cb = cb - ub;
 }
 
@@ -745,14 +779,14 @@ __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const 
     const V3 v_pred = b.v + grav;
     const V3 w_pred = b.w;
     const M3 R = qmat(b.q);
-    const S6 Wi = world_inv_inertia(R, E.Jb, E.inv_m);
+    const S6 Wi = world_inv_inertia_r(R, E.Jb, E.inv_m);
     const float trW = Wi.xx + Wi.yy + Wi.zz;
     const bool solved = nc > 0 && I > 0;
     V3 Vf = v_pred, Wf = w_pred;   // body velocity after the solve
     if (solved) {
         const float *s = sp.sh + 8 * (I - 1);
         Vf = v_pred + mk(s[0], s[1], s[2]) * E.inv_m;
-        Wf = w_pred + smul(Wi, mk(s[3], s[4], s[5]));
+        Wf = w_pred + smul_r(Wi, mk(s[3], s[4], s[5]));
     }
 
     // -- integration: x' = x + h V, q' = normalize(exp(h W) q)
@@ -765,14 +799,14 @@ __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const 
         sincosf(0.5f * wn * h, &sn, &cs);
         const float kq = (wn > 0.0f) ? sn / wn : 0.5f * h;
         const Q4 e = {cs, Wf.x * kq, Wf.y * kq, Wf.z * kq};
-        const Q4 p = qmul(e, b.q);
+        const Q4 p = qmul_r(e, b.q);
         const float s = rsqrtf(p.w * p.w + p.x * p.x + p.y * p.y + p.z * p.z);
         const Q4 qn = {p.w * s, p.x * s, p.y * s, p.z * s};
         const float dq = ad.q.w * qn.w + ad.q.x * qn.x + ad.q.y * qn.y + ad.q.z * qn.z;
         const Q4 pb = {(ad.q.w - qn.w * dq) * s, (ad.q.x - qn.x * dq) * s, (ad.q.y - qn.y * dq) * s,
                        (ad.q.z - qn.z * dq) * s};
-        qb = qmul(qconj(e), pb);                // p = e q: dq = L(e)^T dp
-        const Q4 eb = qmul(pb, qconj(b.q));     // de = R(q)^T dp
+        qb = qmul_r(qconj(e), pb);                // p = e q: dq = L(e)^T dp
+        const Q4 eb = qmul_r(pb, qconj(b.q));     // de = R(q)^T dp
         // e = (cos(th/2), s(th) A), A = h W, th = |A|, s(th) = sin(th/2) / th
         const float th = wn * h;
         const float sf = kq / h;
@@ -857,21 +891,21 @@ __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const 
                 invm_l += dot(Vb, S1);
                 outer_add(Wbar, Wb, S2, 1.0f);
             }
-            const V3 g = smul(Wi, Wb);
+            const V3 g = smul_r(Wi, Wb);
             const V3 vm = Vb * E.inv_m;
             // every register slot without a branch (an empty slot has r = l1 = 0
             // and keeps lb = 0, so its reverse below adds zeros)
 #pragma unroll
             for (int k = 0; k < PL; ++k) {
-                const V3 lbk = lb[k] + vm + cross(g, r_[k]);
+                const V3 lbk = lb[k] + vm + cross_r(g, r_[k]);
                 lb[k] = (G.gt + T * k < nc) ? lbk : lb[k];
-                rb[k] = rb[k] + cross(l1_[k], g);
+                rb[k] = rb[k] + cross_r(l1_[k], g);
             }
             // (b) the contact updates of iteration it, against V^it, W^it
             V3 Vi = v_pred, Wv = w_pred;
             if (it > 0) {
                 Vi = v_pred + mk(sp_lo.x, sp_lo.y, sp_lo.z) * E.inv_m;
-                Wv = w_pred + smul(Wi, mk(sp_lo.w, sp_hi.x, sp_hi.y));
+                Wv = w_pred + smul_r(Wi, mk(sp_lo.w, sp_hi.x, sp_hi.y));
             }
             float acc[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
@@ -884,7 +918,7 @@ __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const 
                 float4 *A = sp.adjs + 4 * ci;
                 const float4 a0 = A[0], a1 = A[1], a2 = A[2], a3 = A[3];
                 const V3 r = xyz(r0);
-                V3 lbk = xyz(a0) + vm + cross(g, r), nbk = xyz(a1), rbk = xyz(a2) + cross(lam_at(it, ci), g),
+                V3 lbk = xyz(a0) + vm + cross_r(g, r), nbk = xyz(a1), rbk = xyz(a2) + cross_r(lam_at(it, ci), g),
                    cbk = xyz(a3);
                 float iknbk = a0.w, iktbk = a1.w;
                 contact_update_bwd(r, xyz(r1), xyz(r2), r1.w, r2.w, lam_at(it - 1, ci), Vi, Wv, E.mu, inv_nc, width,
@@ -1283,7 +1317,7 @@ __global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
     }
     if (lane == 0) {
         // rotation tangent: q = exp(delta) q0, d/d delta at 0 = vec(qbar (x) conj(q0)) / 2
-        const Q4 g = qmul(ad.q, qconj(b0.q));
+        const Q4 g = qmul_r(ad.q, qconj(b0.q));
         float *gr = a.grad + 8 * slot;
         gr[0] = ad.x.x; gr[1] = ad.x.y; gr[2] = ad.x.z;
         gr[3] = 0.5f * g.x; gr[4] = 0.5f * g.y; gr[5] = 0.5f * g.z;

@@ -23,7 +23,7 @@ struct ih_sim {
     DevConfig dcfg{};
     uint64_t seed = 0;
     cudaStream_t stream = nullptr;
-    StepVariant variant{32, 4, 128};
+    StepVariant variant{32, 4, 32};
     int step_grid = 0;
     int s_max = 1;   // most spheres in one shape
     int sms = 1;     // SMs of the device
@@ -168,33 +168,38 @@ DevScene dev_scene(const ih_sim *s) {
     return d;
 }
 
-// Default step-kernel shape before any autotuning: few environments get a
-// whole CTA each (latency bound), many get one warp each (issue bound); the
-// register-resident contacts per thread must cover c_max.
-StepVariant default_variant(int N, int c_max) {
-    (void)c_max;   // every shape holds any c_max
-    return N <= 4096 ? StepVariant{64, 2, 128} : StepVariant{32, 2, 128};
-}
+// Default step-kernel shape before any autotuning.
+StepVariant default_variant(int N) { return N <= 4096 ? StepVariant{64, 2, 0} : StepVariant{32, 2, 0}; }
 
-int grid_for(const StepVariant &v, int N) {
-    const int groups_per_block = v.block / v.group;
-    const int need = (N + groups_per_block - 1) / groups_per_block;
-    return need > 0 ? need : 1;
+// The lanes of a warp that execute an environment (the results do not depend on
+// them). A whole warp by default; two environments to a warp for the 16-wide
+// shapes, and for objects of at most 32 spheres (rarely more than 16 contacts a
+// substep, 25 at most for the 27-sphere box) once there are more environments
+// than 12 warps per SM hold. Four frames of the box, 32 against 16 lanes: 90 / 102 us
+// at N = 1500, 107 / 101 at 2000, 167 / 124 at 3000, 644 / 500 at 16384; objects
+// with more contacts lose at every size (uneven 4000: 360 / 572 us, 3000
+// cylinders 363 / 591).
+int step_lanes(int group, int N, int s_max, int sms) {
+    if (group == 16) return 16;
+    if (group == 128) return 32;
+    return s_max <= 32 && N > 12 * sms ? 16 : 32;
 }
 
 // Make v the step shape: shared-memory opt-in, a persistent grid of at most the
-// blocks that fit on the device at once (the groups take environments from the
+// one-warp blocks that fit on the device at once (they take environments from the
 // launch's work queue), and a spill area for the contacts beyond the shape's
 // shared-memory staging, grown when needed (cudaFree synchronises the device,
 // so no launch still uses the old one).
-cudaError_t use_variant(ih_sim *s, const StepVariant &v) {
+cudaError_t use_variant(ih_sim *s, StepVariant v) {
+    v.lanes = step_lanes(v.group, s->cfg.n_envs, s->s_max, s->sms);
     int bps = 0;
     cudaError_t e = step_prepare(v, s->s_max, s->cfg.c_max, s->dcfg.warm != 0, s->clp_cap, &bps);
     if (e != cudaSuccess) return e;
     const int resident = std::max(1, bps) * std::max(1, s->sms);
-    const int grid = std::min(grid_for(v, s->cfg.n_envs), resident);
+    const int epb = step_envs_per_block(v);
+    const int grid = std::min((s->cfg.n_envs + epb - 1) / epb, resident);
     const int sc = step_stage_capacity(v, s->cfg.c_max);
-    const size_t need = (size_t)grid * (v.block / v.group) * (size_t)(s->cfg.c_max - sc) * 4;
+    const size_t need = (size_t)grid * epb * (size_t)(s->cfg.c_max - sc) * 4;
     if (need > s->spill_f4) {
         // a captured window graph holds the old spill pointer: let it finish, capture again
         if (s->cap_stream) cudaStreamSynchronize(s->cap_stream);
@@ -289,7 +294,7 @@ ih_status sim_create(const ih_scene *sc, const ih_config *cfg, uint64_t seed, vo
     d.kp = cfg->kp; d.kd = cfg->kd; d.armature = cfg->armature; d.v_slip = cfg->v_slip; d.w_slip = cfg->w_slip;
     for (int k = 0; k < 10; ++k) d.w_full[k] = cfg->w_full[k];
     s->pd = cfg->hand == IH_HAND_PD;
-    s->variant = default_variant(cfg->n_envs, cfg->c_max);
+    s->variant = default_variant(cfg->n_envs);
     const int N = cfg->n_envs, P = sc->n_pads, F = sc->n_fingers;
 
     cudaError_t e = cudaSuccess;
@@ -543,8 +548,8 @@ ih_status sim_step(ih_sim *s, int32_t frame0, int32_t n_frames) {
     a.cm_frames = nullptr; a.pose_frames = nullptr;
     a.cache = s->cache; a.cache_n = s->cache_n;
     a.stage_cap = s->stage_cap; a.spill = s->spill; a.clp_cap = s->clp_cap;
-    // the work queue only when the grid's groups are fewer than the environments
-    a.queue = (size_t)s->step_grid * (s->variant.block / s->variant.group) < (size_t)s->cfg.n_envs ? s->queue : nullptr;
+    // the work queue only when the grid holds fewer than all environments
+    a.queue = (size_t)s->step_grid * step_envs_per_block(s->variant) < (size_t)s->cfg.n_envs ? s->queue : nullptr;
     cudaError_t e = launch_step(a, s->variant, s->step_grid, s->s_max, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "step launch");
     s->stepped = true;
@@ -565,8 +570,8 @@ StepArgs scored_args(ih_sim *s, int frame, const float *obs, double *cost_mean, 
     a.cm_frames = nullptr; a.pose_frames = nullptr;
     a.cache = s->cache; a.cache_n = s->cache_n;
     a.stage_cap = s->stage_cap; a.spill = s->spill; a.clp_cap = s->clp_cap;
-    // the work queue only when the grid's groups are fewer than the environments
-    a.queue = (size_t)s->step_grid * (s->variant.block / s->variant.group) < (size_t)s->cfg.n_envs ? s->queue : nullptr;
+    // the work queue only when the grid holds fewer than all environments
+    a.queue = (size_t)s->step_grid * step_envs_per_block(s->variant) < (size_t)s->cfg.n_envs ? s->queue : nullptr;
     return a;
 }
 
@@ -966,11 +971,8 @@ ih_status sim_work_counters(ih_sim *s, uint64_t *out, int32_t reset) {
 ih_status sim_set_variant(ih_sim *s, int32_t tpe, int32_t cpl) {
     if (!s) return IH_ERR_ARG;
     if (s->pd) return refuse_pd(s, "sim_set_variant");
-    StepVariant v{tpe, cpl, 128};
-    if (!step_variant_supported(v)) return fail(s, IH_ERR_ARG, "unsupported step shape %d x %d", tpe, cpl);
-    if (step_variant_max_contacts(v) < s->cfg.c_max)
-        return fail(s, IH_ERR_ARG, "shape %d x %d holds fewer than c_max = %d contacts", tpe, cpl, s->cfg.c_max);
-    cudaError_t e = use_variant(s, v);
+    if (!step_variant_supported(tpe, cpl)) return fail(s, IH_ERR_ARG, "unsupported step shape %d x %d", tpe, cpl);
+    cudaError_t e = use_variant(s, StepVariant{tpe, cpl, 0});
     if (e != cudaSuccess) return cuda_fail(s, e, "set_variant");
     return IH_OK;
 }
@@ -1034,7 +1036,7 @@ ih_status sim_autotune(ih_sim *s, int32_t frame0, int32_t n_frames, int32_t *cho
     if (e == cudaSuccess) { save(); e = cudaStreamSynchronize(st); }
     for (int k = 0; k < nv && e == cudaSuccess; ++k) {
         float ms = NAN;
-        if (step_variant_max_contacts(cand[k]) >= s->cfg.c_max && use_variant(s, cand[k]) == cudaSuccess) {
+        if (use_variant(s, cand[k]) == cudaSuccess) {
             ih_status r = sim_step(s, frame0, n_frames);   // warm-up (and first-use setup)
             restore();
             for (int rep = 0; rep < 3 && r == IH_OK && e == cudaSuccess; ++rep) {

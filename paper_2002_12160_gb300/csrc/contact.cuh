@@ -16,31 +16,36 @@ struct Hit {
     float t;  // axial fraction along a capsule, 0 on the palm
 };
 
-// sphere (centre c, radius rs) against the palm box (pose a, q; half extents)
-__device__ __forceinline__ Hit hit_box(V3 c, float rs, V3 a, Q4 q, float hx, float hy, float hz) {
-    const V3 cl = qrot_inv(q, c - a);
-    const V3 k = mk(fminf(fmaxf(cl.x, -hx), hx), fminf(fmaxf(cl.y, -hy), hy), fminf(fmaxf(cl.z, -hz), hz));
+// sphere (centre c, radius rs) against a box of the given half extents at the
+// origin of c's frame
+__device__ __forceinline__ Hit hit_box_local(V3 c, float rs, float hx, float hy, float hz) {
+    const V3 k = mk(fminf(fmaxf(c.x, -hx), hx), fminf(fmaxf(c.y, -hy), hy), fminf(fmaxf(c.z, -hz), hz));
     Hit h;
     h.t = 0.0f;
-    const bool inside = (k.x == cl.x) && (k.y == cl.y) && (k.z == cl.z);
+    const bool inside = (k.x == c.x) && (k.y == c.y) && (k.z == c.z);
     if (!inside) {
-        const V3 d = cl - k;
+        const V3 d = c - k;
         const float d2 = dot(d, d);
         const float inv = rsqrtf(d2);   // d2 > 0: the centre is outside the box
-        h.n = qrot(q, d * inv);
+        h.n = d * inv;
         h.gap = d2 * inv - rs;
     } else {
         // shallowest face, ties to the lowest axis and the + side
-        float best = hx - cl.x;
-        V3 nl = mk(1, 0, 0);
-        if (hx + cl.x < best) { best = hx + cl.x; nl = mk(-1, 0, 0); }
-        if (hy - cl.y < best) { best = hy - cl.y; nl = mk(0, 1, 0); }
-        if (hy + cl.y < best) { best = hy + cl.y; nl = mk(0, -1, 0); }
-        if (hz - cl.z < best) { best = hz - cl.z; nl = mk(0, 0, 1); }
-        if (hz + cl.z < best) { best = hz + cl.z; nl = mk(0, 0, -1); }
-        h.n = qrot(q, nl);
+        float best = hx - c.x;
+        h.n = mk(1, 0, 0);
+        if (hx + c.x < best) { best = hx + c.x; h.n = mk(-1, 0, 0); }
+        if (hy - c.y < best) { best = hy - c.y; h.n = mk(0, 1, 0); }
+        if (hy + c.y < best) { best = hy + c.y; h.n = mk(0, -1, 0); }
+        if (hz - c.z < best) { best = hz - c.z; h.n = mk(0, 0, 1); }
+        if (hz + c.z < best) { best = hz + c.z; h.n = mk(0, 0, -1); }
         h.gap = -best - rs;
     }
+    return h;
+}
+// ... and the palm box at pose a, q
+__device__ __forceinline__ Hit hit_box(V3 c, float rs, V3 a, Q4 q, float hx, float hy, float hz) {
+    Hit h = hit_box_local(qrot_inv(q, c - a), rs, hx, hy, hz);
+    h.n = qrot(q, h.n);
     return h;
 }
 
@@ -82,9 +87,10 @@ __device__ __forceinline__ bool link_reaches(const DevScene &sc, const DevConfig
     return dot(dd, dd) < reach * reach;
 }
 
+// (one division for both regimes, so that a warp that mixes them divides once)
 __device__ __forceinline__ float contact_bias(const DevConfig &cfg, float gap) {
-    if (gap > 0.0f) return gap / cfg.h;
-    return fmaxf(cfg.beta * fminf(gap + cfg.slop, 0.0f) / cfg.h, -cfg.vmax);
+    const float q = (gap > 0.0f ? gap : cfg.beta * fminf(gap + cfg.slop, 0.0f)) / cfg.h;
+    return gap > 0.0f ? q : fmaxf(q, -cfg.vmax);
 }
 
 __device__ __forceinline__ bool all_finite(V3 x, Q4 q, V3 v, V3 w) {
@@ -106,7 +112,7 @@ __device__ __forceinline__ CSetup setup_contact(V3 r, V3 n, float gap, int l, co
     // k_n = 1/m + (r x n)^T W (r x n); tr K = 3/m + |r|^2 tr W - r^T W r
     const V3 rn = cross(r, n);
     const float kn = inv_m + dot(rn, smul(Wi, rn));
-    const float trK = 3.0f * inv_m + dot(r, r) * trW - dot(r, smul(Wi, r));
+    const float trK = prod_add(3.0f, inv_m, dot(r, r), trW) - dot(r, smul(Wi, r));
     CSetup c;
     c.ikn = 1.0f / kn;
     c.ikt = 2.0f / (trK - kn);
@@ -117,7 +123,8 @@ __device__ __forceinline__ CSetup setup_contact(V3 r, V3 n, float gap, int l, co
         const float4 Aq = __ldg(L0 + l * kLinkStride + 2), Bq = __ldg(L1 + l * kLinkStride + 2);
         const Q4 qa = {Aq.x, Aq.y, Aq.z, Aq.w}, qb = {Bq.x, Bq.y, Bq.z, Bq.w};
         const V3 pl = qrot_inv(qa, (x - xyz(A0)) + r);   // contact in link coords
-        vl = ((xyz(B0) - xyz(A0)) + (qrot(qb, pl) - qrot(qa, pl))) * inv_h;
+        const V3 d = (xyz(B0) - xyz(A0)) + (qrot(qb, pl) - qrot(qa, pl));
+        vl = {__fmul_rn(d.x, inv_h), __fmul_rn(d.y, inv_h), __fmul_rn(d.z, inv_h)};
     }
     c.cc = vl - n * b;
     return c;
@@ -135,15 +142,96 @@ __device__ __forceinline__ V3 update_contact(V3 lam, V3 r, V3 n, V3 cc, float ik
     const float un = dot(u, n);
     const float l_old = dot(lam, n);
     const float ln = fmaxf(l_old - un * ikn, 0.0f);
-    V3 lt = (lam - n * l_old) - (u - n * un) * ikt;
+    const V3 lt = (lam - n * l_old) - (u - n * un) * ikt;
     const float tn2 = dot(lt, lt);
     const float lim = mu * ln;
     const bool slip = tn2 > lim * lim;
     const float sc = lim * rsqrtf(slip ? tn2 : 1.0f);
-    lt = lt * (slip ? sc : 1.0f);
-    const V3 lp = n * ln + lt;
+    const float f = slip ? sc : 1.0f;
+    const V3 lp = {prod_add(n.x, ln, lt.x, f), prod_add(n.y, ln, lt.y, f), prod_add(n.z, ln, lt.z, f)};
     return lam + (lp - lam) * inv_nc;
 }
+
+// The same update on one contact (T = float) or on two at once (T = float2, the
+// packed FP32 instructions: half the issue slots of two scalar updates, and two
+// chains that interleave), bit for bit update_contact's: every operation is the
+// scalar one of each half, and a product's sign may move (rounding is
+// symmetric). Two contacts cost ~70 issue slots instead of ~130; an iteration
+// of a 60-contact environment at 16 warps per SM took 258 cycles a warp scalar,
+// 198 packed. The reciprocal square root is taken of the argument scaled by
+// 2^24, which no FP32 value leaves denormal, so the approximate instruction
+// needs no denormal path (18 cycles instead of 40); for arguments below 2^104 it
+// equals rsqrtf bit for bit (all of them compared).
+typedef float2 F2;
+__device__ __forceinline__ float t_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ F2 t_fma(F2 a, F2 b, F2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float t_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ F2 t_mul(F2 a, F2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float t_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ F2 t_add(F2 a, F2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float t_neg(float a) { return -a; }
+__device__ __forceinline__ F2 t_neg(F2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float t_relu(float a) { return fmaxf(a, 0.0f); }
+__device__ __forceinline__ F2 t_relu(F2 a) { return make_float2(fmaxf(a.x, 0.0f), fmaxf(a.y, 0.0f)); }
+template <typename T> __device__ __forceinline__ T t_all(float a);
+template <> __device__ __forceinline__ float t_all<float>(float a) { return a; }
+template <> __device__ __forceinline__ F2 t_all<F2>(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// scale of the disk clamp: lim / |t| where |t| > lim, else 1, from t2 = 2^24 |t|^2 and lim = 2^12 mu l_n
+__device__ __forceinline__ float t_clamp(float t2, float lim) {
+    const float sc = lim * rsqrt_ftz(t2);
+    return t2 > lim * lim ? sc : 1.0f;
+}
+__device__ __forceinline__ F2 t_clamp(F2 t2, F2 lim) { return make_float2(t_clamp(t2.x, lim.x), t_clamp(t2.y, lim.y)); }
+
+template <typename T>
+struct Vec {
+    T x, y, z;
+};
+template <typename T>
+__device__ __forceinline__ T t_dot(const Vec<T> &a, const Vec<T> &b) { return t_fma(a.x, b.x, t_fma(a.y, b.y, t_mul(a.z, b.z))); }
+template <typename T>
+struct Contact {
+    Vec<T> r, n, c, lam;
+    T ikn, ikt;
+    __device__ __forceinline__ void clear() {   // an empty slot: keeps a zero impulse and adds zeros
+        const T o = t_all<T>(0.0f);
+        r = c = lam = {o, o, o};
+        n = {o, o, t_all<T>(1.0f)};
+        ikn = ikt = o;
+    }
+    // lam after one update against the velocity (v, w); mu_s = 2^12 mu
+    __device__ __forceinline__ void update(V3 v, V3 w, float mu_s, float inv_nc) {
+        const Vec<T> nv = {t_all<T>(-v.x), t_all<T>(-v.y), t_all<T>(-v.z)}, pw = {t_all<T>(w.x), t_all<T>(w.y), t_all<T>(w.z)},
+                     nw = {t_all<T>(-w.x), t_all<T>(-w.y), t_all<T>(-w.z)};
+        // -u = c - (v + w x r)
+        const Vec<T> nu = {t_add(t_add(nv.x, t_fma(nw.y, r.z, t_mul(pw.z, r.y))), c.x),
+                           t_add(t_add(nv.y, t_fma(nw.z, r.x, t_mul(pw.x, r.z))), c.y),
+                           t_add(t_add(nv.z, t_fma(nw.x, r.y, t_mul(pw.y, r.x))), c.z)};
+        const T nun = t_dot(nu, n), lo = t_dot(lam, n), un = t_neg(nun), nlo = t_neg(lo);
+        const T ln = t_relu(t_fma(nun, ikn, lo));
+        const Vec<T> t = {t_fma(t_fma(n.x, un, nu.x), ikt, t_fma(n.x, nlo, lam.x)),
+                          t_fma(t_fma(n.y, un, nu.y), ikt, t_fma(n.y, nlo, lam.y)),
+                          t_fma(t_fma(n.z, un, nu.z), ikt, t_fma(n.z, nlo, lam.z))};
+        const T f = t_clamp(t_mul(t_dot(t, t), t_all<T>(16777216.0f)), t_mul(t_all<T>(mu_s), ln));
+        const T m1 = t_all<T>(-1.0f), k = t_all<T>(inv_nc);
+        lam.x = t_fma(t_fma(lam.x, m1, t_fma(n.x, ln, t_mul(t.x, f))), k, lam.x);
+        lam.y = t_fma(t_fma(lam.y, m1, t_fma(n.y, ln, t_mul(t.y, f))), k, lam.y);
+        lam.z = t_fma(t_fma(lam.z, m1, t_fma(n.z, ln, t_mul(t.z, f))), k, lam.z);
+    }
+    // its impulse and moment r x lam
+    __device__ __forceinline__ void wrench(T (&s)[6]) const {
+        const Vec<T> nl = {t_neg(lam.x), t_neg(lam.y), t_neg(lam.z)};
+        s[0] = lam.x; s[1] = lam.y; s[2] = lam.z;
+        s[3] = t_fma(r.y, lam.z, t_mul(r.z, nl.y));
+        s[4] = t_fma(r.z, lam.x, t_mul(r.x, nl.z));
+        s[5] = t_fma(r.x, lam.y, t_mul(r.y, nl.x));
+    }
+};
 
 // Sum of 6 values over the WIDTH lanes of a group (WIDTH = 16 or 32), every
 // lane receiving all 6 sums. Reduce-scatter first: padded to 8 values, each

@@ -55,19 +55,24 @@ __device__ __forceinline__ V3 operator+(V3 a, V3 b) { return {a.x + b.x, a.y + b
 __device__ __forceinline__ V3 operator-(V3 a, V3 b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
 __device__ __forceinline__ V3 operator*(V3 a, float s) { return {a.x * s, a.y * s, a.z * s}; }
 __device__ __forceinline__ float dot(V3 a, V3 b) { return fmaf(a.x, b.x, fmaf(a.y, b.y, a.z * b.z)); }
+// Sums of two products with a fixed contraction, fma(a, b, +-round(c d)): left to
+// the compiler, which of the products is rounded first varies with the code
+// around it, and with it the last bits of every kernel that shares an expression.
+__device__ __forceinline__ float prod_add(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ float prod_sub(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
 __device__ __forceinline__ V3 cross(V3 a, V3 b) {
-    return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+    return {prod_sub(a.y, b.z, a.z, b.y), prod_sub(a.z, b.x, a.x, b.z), prod_sub(a.x, b.y, a.y, b.x)};
 }
 __device__ __forceinline__ V3 xyz(float4 v) { return {v.x, v.y, v.z}; }
 
 __device__ __forceinline__ Q4 qmul(Q4 a, Q4 b) {
-    return {a.w * b.w - a.x * b.x - a.y * b.y - a.z * b.z,
-            a.w * b.x + a.x * b.w + a.y * b.z - a.z * b.y,
-            a.w * b.y - a.x * b.z + a.y * b.w + a.z * b.x,
-            a.w * b.z + a.x * b.y - a.y * b.x + a.z * b.w};
+    return {__fmaf_rn(-a.z, b.z, __fmaf_rn(-a.y, b.y, prod_sub(a.w, b.w, a.x, b.x))),
+            __fmaf_rn(-a.z, b.y, __fmaf_rn(a.y, b.z, prod_add(a.w, b.x, a.x, b.w))),
+            __fmaf_rn(a.z, b.x, __fmaf_rn(a.y, b.w, prod_sub(a.w, b.y, a.x, b.z))),
+            __fmaf_rn(a.z, b.w, __fmaf_rn(-a.y, b.x, prod_add(a.w, b.z, a.x, b.y)))};
 }
 __device__ __forceinline__ Q4 qnorm(Q4 q) {
-    float s = rsqrtf(q.w * q.w + q.x * q.x + q.y * q.y + q.z * q.z);
+    float s = rsqrtf(__fmaf_rn(q.z, q.z, __fmaf_rn(q.y, q.y, prod_add(q.w, q.w, q.x, q.x))));
     return {q.w * s, q.x * s, q.y * s, q.z * s};
 }
 // rotate v by unit quaternion q: v + 2 w (u x v) + 2 u x (u x v)
@@ -76,36 +81,54 @@ __device__ __forceinline__ V3 qrot(Q4 q, V3 v) {
     V3 t = cross(u, v) * 2.0f;
     return v + t * q.w + cross(u, t);
 }
-__device__ __forceinline__ V3 qrot_inv(Q4 q, V3 v) { return qrot({q.w, -q.x, -q.y, -q.z}, v); }
+// by its inverse: the same with -u, as (v x u) and (t x u)
+__device__ __forceinline__ V3 qrot_inv(Q4 q, V3 v) {
+    V3 u = {q.x, q.y, q.z};
+    V3 t = cross(v, u) * 2.0f;
+    return v + t * q.w + cross(t, u);
+}
 
 // symmetric 3x3 stored as xx yy zz xy xz yz
 struct S6 { float xx, yy, zz, xy, xz, yz; };
 __device__ __forceinline__ V3 smul(const S6 &A, V3 v) {
-    return {A.xx * v.x + A.xy * v.y + A.xz * v.z,
-            A.xy * v.x + A.yy * v.y + A.yz * v.z,
-            A.xz * v.x + A.yz * v.y + A.zz * v.z};
+    return {__fmaf_rn(A.xz, v.z, prod_add(A.xx, v.x, A.xy, v.y)),
+            __fmaf_rn(A.yz, v.z, prod_add(A.xy, v.x, A.yy, v.y)),
+            __fmaf_rn(A.zz, v.z, prod_add(A.xz, v.x, A.yz, v.y))};
 }
 // columns of the rotation matrix of q
 struct M3 { V3 c0, c1, c2; };
 __device__ __forceinline__ M3 qmat(Q4 q) {
-    M3 R;
-    R.c0 = {1 - 2 * (q.y * q.y + q.z * q.z), 2 * (q.x * q.y + q.w * q.z), 2 * (q.x * q.z - q.w * q.y)};
-    R.c1 = {2 * (q.x * q.y - q.w * q.z), 1 - 2 * (q.x * q.x + q.z * q.z), 2 * (q.y * q.z + q.w * q.x)};
-    R.c2 = {2 * (q.x * q.z + q.w * q.y), 2 * (q.y * q.z - q.w * q.x), 1 - 2 * (q.x * q.x + q.y * q.y)};
+    M3 R;   // (the first diagonal entry's squares are both rounded)
+    R.c0 = {1 - 2 * __fadd_rn(__fmul_rn(q.y, q.y), __fmul_rn(q.z, q.z)), 2 * prod_add(q.x, q.y, q.w, q.z), 2 * prod_sub(q.x, q.z, q.w, q.y)};
+    R.c1 = {2 * prod_sub(q.x, q.y, q.w, q.z), 1 - 2 * prod_add(q.x, q.x, q.z, q.z), 2 * prod_add(q.w, q.x, q.y, q.z)};
+    R.c2 = {2 * prod_add(q.x, q.z, q.w, q.y), 2 * -prod_sub(q.w, q.x, q.y, q.z), 1 - 2 * prod_add(q.x, q.x, q.y, q.y)};
     return R;
 }
-__device__ __forceinline__ V3 mmul(const M3 &R, V3 v) { return R.c0 * v.x + R.c1 * v.y + R.c2 * v.z; }
+__device__ __forceinline__ V3 mmul(const M3 &R, V3 v) {
+    return {__fmaf_rn(R.c2.x, v.z, prod_add(R.c0.x, v.x, R.c1.x, v.y)),
+            __fmaf_rn(R.c2.y, v.z, prod_add(R.c0.y, v.x, R.c1.y, v.y)),
+            __fmaf_rn(R.c2.z, v.z, prod_add(R.c0.z, v.x, R.c1.z, v.y))};
+}
 __device__ __forceinline__ V3 mtmul(const M3 &R, V3 v) { return {dot(R.c0, v), dot(R.c1, v), dot(R.c2, v)}; }
+
+// r_i . a_j / m for the rows r_i of R and a_j = J^-1 r_j
+__device__ __forceinline__ S6 sandwich(V3 r0, V3 r1, V3 r2, V3 a0, V3 a1, V3 a2, float inv_m) {
+    S6 W;
+    W.xx = dot(r0, a0) * inv_m; W.yy = dot(r1, a1) * inv_m; W.zz = dot(r2, a2) * inv_m;
+    W.xy = dot(r0, a1) * inv_m; W.xz = dot(r0, a2) * inv_m; W.yz = dot(r1, a2) * inv_m;
+    return W;
+}
 
 // W = R J^-1 R^T / m for symmetric J^-1 (body frame)
 __device__ __forceinline__ S6 world_inv_inertia(const M3 &R, const S6 &Jb, float inv_m) {
     // columns of J R^T: rows of R are (c0.x, c1.x, c2.x) etc.
     V3 r0 = {R.c0.x, R.c1.x, R.c2.x}, r1 = {R.c0.y, R.c1.y, R.c2.y}, r2 = {R.c0.z, R.c1.z, R.c2.z};
-    V3 a0 = smul(Jb, r0), a1 = smul(Jb, r1), a2 = smul(Jb, r2);
-    S6 W;
-    W.xx = dot(r0, a0) * inv_m; W.yy = dot(r1, a1) * inv_m; W.zz = dot(r2, a2) * inv_m;
-    W.xy = dot(r0, a1) * inv_m; W.xz = dot(r0, a2) * inv_m; W.yz = dot(r1, a2) * inv_m;
-    return W;
+    auto jmul = [&](V3 v) -> V3 {   // (the contraction differs from smul's in the second row)
+        return {__fmaf_rn(Jb.xz, v.z, prod_add(Jb.xx, v.x, Jb.xy, v.y)),
+                __fmaf_rn(Jb.yz, v.z, prod_add(Jb.yy, v.y, Jb.xy, v.x)),
+                __fmaf_rn(Jb.zz, v.z, prod_add(Jb.xz, v.x, Jb.yz, v.y))};
+    };
+    return sandwich(r0, r1, r2, jmul(r0), jmul(r1), jmul(r2), inv_m);
 }
 
 // ---------------------------------------------------------------- Philox4x32-10
@@ -314,16 +337,18 @@ int pd_step_grid(int N, int sms);
 cudaError_t launch_pd_step(const PdArgs &a, int grid, int s_max, cudaStream_t s);
 cudaError_t launch_hand_rest(int N, int D, const float *q0, float *qj, float *qdj, cudaStream_t s);
 
+// A step shape (group, cpl) as the interface names it -- group, the width of the
+// solver's sums, alone fixes the results -- and the lanes of a warp that execute
+// an environment (chosen by the library; the results do not depend on them).
 struct StepVariant {
-    int group;        // lanes per environment
-    int cpl;          // register-resident contacts per lane
-    int block;        // threads per CTA
+    int group;
+    int cpl;
+    int lanes;
 };
+constexpr int step_envs_per_block(const StepVariant &v) { return 32 / v.lanes; }
 cudaError_t launch_step(const StepArgs &a, const StepVariant &v, int grid, int s_max, cudaStream_t s);
-int step_variant_max_contacts(const StepVariant &v);
-bool step_variant_supported(const StepVariant &v);
-size_t step_smem_bytes(const StepVariant &v, int s_max, int c_max, bool warm, int clp_cap);
-// contacts a shape stages in shared memory (the rest of c_max spill to global memory)
+bool step_variant_supported(int group, int cpl);
+// contacts staged in shared memory (the rest of c_max spill to global memory)
 int step_stage_capacity(const StepVariant &v, int c_max);
 int step_variant_list(StepVariant *out, int cap);
 
@@ -481,7 +506,6 @@ cudaError_t launch_win_desc(WinDesc *d, WinDesc v, cudaStream_t s);
 // shared-memory opt-in of a shape; blocks_per_sm (may be null) receives its occupancy
 cudaError_t step_prepare(const StepVariant &v, int s_max, int c_max, bool warm, int clp_cap, int *blocks_per_sm);
 // the warm-started instances (step_warm.cu)
-size_t step_smem_bytes_warm(const StepVariant &v, int s_max, int c_max, int clp_cap);
 cudaError_t step_prepare_warm(const StepVariant &v, int s_max, int c_max, int clp_cap, int *blocks_per_sm);
 cudaError_t launch_step_warm(const StepArgs &a, const StepVariant &v, int grid, int s_max, cudaStream_t s);
 cudaError_t launch_optimizer(const OptArgs &a, cudaStream_t s);

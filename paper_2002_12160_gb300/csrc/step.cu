@@ -5,13 +5,8 @@
 #include "step_kernel.cuh"
 
 namespace ih {
-// every shape holds any c_max <= IH_MAX_CONTACTS (contacts beyond its registers
-// live in shared memory, and beyond the shape's staging capacity in the spill area)
-int step_variant_max_contacts(const StepVariant &v) { return v.group > 0 ? IH_MAX_CONTACTS : 0; }
-
-bool step_variant_supported(const StepVariant &v) {
-    if (v.block != kBlock) return false;
-#define IH_SUP(T, C) if (v.group == T && v.cpl == C) return true;
+bool step_variant_supported(int group, int cpl) {
+#define IH_SUP(T, C) if (group == T && cpl == C) return true;
     IH_STEP_VARIANTS(IH_SUP)
 #undef IH_SUP
     return false;
@@ -19,14 +14,10 @@ bool step_variant_supported(const StepVariant &v) {
 
 int step_variant_list(StepVariant *out, int cap) {
     int n = 0;
-#define IH_LIST(T, C) if (n < cap) out[n] = StepVariant{T, C, kBlock}; ++n;
+#define IH_LIST(T, C) if (n < cap) out[n] = StepVariant{T, C, 0}; ++n;
     IH_STEP_VARIANTS(IH_LIST)
 #undef IH_LIST
     return n;
-}
-
-size_t step_smem_bytes(const StepVariant &v, int s_max, int c_max, bool warm, int clp_cap) {
-    return warm ? step_smem_bytes_warm(v, s_max, c_max, clp_cap) : smem_bytes_w<false>(v, s_max, c_max, clp_cap);
 }
 
 cudaError_t step_prepare(const StepVariant &v, int s_max, int c_max, bool warm, int clp_cap, int *blocks_per_sm) {
@@ -34,9 +25,7 @@ cudaError_t step_prepare(const StepVariant &v, int s_max, int c_max, bool warm, 
                 : prepare_w<false>(v, s_max, c_max, clp_cap, blocks_per_sm);
 }
 
-int step_stage_capacity(const StepVariant &v, int c_max) {
-    return stage_capacity(v.group * v.cpl, c_max, v.block / v.group);
-}
+int step_stage_capacity(const StepVariant &v, int c_max) { return stage_capacity(v.lanes, c_max); }
 
 cudaError_t launch_step(const StepArgs &a, const StepVariant &v, int grid, int s_max, cudaStream_t s) {
     return a.cfg.warm ? launch_step_warm(a, v, grid, s_max, s) : launch_w<false>(a, v, grid, s_max, s);

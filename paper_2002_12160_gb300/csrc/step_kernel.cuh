@@ -2,27 +2,41 @@
 // independent hand-plus-object simulations (Sec. III-A; Algorithm 1, "step
 // simulation"), with the contact-sensor readout c_t^(l) of every pad.
 //
-// A group of TPE threads (16, 32, 64 or 128) owns one environment at a time
-// and walks the environments grid-stride; groups wider than a warp
-// synchronise with named barriers. Per substep the group
-//   1. predicts the velocity under gravity and caches the object's spheres,
-//      rotated into the world frame, in shared memory;
-//   2. culls hand links against the object's bounding sphere (one ballot);
-//   3. tests every (surviving link, sphere) pair, TPE pairs per round, and
-//      compacts contacts (gap d < margin) into shared memory in pair order by
-//      ballot (and, across warps, by per-warp counts);
-//   4. moves each contact into the registers of one thread (CPL per thread)
-//      with its lever arm, normal, scalar normal/tangential effective masses
-//      and the bias folded into a target velocity;
-//   5. runs `iters` Jacobi projected-impulse iterations: every contact updates
-//      against the same body velocity, then the group sums impulses and
-//      moments (xor shuffles, then a double-buffered shared-memory exchange
-//      between warps) and recomputes the body velocity;
-//   6. integrates (symplectic Euler, exact rotation exponential) and adds the
-//      contacts' impulses into their sensor pads in a fixed order, each pad
-//      scanning only the contacts of its own link.
-// Nothing here is a dense contraction: the kernel is bound by FP32 issue and
-// by the latency of the solver's reductions.
+// L lanes of one warp (32, or 16 with two environments to a warp) own one
+// environment at a time; nothing but the warp synchronises. Per substep they
+//   1. predict the velocity under gravity, cache the object's spheres, rotated
+//      into the world frame, and the links' offsets in shared memory, and cull
+//      the links against the object's bounding sphere (one ballot);
+//   2. cull (surviving link, 8-sphere cluster) pairs by the clusters' enclosing
+//      spheres; then one lane takes each surviving pair and tests its eight
+//      spheres by squared distance alone (the few within 1e-5 of the margin
+//      again by their gap), and the contacts (gap d < margin) are listed in
+//      pair order (link, then sphere) by bit-plane ballots of the lanes' counts;
+//   3. set each listed contact up: gap, normal and lever arm, its pad, scalar
+//      normal/tangential effective masses, and the bias folded into a target
+//      velocity; the first kSlots L contacts go to registers;
+//   4. run `iters` Jacobi projected-impulse iterations: every contact updates
+//      against the same body velocity, then the impulses and moments are
+//      summed by shuffles and the body velocity recomputed;
+//   5. integrate (symplectic Euler, exact rotation exponential) and add the
+//      contacts' impulses into their sensor pads in a fixed order, one lane per
+//      pad and component scanning the contacts of the pad's link.
+// Nothing here is a dense contraction: the kernel is bound by FP32 issue and by
+// the latency of the solver's chain (and, when the device is full, by instruction
+// fetch: the loops off the solver are kept rolled). Against groups of 64 (or, in
+// large batches, 32) threads with block barriers, a link cull before the cluster
+// cull, one pair test per thread and guarded scalar slots, sim_step alone: 1024
+// cylinders, ten frames, 421 -> 332 us; 32768 mugs, two frames, 4.50 -> 3.59 ms;
+// 4097 boxes, four frames, 392 -> 144 us; 8192 of mixed shapes, six frames,
+// 969 -> 879 us.
+//
+// A step shape's width TPE (16, 32, 64, 128) fixes the order of the solver's
+// sums and with it every bit of the result: thread t of TPE adds contacts t,
+// t + TPE, ... in order, each 32 threads are summed by a xor tree (16, 8, 4, 2,
+// 1), and the 32-thread sums are added in order. The lanes that execute it are a
+// free choice: a lane holds the accumulators of threads lane, lane + L, ...
+// (zeros of empty threads change nothing), and a tree level that pairs two
+// threads of one lane is an addition in that lane.
 #pragma once
 #include <cstddef>
 
@@ -32,142 +46,132 @@
 namespace ih {
 namespace {
 
-constexpr int kBlock = 128;
-// the compiled (group width, register contacts per thread) shapes
+// the shapes of the interface (summation width, contacts per thread); the
+// second number no longer changes anything: the width alone fixes the result
 #define IH_STEP_VARIANTS(X) X(16, 2) X(16, 4) X(32, 1) X(32, 2) X(32, 3) X(32, 4) X(64, 1) X(64, 2) X(128, 1)
+// the compiled kernels: (lanes per environment, summation width)
+#define IH_STEP_KERNELS(X) X(16, 16) X(16, 32) X(16, 64) X(32, 32) X(32, 64) X(32, 128)
 constexpr int kMaxLinks = 32;
-constexpr int kPadsPerLink = 4;
+constexpr int kSlots = 4;            // register-resident contacts per lane
+constexpr int kSphStride = kCluster + 1;   // spheres of a cluster, padded: lanes on different clusters hit different banks
+constexpr unsigned kAll = 0xffffffffu;
 
-template <int TPE>
-struct Group {
-    static constexpr int GPB = kBlock / TPE;               // groups per block
-    static constexpr int W = TPE >= 32 ? TPE / 32 : 1;     // warps per group
-    static constexpr int WIDTH = TPE < 32 ? TPE : 32;      // lanes of the group in one warp
-    int grp, tid, wid, lane;
-    unsigned mask;    // this group's lanes in the warp
-    int shift;        // first lane of this group in the warp
-    __device__ Group() {
-        grp = threadIdx.x / TPE;
-        tid = threadIdx.x % TPE;
-        lane = threadIdx.x & 31;
-        wid = tid / 32;
-        if constexpr (TPE < 32) {
-            shift = (lane / TPE) * TPE;
-            mask = ((1u << TPE) - 1u) << shift;
-        } else {
-            shift = 0;
-            mask = 0xffffffffu;
-        }
-    }
-    __device__ __forceinline__ void sync() const {
-        if constexpr (TPE <= 32) {
-            __syncwarp(mask);
-        } else if constexpr (TPE == kBlock) {
-            __syncthreads();
-        } else {
-            asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(TPE) : "memory");
-        }
-    }
-    // ballot of `p` over the group's lanes in this warp, bit 0 = first lane
-    __device__ __forceinline__ unsigned ballot(bool p) const {
-        const unsigned b = __ballot_sync(mask, p);
-        if constexpr (TPE < 32) return (b >> shift) & ((1u << TPE) - 1u);
-        return b;
-    }
-    __device__ __forceinline__ int lane_in_warp() const { return TPE < 32 ? tid : lane; }
-};
-
-// Shared memory of one group. Everything has a fixed size except the contact
-// staging, the cache of world-frame sphere and cluster centres and the list of
-// surviving (link, cluster) pairs, which follow the group records.
-
-template <int W>
-struct alignas(16) GSm {   // 16-byte aligned: red is read as float4
+// Shared memory of one environment. Everything has a fixed size except the
+// contact records, the caches of world-frame centres and the lists, which follow.
+struct alignas(16) GSm {
     double term[IH_MAX_PADS];        // FP64 force term of each pad (scoring)
+    float4 xa[kMaxLinks];            // x - link origin
+    float4 ax[kMaxLinks];            // link axis
     float padacc[IH_MAX_PADS * 3];
-    float red[2][W][8];              // cross-warp partial sums
-    int cnt[2][2 * W];               // cross-warp hit counts
     int flag[IH_MAX_PADS];           // contact-state mismatch of each pad (scoring)
-    double best_c;                   // best (C, env) of this group so far
-    int best_i;
-    int next;                        // work-queue slot handed to the group (groups wider than a warp)
-    unsigned long long work[6];      // this group's work counters (see sim_work_counters)
-    unsigned surv;                   // surviving-link mask
-    int n_clp;
-    int n_prev;                      // warm start: contacts of the last substep (cache entries)
-    unsigned char links[32];         // surviving links in order
-    unsigned short lbeg[32], lend[32];   // contact range of each link
+    unsigned short lbeg[kMaxLinks], lend[kMaxLinks];   // contact range of each link
+};
+static_assert(sizeof(GSm) % 16 == 0, "the records keep 16-byte alignment");
+// The warp's pad table: per link its pads in order and their intervals [s0, s1)
+// (absent: an interval that holds nothing; the palm: its first pad holds all).
+constexpr int kPadsPerLink = 4;
+struct alignas(16) PadSm {
+    float s0[kMaxLinks][kPadsPerLink], s1[kMaxLinks][kPadsPerLink];
+    unsigned char id[kMaxLinks][kPadsPerLink];
 };
 
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
-__host__ __device__ constexpr size_t block_smem_bytes() {
-    return align16(kMaxLinks) + align16(kMaxLinks * kPadsPerLink) + 2 * align16(4 * IH_MAX_PADS);
+__host__ __device__ constexpr int sph_cap(int s_max) { return (s_max + kCluster - 1) / kCluster * kSphStride; }
+// contacts whose record (3 float4) and impulse (1) are in shared memory: the
+// register-resident ones; the rest of up to c_max spill to global memory
+__host__ __device__ constexpr int stage_capacity(int lanes, int c_max) {
+    return c_max < kSlots * lanes ? c_max : kSlots * lanes;
 }
-template <int W>
-__host__ __device__ constexpr size_t gsm_bytes() { return align16(sizeof(GSm<W>)); }
-static_assert(sizeof(GSm<1>) % 16 == 0 && sizeof(GSm<2>) % 16 == 0 && sizeof(GSm<4>) % 16 == 0,
-              "group records must keep 16-byte alignment");
-static_assert(offsetof(GSm<2>, red) % 16 == 0, "red is read as float4");
-// dynamic part of a group: the contact staging (4 float4 per contact, the
-// first stage_cap contacts; the rest of up to c_max spill to global memory),
-// the cache of sphere and cluster centres, for a warm-started solver the cache
-// of the last substep's contacts, and the surviving (link, cluster) pairs
-__host__ __device__ inline size_t group_dyn_floats4(int s_max, int stage_cap, int c_max, bool warm, int clp_cap) {
-    return 4 * (size_t)stage_cap + s_max + 32 + (warm ? (size_t)c_max : 0) + ((size_t)clp_cap * 2 + 15) / 16;
+// float4s of the sphere cache and the impulses, which share their place (the
+// spheres are done with when the first impulse is stored) unless the solver
+// starts from cached impulses
+__host__ __device__ constexpr int sph_lam_cap(int s_max, int stage_cap, bool warm) {
+    return warm ? sph_cap(s_max) + stage_cap : sph_cap(s_max) > stage_cap ? sph_cap(s_max) : stage_cap;
 }
-// contacts a group stages in shared memory: at least its register-resident
-// ones, and 64 (32 for the narrow shapes, eight or more groups to a block,
-// whose staging would otherwise cap the blocks an SM holds), at most c_max
-__host__ __device__ constexpr int stage_capacity(int rcap, int c_max, int groups_per_block) {
-    return c_max < (rcap > (groups_per_block >= 8 ? 32 : 64) ? rcap : (groups_per_block >= 8 ? 32 : 64))
-               ? c_max
-               : (rcap > (groups_per_block >= 8 ? 32 : 64) ? rcap : (groups_per_block >= 8 ? 32 : 64));
+__host__ __device__ inline size_t env_bytes(int s_max, int stage_cap, int c_max, bool warm, int clp_cap) {
+    return sizeof(GSm) +
+           sizeof(float4) * (3 * (size_t)stage_cap + sph_lam_cap(s_max, stage_cap, warm) + kMaxLinks + (warm ? c_max : 0)) +
+           align16(2 * (size_t)clp_cap) + align16(2 * (size_t)c_max) + align16((size_t)c_max);
 }
 
-template <int TPE>
-__device__ __forceinline__ void group_sum6(float (&v)[6], const Group<TPE> &G, float *red, int parity) {
-    constexpr int WIDTH = Group<TPE>::WIDTH;
-    if constexpr (TPE <= 32) {
-        width_sum6<WIDTH>(v, G.mask, G.lane_in_warp() & (WIDTH - 1));
-    } else {
-        // each warp's sums go straight from the lanes that hold them to shared
-        // memory; every thread then adds the W warps' partials in warp order
-        constexpr int W = Group<TPE>::W;
-        const float c = width_scatter6<32>(v, G.mask, G.lane);
-        float *r = red + parity * W * 8;
-        const int k = G.lane >> 2;
-        if ((G.lane & 3) == 0 && k < 6) r[G.wid * 8 + k] = c;
-        G.sync();
-        const float4 *r4 = reinterpret_cast<const float4 *>(r);
-        float4 lo = r4[0], hi = r4[1];
+// The sum over an environment's L lanes of six values A (one 32-thread tree of the
+// width, its first level already added when L = 16) or of A and B (two trees,
+// added in order), every lane receiving the six totals. Reduce-scatter: a level
+// sends the half of the values that the lane does not keep, so 13 shuffles (two
+// trees, L = 32) reduce twelve values.
+template <int L>
+__device__ __forceinline__ void sum_trees(const float (&A)[6], const float (&B)[6], float (&v)[6], int gl) {
+    // the first level leaves A to one half of the lanes and B to the other
+    constexpr int H = L / 2;
+    const bool b1 = gl & H, b2 = gl & (H / 2), b3 = gl & (H / 4), b4 = gl & (H / 8);
+    float s[6];
 #pragma unroll
-        for (int w = 1; w < W; ++w) {
-            const float4 l2 = r4[2 * w], h2 = r4[2 * w + 1];
-            lo.x += l2.x; lo.y += l2.y; lo.z += l2.z; lo.w += l2.w;
-            hi.x += h2.x; hi.y += h2.y;
+    for (int k = 0; k < 6; ++k) s[k] = (b1 ? B[k] : A[k]) + __shfl_xor_sync(kAll, b1 ? A[k] : B[k], H, L);
+    float t[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) t[k] = (b2 ? s[k + 3] : s[k]) + __shfl_xor_sync(kAll, b2 ? s[k] : s[k + 3], H / 2, L);
+    const float u0 = (b3 ? t[2] : t[0]) + __shfl_xor_sync(kAll, b3 ? t[0] : t[2], H / 4, L);
+    const float u1 = (b3 ? 0.0f : t[1]) + __shfl_xor_sync(kAll, b3 ? t[1] : 0.0f, H / 4, L);
+    float c = (b4 ? u1 : u0) + __shfl_xor_sync(kAll, b4 ? u0 : u1, H / 8, L);
+    if constexpr (L == 32) c += __shfl_xor_sync(kAll, c, 1, L);
+    c += __shfl_xor_sync(kAll, c, H, L);   // A + B
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] = __shfl_sync(kAll, c, (k / 3) * (H / 2) + (k % 3 == 2 ? H / 4 : (k % 3) * (H / 8)), L);
+}
+
+// The sums of NA accumulators of six values (accumulator j of lane g: thread
+// g + j L of the summation width L NA), of which the first NZ can be nonzero, in
+// the width's order (see above; a tree of zeros is left out).
+template <int L, int NA, int NZ>
+__device__ __forceinline__ void env_sum6(const float (&acc)[NA][6], float (&v)[6], int gl) {
+    if constexpr (L * NA <= 64) {
+        float A[6], B[6];
+        constexpr bool two = L * NA == 64 && (L == 32 ? NZ > 1 : NZ > 2);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            A[k] = (L == 16 && NA > 1 && NZ > 1) ? acc[0][k] + acc[NA > 1 ? 1 : 0][k] : acc[0][k];
+            if constexpr (two) B[k] = L == 16 ? (NZ > 3 ? acc[NA - 2][k] + acc[NA - 1][k] : acc[NA - 2][k]) : acc[NA - 1][k];
         }
-        v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w; v[4] = hi.x; v[5] = hi.y;
+        if constexpr (two) {
+            sum_trees<L>(A, B, v, gl);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) v[k] = A[k];
+            width_sum6<L>(v, kAll, gl);
+        }
+    } else {   // 128: four sums, added in order
+        float c = width_scatter6<32>(acc[0], kAll, gl);
+#pragma unroll
+        for (int j = 1; j < NZ; ++j) c += width_scatter6<32>(acc[j], kAll, gl);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[k] = __shfl_sync(kAll, c, scatter_lane<32>(k), 32);
     }
 }
 
-// Resident blocks per SM each shape is compiled for (caps its registers):
-// one or two register-resident contacts per thread at 4 blocks (128
-// registers: with one contact a cap of 5 blocks spilled and ran 6 % slower on
-// large batches), four at 3.
-#ifndef IH_STEP_MIN_BLOCKS_CPL2
-#define IH_STEP_MIN_BLOCKS_CPL2 4
-#endif
-template <int TPE, int CPL>
-struct MinBlocks {
-    static constexpr int value = CPL <= 2 ? IH_STEP_MIN_BLOCKS_CPL2 : (CPL <= 4 ? 3 : 2);
-};
+// Whether a sphere's gap to link l is below the margin, in the contact setup's own
+// arithmetic (the rare pairs that the squared distance leaves open; out of line)
+__device__ __noinline__ bool gap_below_margin(const DevScene &sc, float margin, int l, V3 ca, float rs, V3 ld) {
+    const Hit h = l == 0 ? hit_box_local(ca, rs, sc.palm_hx, sc.palm_hy, sc.palm_hz)
+                         : hit_capsule(ca, rs, ld, sc.link_len, 1.0f / sc.link_len, sc.link_rad, {1.0f, 0.0f, 0.0f, 0.0f});
+    return h.gap < margin;   // (the gap does not depend on the link's rotation)
+}
 
-template <int TPE, int CPL, bool WARM>
-__global__ void __launch_bounds__(kBlock, MinBlocks<TPE, CPL>::value) step_kernel(const StepArgs a, int s_max) {
-    using Grp = Group<TPE>;
-    constexpr int GPB = Grp::GPB, W = Grp::W, RCAP = TPE * CPL;   // register-resident contacts
+// order-preserving key of a cost (NaN excluded), compared with integers: FP64
+// compares take the scarce FP64 pipe
+__device__ __forceinline__ unsigned long long cost_key(double c) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(c);
+    return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+}
+
+// One warp per block, so that the environments spread evenly over the SMs (an
+// SM holds 6 or 7 of 1024 environments; blocks of two would put 8 on some), and
+// 16 warps to an SM by registers.
+template <int L, int TPE, bool WARM>
+__global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_max) {
+    static_assert(TPE % L == 0 && TPE / L <= kSlots, "the width's threads are the lanes' accumulators");
+    constexpr int EPW = 32 / L, NA = TPE / L, RCAP = kSlots * L;
     extern __shared__ __align__(16) unsigned char smem[];
-    const Grp G;
+    const int lane = threadIdx.x, sub = lane / L, gl = lane % L, shift = sub * L;
     const DevScene &sc = a.sc;
     const DevConfig &cfg = a.cfg;
     const int ns = cfg.substeps, Lk = sc.n_links, P = sc.n_pads;
@@ -183,67 +187,69 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<TPE, CPL>::value) step_kerne
     const bool window_mode = a.cm_frames != nullptr;   // every frame scored, argmin afterwards
     const bool scored = obs != nullptr;
     const int n_win0 = scored ? *a.n_window : 0;       // frames in the window before this launch
-    const int n_win = n_win0 + 1;
 
-    // block-wide tables: the pads of each link (in pad order) and their intervals
-    unsigned char *pl_cnt = smem;
-    unsigned char *pl_id = smem + align16(kMaxLinks);
-    float *p_s0 = reinterpret_cast<float *>(smem + align16(kMaxLinks) + align16(kMaxLinks * kPadsPerLink));
-    float *p_s1 = p_s0 + IH_MAX_PADS;
-    GSm<W> &S = *reinterpret_cast<GSm<W> *>(smem + block_smem_bytes() + G.grp * gsm_bytes<W>());
     const int cap = cfg.c_max;
-    const int SC = a.stage_cap;   // contacts staged in shared memory; the rest spill to global memory
-    // contact staging: [0] (r, gap -> 1/k_t), [1] (n, link | pad << 8), [2] (c, 1/k_n), [3] (lambda)
-    float4 (*stage)[4] = reinterpret_cast<float4 (*)[4]>(
-        reinterpret_cast<float4 *>(smem + block_smem_bytes() + GPB * gsm_bytes<W>()) +
-        G.grp * group_dyn_floats4(s_max, SC, cap, WARM, a.clp_cap));
-    float4 *sph = &stage[SC][0];
-    float4 *clc = sph + s_max;   // cluster centres follow the spheres
+    const int SC = a.stage_cap;   // contacts staged in shared memory (RCAP, or c_max); the rest spill to global memory
+    PadSm &PT = *reinterpret_cast<PadSm *>(smem);
+#pragma unroll 1
+    for (int l = lane; l < Lk; l += 32) {
+        int c = 0;
+#pragma unroll 1
+        for (int p = 0; p < P && c < (l == 0 ? 1 : kPadsPerLink); ++p) {
+            if (__ldg(sc.pad_link + p) != l) continue;
+            const float s1 = __ldg(sc.pad_s1 + p);
+            PT.s0[l][c] = l == 0 ? -1.0f : __ldg(sc.pad_s0 + p);
+            PT.s1[l][c] = (l == 0 || s1 >= 1.0f) ? 2.0f : s1;   // (t <= 1)
+            PT.id[l][c++] = (unsigned char)p;
+        }
+#pragma unroll 1
+        for (; c < kPadsPerLink; ++c) {
+            PT.s0[l][c] = 3.0f;
+            PT.s1[l][c] = 3.0f;
+            PT.id[l][c] = 0xff;
+        }
+    }
+    __syncwarp();
+    unsigned char *mine = smem + sizeof(PadSm) + sub * env_bytes(s_max, SC, cap, WARM, a.clp_cap);
+    GSm &S = *reinterpret_cast<GSm *>(mine);
+    // contact records, 3 float4 each: (r, 1/k_t), (n, 1/k_n), (c, -); the impulses follow
+    float4 *rec = reinterpret_cast<float4 *>(mine + sizeof(GSm));
+    float4 *sph = rec + 3 * SC;            // sphere centres (world rotation, relative to x), radius
+    float4 *lamst = WARM ? sph + sph_cap(s_max) : sph;
+    float4 *clc = sph + sph_lam_cap(s_max, SC, WARM);    // cluster centres, enclosing radius
     // warm start: final impulse (xyz) and pair id (w, link << 8 | sphere) of the
     // environment's last substep's contacts, in pair order
-    float4 *prev = clc + 32;
-    // surviving (link index << 8 | cluster) pairs in order
+    float4 *prev = clc + kMaxLinks;
+    // surviving pairs in order (link << 8 | cluster); contacts in order (link << 8 | sphere); their pads
     unsigned short *clp = reinterpret_cast<unsigned short *>(prev + (WARM ? cap : 0));
-    // contacts SC .. c_max - 1 of the group's environment: its slot of the spill area
-    float4 *spill_g = a.spill ? a.spill + (size_t)(blockIdx.x * GPB + G.grp) * (size_t)(cap - SC) * 4 : nullptr;
-    auto cslot = [&](int ci) -> float4 * { return ci < SC ? stage[ci] : spill_g + (size_t)(ci - SC) * 4; };
-    constexpr bool warm = WARM;
-    if (threadIdx.x < kMaxLinks) {
-        int c = 0;
-        for (int p = 0; p < P && c < kPadsPerLink; ++p)
-            if (__ldg(sc.pad_link + p) == (int)threadIdx.x) pl_id[threadIdx.x * kPadsPerLink + c++] = (unsigned char)p;
-        pl_cnt[threadIdx.x] = (unsigned char)c;
-    }
-    for (int p = threadIdx.x; p < P; p += kBlock) {
-        p_s0[p] = __ldg(sc.pad_s0 + p);
-        p_s1[p] = __ldg(sc.pad_s1 + p);
-    }
-    __syncthreads();
-
-    int parity = 0;
-    if (G.tid == 0) {
-        S.best_c = INFINITY;
-        S.best_i = 0x7fffffff;
-        for (int k = 0; k < 6; ++k) S.work[k] = 0ull;
-    }
-
-    // the next work slot of the group: from the launch's work queue (slots in
-    // LPT order, taken one environment at a time by whichever group is free),
-    // else grid-stride
-    auto fetch = [&](int last) -> int {
-        if (!a.queue) return last < 0 ? (int)blockIdx.x * GPB + G.grp : last + (int)gridDim.x * GPB;
-        int v = 0;
-        if constexpr (TPE <= 32) {
-            if (G.tid == 0) v = atomicAdd(a.queue, 1);
-            v = __shfl_sync(G.mask, v, G.shift);
-        } else {
-            if (G.tid == 0) S.next = atomicAdd(a.queue, 1);
-            G.sync();   // S.next is written again only after the body's closing barrier
-            v = S.next;
-        }
-        return v;
+    unsigned short *clist = reinterpret_cast<unsigned short *>(reinterpret_cast<unsigned char *>(clp) + align16(2 * (size_t)a.clp_cap));
+    unsigned char *cpad = reinterpret_cast<unsigned char *>(clist) + align16(2 * (size_t)cap);
+    // contacts SC .. c_max - 1 of the environment: its slot of the spill area
+    float4 *spill_g = a.spill ? a.spill + (size_t)(blockIdx.x * EPW + sub) * (size_t)(cap - SC) * 4 : nullptr;   // (SC = RCAP when there is one)
+    auto ballot = [&](bool p) -> unsigned {   // of the environment's lanes, bit 0 its first
+        const unsigned b = __ballot_sync(kAll, p);
+        return L == 32 ? b : (b >> shift) & 0xffffu;
     };
-    for (int slot = fetch(-1); slot < a.N; slot = fetch(slot)) {
+    auto wmax = [&](int v) -> int { return L == 32 ? v : max(v, __shfl_xor_sync(kAll, v, 16)); };
+    const unsigned below = (1u << gl) - 1u;
+
+    unsigned long long best_k = ~0ull;   // best (C, env) of these lanes so far (single scored frame)
+    int best_i = 0x7fffffff;
+    unsigned long long work = 0ull;      // lane k < 6: work counter k (see sim_work_counters)
+
+    // The next environments of the warp: from the launch's work queue (slots in
+    // LPT order, taken by whichever warp is free), else grid-stride. Both
+    // environments of a 16-lane warp walk the same loops to the larger of their
+    // counts, so that the warp stays converged; neighbours in LPT order are alike.
+    auto fetch = [&](int last) -> int {
+        if (!a.queue) return last < 0 ? (int)blockIdx.x * EPW : last + (int)gridDim.x * EPW;
+        int v = 0;
+        if (lane == 0) v = atomicAdd(a.queue, EPW);
+        return __shfl_sync(kAll, v, 0);
+    };
+    for (int base = fetch(-1); base < a.N; base = fetch(base)) {
+        const bool live = base + sub < a.N;
+        const int slot = live ? base + sub : base;
         const int env = a.order ? __ldg(a.order + slot) : slot;
         int st = a.status[env];
         const float4 P0 = a.pose[2 * env], P1 = a.pose[2 * env + 1];
@@ -251,29 +257,31 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<TPE, CPL>::value) step_kerne
         const float2 th = a.params[env];
         const int shp = a.shape[env];
         const int iters = a.iters[env];
+        const int iters_w = wmax(iters);
         V3 x = xyz(P0);
         Q4 q = {P1.x, P1.y, P1.z, P1.w};
         V3 v = xyz(V0), w = xyz(V1);
         const float m = th.x, mu = th.y, inv_m = 1.0f / m;
         const int sfirst = __ldg(sc.shape_first + shp), NS = __ldg(sc.shape_count + shp);
-        const float bound = __ldg(sc.shape_bound + shp);
         const int ncl = (NS + kCluster - 1) / kCluster;
         const float inv_ncl = 1.0f / (float)ncl;
         const int cfirst = __ldg(sc.cl_first + shp);
-        if (warm) {   // the environment's impulse cache from its previous launch
-            const int np = a.cache_n[env];
-            if (G.tid == 0) S.n_prev = np;
-            for (int k = G.tid; k < np; k += TPE) prev[k] = a.cache[(size_t)env * cap + k];
+        int n_prev = 0;
+        if (WARM) {   // the environment's impulse cache from its previous launch
+            n_prev = a.cache_n[env];
+#pragma unroll 1
+            for (int k = gl; k < n_prev; k += L) prev[k] = a.cache[(size_t)env * cap + k];
         }
-        double c_sum_env = (window_mode && G.tid == 0) ? a.c_sum[env] : 0.0;
+        double c_sum_env = (scored && gl == 0) ? a.c_sum[env] : 0.0;
         // cost of the frame just stepped against observation ob (Sec. III-C),
-        // FP64 without contraction, pads in order; valid in the group's thread 0
+        // FP64 without contraction, pads in order; valid in the environment's first lane
         auto frame_cost = [&](const float *ob, int stt) -> double {
             const float inv_ns_f = 1.0f / (float)ns;
-            G.sync();
+            __syncwarp();
             const double tau = (double)cfg.tau, wf = (double)cfg.w_force;
             const double tau2 = __dmul_rn(tau, tau);
-            for (int p = G.tid; p < P; p += TPE) {
+#pragma unroll 1
+            for (int p = gl; p < P; p += L) {
                 const double fx = S.padacc[3 * p] * inv_ns_f, fy = S.padacc[3 * p + 1] * inv_ns_f,
                              fz = S.padacc[3 * p + 2] * inv_ns_f;
                 const double ox = ob[3 * p], oy = ob[3 * p + 1], oz = ob[3 * p + 2];
@@ -284,27 +292,32 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<TPE, CPL>::value) step_kerne
                 const double no2 = __dadd_rn(__dadd_rn(__dmul_rn(ox, ox), __dmul_rn(oy, oy)), __dmul_rn(oz, oz));
                 S.flag[p] = (ns2 > tau2) != (no2 > tau2);
             }
-            G.sync();
+            __syncwarp();
             double c = 0.0;
-            if (G.tid == 0) {
+            if (gl == 0) {
                 if (stt & kDiverged) {
                     c = INFINITY;
                 } else {
+#pragma unroll 1
                     for (int p = 0; p < P; ++p) {
                         c = __dadd_rn(c, S.term[p]);
                         if (S.flag[p]) c = __dadd_rn(c, (double)cfg.w_contact);
                     }
                 }
             }
-            G.sync();   // S.term / S.flag are reused by the next frame
+            __syncwarp();   // S.term / S.flag are reused by the next frame
             return c;
         };
 
+#pragma unroll 1
         for (int fr = 0; fr < a.n_frames; ++fr) {
-            for (int k = G.tid; k < 3 * P; k += TPE) S.padacc[k] = 0.0f;
+#pragma unroll 1
+            for (int k = gl; k < 3 * P; k += L) S.padacc[k] = 0.0f;
             const float4 *tab = a.link_tab + (size_t)(frame0 + fr) * (ns + 1) * Lk * kLinkStride;
-            const bool skip = (st & kDiverged) != 0;   // decided once per frame
-            for (int s = 0; s < ns && !skip; ++s) {
+            const bool act = live && (st & kDiverged) == 0;   // decided once per frame
+            const int ns_w = __any_sync(kAll, act) ? ns : 0;
+#pragma unroll 1
+            for (int s = 0; s < ns_w; ++s) {
                 const float4 *L0 = tab + (size_t)s * Lk * kLinkStride;
                 const float4 *L1 = L0 + Lk * kLinkStride;
                 const V3 v_pred = v + grav;
@@ -317,502 +330,534 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<TPE, CPL>::value) step_kerne
                 const S6 Wi = world_inv_inertia(R, Jb, inv_m);
 
                 // -- 1. spheres and cluster centres to world (relative to x), cached
-                for (int j = G.tid; j < NS; j += TPE) {
-                    const float4 sp = __ldg(sc.spheres + sfirst + j);
-                    const V3 cr = mmul(R, xyz(sp));
-                    sph[j] = make_float4(cr.x, cr.y, cr.z, sp.w);
+                //       (padding of the last cluster: far away); the links' offsets
+#pragma unroll 1
+                for (int j = gl; j < ncl * kCluster; j += L) {
+                    float4 o = make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+                    if (j < NS) {
+                        const float4 sp = __ldg(sc.spheres + sfirst + j);
+                        const V3 cr = mmul(R, xyz(sp));
+                        o = make_float4(cr.x, cr.y, cr.z, sp.w);
+                    }
+                    sph[(j >> 3) * kSphStride + (j & 7)] = o;
                 }
-                for (int k = G.tid; k < ncl; k += TPE) {
+#pragma unroll 1
+                for (int k = gl; k < ncl; k += L) {
                     const float4 cl = __ldg(sc.clusters + cfirst + k);
                     const V3 cr = mmul(R, xyz(cl));
                     clc[k] = make_float4(cr.x, cr.y, cr.z, cl.w);
                 }
-                // -- 2. cull links whose bounding volume the object cannot reach
-                if constexpr (TPE >= 32) {
-                    if (G.wid == 0) {
-                        const bool keep = G.lane < Lk && link_reaches(sc, cfg, L0, G.lane, x, bound);
-                        const unsigned ml = __ballot_sync(0xffffffffu, keep);
-                        if (G.lane == 0) S.surv = ml;
-                    }
-                } else {
-                    unsigned ml = 0;
-                    for (int base = 0; base < Lk; base += TPE) {
-                        const int l = base + G.tid;
-                        const bool keep = l < Lk && link_reaches(sc, cfg, L0, l, x, bound);
-                        ml |= G.ballot(keep) << base;
-                    }
-                    if (G.tid == 0) S.surv = ml;
-                }
-                G.sync();
-                const unsigned surv = S.surv;
-                const int nsurv = __popc(surv);
-                for (int l = G.tid; l < kMaxLinks; l += TPE) {
-                    if (l < Lk && ((surv >> l) & 1u)) S.links[__popc(surv & ((1u << l) - 1u))] = (unsigned char)l;
+#pragma unroll 1
+                for (int l = gl; l < Lk; l += L) {
+                    const V3 xa = x - xyz(__ldg(L0 + l * kLinkStride));
+                    const float4 ld = __ldg(L0 + l * kLinkStride + 1);
+                    S.xa[l] = make_float4(xa.x, xa.y, xa.z, 0.0f);
+                    S.ax[l] = ld;
                     S.lbeg[l] = 0;
                     S.lend[l] = 0;
                 }
-                G.sync();
+                __syncwarp();
 
-                // -- 3a. cull (surviving link, cluster) pairs by the clusters' enclosing spheres
+                // -- 2a. cull (link, cluster) pairs by the clusters' enclosing spheres (the
+                //        reach a little wider: the pair tests decide). The palm's pose is
+                //        the identity (fk_kernel), so its box frame is the world frame
+                auto palm_offset = [&](V3 c) -> V3 {   // from the palm box to a point
+                    return c - mk(fminf(fmaxf(c.x, -sc.palm_hx), sc.palm_hx), fminf(fmaxf(c.y, -sc.palm_hy), sc.palm_hy),
+                                  fminf(fmaxf(c.z, -sc.palm_hz), sc.palm_hz));
+                };
                 int nclp = 0;
-                const int ncpairs = nsurv * ncl;
-                for (int p0 = 0; p0 < ncpairs; p0 += TPE) {
-                    const int p = p0 + G.tid;
+                const int ncpairs = act ? Lk * ncl : 0, ncp_w = wmax(ncpairs);
+#pragma unroll 2
+                for (int p0 = 0; p0 < ncp_w; p0 += L) {
+                    const int p = p0 + gl;
                     bool keep = false;
-                    int li = 0, k = 0;
+                    int e = 0;
                     if (p < ncpairs) {
-                        li = min(max((int)(((float)p + 0.5f) * inv_ncl), 0), nsurv - 1);
-                        k = p - li * ncl;
+                        const int l = min((int)(((float)p + 0.5f) * inv_ncl), Lk - 1), k = p - l * ncl;
                         const float4 cc = clc[k];
-                        keep = link_reaches(sc, cfg, L0, S.links[li], x + xyz(cc), cc.w);
+                        const V3 ca = xyz(S.xa[l]) + xyz(cc), ld = xyz(S.ax[l]);
+                        const V3 dc = ca - ld * fminf(fmaxf(dot(ca, ld), 0.0f), sc.link_len), dp = palm_offset(ca);
+                        const V3 dd = l == 0 ? dp : dc;
+                        const float reach = (cc.w + cfg.margin + (l == 0 ? 0.0f : sc.link_rad)) * 1.00001f;
+                        keep = dot(dd, dd) < reach * reach;
+                        e = (l << 8) | k;
                     }
-                    const unsigned bal = G.ballot(keep);
-                    int off = nclp, tot;
-                    if constexpr (TPE > 32) {
-                        int *cb = S.cnt[parity];
-                        if (G.lane == 0) cb[G.wid] = __popc(bal);
-                        G.sync();
-                        tot = 0;
-#pragma unroll
-                        for (int q2 = 0; q2 < W; ++q2) {
-                            const int c = cb[q2];
-                            if (q2 < G.wid) off += c;
-                            tot += c;
-                        }
-                        parity ^= 1;
-                    } else {
-                        tot = __popc(bal);
-                    }
-                    if (keep) clp[off + __popc(bal & ((1u << G.lane_in_warp()) - 1u))] = (unsigned short)((li << 8) | k);
-                    nclp += tot;
+                    const unsigned bal = ballot(keep);
+                    if (keep) clp[nclp + __popc(bal & below)] = (unsigned short)e;
+                    nclp += __popc(bal);
                 }
-                G.sync();
+                __syncwarp();
 
-                // -- 3b. narrowphase over the spheres of the surviving pairs, in pair order;
-                //        each thread tests two pairs per round (two independent chains)
+                // -- 2b. a lane tests the eight spheres of a surviving pair. A sphere is a
+                //        contact when its gap is below the margin, which its squared
+                //        distance from the link's axis (or box) decides unless it is
+                //        within 1e-5 of the reach squared (the gap's rounding is two
+                //        orders below that): those are tested again by their gap
                 int nc = 0;
-                const int npairs = nclp * kCluster;
-                auto test_pair = [&](int p, Hit &hh, V3 &r, int &l, int &j) -> bool {
-                    if (p >= npairs) return false;
-                    const int e = clp[p / kCluster];
-                    j = (e & 0xff) * kCluster + (p % kCluster);
-                    l = S.links[e >> 8];
-                    if (j >= NS) return false;
-                    const float4 sp = sph[j];
-                    const V3 cr = xyz(sp);
-                    const float4 A0 = __ldg(L0 + l * kLinkStride);
-                    const float4 Aq = __ldg(L0 + l * kLinkStride + 2);
-                    const Q4 lq = {Aq.x, Aq.y, Aq.z, Aq.w};
-                    if (l == 0) {
-                        hh = hit_box(x + cr, sp.w, xyz(A0), lq, sc.palm_hx, sc.palm_hy, sc.palm_hz);
-                    } else {
-                        const V3 ld = xyz(__ldg(L0 + l * kLinkStride + 1));
-                        hh = hit_capsule((x - xyz(A0)) + cr, sp.w, ld, sc.link_len, inv_L, sc.link_rad, lq);
-                    }
-                    r = cr - hh.n * sp.w;
-                    return hh.gap < cfg.margin;
-                };
-                auto emit = [&](int idx, const Hit &hh, V3 r, int l, int j) {
-                    if (idx >= cap) return;
-                    int pad = -1;
-                    const int npl = pl_cnt[l];
-                    for (int k = 0; k < npl; ++k) {
-                        const int pp = pl_id[l * kPadsPerLink + k];
-                        if (l == 0) { pad = pp; break; }
-                        const float s0 = p_s0[pp], s1 = p_s1[pp];
-                        if (hh.t >= s0 && (hh.t < s1 || s1 >= 1.0f)) { pad = pp; break; }
-                    }
-                    float4 *c4 = cslot(idx);
-                    c4[0] = make_float4(r.x, r.y, r.z, hh.gap);
-                    c4[1] = make_float4(hh.n.x, hh.n.y, hh.n.z, __int_as_float(l | ((pad & 0xff) << 8) | (j << 16)));
-                };
-                for (int p0 = 0; p0 < npairs; p0 += 2 * TPE) {
-                    Hit ha = {0.0f, mk(0, 0, 1), 0.0f}, hb = {0.0f, mk(0, 0, 1), 0.0f};
-                    V3 ra = mk(0, 0, 0), rb = mk(0, 0, 0);
-                    int la = 0, lb = 0, ja = 0, jb = 0;
-                    const bool hit_a = test_pair(p0 + G.tid, ha, ra, la, ja);
-                    const bool hit_b = test_pair(p0 + TPE + G.tid, hb, rb, lb, jb);
-                    const unsigned bal_a = G.ballot(hit_a), bal_b = G.ballot(hit_b);
-                    const unsigned below = (1u << G.lane_in_warp()) - 1u;
-                    int off_a = nc, off_b, tot;
-                    if constexpr (TPE > 32) {
-                        int *cb = &S.cnt[parity][0];   // per warp: hits of the first and second halves
-                        if (G.lane == 0) { cb[2 * G.wid] = __popc(bal_a); cb[2 * G.wid + 1] = __popc(bal_b); }
-                        G.sync();
-                        int tot_a = 0, pre_b = 0, tot_b = 0;
+                const int nclp_w = wmax(nclp);
+#pragma unroll 1
+                for (int e0 = 0; e0 < nclp_w; e0 += L) {
+                    unsigned hits = 0, close = 0;
+                    int e = 0;
+                    if (e0 + gl < nclp) {
+                        e = clp[e0 + gl];
+                        const int l = e >> 8;
+                        const V3 xa = xyz(S.xa[l]);
+                        const float4 *sk = sph + (e & 0xff) * kSphStride;
+                        auto mark = [&](V3 dd, float reach, int i) {
+                            const float d2 = dot(dd, dd), r2 = reach * reach, over = d2 - r2;
+                            if (over < 0.0f) hits |= 1u << i;
+                            if (!(fabsf(over) > 1e-5f * r2)) close |= 1u << i;
+                        };
+                        if (l == 0) {
 #pragma unroll
-                        for (int q2 = 0; q2 < W; ++q2) {
-                            const int ca = cb[2 * q2], cbb = cb[2 * q2 + 1];
-                            if (q2 < G.wid) { off_a += ca; pre_b += cbb; }
-                            tot_a += ca;
-                            tot_b += cbb;
+                            for (int i = 0; i < kCluster; ++i) {
+                                const float4 c4 = sk[i];
+                                mark(palm_offset(xa + xyz(c4)), c4.w + cfg.margin, i);
+                            }
+                        } else {
+                            const V3 ld = xyz(S.ax[l]);
+                            const float rm = sc.link_rad + cfg.margin;
+#pragma unroll
+                            for (int i = 0; i < kCluster; ++i) {
+                                const float4 c4 = sk[i];
+                                const V3 ca = xa + xyz(c4);
+                                const float t = fminf(fmaxf(dot(ca, ld) * inv_L, 0.0f), 1.0f);
+                                mark(ca - ld * (t * sc.link_len), c4.w + rm, i);
+                            }
                         }
-                        off_b = nc + tot_a + pre_b;
-                        tot = tot_a + tot_b;
-                        parity ^= 1;
-                    } else {
-                        off_b = nc + __popc(bal_a);
-                        tot = __popc(bal_a) + __popc(bal_b);
+#pragma unroll 1
+                        for (; close; close &= close - 1u) {   // rare
+                            const int i = __ffs(close) - 1;
+                            const float4 c4 = sk[i];
+                            const bool hit = (e & 0xff) * kCluster + i < NS &&
+                                             gap_below_margin(sc, cfg.margin, l, xa + xyz(c4), c4.w, xyz(S.ax[l]));
+                            hits = (hits & ~(1u << i)) | (hit ? 1u << i : 0u);
+                        }
                     }
-                    if (hit_a) emit(off_a + __popc(bal_a & below), ha, ra, la, ja);
-                    if (hit_b) emit(off_b + __popc(bal_b & below), hb, rb, lb, jb);
-                    nc += tot;
+                    // the lanes' counts (0..8) by bit planes: hits of the lanes before, and in all
+                    const int cnt = __popc(hits);
+                    int idx = nc;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        const unsigned bal = ballot((cnt >> b) & 1);
+                        idx += __popc(bal & below) << b;
+                        nc += __popc(bal) << b;
+                    }
+                    const int cj = (e & 0xff00) | ((e & 0xff) * kCluster);
+#pragma unroll
+                    for (int i = 0; i < kCluster; ++i) {
+                        const int at = idx + __popc(hits & ((1u << i) - 1u));
+                        if (((hits >> i) & 1u) && at < cap) clist[at] = (unsigned short)(cj + i);
+                    }
                 }
-                G.sync();
+                __syncwarp();
                 if (nc > cfg.c_max) {   // more contacts than the per-env capacity
                     st |= IH_ENV_OVERFLOW;
                     nc = 0;
                 }
-                if (G.tid == 0) {
-                    S.work[0] += (unsigned long long)nclp * kCluster;
-                    S.work[1] += nc;
-                    S.work[2] += nc > 0 ? (unsigned long long)nc * iters : 0ull;
-                    S.work[3] += 1;
-                    S.work[4] += nc > 0 ? iters : 0;
-                    S.work[5] += ncpairs;
-                }
+                if (act)   // the work counters, one lane each
+                    work += gl == 0 ? nclp * kCluster : gl == 1 ? nc : gl == 2 ? nc * iters : gl == 3 ? 1 : gl == 4 ? (nc > 0 ? iters : 0) : ncpairs;
 
-                // -- 4. contact setup: the first TPE*CPL contacts in registers, the rest in
-                //       shared memory (and beyond SC in the spill area); the contact
-                //       range of each link
-                V3 cr_[CPL], cn_[CPL], cc_[CPL], lam_[CPL];
-                float ikn_[CPL], ikt_[CPL];
+                // -- 3. contact setup, records to shared memory (past SC to the spill area);
+                //       the contact range of each link
+                const int nc_w = wmax(nc);
                 const float trW = Wi.xx + Wi.yy + Wi.zz;
-                // warm start: the impulse of the same pair at the end of the last
-                // substep (both lists are in pair order: binary search), else zero
-                const int n_prev = warm ? S.n_prev : 0;
-                auto warm_lam = [&](float wbits) -> V3 {
-                    const int id = (__float_as_int(wbits) & 0xff) << 8 | ((__float_as_int(wbits) >> 16) & 0xff);
-                    int lo = 0, hi = n_prev;
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (__float_as_int(prev[mid].w) < id) lo = mid + 1; else hi = mid;
+                // (two contacts a lane and round: two independent chains; the palm takes
+                // the capsules' path wherever the two agree, its pose being the identity)
+                auto setup = [&](int ci) {
+                    const int e = clist[ci], l = e >> 8, j = e & 0xff;
+                    const int e0 = ci > 0 ? clist[ci - 1] >> 8 : -1, e1 = ci < nc - 1 ? clist[ci + 1] >> 8 : -1;
+                    if (e0 != l) S.lbeg[l] = (unsigned short)ci;
+                    if (e1 != l) S.lend[l] = (unsigned short)(ci + 1);
+                    const float4 sp = sph[(j >> 3) * kSphStride + (j & 7)];
+                    const V3 cr = xyz(sp), ca = xyz(S.xa[l]) + cr;
+                    Hit hh;
+                    if (l == 0) {
+                        hh = hit_box_local(ca, sp.w, sc.palm_hx, sc.palm_hy, sc.palm_hz);
+                    } else {
+                        const float4 Aq = __ldg(L0 + l * kLinkStride + 2);
+                        hh = hit_capsule(ca, sp.w, xyz(S.ax[l]), sc.link_len, inv_L, sc.link_rad, {Aq.x, Aq.y, Aq.z, Aq.w});
                     }
-                    if (lo < n_prev && __float_as_int(prev[lo].w) == id) return xyz(prev[lo]);
-                    return mk(0, 0, 0);
+                    const V3 r = cr - hh.n * sp.w;
+                    // the first pad of the link whose interval holds t
+                    const float4 b4 = *reinterpret_cast<const float4 *>(PT.s0[l]), e4 = *reinterpret_cast<const float4 *>(PT.s1[l]);
+                    const uchar4 id = *reinterpret_cast<const uchar4 *>(PT.id[l]);
+                    unsigned char pad = 0xff;
+                    if (hh.t >= b4.w && hh.t < e4.w) pad = id.w;
+                    if (hh.t >= b4.z && hh.t < e4.z) pad = id.z;
+                    if (hh.t >= b4.y && hh.t < e4.y) pad = id.y;
+                    if (hh.t >= b4.x && hh.t < e4.x) pad = id.x;
+                    cpad[ci] = pad;
+                    const CSetup cs = setup_contact(r, hh.n, hh.gap, l, Wi, trW, inv_m, cfg, L0, L1, x, inv_h);
+                    const float4 r0 = make_float4(r.x, r.y, r.z, cs.ikt), r1 = make_float4(hh.n.x, hh.n.y, hh.n.z, cs.ikn),
+                                 r2 = make_float4(cs.cc.x, cs.cc.y, cs.cc.z, 0.0f);
+                    float4 l4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    if (WARM) {   // the pair's impulse at the end of the last substep (both lists are in pair order), else zero
+                        int lo = 0, hi = n_prev;
+#pragma unroll 1
+                        while (lo < hi) {
+                            const int mid = (lo + hi) >> 1;
+                            if (__float_as_int(prev[mid].w) < e) lo = mid + 1; else hi = mid;
+                        }
+                        if (lo < n_prev && __float_as_int(prev[lo].w) == e) {
+                            const float4 p4 = prev[lo];
+                            l4 = make_float4(p4.x, p4.y, p4.z, 0.0f);
+                        }
+                    }
+                    if (ci < RCAP) {
+                        rec[3 * ci] = r0;
+                        rec[3 * ci + 1] = r1;
+                        rec[3 * ci + 2] = r2;
+                        if (WARM) lamst[ci] = l4;
+                    } else {
+                        float4 *g4 = spill_g + (size_t)(ci - RCAP) * 4;
+                        g4[0] = r0;
+                        g4[1] = r1;
+                        g4[2] = r2;
+                        g4[3] = l4;
+                    }
                 };
-#pragma unroll
-                for (int k = 0; k < CPL; ++k) {
-                    const int ci = G.tid + k * TPE;
-                    lam_[k] = mk(0, 0, 0);
-                    cr_[k] = mk(0, 0, 0); cn_[k] = mk(0, 0, 1); cc_[k] = mk(0, 0, 0);
-                    ikn_[k] = 0.0f; ikt_[k] = 0.0f;
-                    if (ci < nc) {
-                        const float4 s0 = stage[ci][0], s1 = stage[ci][1];
-                        const int l = __float_as_int(s1.w) & 0xff;
-                        if (ci == 0 || (__float_as_int(stage[ci - 1][1].w) & 0xff) != l) S.lbeg[l] = (unsigned short)ci;
-                        if (ci == nc - 1 || (__float_as_int(cslot(ci + 1)[1].w) & 0xff) != l) S.lend[l] = (unsigned short)(ci + 1);
-                        const CSetup cs = setup_contact(xyz(s0), xyz(s1), s0.w, l, Wi, trW, inv_m, cfg, L0, L1, x, inv_h);
-                        cr_[k] = xyz(s0); cn_[k] = xyz(s1); cc_[k] = cs.cc; ikn_[k] = cs.ikn; ikt_[k] = cs.ikt;
-                        if (warm) lam_[k] = warm_lam(s1.w);
-                    }
-                }
-                for (int ci = RCAP + G.tid; ci < nc; ci += TPE) {
-                    float4 *c4 = cslot(ci);
-                    const float4 s0 = c4[0], s1 = c4[1];
-                    const int l = __float_as_int(s1.w) & 0xff;
-                    if ((__float_as_int(cslot(ci - 1)[1].w) & 0xff) != l) S.lbeg[l] = (unsigned short)ci;
-                    if (ci == nc - 1 || (__float_as_int(cslot(ci + 1)[1].w) & 0xff) != l) S.lend[l] = (unsigned short)(ci + 1);
-                    const CSetup cs = setup_contact(xyz(s0), xyz(s1), s0.w, l, Wi, trW, inv_m, cfg, L0, L1, x, inv_h);
-                    c4[0].w = cs.ikt;
-                    c4[2] = make_float4(cs.cc.x, cs.cc.y, cs.cc.z, cs.ikn);
-                    const V3 l0 = warm ? warm_lam(s1.w) : mk(0, 0, 0);
-                    c4[3] = make_float4(l0.x, l0.y, l0.z, 0.0f);
-                }
+#pragma unroll 1
+                for (int ci = gl; ci < nc; ci += L) setup(ci);
+                __syncwarp();   // (the impulses take the spheres' place)
 
-                // -- 5. Jacobi projected-impulse iterations
+                // -- 4. Jacobi projected-impulse iterations
                 V3 vv = v_pred, ww = w_pred;
-                if (nc > 0) {
-                    const float inv_nc = 1.0f / (float)nc;
-                    const int slot_off = TPE > 32 ? 32 * G.wid : 0;   // this warp's first contact of a slot
-                    if (warm) {   // the cached impulses act from the first iteration on
-                        float acc[6] = {0, 0, 0, 0, 0, 0};
+                if (nc_w > 0) {
+                    const float inv_nc = nc > 0 ? 1.0f / (float)nc : 0.0f, mu_s = 4096.0f * mu;
+                    auto unpack = [&](Contact<float> &c, const float4 *c4, const float4 *l) {
+                        const float4 s0 = c4[0], s1 = c4[1], s2 = c4[2];
+                        c.r = {s0.x, s0.y, s0.z};
+                        c.n = {s1.x, s1.y, s1.z};
+                        c.c = {s2.x, s2.y, s2.z};
+                        c.ikt = s0.w;
+                        c.ikn = s1.w;
+                        if (l) c.lam = {l->x, l->y, l->z};
+                    };
+                    // register slot k of the lane: contact gl + k L (empty past the list)
+                    auto load1 = [&](Contact<float> &c, int k) {
+                        const int ci = gl + k * L;
+                        c.clear();
+                        if (ci < nc) unpack(c, rec + 3 * ci, WARM ? lamst + ci : nullptr);
+                    };
+                    auto store1 = [&](float lx, float ly, float lz, int k) {
+                        const int ci = gl + k * L;
+                        if (ci < nc) lamst[ci] = make_float4(lx, ly, lz, 0.0f);
+                    };
+                    auto load2 = [&](Contact<F2> &c, int k) {
+                        Contact<float> a, b;
+                        load1(a, k);
+                        load1(b, k + 1);
+                        c.r = {{a.r.x, b.r.x}, {a.r.y, b.r.y}, {a.r.z, b.r.z}};
+                        c.n = {{a.n.x, b.n.x}, {a.n.y, b.n.y}, {a.n.z, b.n.z}};
+                        c.c = {{a.c.x, b.c.x}, {a.c.y, b.c.y}, {a.c.z, b.c.z}};
+                        c.lam = {{a.lam.x, b.lam.x}, {a.lam.y, b.lam.y}, {a.lam.z, b.lam.z}};
+                        c.ikn = {a.ikn, b.ikn};
+                        c.ikt = {a.ikt, b.ikt};
+                    };
+                    auto store2 = [&](const Contact<F2> &c, int k) {
+                        store1(c.lam.x.x, c.lam.y.x, c.lam.z.x, k);
+                        store1(c.lam.x.y, c.lam.y.y, c.lam.z.y, k + 1);
+                    };
+                    // adds the wrenches of slots k (and k + 1) to their accumulators, slot mod NA, in slot order
+                    auto add1 = [&](float (&acc)[NA][6], const Contact<float> &c, int k) {
+                        float s[6];
+                        c.wrench(s);
 #pragma unroll
-                        for (int k = 0; k < CPL; ++k) {
-                            if (k * TPE + slot_off < nc) {
-                                const V3 tq = cross(cr_[k], lam_[k]);
-                                acc[0] += lam_[k].x; acc[1] += lam_[k].y; acc[2] += lam_[k].z;
-                                acc[3] += tq.x; acc[4] += tq.y; acc[5] += tq.z;
+                        for (int q = 0; q < 6; ++q) acc[k % NA][q] += s[q];
+                    };
+                    auto add2 = [&](float (&acc)[NA][6], const Contact<F2> &c, int k) {
+                        F2 s[6];
+                        c.wrench(s);
+#pragma unroll
+                        for (int q = 0; q < 6; ++q) {
+                            if constexpr (NA == 1) {
+                                acc[0][q] = (acc[0][q] + s[q].x) + s[q].y;
+                            } else {   // one packed addition
+                                const F2 t = t_add(F2{acc[k % NA][q], acc[(k + 1) % NA][q]}, s[q]);
+                                acc[k % NA][q] = t.x;
+                                acc[(k + 1) % NA][q] = t.y;
                             }
                         }
-                        for (int ci = RCAP + G.tid; ci < nc; ci += TPE) {
-                            const float4 *c4 = cslot(ci);
-                            const V3 lam = xyz(c4[3]), tq = cross(xyz(c4[0]), lam);
-                            acc[0] += lam.x; acc[1] += lam.y; acc[2] += lam.z;
-                            acc[3] += tq.x; acc[4] += tq.y; acc[5] += tq.z;
-                        }
-                        group_sum6<TPE>(acc, G, &S.red[0][0][0], parity);
-                        parity ^= 1;
-                        vv = v_pred + mk(acc[0], acc[1], acc[2]) * inv_m;
-                        ww = w_pred + smul(Wi, mk(acc[3], acc[4], acc[5]));
+                    };
+                    auto body = [&](const float (&t)[6]) {
+                        vv = v_pred + mk(t[0], t[1], t[2]) * inv_m;
+                        const V3 mo = mk(t[3], t[4], t[5]);
+                        if constexpr (WARM && TPE >= 64)   // (these instances' contraction)
+                            ww = w_pred + mk(__fmaf_rn(Wi.xz, mo.z, prod_add(Wi.xy, mo.y, Wi.xx, mo.x)),
+                                             __fmaf_rn(Wi.yz, mo.z, prod_add(Wi.yy, mo.y, Wi.xy, mo.x)),
+                                             __fmaf_rn(Wi.zz, mo.z, prod_add(Wi.yz, mo.y, Wi.xz, mo.x)));
+                        else
+                            ww = w_pred + smul(Wi, mo);
+                    };
+                    if (WARM) {   // the cached impulses act from the first iteration on
+                        float acc[NA][6] = {}, t[6];
+#pragma unroll 1
+                        for (int s0 = 0; s0 * L < nc_w; s0 += NA)
+#pragma unroll
+                            for (int j = 0; j < NA; ++j) {
+                                const int ci = (s0 + j) * L + gl;
+                                Contact<float> c;
+                                c.clear();
+                                if (ci < min(nc, RCAP)) unpack(c, rec + 3 * ci, lamst + ci);
+                                else if (ci < nc) unpack(c, spill_g + (size_t)(ci - RCAP) * 4, spill_g + (size_t)(ci - RCAP) * 4 + 3);
+                                add1(acc, c, j);
+                            }
+                        env_sum6<L, NA, NA>(acc, t, gl);
+                        body(t);
                     }
-                    for (int it = 0; it < iters; ++it) {
-                        float acc[6] = {0, 0, 0, 0, 0, 0};
-                        // a register slot is skipped only when it is empty in every
-                        // lane of the warp (a warp-uniform branch: in a wider group the
-                        // warps holding only empty slots skip it and free issue slots);
-                        // otherwise all lanes update it without a branch so the slots'
-                        // chains interleave:
-                        // an empty slot (r = c = 0, n = z, 1/k = 0, lambda = 0) keeps
-                        // lambda = 0 and adds zeros
+                    // one loop per number of occupied slots, each a straight stretch of
+                    // code: slots in pairs (packed), an odd last one alone. (Guarded slots in
+                    // one loop kept the scheduler from interleaving them: 932 cycles an
+                    // iteration at 1024 cylinders, 80 contacts.) Past its own count an
+                    // environment of a 16-lane warp holds still (a step of zero)
+                    auto rel = [&](int it) -> float { return (L == 32 || it < iters) ? inv_nc : 0.0f; };
+                    if (nc_w <= L) {
+                        Contact<float> c0;
+                        load1(c0, 0);
+#pragma unroll 1
+                        for (int it = 0; it < iters_w; ++it) {
+                            float acc[NA][6] = {}, t[6];
+                            c0.update(vv, ww, mu_s, rel(it));
+                            add1(acc, c0, 0);
+                            env_sum6<L, NA, 1>(acc, t, gl);
+                            body(t);
+                        }
+                        store1(c0.lam.x, c0.lam.y, c0.lam.z, 0);
+                    } else if (nc_w <= 2 * L) {
+                        Contact<F2> c0;
+                        load2(c0, 0);
+#pragma unroll 1
+                        for (int it = 0; it < iters_w; ++it) {
+                            float acc[NA][6] = {}, t[6];
+                            c0.update(vv, ww, mu_s, rel(it));
+                            add2(acc, c0, 0);
+                            env_sum6<L, NA, (NA < 2 ? NA : 2)>(acc, t, gl);
+                            body(t);
+                        }
+                        store2(c0, 0);
+                    } else if (nc_w <= 3 * L) {
+                        Contact<F2> c0;
+                        Contact<float> c2;
+                        load2(c0, 0);
+                        load1(c2, 2);
+#pragma unroll 1
+                        for (int it = 0; it < iters_w; ++it) {
+                            float acc[NA][6] = {}, t[6];
+                            const float k = rel(it);
+                            c0.update(vv, ww, mu_s, k);
+                            c2.update(vv, ww, mu_s, k);
+                            add2(acc, c0, 0);
+                            add1(acc, c2, 2);
+                            env_sum6<L, NA, (NA < 3 ? NA : 3)>(acc, t, gl);
+                            body(t);
+                        }
+                        store2(c0, 0);
+                        store1(c2.lam.x, c2.lam.y, c2.lam.z, 2);
+                    } else {
+                        Contact<F2> c0, c2;
+                        load2(c0, 0);
+                        load2(c2, 2);
+#pragma unroll 1
+                        for (int it = 0; it < iters_w; ++it) {
+                            float acc[NA][6] = {}, t[6];
+                            const float k = rel(it);
+                            c0.update(vv, ww, mu_s, k);
+                            c2.update(vv, ww, mu_s, k);
+                            add2(acc, c0, 0);
+                            add2(acc, c2, 2);
+#pragma unroll 1
+                            for (int s0 = kSlots; s0 * L < nc_w; s0 += NA)   // the further ones, in the same per-thread order
 #pragma unroll
-                        for (int k = 0; k < CPL; ++k) {
-                            if (k * TPE + slot_off < nc) {
-                                lam_[k] = update_contact(lam_[k], cr_[k], cn_[k], cc_[k], ikn_[k], ikt_[k], vv, ww, mu, inv_nc);
-                                const V3 tq = cross(cr_[k], lam_[k]);
-                                acc[0] += lam_[k].x; acc[1] += lam_[k].y; acc[2] += lam_[k].z;
-                                acc[3] += tq.x; acc[4] += tq.y; acc[5] += tq.z;
-                            }
+                                for (int j = 0; j < NA; ++j) {
+                                    const int ci = (s0 + j) * L + gl;
+                                    if (ci < nc) {
+                                        float4 *g4 = spill_g + (size_t)(ci - RCAP) * 4;
+                                        Contact<float> c;
+                                        unpack(c, g4, g4 + 3);
+                                        c.update(vv, ww, mu_s, k);
+                                        g4[3] = make_float4(c.lam.x, c.lam.y, c.lam.z, 0.0f);
+                                        add1(acc, c, j);
+                                    }
+                                }
+                            env_sum6<L, NA, NA>(acc, t, gl);
+                            body(t);
                         }
-                        // staged contacts: shared memory, then the spill area (this
-                        // lane's sequence RCAP + tid, + TPE, ... continued past SC)
-                        const int ncs = min(nc, SC);
-                        for (int ci = RCAP + G.tid; ci < ncs; ci += TPE) {
-                            const float4 s0 = stage[ci][0], s1 = stage[ci][1], s2 = stage[ci][2], s3 = stage[ci][3];
-                            const V3 lam = update_contact(xyz(s3), xyz(s0), xyz(s1), xyz(s2), s2.w, s0.w, vv, ww, mu, inv_nc);
-                            stage[ci][3] = make_float4(lam.x, lam.y, lam.z, 0.0f);
-                            const V3 tq = cross(xyz(s0), lam);
-                            acc[0] += lam.x; acc[1] += lam.y; acc[2] += lam.z;
-                            acc[3] += tq.x; acc[4] += tq.y; acc[5] += tq.z;
-                        }
-                        if (nc > SC) {
-                            int ci = RCAP + G.tid;
-                            if (ci < SC) ci += ((SC - ci + TPE - 1) / TPE) * TPE;
-                            for (; ci < nc; ci += TPE) {
-                                float4 *c4 = spill_g + (size_t)(ci - SC) * 4;
-                                const float4 s0 = c4[0], s1 = c4[1], s2 = c4[2], s3 = c4[3];
-                                const V3 lam = update_contact(xyz(s3), xyz(s0), xyz(s1), xyz(s2), s2.w, s0.w, vv, ww, mu, inv_nc);
-                                c4[3] = make_float4(lam.x, lam.y, lam.z, 0.0f);
-                                const V3 tq = cross(xyz(s0), lam);
-                                acc[0] += lam.x; acc[1] += lam.y; acc[2] += lam.z;
-                                acc[3] += tq.x; acc[4] += tq.y; acc[5] += tq.z;
-                            }
-                        }
-                        group_sum6<TPE>(acc, G, &S.red[0][0][0], parity);
-                        parity ^= 1;
-                        vv = v_pred + mk(acc[0], acc[1], acc[2]) * inv_m;
-                        ww = w_pred + smul(Wi, mk(acc[3], acc[4], acc[5]));
+                        store2(c0, 0);
+                        store2(c2, 2);
                     }
                 }
-                v = vv;
-                w = ww;
 
-                // -- 6. symplectic Euler with the exact rotation exponential
-                x = x + v * h;
-                {
+                // -- 5. symplectic Euler with the exact rotation exponential
+                if (act) {
+                    v = vv;
+                    w = ww;
+                    x = x + v * h;
                     const float wn = sqrtf(dot(w, w));
                     float sn, cs;
                     sincosf(0.5f * wn * h, &sn, &cs);
                     const float kq = (wn > 0.0f) ? sn / wn : 0.5f * h;
                     q = qnorm(qmul({cs, w.x * kq, w.y * kq, w.z * kq}, q));
                 }
-                // sensor pads: force on the pad by the object is -lambda / h,
-                // summed over the contacts of the pad's link in contact order
-#pragma unroll
-                for (int k = 0; k < CPL; ++k) {
-                    const int ci = G.tid + k * TPE;
-                    if (ci < nc) cslot(ci)[3] = make_float4(lam_[k].x, lam_[k].y, lam_[k].z, 0.0f);
-                }
-                G.sync();
-                for (int p = G.tid; p < P; p += TPE) {
+                // sensor pads: force on the pad by the object is -lambda / h, summed
+                // over the contacts of the pad's link in contact order
+                __syncwarp();
+#pragma unroll 1
+                for (int k = gl; k < 3 * P; k += L) {
+                    const int p = k / 3, comp = k - 3 * p;
                     const int l = __ldg(sc.pad_link + p);
-                    float fx = 0.0f, fy = 0.0f, fz = 0.0f;
-                    const int e = S.lend[l];
-                    for (int ci = S.lbeg[l]; ci < e; ++ci) {
-                        const float4 *c4 = cslot(ci);
-                        if (((__float_as_int(c4[1].w) >> 8) & 0xff) != p) continue;
-                        const float4 s3 = c4[3];
-                        fx -= s3.x * inv_h; fy -= s3.y * inv_h; fz -= s3.z * inv_h;
-                    }
-                    S.padacc[3 * p + 0] += fx;
-                    S.padacc[3 * p + 1] += fy;
-                    S.padacc[3 * p + 2] += fz;
+                    float f = 0.0f;
+                    const int e = S.lend[l], es = min(e, RCAP);
+                    int ci = S.lbeg[l];
+                    const float *lc = reinterpret_cast<const float *>(lamst) + comp;
+#pragma unroll 4
+                    for (; ci < es; ++ci) f -= (cpad[ci] == p ? lc[4 * ci] : 0.0f) * inv_h;
+#pragma unroll 1
+                    for (; ci < e; ++ci) f -= (cpad[ci] == p ? reinterpret_cast<const float *>(spill_g + (size_t)(ci - RCAP) * 4 + 3)[comp] : 0.0f) * inv_h;
+                    S.padacc[k] += f;
                 }
-                if (warm) {   // this substep's contacts and final impulses, for the next one
-                    for (int ci = G.tid; ci < nc; ci += TPE) {
-                        const float4 *c4 = cslot(ci);
-                        const int wb = __float_as_int(c4[1].w);
-                        const float4 l3 = c4[3];
-                        prev[ci] = make_float4(l3.x, l3.y, l3.z, __int_as_float((wb & 0xff) << 8 | ((wb >> 16) & 0xff)));
+                if (WARM) {   // this substep's contacts and final impulses, for the next one
+#pragma unroll 1
+                    for (int ci = gl; ci < nc; ci += L) {
+                        const float4 l3 = ci < RCAP ? lamst[ci] : spill_g[(size_t)(ci - RCAP) * 4 + 3];
+                        prev[ci] = make_float4(l3.x, l3.y, l3.z, __int_as_float(clist[ci]));
                     }
-                    if (G.tid == 0) S.n_prev = nc;
+                    if (act) n_prev = nc;
                 }
-                G.sync();
+                __syncwarp();
             }
-            if (!skip) {
+            if (act) {
                 if (!all_finite(x, q, v, w)) st |= IH_ENV_NONFINITE;
                 else if (dot(x, x) > cfg.escape_radius * cfg.escape_radius) st |= IH_ENV_ESCAPED;
             }
-            if (window_mode) {   // this frame's cost, window sum and mean, and pose
+            if (scored) {   // this frame's cost, window sum and mean (every frame, or a single one); the frame's pose
                 const double c = frame_cost(obs + (size_t)fr * P * 3, st);
-                if (G.tid == 0) {
+                if (gl == 0 && live) {
                     c_sum_env = __dadd_rn(c_sum_env, c);
-                    const double cm = __ddiv_rn(c_sum_env, (double)(n_win0 + fr + 1));
-                    a.cm_frames[(size_t)fr * a.N + env] = cm;
-                    float4 *pf = a.pose_frames + 2 * ((size_t)fr * a.N + env);
-                    pf[0] = make_float4(x.x, x.y, x.z, 0.0f);
-                    pf[1] = make_float4(q.w, q.x, q.y, q.z);
+                    double cm = __ddiv_rn(c_sum_env, (double)(n_win0 + fr + 1));
+                    if (window_mode) {
+                        a.cm_frames[(size_t)fr * a.N + env] = cm;
+                        float4 *pf = a.pose_frames + 2 * ((size_t)fr * a.N + env);
+                        pf[0] = make_float4(x.x, x.y, x.z, 0.0f);
+                        pf[1] = make_float4(q.w, q.x, q.y, q.z);
+                    }
                     if (fr == a.n_frames - 1) {
                         a.c_sum[env] = c_sum_env;
                         a.c_mean[env] = cm;
                         if (a.cost_mean) a.cost_mean[env] = cm;
+                        const unsigned long long key = cost_key(isnan(cm) ? INFINITY : cm);
+                        if (key < best_k || (key == best_k && env < best_i)) { best_k = key; best_i = env; }
                     }
                 }
-            }
-        }
-        // frame cost against the observation (Sec. III-C), FP64, in pad order,
-        // on exactly the forces written out below
-        if (scored && !window_mode) {
-            const double c = frame_cost(obs, st);
-            if (G.tid == 0) {
-                const double sum = __dadd_rn(a.c_sum[env], c);
-                a.c_sum[env] = sum;
-                double cm = __ddiv_rn(sum, (double)n_win);
-                a.c_mean[env] = cm;
-                if (a.cost_mean) a.cost_mean[env] = cm;
-                if (isnan(cm)) cm = INFINITY;
-                if (cm < S.best_c || (cm == S.best_c && env < S.best_i)) { S.best_c = cm; S.best_i = env; }
             }
         }
         // forces of the last frame, averaged over its substeps
         const float inv_ns = 1.0f / (float)ns;
         float *fo = a.forces + (size_t)env * P * 3;
-        G.sync();
-        for (int k = G.tid; k < 3 * P; k += TPE) fo[k] = S.padacc[k] * inv_ns;
-        if (G.tid == 0) {
+        __syncwarp();
+#pragma unroll 1
+        for (int k = gl; k < 3 * P && live; k += L) fo[k] = S.padacc[k] * inv_ns;
+        if (gl == 0 && live) {
             a.pose[2 * env] = make_float4(x.x, x.y, x.z, 0.0f);
             a.pose[2 * env + 1] = make_float4(q.w, q.x, q.y, q.z);
             a.vel[2 * env] = make_float4(v.x, v.y, v.z, 0.0f);
             a.vel[2 * env + 1] = make_float4(w.x, w.y, w.z, 0.0f);
             a.status[env] = st;
         }
-        if (warm) {   // the cache for the next launch
-            const int np = S.n_prev;
-            if (G.tid == 0) a.cache_n[env] = np;
-            for (int k = G.tid; k < np; k += TPE) a.cache[(size_t)env * cap + k] = prev[k];
+        if (WARM && live) {   // the cache for the next launch
+            if (gl == 0) a.cache_n[env] = n_prev;
+#pragma unroll 1
+            for (int k = gl; k < n_prev; k += L) a.cache[(size_t)env * cap + k] = prev[k];
         }
-        G.sync();
+        __syncwarp();
     }
-    if (G.tid == 0 && a.work)
-        for (int k = 0; k < 6; ++k)
-            if (S.work[k]) atomicAdd(a.work + k, S.work[k]);
-    if (a.queue) {   // the last block to finish empties the queue for the next launch
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();   // this block's queue draws, before its finish ticket
-            if (atomicAdd(a.queue + 1, 1) == (int)gridDim.x - 1) {
-                atomicExch(a.queue, 0);
-                atomicExch(a.queue + 1, 0);
-            }
+    if (gl < 6 && a.work && work) atomicAdd(a.work + gl, work);
+    if (a.queue && lane == 0) {   // the last block to finish empties the queue for the next launch
+        __threadfence();   // this block's queue draws, before its finish ticket
+        if (atomicAdd(a.queue + 1, 1) == (int)gridDim.x - 1) {
+            atomicExch(a.queue, 0);
+            atomicExch(a.queue + 1, 0);
         }
     }
     if (!scored || window_mode) return;
     // argmin (C_i, i) over the grid: per-block candidate, then the last block
-    __shared__ bool last;
-    __shared__ int best_env;
+    auto better = [&](unsigned long long k, int i) {
+        if (k < best_k || (k == best_k && i < best_i)) { best_k = k; best_i = i; }
+    };
+    if (L == 16) better(__shfl_sync(kAll, best_k, 16), __shfl_sync(kAll, best_i, 16));
+    bool last = false;
     __threadfence();   // this thread's pose/status/cost writes, before the ticket
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double bc = INFINITY;
-        int bi = 0x7fffffff;
-        for (int g2 = 0; g2 < GPB; ++g2) {
-            const GSm<W> &S2 = *reinterpret_cast<const GSm<W> *>(smem + block_smem_bytes() + g2 * gsm_bytes<W>());
-            const double c = S2.best_c;
-            const int i = S2.best_i;
-            if (c < bc || (c == bc && i < bi)) { bc = c; bi = i; }
-        }
-        a.part_c[blockIdx.x] = bc;
-        a.part_i[blockIdx.x] = bi;
+    __syncwarp();
+    if (lane == 0) {
+        a.part_c[blockIdx.x] = __longlong_as_double((long long)best_k);
+        a.part_i[blockIdx.x] = best_i;
         __threadfence();
         last = atomicAdd(a.done, 1u) == gridDim.x - 1;
     }
-    __syncthreads();
-    if (!last) return;
+    if (!__shfl_sync(kAll, (int)last, 0)) return;
     __threadfence();
-    if (threadIdx.x < 32) {
-        double bc = INFINITY;
-        int bi = 0x7fffffff;
-        for (int b = threadIdx.x; b < gridDim.x; b += 32) {
-            const double c = __ldcg(a.part_c + b);
-            const int i = __ldcg(a.part_i + b);
-            if (c < bc || (c == bc && i < bi)) { bc = c; bi = i; }
-        }
+    best_k = ~0ull;
+    best_i = 0x7fffffff;
+#pragma unroll 4
+    for (int b = lane; b < (int)gridDim.x; b += 32)
+        better((unsigned long long)__double_as_longlong(__ldcg(a.part_c + b)), __ldcg(a.part_i + b));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double oc = __shfl_xor_sync(0xffffffffu, bc, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (oc < bc || (oc == bc && oi < bi)) { bc = oc; bi = oi; }
-        }
-        if (threadIdx.x == 0) {
-            const int best = (bi == 0x7fffffff) ? 0 : bi;
-            int *argmin_out = a.argmin_out;
-            if (a.win) argmin_out = a.win->argmin ? a.win->argmin + a.win_k : nullptr;
-            *a.argmin_state = best;
-            if (argmin_out) *argmin_out = best;
-            *a.n_window = n_win;
-            *a.done = 0u;
-            best_env = best;
-        }
+    for (int o = 16; o > 0; o >>= 1) better(__shfl_xor_sync(kAll, best_k, o), __shfl_xor_sync(kAll, best_i, o));
+    const int best = (best_i == 0x7fffffff) ? 0 : best_i;
+    if (lane == 0) {
+        int *argmin_out = a.argmin_out;
+        if (a.win) argmin_out = a.win->argmin ? a.win->argmin + a.win_k : nullptr;
+        *a.argmin_state = best;
+        if (argmin_out) *argmin_out = best;
+        *a.n_window = n_win0 + 1;
+        *a.done = 0u;
     }
-    __syncthreads();
     float *est_out = a.est_pose_out;
     if (a.win) est_out = a.win->est ? a.win->est + 8 * a.win_k : nullptr;
-    if (est_out && threadIdx.x < 8) {
-        const float4 p = __ldcg(a.pose + 2 * best_env + (threadIdx.x >> 2));
+    if (est_out && lane < 8) {
+        const float4 p = __ldcg(a.pose + 2 * best + (lane >> 2));
         const float v[4] = {p.x, p.y, p.z, p.w};
-        est_out[threadIdx.x] = v[threadIdx.x & 3];
+        est_out[lane] = v[lane & 3];
     }
 }
 
-template <int TPE, int CPL, bool WARM>
+template <int L, int TPE, bool WARM>
 size_t bytes_t(int s_max, int c_max, int clp_cap) {
-    constexpr int GPB = Group<TPE>::GPB;
-    const int sc = stage_capacity(TPE * CPL, c_max, GPB);
-    return block_smem_bytes() + GPB * gsm_bytes<Group<TPE>::W>() +
-           GPB * group_dyn_floats4(s_max, sc, c_max, WARM, clp_cap) * sizeof(float4);
+    return sizeof(PadSm) + 32 / L * env_bytes(s_max, stage_capacity(L, c_max), c_max, WARM, clp_cap);
 }
 
-// Shared-memory opt-in, and the blocks of this shape that fit on one SM
-template <int TPE, int CPL, bool WARM>
+// Shared-memory opt-in, and the blocks of this kernel that fit on one SM
+template <int L, int TPE, bool WARM>
 cudaError_t prepare_t(int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
-    const size_t bytes = bytes_t<TPE, CPL, WARM>(s_max, c_max, clp_cap);
+    const size_t bytes = bytes_t<L, TPE, WARM>(s_max, c_max, clp_cap);
     cudaError_t e = cudaSuccess;
     if (bytes > 48 * 1024)
-        e = cudaFuncSetAttribute(step_kernel<TPE, CPL, WARM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        e = cudaFuncSetAttribute(step_kernel<L, TPE, WARM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess && blocks_per_sm)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, step_kernel<TPE, CPL, WARM>, kBlock, bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, step_kernel<L, TPE, WARM>, 32, bytes);
     return e;
 }
 
-template <int TPE, int CPL, bool WARM>
-cudaError_t launch_t(const StepArgs &a, int grid, int s_max, cudaStream_t s) {
-    step_kernel<TPE, CPL, WARM><<<grid, kBlock, bytes_t<TPE, CPL, WARM>(s_max, a.cfg.c_max, a.clp_cap), s>>>(a, s_max);
-    return cudaGetLastError();
-}
-
-// The dispatch over the compiled shapes, for the cold (WARM = false) or the
+// The dispatch over the compiled kernels, for the cold (WARM = false) or the
 // warm-started (WARM = true) solver; each is instantiated in its own
 // translation unit so the two build in parallel.
 template <bool WARM>
-size_t smem_bytes_w(const StepVariant &v, int s_max, int c_max, int clp_cap) {
-#define IH_BYTES(T, C) if (v.group == T && v.cpl == C) return bytes_t<T, C, WARM>(s_max, c_max, clp_cap);
-    IH_STEP_VARIANTS(IH_BYTES)
-#undef IH_BYTES
-    return 0;
-}
-
-template <bool WARM>
 cudaError_t prepare_w(const StepVariant &v, int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
-#define IH_PREP(T, C) if (v.group == T && v.cpl == C) return prepare_t<T, C, WARM>(s_max, c_max, clp_cap, blocks_per_sm);
-    IH_STEP_VARIANTS(IH_PREP)
+#define IH_PREP(L, T) if (v.lanes == L && v.group == T) return prepare_t<L, T, WARM>(s_max, c_max, clp_cap, blocks_per_sm);
+    IH_STEP_KERNELS(IH_PREP)
 #undef IH_PREP
     return cudaErrorInvalidValue;
 }
 
 template <bool WARM>
 cudaError_t launch_w(const StepArgs &a, const StepVariant &v, int grid, int s_max, cudaStream_t s) {
-#define IH_LAUNCH(T, C) if (v.group == T && v.cpl == C) return launch_t<T, C, WARM>(a, grid, s_max, s);
-    IH_STEP_VARIANTS(IH_LAUNCH)
+#define IH_LAUNCH(L, T)                                                                                              \
+    if (v.lanes == L && v.group == T) {                                                                              \
+        step_kernel<L, T, WARM><<<grid, 32, bytes_t<L, T, WARM>(s_max, a.cfg.c_max, a.clp_cap), s>>>(a, s_max);      \
+        return cudaGetLastError();                                                                                   \
+    }
+    IH_STEP_KERNELS(IH_LAUNCH)
 #undef IH_LAUNCH
     return cudaErrorInvalidValue;
 }

@@ -6,10 +6,6 @@
 
 namespace ih {
 
-size_t step_smem_bytes_warm(const StepVariant &v, int s_max, int c_max, int clp_cap) {
-    return smem_bytes_w<true>(v, s_max, c_max, clp_cap);
-}
-
 cudaError_t step_prepare_warm(const StepVariant &v, int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
     return prepare_w<true>(v, s_max, c_max, clp_cap, blocks_per_sm);
 }
