@@ -19,8 +19,11 @@
 //                      its state, adds L eps (Philox normals), clamps m and mu;
 //                      every window sum restarts.
 #include <cmath>
+#include <cooperative_groups.h>
 
 #include "internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace ih {
 namespace {
@@ -652,235 +655,286 @@ __global__ void __launch_bounds__(kOptBlock * kApplyLanes) apply_kernel(const Op
 // ---------------------------------------------------------------- WRS / REPS
 // (Sec. III-D): a PMF over all simulations, N draws with replacement,
 // isotropic exploration of every simulation.
-constexpr int kSoft = 1024;
+//
+// The weights run in one launch of a thread-block cluster, each CTA on its share
+// of the simulations (consecutive, for the CDF): every Newton step of the REPS
+// dual is a sum over all of them, and GB300's FP64 rate (1/64 of FP32) made one
+// CTA spend 302 us on the steps of 4096 simulations, with the weights 5 and their
+// CDF 15 more in launches of their own; stepping, scoring and updating 4096 boxes
+// went from 433 to 161 us. The steps search in FP32 and finish in FP64: two or
+// three steps of ~50 FP64 instructions per simulation, spread over the cluster's
+// SMs, which exchange their sums through distributed shared memory.
+constexpr int kSoft = 512;       // threads per CTA
+constexpr int kSoftCtas = 8;     // CTAs of the cluster (the portable size)
 
-// sums of three doubles over the block (every thread gets them): warp sums,
-// then the first warp sums the warps' partials and broadcasts the totals
-// through shared memory (FP64 adds are scarce on this part: one warp does them)
-__device__ void block_sum3(double &x, double &y, double &z, double (*red)[3]) {
+struct SoftSm {
+    double wpart[kSoft / 32][3];     // a CTA's partial sums, per warp
+    double part[2][3];               // its sums (double-buffered, read by the cluster)
+    double tot[3];
+    unsigned long long kmin[kSoft / 32], kmax[kSoft / 32], kbest[kSoft / 32];
+    int idx[kSoft / 32], cnt[kSoft / 32];
+    unsigned long long ckmin, ckmax, ckbest;
+    int cidx, ccnt;
+    double sc[4];                    // broadcast scalars
+};
+
+// Sums of three values over the cluster, every thread receiving them; in a fixed
+// order (lanes, warps and CTAs by trees), so every CTA takes the same steps
+template <typename T>
+__device__ void cluster_sum3(T &x, T &y, T &z, SoftSm &S, int &buf) {
+    const cg::cluster_group cl = cg::this_cluster();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         x += __shfl_xor_sync(0xffffffffu, x, o);
         y += __shfl_xor_sync(0xffffffffu, y, o);
         z += __shfl_xor_sync(0xffffffffu, z, o);
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) { red[wid][0] = x; red[wid][1] = y; red[wid][2] = z; }
+    if (lane == 0) { S.wpart[wid][0] = (double)x; S.wpart[wid][1] = (double)y; S.wpart[wid][2] = (double)z; }
     __syncthreads();
     if (wid == 0) {
-        double a = red[lane][0], b = red[lane][1], c = red[lane][2];   // kSoft / 32 == 32 partials
+        const bool on = lane < kSoft / 32;
+        T a = on ? (T)S.wpart[lane][0] : (T)0, b = on ? (T)S.wpart[lane][1] : (T)0, c = on ? (T)S.wpart[lane][2] : (T)0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = kSoft / 64; o > 0; o >>= 1) {
             a += __shfl_xor_sync(0xffffffffu, a, o);
             b += __shfl_xor_sync(0xffffffffu, b, o);
             c += __shfl_xor_sync(0xffffffffu, c, o);
         }
-        __syncwarp();
-        if (lane == 0) { red[0][0] = a; red[0][1] = b; red[0][2] = c; }
+        if (lane == 0) { S.part[buf][0] = (double)a; S.part[buf][1] = (double)b; S.part[buf][2] = (double)c; }
     }
-    __syncthreads();
-    x = red[0][0]; y = red[0][1]; z = red[0][2];
-    __syncthreads();
-}
-
-// S0 = sum e_i, S1 = sum e_i D_i, S2 = sum e_i D_i^2 over the finite costs,
-// D_i = C_min - C_i, e_i = exp(D_i / eta)
-// (FP32 exponentials, FP64 sums, for the search; FP64 throughout for the
-// final step)
-template <bool FP32_EXP>
-__device__ void reps_sums(const OptArgs &a, double cmin, double inv_eta, double &S0, double &S1, double &S2,
-                          double (*red)[3]) {
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int i = threadIdx.x; i < a.N; i += kSoft) {
-        const double c = a.c_mean[i];
-        if (!isfinite(c)) continue;
-        const double d = cmin - c;
-        const double e = FP32_EXP ? (double)__expf((float)(d * inv_eta)) : exp(d * inv_eta);
-        s0 += e; s1 += e * d; s2 += e * d * d;
-    }
-    block_sum3(s0, s1, s2, red);
-    S0 = s0; S1 = s1; S2 = s2;
-}
-
-// One CTA: C_min, C_max and the number K of finite window means, i*, the REPS
-// temperature, the weights and their inclusive CDF in index order (elite_w),
-// the total (misc[M_WSUM]).
-__global__ void __launch_bounds__(kSoft) soft_weights_kernel(const OptArgs a) {
-    __shared__ double red[kSoft / 32][3];
-    __shared__ unsigned long long s_min_key;
-    __shared__ int s_min_idx;
-    const int N = a.N, t = threadIdx.x;
-    double lo = INFINITY, hi = -INFINITY, cnt = 0.0;
-    unsigned long long bk = ~0ull;
-    int bi = 0x7fffffff;
-    for (int i = t; i < N; i += kSoft) {
-        const double c = a.c_mean[i];
-        if (isfinite(c)) { lo = fmin(lo, c); hi = fmax(hi, c); cnt += 1.0; }
-        const unsigned long long key = order_key(c);
-        if (key < bk || (key == bk && i < bi)) { bk = key; bi = i; }
-    }
-    // min and max as sums of one-hot terms would be inexact: reduce them directly
+    cl.sync();
+    if (wid == 0) {
+        const double *r = cl.map_shared_rank(&S.part[buf][0], lane % kSoftCtas);
+        T a = (T)r[0], b = (T)r[1], c = (T)r[2];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        const unsigned long long ok = __shfl_xor_sync(0xffffffffu, bk, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ok < bk || (ok == bk && oi < bi)) { bk = ok; bi = oi; }
-    }
-    if (t == 0) { s_min_key = ~0ull; s_min_idx = 0x7fffffff; }
-    if ((t & 31) == 0) { red[t >> 5][0] = lo; red[t >> 5][1] = hi; red[t >> 5][2] = cnt; }
-    __syncthreads();
-    if ((t & 31) == 0) atomicMin(&s_min_key, bk);
-    if (t < 32) {   // the first warp combines the warps' partials
-        double mn = red[t][0], mx = red[t][1], ct = red[t][2];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-            mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            ct += __shfl_xor_sync(0xffffffffu, ct, o);
+        for (int o = kSoftCtas / 2; o > 0; o >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, o);
+            b += __shfl_xor_sync(0xffffffffu, b, o);
+            c += __shfl_xor_sync(0xffffffffu, c, o);
         }
-        __syncwarp();
-        if (t == 0) { red[0][0] = mn; red[0][1] = mx; red[0][2] = ct; }
+        if (lane == 0) { S.tot[0] = (double)a; S.tot[1] = (double)b; S.tot[2] = (double)c; }
     }
     __syncthreads();
-    const double cmin = red[0][0], cmax = red[0][1], K = red[0][2];
-    __syncthreads();
-    if ((t & 31) == 0 && bk == s_min_key) atomicMin(&s_min_idx, bi);
-    double nmin = 0.0;
-    for (int i = t; i < N; i += kSoft) nmin += (a.c_mean[i] == cmin) ? 1.0 : 0.0;
-    double z0 = 0.0, z1 = 0.0;
-    block_sum3(nmin, z0, z1, red);
-    const int istar = s_min_idx;
+    x = (T)S.tot[0]; y = (T)S.tot[1]; z = (T)S.tot[2];
+    buf ^= 1;
+}
 
-    // REPS temperature: the root of g'(eta) = eps + log(S0/K) - S1/(eta S0) by
-    // Newton steps in t = log(eta) (dg'/dt = Var_w(D)/eta^2) inside a
-    // shrinking bracket, bisecting when a step leaves it
+__device__ __forceinline__ double key_value(unsigned long long k) {   // the cost of an order_key
+    return __longlong_as_double((long long)((k >> 63) ? k ^ 0x8000000000000000ull : ~k));
+}
+
+// C_min, C_max and the number K of finite window means, i*, the REPS temperature
+// eta, the weights and their inclusive CDF in index order (elite_w), the total
+// (misc[M_WSUM]).
+__global__ void __launch_bounds__(kSoft) soft_weights_kernel(const OptArgs a) {
+    __shared__ SoftSm S;
+    const cg::cluster_group cl = cg::this_cluster();
+    const int N = a.N, t = threadIdx.x, lane = t & 31, wid = t >> 5, rank = (int)cl.block_rank();
+    const int per = ((N + kSoftCtas - 1) / kSoftCtas + kSoft - 1) / kSoft * kSoft;   // whole chunks
+    const int i0 = min(N, rank * per), i1 = min(N, i0 + per);
+    int buf = 0;
+
+    // ---- extremes of the finite costs, their number, and i* = smallest (key, index), on integer keys
+    unsigned long long kmin = ~0ull, kmax = 0ull, kbest = ~0ull;
+    int bi = 0x7fffffff, cnt = 0;
+    for (int i = i0 + t; i < i1; i += kSoft) {
+        const double c = a.c_mean[i];
+        const unsigned long long key = order_key(c);
+        if (finite_bits(c)) { kmin = min(kmin, key); kmax = max(kmax, key); ++cnt; }
+        if (key < kbest) { kbest = key; bi = i; }
+    }
+    auto reduce = [&](int from) {
+        for (int o = from; o > 0; o >>= 1) {
+            kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
+            kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
+            cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+            const unsigned long long ok = __shfl_xor_sync(0xffffffffu, kbest, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (ok < kbest || (ok == kbest && oi < bi)) { kbest = ok; bi = oi; }
+        }
+    };
+    reduce(16);
+    if (lane == 0) { S.kmin[wid] = kmin; S.kmax[wid] = kmax; S.kbest[wid] = kbest; S.idx[wid] = bi; S.cnt[wid] = cnt; }
+    __syncthreads();
+    if (wid == 0) {
+        const int l = lane % (kSoft / 32);
+        kmin = S.kmin[l]; kmax = S.kmax[l]; kbest = S.kbest[l]; bi = S.idx[l]; cnt = S.cnt[l];
+        reduce(kSoft / 64);
+        if (lane == 0) { S.ckmin = kmin; S.ckmax = kmax; S.ckbest = kbest; S.cidx = bi; S.ccnt = cnt; }
+    }
+    cl.sync();
+    if (wid == 0) {
+        const SoftSm *o = cl.map_shared_rank(&S, lane % kSoftCtas);
+        kmin = o->ckmin; kmax = o->ckmax; kbest = o->ckbest; bi = o->cidx; cnt = o->ccnt;
+        reduce(kSoftCtas / 2);
+        if (lane == 0) { S.kmin[0] = kmin; S.kmax[0] = kmax; S.idx[0] = bi; S.cnt[0] = cnt; }
+    }
+    __syncthreads();
+    const double cmin = S.cnt[0] > 0 ? key_value(S.kmin[0]) : INFINITY, cmax = S.cnt[0] > 0 ? key_value(S.kmax[0]) : -INFINITY;
+    const int istar = S.idx[0];
+    const double K = (double)S.cnt[0];
+
+    // ---- REPS temperature: the root of g'(eta) = eps + log(S0/K) - S1/(eta S0),
+    // S0 = sum e_i, S1 = sum e_i D_i, S2 = sum e_i D_i^2 over the finite costs, D_i =
+    // (C_min - C_i) / (C_max - C_min), e_i = exp(D_i / eta), by Newton steps in t =
+    // log(eta) (dg'/dt = Var_e(D)/eta^2) inside a shrinking bracket, bisecting when a
+    // step leaves it; eta here in units of C_max - C_min
     double eta = NAN;
     if (a.kind == 2 && K > 0.0) {
+        float nmin = 0.0f, z0 = 0.0f, z1 = 0.0f;   // (counts below 2^24 are exact)
+        const double range = cmax - cmin;
+        float *xs = reinterpret_cast<float *>(a.elite_w);   // D_i in FP32 (NaN: not finite), in the weights' place
+        for (int i = i0 + t; i < i1; i += kSoft) {
+            const double c = a.c_mean[i];
+            nmin += c == cmin ? 1.0f : 0.0f;
+            xs[2 * i] = finite_bits(c) ? (float)((cmin - c) / range) : NAN;
+        }
+        cluster_sum3(nmin, z0, z1, S, buf);
         const double eps = a.reps_epsilon;
+        if (t == 0) S.sc[0] = log(K / (double)nmin);
+        __syncthreads();
         if (!(cmax > cmin)) {
             eta = INFINITY;
-        } else if (eps >= log(K / nmin)) {
+        } else if (eps >= S.sc[0]) {
             eta = 0.0;
         } else {
-            // the scalar steps run in thread 0 and reach the block through
-            // shared memory (FP64 transcendentals are costly on this part)
-            __shared__ double s_sc[4];   // e^t, 1/e^t, t, done flag
-            double S0, S1, S2;
-            double tlo = 0.0, thi = 0.0, tt = 0.0;
-            if (t == 0) {
-                const double lr = log(cmax - cmin);
-                tlo = lr - 50.0;
-                thi = lr + 50.0;
-                s_sc[0] = exp(tlo); s_sc[1] = 1.0 / s_sc[0];
-            }
-            __syncthreads();
-            for (int k = 0; k < 200; ++k) {   // widen the bracket until g'(e^tlo) < 0 (a sign: FP32 will do)
-                reps_sums<true>(a, cmin, s_sc[1], S0, S1, S2, red);
-                if (t == 0) {
-                    const bool below = eps + log(S0 / K) - S1 / (s_sc[0] * S0) < 0.0;
-                    if (!below) { tlo -= 50.0; s_sc[0] = exp(tlo); s_sc[1] = 1.0 / s_sc[0]; }
-                    s_sc[3] = below ? 1.0 : 0.0;
+            // FP32 steps to FP32 accuracy (every thread takes the scalar step)
+            float tf = 0.0f, flo = -80.0f, fhi = 50.0f;
+            const float Kf = (float)K, epsf = (float)eps;
+            for (int it = 0; it < 60; ++it) {
+                const float inv = __expf(-tf);
+                float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+                for (int i = i0 + t; i < i1; i += kSoft) {
+                    const float x = xs[2 * i];
+                    const float e = __expf(x * inv);
+                    if (x <= 0.0f) { s0 += e; s1 += e * x; s2 += e * x * x; }
                 }
-                __syncthreads();
-                const bool done = s_sc[3] != 0.0;
-                __syncthreads();
-                if (done) break;
+                cluster_sum3(s0, s1, s2, S, buf);
+                const float mean = s1 / s0, g1 = epsf + logf(s0 / Kf) - mean * inv;
+                if (g1 < 0.0f) flo = tf; else fhi = tf;
+                const float slope = (s2 / s0 - mean * mean) * inv * inv;
+                float tn = slope > 0.0f ? tf - g1 / slope : 0.5f * (flo + fhi);
+                if (!(tn > flo && tn < fhi)) tn = 0.5f * (flo + fhi);
+                const bool near = fabsf(tn - tf) <= 1e-3f * (1.0f + fabsf(tf)) || fhi - flo <= 1e-4f;
+                tf = tn;
+                if (near) break;   // (the same in every thread of the cluster)
             }
-            if (t == 0) { tt = 0.5 * (tlo + thi); s_sc[0] = exp(tt); s_sc[1] = 1.0 / s_sc[0]; s_sc[2] = tt; s_sc[3] = 0.0; }
-            __syncthreads();
-            // Newton steps with FP32 exponentials down to FP32 accuracy, then
-            // one step with FP64 sums: Newton's quadratic convergence takes
-            // the ~1e-7 error of the FP32 root to ~1e-14
-            for (int it = 0; it < 201; ++it) {
-                const bool last = s_sc[3] == 2.0;
-                if (last) reps_sums<false>(a, cmin, s_sc[1], S0, S1, S2, red);
-                else reps_sums<true>(a, cmin, s_sc[1], S0, S1, S2, red);
+            // FP64 steps until one moves t by less than 1e-7 (a Newton step squares
+            // the error). The bracket holds every root: at e^-100 of the range no cost
+            // but the minima counts (FP64 gaps are above 1e-17 of it), at e^50 all
+            // count alike
+            double tt = (double)tf, tlo = -100.0, thi = 50.0;
+            for (int it = 0; it < 400; ++it) {
+                if (t == 0) { const double e = exp(tt); S.sc[0] = e; S.sc[1] = 1.0 / e; }
+                __syncthreads();
+                const double inv = S.sc[1] / range;
+                double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+                for (int i = i0 + t; i < i1; i += kSoft) {
+                    const double c = a.c_mean[i];
+                    if (!finite_bits(c)) continue;
+                    const double d = cmin - c, e = exp(d * inv);
+                    s0 += e; s1 += e * d; s2 += e * d * d;
+                }
+                cluster_sum3(s0, s1, s2, S, buf);
                 if (t == 0) {
-                    const double e = s_sc[0];
-                    const double g1 = eps + log(S0 / K) - S1 / (e * S0);
+                    const double e = S.sc[0] * range;
+                    const double mean = s1 / s0, var = s2 / s0 - mean * mean;
+                    const double g1 = eps + log(s0 / K) - mean / e, slope = var / (e * e);
                     if (g1 < 0.0) tlo = tt; else thi = tt;
-                    const double mean = S1 / S0, var = S2 / S0 - mean * mean;
-                    const double slope = var / (e * e);
-                    double tn = (slope > 0.0) ? tt - g1 / slope : 0.5 * (tlo + thi);
+                    double tn = slope > 0.0 ? tt - g1 / slope : 0.5 * (tlo + thi);
                     if (!(tn > tlo && tn < thi)) tn = 0.5 * (tlo + thi);
-                    const bool near = fabs(tn - tt) <= 1e-6 * (1.0 + fabs(tt)) || thi - tlo <= 1e-6 * (1.0 + fabs(tt));
-                    tt = tn;
-                    s_sc[0] = exp(tt); s_sc[1] = 1.0 / s_sc[0]; s_sc[2] = tt;
-                    s_sc[3] = last ? 1.0 : (near || it == 199 ? 2.0 : 0.0);
+                    const double tol = 1.0 + fabs(tt);
+                    S.sc[3] = (fabs(tn - tt) <= 1e-7 * tol || thi - tlo <= 1e-13 * tol) ? 1.0 : 0.0;
+                    S.sc[2] = tn;
                 }
                 __syncthreads();
-                const bool done = s_sc[3] == 1.0;
-                __syncthreads();
-                if (done) break;
+                tt = S.sc[2];
+                if (S.sc[3] != 0.0) break;
             }
-            eta = s_sc[0];
+            __syncthreads();
+            if (t == 0) S.sc[0] = exp(tt) * range;
+            __syncthreads();
+            eta = S.sc[0];
         }
     }
-    if (t == 0) {   // for the weights (grid) and the CDF
-        a.misc[M_U] = eta;
-        a.misc[M_CMIN] = cmin;
-        a.misc[M_NFIN] = K;
-        a.misc[M_ISTAR] = (double)istar;
-        *a.argmin_state = istar;
-        if (a.argmin_out) *a.argmin_out = istar;
-    }
-}
 
-// One thread per environment: its weight (FP64), into elite_w.
-__global__ void soft_w_kernel(const OptArgs a) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.N) return;
-    const double eta = a.misc[M_U], cmin = a.misc[M_CMIN], K = a.misc[M_NFIN];
-    const double c = a.c_mean[i];
-    double w;
-    if (K == 0.0) w = 1.0;
-    else if (!isfinite(c)) w = 0.0;
-    else if (a.kind == 1) w = exp(-a.wrs_lambda * (c - cmin));
-    else if (isinf(eta)) w = 1.0;
-    else if (eta == 0.0) w = (c == cmin) ? 1.0 : 0.0;
-    else w = exp((cmin - c) / eta);
-    a.elite_w[i] = w;
-}
-
-// One CTA: the inclusive CDF of the weights in index order (chunks of kSoft,
-// carried), in place, and the total (misc[M_WSUM]).
-__global__ void __launch_bounds__(kSoft) soft_cdf_kernel(const OptArgs a) {
-    __shared__ double red[kSoft / 32][3];
-    const int N = a.N, t = threadIdx.x;
+    // ---- the weights, and their inclusive CDF: chunks of kSoft scanned and carried
+    // within the CTA, then the totals of the CTAs before it added
     double carry = 0.0;
-    const int lane = t & 31, wid = t >> 5;
-    for (int base = 0; base < N; base += kSoft) {
+    for (int base = i0; base < i0 + per; base += kSoft) {
         const int i = base + t;
-        const double w = (i < N) ? a.elite_w[i] : 0.0;
+        double w = 0.0;
+        if (i < i1) {
+            const double c = a.c_mean[i];
+            if (K == 0.0) w = 1.0;
+            else if (!finite_bits(c)) w = 0.0;
+            else if (a.kind == 1) w = exp(-a.wrs_lambda * (c - cmin));
+            else if (isinf(eta)) w = 1.0;
+            else if (eta == 0.0) w = (c == cmin) ? 1.0 : 0.0;
+            else w = exp((cmin - c) / eta);
+        }
         double inc = w;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const double u = __shfl_up_sync(0xffffffffu, inc, o);
             if (lane >= o) inc += u;
         }
-        if (lane == 31) red[wid][0] = inc;
+        __syncthreads();   // (the last chunk's totals have been read)
+        if (lane == 31) S.wpart[wid][0] = inc;
         __syncthreads();
         if (wid == 0) {   // exclusive scan of the warps' totals by the first warp
-            const double v = red[lane][0];
+            const double v = lane < kSoft / 32 ? S.wpart[lane][0] : 0.0;
             double x = v;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
+            for (int o = 1; o < kSoft / 32; o <<= 1) {
                 const double u = __shfl_up_sync(0xffffffffu, x, o);
                 if (lane >= o) x += u;
             }
-            __syncwarp();
-            red[lane][1] = x - v;
-            if (lane == 31) red[0][2] = x;
+            if (lane < kSoft / 32) S.wpart[lane][1] = x - v;
+            if (lane == kSoft / 32 - 1) S.tot[0] = x;
         }
         __syncthreads();
-        if (i < N) a.elite_w[i] = carry + (red[wid][1] + inc);
-        carry += red[0][2];
-        __syncthreads();
+        if (i < i1) a.elite_w[i] = carry + (S.wpart[wid][1] + inc);
+        carry += S.tot[0];
     }
-    if (t == 0) a.misc[M_WSUM] = carry;
+    if (t == 0) S.part[buf][0] = carry;
+    cl.sync();
+    double before = 0.0, total = 0.0;
+    for (int r = 0; r < kSoftCtas; ++r) {
+        const double v = *cl.map_shared_rank(&S.part[buf][0], r);
+        if (r < rank) before += v;
+        total += v;
+    }
+    if (rank > 0)
+        for (int i = i0 + t; i < i1; i += kSoft) a.elite_w[i] += before;
+    if (rank == 0 && t == 0) {
+        a.misc[M_U] = eta;
+        a.misc[M_CMIN] = cmin;
+        a.misc[M_NFIN] = K;
+        a.misc[M_ISTAR] = (double)istar;
+        a.misc[M_WSUM] = total;
+        *a.argmin_state = istar;
+        if (a.argmin_out) *a.argmin_out = istar;
+    }
+    cl.sync();   // no CTA leaves while another reads its shared memory
+}
+
+// The state before the update (one launch instead of a copy per array).
+__global__ void soft_snapshot_kernel(const OptArgs a) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 2 * a.N) return;
+    a.sn_pose[i] = a.pose[i];
+    a.sn_vel[i] = a.vel[i];
+    if (i < a.N) {
+        a.sn_params[i] = a.params[i];
+        a.sn_status[i] = a.status[i];
+    }
+    if (a.qj)
+        for (size_t k = i; k < (size_t)a.N * a.D; k += 2 * (size_t)a.N) {
+            a.sn_qj[k] = a.qj[k];
+            a.sn_qdj[k] = a.qdj[k];
+        }
 }
 
 // Four lanes per environment: lane 0 draws the parent (inverse CDF), every
@@ -969,19 +1023,18 @@ cudaError_t launch_select(const OptArgs &a, cudaStream_t s) {
 
 cudaError_t launch_optimizer(const OptArgs &a, cudaStream_t s) {
     if (a.kind != 0) {   // WRS / REPS: weights, snapshot of the state, draws and exploration
-        const size_t N = a.N;
-        soft_weights_kernel<<<1, kSoft, 0, s>>>(a);
-        soft_w_kernel<<<(a.N + 127) / 128, 128, 0, s>>>(a);
-        soft_cdf_kernel<<<1, kSoft, 0, s>>>(a);
-        cudaError_t e = cudaMemcpyAsync(a.sn_pose, a.pose, 2 * N * sizeof(float4), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(a.sn_vel, a.vel, 2 * N * sizeof(float4), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(a.sn_params, a.params, N * sizeof(float2), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(a.sn_status, a.status, N * sizeof(int), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess && a.qj) {
-            const size_t hb = N * (size_t)a.D * sizeof(float);
-            e = cudaMemcpyAsync(a.sn_qj, a.qj, hb, cudaMemcpyDeviceToDevice, s);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(a.sn_qdj, a.qdj, hb, cudaMemcpyDeviceToDevice, s);
-        }
+        soft_snapshot_kernel<<<(2 * a.N + 255) / 256, 256, 0, s>>>(a);
+        cudaLaunchConfig_t c = {};
+        c.gridDim = dim3(kSoftCtas);
+        c.blockDim = dim3(kSoft);
+        c.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = kSoftCtas;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        c.attrs = at;
+        c.numAttrs = 1;
+        cudaError_t e = cudaLaunchKernelEx(&c, soft_weights_kernel, a);
         if (e != cudaSuccess) return e;
         soft_apply_kernel<<<opt_blocks(a.N), kOptBlock * kApplyLanes, 0, s>>>(a);
         return cudaGetLastError();
