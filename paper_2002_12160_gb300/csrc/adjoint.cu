@@ -21,11 +21,12 @@
 // Contact membership (gap < margin), the capsule's end clamps, the palm's face
 // or clamp pattern and the bias regimes are held fixed.
 //
-// Work layout: a group of GW warps (32 GW threads) per environment. The
-// group enumerates the contacts together, in the step's order; thread
-// k % (32 GW) then owns contact k for the setup, the Jacobi iterations and
-// their reverse -- its first PL contacts in registers, the further ones in the
-// environment's scratch memory -- and the group sums impulses and derivatives
+// Work layout: a block of GW warps (32 GW threads; 4 or 1) per environment. The
+// block enumerates the contacts together, in the step's order (a thread tests the
+// eight spheres of a (link, cluster) pair that survived the cull); thread k % (32 GW)
+// then owns contact k for the setup, the Jacobi iterations and their reverse --
+// 128 contacts of a block in registers and shared memory, the further ones in the
+// environment's scratch memory -- and the block sums impulses and derivatives
 // by warp shuffles and a shared-memory exchange between its warps. The state
 // at every K-th frame is kept (checkpoints). The reverse sweep walks the
 // segments between checkpoints backwards: it recomputes the segment's
@@ -38,37 +39,72 @@
 // last segment's tape is recorded by the first pass itself.) Checkpoints,
 // segment states and the tape live in a slice of a scratch buffer owned by
 // the handle, one slice per environment.
+//
+// What bounds it: an iteration and its reverse are one chain of dependent
+// arithmetic and shuffles per environment (two or fewer warps a scheduler at 255
+// registers), and where many environments run, also the instruction fetch, since
+// every warp is somewhere else in the code. Hence: two contacts of a lane packed
+// in FP32 pairs (half the instructions); one loop per number of occupied slots,
+// each body one straight stretch of code (predicated stores and copies instead of
+// branches), so that the scheduler overlaps the chains: an iteration of the reverse
+// 1100 -> 650 cycles for four warps with a contact a thread; the tape read by
+// asynchronous copies three iterations ahead; everything off those loops rolled.
+// Against one thread per pair, scalar slots with a branch each, and tape loads in the
+// iteration that needs them, at the public call: 1024 cylinders, 30 frames, three
+// segments 5.28 -> 4.28 ms; 102 cylinders, 10 frames, 552 -> 455 us; 64 boxes, 5 frames
+// (bound by the host), the kernel 258 -> 200 us.
 #include "contact.cuh"
 #include "internal.cuh"
 
 namespace ih {
 namespace {
 
-constexpr int kAW = 4;   // warps per CTA
-constexpr int kABlock = 32 * kAW;
 constexpr unsigned kFull = 0xffffffffu;
+constexpr int kRC = 128;   // contacts of a block held in registers and shared memory
+// Iterations of the tape held in shared memory by the reverse sweep, copied there
+// asynchronously three iterations ahead. (Requested into registers an iteration
+// ahead, the rotation of the registers waited for the loads: 990 cycles an
+// iteration for four warps with a contact a thread.)
+constexpr int kRing = 4;
+// (bytes: 16, or 0 to fill with zeros; skipped without a branch unless `on`)
+__device__ __forceinline__ void copy_async(float4 *dst, const float4 *src, int bytes, bool on = true) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.s32 p, %3, 0;\n@p cp.async.ca.shared.global [%0], [%1], 16, %2;\n}" ::"r"(
+            (unsigned)__cvta_generic_to_shared(dst)),
+        "l"(src), "r"(bytes), "r"((int)on)
+        : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// a store without a branch (`on` varies by lane), so that a loop's body stays one
+// stretch of code for the scheduler
+__device__ __forceinline__ void store_if(bool on, float4 *dst, float4 v) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.s32 p, %5, 0;\n@p st.global.v4.f32 [%0], {%1, %2, %3, %4};\n}" ::"l"(dst), "f"(v.x),
+                 "f"(v.y), "f"(v.z), "f"(v.w), "r"((int)on)
+                 : "memory");
+}
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// The GW warps of one environment: group thread gt, lane, warp within the
-// group, group within the block; sync() is the group's barrier.
+// The GW warps of one environment (a block): thread gt, lane, warp; sync() is the
+// block's barrier.
 template <int GW>
 struct AGroup {
     static constexpr int T = 32 * GW;
-    int gt, lane, wg, gid;
+    int gt, lane, wg;
     __device__ AGroup() {
-        gt = threadIdx.x % T;
+        gt = threadIdx.x;
         lane = threadIdx.x & 31;
         wg = gt >> 5;
-        gid = threadIdx.x / T;
     }
     __device__ __forceinline__ void sync() const {
-        if constexpr (GW == 1) {
-            __syncwarp();
-        } else if constexpr (T == kABlock) {
-            __syncthreads();
-        } else {
-            asm volatile("bar.sync %0, %1;" ::"r"(gid + 1), "r"(T) : "memory");
-        }
+        if constexpr (GW == 1) __syncwarp();
+        else __syncthreads();
     }
+};
+
+template <bool V>
+struct Flag {
+    static constexpr bool value = V;
 };
 
 struct Body {
@@ -108,99 +144,88 @@ __device__ __forceinline__ S6 world_inv_inertia_f(const M3 &R, const S6 &J, floa
                    __fmaf_rn(J.zz, r0.z, prod_add(J.xz, r0.x, J.yz, r0.y))};   // (first and second row)
     return sandwich(r0, r1, r2, a0, smul(J, r1), smul(J, r2), inv_m);
 }
-// The reverse sweep's products, their contraction left to the compiler
-__device__ __forceinline__ V3 cross_r(V3 a, V3 b) {
-    return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
-}
-__device__ __forceinline__ V3 smul_r(const S6 &A, V3 v) {
-    return {A.xx * v.x + A.xy * v.y + A.xz * v.z,
-            A.xy * v.x + A.yy * v.y + A.yz * v.z,
-            A.xz * v.x + A.yz * v.y + A.zz * v.z};
-}
-__device__ __forceinline__ Q4 qmul_r(Q4 a, Q4 b) {
-    return {a.w * b.w - a.x * b.x - a.y * b.y - a.z * b.z,
-            a.w * b.x + a.x * b.w + a.y * b.z - a.z * b.y,
-            a.w * b.y - a.x * b.z + a.y * b.w + a.z * b.x,
-            a.w * b.z + a.x * b.y - a.y * b.x + a.z * b.w};
-}
-__device__ __forceinline__ S6 world_inv_inertia_r(const M3 &R, const S6 &J, float inv_m) {
-    const V3 r0 = {R.c0.x, R.c1.x, R.c2.x}, r1 = {R.c0.y, R.c1.y, R.c2.y}, r2 = {R.c0.z, R.c1.z, R.c2.z};
-    return sandwich(r0, r1, r2, smul_r(J, r0), smul_r(J, r1), smul_r(J, r2), inv_m);
-}
-
+struct Centres {
+    float4 sph[IH_MAX_SPHERES / kCluster * kSphStride];   // the substep's sphere centres (world rotation, relative to x), radius
+    float4 clc[IH_MAX_SPHERES / kCluster];   // cluster centres (likewise), enclosing radius
+    unsigned short clp[kMaxLinks * (IH_MAX_SPHERES / kCluster)];   // surviving (link << 8 | cluster) pairs
+};
 template <int GW>
 struct alignas(16) GroupSm {
-    // contacts whose record (besides the slot's global one, which the tape
-    // keeps) the forward substep also holds here: the register slots' and more
-    static constexpr int kRC = GW == 1 ? 64 : 128;
-    float4 crec[kRC][2];           // (r, gap), (n, link | pad << 8 as int bits)
-    float4 clam[kRC];              // the pass's final impulses of the register slots (pad sums)
-    float4 sph[IH_MAX_SPHERES];    // the substep's sphere centres (world rotation, relative to x), radius
-    float4 clc[IH_MAX_SPHERES / kCluster];   // cluster centres (likewise), enclosing radius
+    // GW = 1: the constants of the lane's contacts lane + 32 k (k < 4), slots 2 p
+    // and 2 p + 1 interleaved so that a float4 holds two pairs: r, n, c, 1/k_n, 1/k_t
+    float4 cp[GW == 1 ? 2 : 1][6][32];
+    float4 clam[kRC];              // the pass's final impulses (pad sums)
+    float4 meta[kRC];              // reverse: the contacts' gap, link | pad << 8 and sphere
+    union {                        // (a substep's enumeration and a reverse sweep never overlap)
+        float4 ring[kRing][kRC];   // reverse: the impulses after iterations it & (kRing - 1), on their way from the tape
+        Centres en;                // forward: the enumeration's centres and pairs
+    };
+    float4 rsum[GW][kRing][2];     // ... and their sums, a copy per warp
+    float4 xa[kMaxLinks], ax[kMaxLinks];     // x - link origin, link axis
     double term[IH_MAX_PADS];      // a frame's FP64 force term of each pad
     float padacc[IH_MAX_PADS * 3];
     float fbar[IH_MAX_PADS * 3];   // dL/dF_p / (h ns): minus the derivative w.r.t. a final impulse
-    float red[2][GW][8];           // partial sums of the group's warps (double-buffered)
+    float4 red[2][GW][2];          // partial sums of the block's warps (double-buffered)
+    float fin[16];                 // results of the contacts' warps for the others
     int cnt[2][GW];                // hits of each warp in a compaction round (double-buffered)
     int flag[IH_MAX_PADS];         // a frame's contact-state mismatch of each pad
-    unsigned short lbeg[32], lend[32];
-    unsigned short clp[32 * (IH_MAX_SPHERES / kCluster)];   // surviving (link index << 8 | cluster) pairs
-    unsigned char links[32];       // surviving links in order
-    unsigned surv;
+    unsigned short lbeg[kMaxLinks], lend[kMaxLinks];   // contact range of each link
+    unsigned short clist[IH_MAX_CONTACTS];   // the contacts in order (link << 8 | sphere)
+    unsigned char cpad[IH_MAX_CONTACTS];     // their pads
 };
 
-// Block-wide pad tables: the pads of each link (in pad order) and their intervals.
-constexpr int kAPadsPerLink = 4;
-struct PadTab {
-    unsigned char cnt[32];
-    unsigned char id[32 * kAPadsPerLink];
-    float s0[IH_MAX_PADS], s1[IH_MAX_PADS];
-};
-
-// Positions of the group's hits in a round of order-preserving compaction:
-// `hit` of this thread; returns its slot (base + hits of the threads before
-// it in the group) and adds the round's hits to `base`.
-template <int GW>
-__device__ __forceinline__ int gcompact(bool hit, int &base, const AGroup<GW> &G, GroupSm<GW> &S, int &parity) {
-    const unsigned bal = __ballot_sync(kFull, hit);
-    int off = base + __popc(bal & ((1u << G.lane) - 1u));
-    if constexpr (GW == 1) {
-        base += __popc(bal);
-    } else {
+// Sum of `mine` (0..15) over the block's threads before this one (returned, plus
+// base) and over all of them (added to base): the slots of an order-preserving
+// compaction, by bit planes of the warps' ballots.
+template <int GW, int BITS>
+__device__ __forceinline__ int gcompact(int mine, int &base, const AGroup<GW> &G, GroupSm<GW> &S, int &parity) {
+    int off = base, tot = 0;
+#pragma unroll
+    for (int b = 0; b < BITS; ++b) {
+        const unsigned bal = __ballot_sync(kFull, (mine >> b) & 1);
+        off += __popc(bal & ((1u << G.lane) - 1u)) << b;
+        tot += __popc(bal) << b;
+    }
+    if constexpr (GW > 1) {
         int *c = S.cnt[parity];
-        if (G.lane == 0) c[G.wg] = __popc(bal);
+        if (G.lane == 0) c[G.wg] = tot;
         G.sync();
-        int tot = 0;
+        tot = 0;
 #pragma unroll
         for (int w = 0; w < GW; ++w) {
             const int k = c[w];
             if (w < G.wg) off += k;
             tot += k;
         }
-        base += tot;
         parity ^= 1;
     }
+    base += tot;
     return off;
 }
 
-// Sum of 6 values over the group's threads, every thread receiving the sums:
-// within each warp by shuffles, then the warps' partials in warp order.
+// Sum of 6 values over the first aw warps of the block, every one of their threads
+// receiving the sums: within each warp by shuffles, then the warps' partials in
+// warp order.
 template <int GW>
-__device__ __forceinline__ void gsum6(float (&v)[6], const AGroup<GW> &G, GroupSm<GW> &S, int &parity) {
+__device__ __forceinline__ void gsum6(float (&v)[6], const AGroup<GW> &G, GroupSm<GW> &S, int &parity, int aw = GW) {
     if constexpr (GW == 1) {
         width_sum6<32>(v, kFull, G.lane);
     } else {
         const float c = width_scatter6<32>(v, kFull, G.lane);
-        float *r = &S.red[parity][0][0];
+        float *r = reinterpret_cast<float *>(&S.red[parity][0][0]);
         const int k = G.lane >> 2;
         if ((G.lane & 3) == 0 && k < 6) r[G.wg * 8 + k] = c;
-        G.sync();
+        asm volatile("bar.sync 1, %0;" ::"r"(32 * aw) : "memory");
+        const float4 *r4 = reinterpret_cast<const float4 *>(r);
+        float4 lo = r4[0], hi = r4[1];
 #pragma unroll
-        for (int q = 0; q < 6; ++q) v[q] = r[q];
-#pragma unroll
-        for (int w = 1; w < GW; ++w)
-#pragma unroll
-            for (int q = 0; q < 6; ++q) v[q] += r[w * 8 + q];
+        for (int w = 1; w < GW; ++w) {
+            const float4 l = r4[2 * w], u = r4[2 * w + 1];
+            const bool on = w < aw;   // (the others' places hold old sums)
+            lo.x += on ? l.x : 0.0f; lo.y += on ? l.y : 0.0f; lo.z += on ? l.z : 0.0f; lo.w += on ? l.w : 0.0f;
+            hi.x += on ? u.x : 0.0f; hi.y += on ? u.y : 0.0f;
+        }
+        v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w; v[4] = hi.x; v[5] = hi.y;
         parity ^= 1;
     }
 }
@@ -264,13 +289,76 @@ struct SlotPtr {
 // Per-environment constants.
 struct Env {
     int sfirst, NS, iters, cfirst;
-    float mu, inv_m, bound;
+    float mu, inv_m;
     S6 Jb;
 };
 
 // contact record: [0] (r, gap) [1] (n, 1/k_n) [2] (c, 1/k_t) [3] (t, link | pad << 8, sphere, -)
-__device__ __forceinline__ int rec_link(float4 r3) { return __float_as_int(r3.y) & 0xff; }
-__device__ __forceinline__ int rec_pad(float4 r3) { return (__float_as_int(r3.y) >> 8) & 0xff; }
+__device__ __forceinline__ int rec_pad(float4 r3) { return (__float_as_int(r3.y) >> 8) & 0xff; }   // (of GroupSm::meta too)
+
+// A pair's constants in shared memory (GroupSm::cp): value v of r, n, c, 1/k_n,
+// 1/k_t (0..10) of slots 2 p and 2 p + 1
+template <int GW>
+__device__ __forceinline__ void cp_store(GroupSm<GW> &S, int slot, int lane, V3 r, V3 n, V3 c, float ikn, float ikt) {
+    const float v[11] = {r.x, r.y, r.z, n.x, n.y, n.z, c.x, c.y, c.z, ikn, ikt};
+#pragma unroll
+    for (int q = 0; q < 11; ++q)
+        reinterpret_cast<float *>(&S.cp[GW == 1 ? slot >> 1 : 0][q >> 1][lane])[(q & 1) * 2 + (slot & 1)] = v[q];
+}
+template <int GW>
+__device__ __forceinline__ void cp_load(const GroupSm<GW> &S, int slot, int lane, Contact<F2> &c) {
+    const float4 *p = &S.cp[GW == 1 ? slot >> 1 : 0][0][lane];
+    const float4 a = p[0], b = p[32], d = p[64], e = p[96], f = p[128], g = p[160];
+    c.r = {{a.x, a.y}, {a.z, a.w}, {b.x, b.y}};
+    c.n = {{b.z, b.w}, {d.x, d.y}, {d.z, d.w}};
+    c.c = {{e.x, e.y}, {e.z, e.w}, {f.x, f.y}};
+    c.ikn = {f.z, f.w};
+    c.ikt = {g.x, g.y};
+}
+template <int GW>
+__device__ __forceinline__ void cp_load(const GroupSm<GW> &S, int slot, int lane, Contact<float> &c) {   // slot even
+    Contact<F2> t;
+    cp_load(S, slot, lane, t);
+    c.r = {t.r.x.x, t.r.y.x, t.r.z.x};
+    c.n = {t.n.x.x, t.n.y.x, t.n.z.x};
+    c.c = {t.c.x.x, t.c.y.x, t.c.z.x};
+    c.ikn = t.ikn.x;
+    c.ikt = t.ikt.x;
+}
+// The constants of the block's first kRC contacts from their records: to shared
+// memory (GW = 1, every load requested before the first is used; empty slots to
+// the next whole pair), or to the thread's own contact; with META the rest of the
+// record too
+template <int GW, bool META>
+__device__ __forceinline__ void load_constants(const SlotPtr &sp, GroupSm<GW> &S, const AGroup<GW> &G, int nc, Contact<float> &own) {
+    constexpr int NK = GW == 1 ? 4 : 1;
+    float4 r[NK][4];
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        const int ci = G.gt + AGroup<GW>::T * k;
+        r[k][0] = r[k][2] = r[k][3] = make_float4(0, 0, 0, 0);
+        r[k][1] = make_float4(0, 0, 1, 0);
+        if (ci < nc)
+            for (int q = 0; q < (META ? 4 : 3); ++q) r[k][q] = sp.rec[4 * ci + q];
+    }
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+        const int ci = G.gt + AGroup<GW>::T * k;
+        if (META && ci < nc) S.meta[ci] = make_float4(r[k][0].w, r[k][3].y, r[k][3].z, 0.0f);
+        if constexpr (GW == 1) {
+            if (32 * (k & ~1) < nc) cp_store(S, k, G.lane, xyz(r[k][0]), xyz(r[k][1]), xyz(r[k][2]), r[k][1].w, r[k][2].w);
+        } else {
+            own.r = {r[k][0].x, r[k][0].y, r[k][0].z};
+            own.n = {r[k][1].x, r[k][1].y, r[k][1].z};
+            own.c = {r[k][2].x, r[k][2].y, r[k][2].z};
+            own.ikn = r[k][1].w;
+            own.ikt = r[k][2].w;
+        }
+    }
+}
+__device__ __forceinline__ float4 lam4(const Contact<float> &c) { return make_float4(c.lam.x, c.lam.y, c.lam.z, 0.0f); }
+__device__ __forceinline__ float4 lam4a(const Contact<F2> &c) { return make_float4(c.lam.x.x, c.lam.y.x, c.lam.z.x, 0.0f); }
+__device__ __forceinline__ float4 lam4b(const Contact<F2> &c) { return make_float4(c.lam.x.y, c.lam.y.y, c.lam.z.y, 0.0f); }
 
 // One substep of one environment (the arithmetic of step_kernel.cuh, contacts in the
 // same order: link, then sphere), its contact records written at sp.rec.
@@ -280,18 +368,14 @@ __device__ __forceinline__ int rec_pad(float4 r3) { return (__float_as_int(r3.y)
 // at sp.rec are those of an earlier run from the same state (replay_nc
 // contacts, setup included), which replaces the enumeration and the setup.
 // Returns the contact count (0 on overflow). Not inlined, with the flags as
-// arguments: every pass (cost, recomputation, tape) then runs the same
-// compiled arithmetic, so a recorded tape is bit for bit the forward's.
-template <int GW, int PL>
+// arguments: one copy serves every pass. (The iterations' arithmetic has a fixed
+// contraction, contact.cuh, so a recorded tape is bit for bit the forward's.)
+template <int GW>
 __device__ __noinline__ int fwd_substep(const AdjArgs &a, const Env &E_, Body &b, const float4 *L0,
-                                        const float4 *L1, const SlotPtr &sp_, GroupSm<GW> &S, const PadTab &PT,
+                                        const float4 *L1, const SlotPtr &sp_, GroupSm<GW> &S, const PadTable &PT,
                                         const AGroup<GW> &G_, int &parity_, int &st_, int tape_flag,
                                         int pads_flag, int replay_nc) {
-    // the flags are run-time values (the callers combine them with a.zero):
-    // one compiled body serves the cost pass, the recomputation and the tape,
-    // so a recorded tape is bit for bit the forward's
     const bool TAPE = tape_flag != 0, PADS = pads_flag != 0;
-    static_assert(AGroup<GW>::T * PL <= GroupSm<GW>::kRC, "the register slots' records are in shared memory");
     // by-value copies of what the loops read: through the references every
     // store to the tape or to shared memory could alias them and force reloads
     const Env E = E_;
@@ -308,210 +392,296 @@ __device__ __noinline__ int fwd_substep(const AdjArgs &a, const Env &E_, Body &b
     const V3 w_pred = b.w;
     const M3 R = qmat(b.q);
     const S6 Wi = world_inv_inertia_f(R, E.Jb, E.inv_m);
-    const int lane = G.lane;
+    const int lane = G.lane, gt = G.gt;
 
-    const int gt = G.gt;
     int nc = 0;
     const bool replay = replay_nc >= 0;
     if (replay) {
         // the records this substep's first run left, setup included: no
         // enumeration (the run is deterministic, so they are its own)
         nc = replay_nc;
-        for (int ci = gt; ci < nc && ci < GroupSm<GW>::kRC; ci += T) {
-            const float4 *rc = sp.rec + 4 * ci;
-            const float4 r0 = rc[0], r1 = rc[1], r3 = rc[3];
-            S.crec[ci][0] = r0;
-            S.crec[ci][1] = make_float4(r1.x, r1.y, r1.z, r3.y);
-        }
-        for (int l = gt; l < 32; l += T) {
-            S.lbeg[l] = 0;
-            S.lend[l] = 0;
-        }
-        G.sync();
     } else {
-        // contact enumeration by the whole group, in the step's order (link,
-        // then sphere): sphere and cluster centres to world, the link cull, the
-        // (link, cluster) cull by the clusters' enclosing spheres, then the
-        // spheres of the surviving pairs, one test per thread per round,
-        // compacted in order
+        // contact enumeration, in the step's order (link, then sphere): sphere and
+        // cluster centres to world, the (link, cluster) cull by the clusters' enclosing
+        // spheres, then a thread tests the eight spheres of a surviving pair
         const int ncl = (E.NS + kCluster - 1) / kCluster;
-        for (int j = gt; j < E.NS; j += T) {
-            const float4 s4 = __ldg(sc.spheres + E.sfirst + j);
-            const V3 cr = mmul(R, xyz(s4));
-            S.sph[j] = make_float4(cr.x, cr.y, cr.z, s4.w);
+        const float inv_ncl = 1.0f / (float)ncl;
+        G.sync();   // (a reverse sweep may just have read the ring in the centres' place)
+#pragma unroll 1
+        for (int j = gt; j < ncl * kCluster; j += T) {
+            float4 o = make_float4(1e18f, 1e18f, 1e18f, 0.0f);   // (padding of the last cluster: far away)
+            if (j < E.NS) {
+                const float4 s4 = __ldg(sc.spheres + E.sfirst + j);
+                const V3 cr = mmul(R, xyz(s4));
+                o = make_float4(cr.x, cr.y, cr.z, s4.w);
+            }
+            S.en.sph[(j >> 3) * kSphStride + (j & 7)] = o;
         }
+#pragma unroll 1
         for (int k = gt; k < ncl; k += T) {
             const float4 cl = __ldg(sc.clusters + E.cfirst + k);
             const V3 cr = mmul(R, xyz(cl));
-            S.clc[k] = make_float4(cr.x, cr.y, cr.z, cl.w);
+            S.en.clc[k] = make_float4(cr.x, cr.y, cr.z, cl.w);
         }
-        if (G.wg == 0) {
-            const bool keep = lane < Lk && link_reaches(sc, cfg, L0, lane, b.x, E.bound);
-            const unsigned surv = __ballot_sync(kFull, keep);
-            if (keep) S.links[__popc(surv & ((1u << lane) - 1u))] = (unsigned char)lane;
-            if (lane == 0) S.surv = surv;
-        }
-        for (int l = gt; l < 32; l += T) {
+#pragma unroll 1
+        for (int l = gt; l < Lk; l += T) {
+            const V3 xa = b.x - xyz(__ldg(L0 + l * kLinkStride));
+            S.xa[l] = make_float4(xa.x, xa.y, xa.z, 0.0f);
+            S.ax[l] = __ldg(L0 + l * kLinkStride + 1);
             S.lbeg[l] = 0;
             S.lend[l] = 0;
         }
         G.sync();
-        const int ncp = __popc(S.surv) * ncl;
+        const int ncp = Lk * ncl;
         int nclp = 0;
+#pragma unroll 1
         for (int p0 = 0; p0 < ncp; p0 += T) {
             const int p = p0 + gt;
             bool keep = false;
-            int li = 0, k = 0;
+            int e = 0;
             if (p < ncp) {
-                li = p / ncl;
-                k = p - li * ncl;
-                const float4 cc = S.clc[k];
-                keep = link_reaches(sc, cfg, L0, S.links[li], b.x + xyz(cc), cc.w);
+                const int l = min((int)(((float)p + 0.5f) * inv_ncl), Lk - 1), k = p - l * ncl;
+                const float4 cc = S.en.clc[k];
+                keep = cluster_reaches(sc, cfg, l, xyz(S.xa[l]) + xyz(cc), cc.w, xyz(S.ax[l]));
+                e = (l << 8) | k;
             }
-            const int off = gcompact<GW>(keep, nclp, G, S, parity);
-            if (keep) S.clp[off] = (unsigned short)((li << 8) | k);
+            const int off = gcompact<GW, 1>(keep, nclp, G, S, parity);
+            if (keep) S.en.clp[off] = (unsigned short)e;
         }
         G.sync();
-        const int npairs = nclp * kCluster;
-        for (int p0 = 0; p0 < npairs; p0 += T) {
-            const int p = p0 + gt;
-            bool hit = false;
-            Hit hh = {0.0f, mk(0, 0, 1), 0.0f};
-            V3 r = mk(0, 0, 0);
-            int l = 0, j = 0;
-            if (p < npairs) {
-                const int e = S.clp[p / kCluster];
-                j = (e & 0xff) * kCluster + (p % kCluster);
-                l = S.links[e >> 8];
-                if (j < E.NS) {   // (j >= NS: padding of the shape's last cluster)
-                    const float4 s4 = S.sph[j];
-                    const V3 cr = xyz(s4);
-                    const float4 A0 = __ldg(L0 + l * kLinkStride);
-                    const float4 Aq = __ldg(L0 + l * kLinkStride + 2);
-                    const Q4 lq = {Aq.x, Aq.y, Aq.z, Aq.w};
-                    if (l == 0) {
-                        hh = hit_box(b.x + cr, s4.w, xyz(A0), lq, sc.palm_hx, sc.palm_hy, sc.palm_hz);
-                    } else {
-                        const V3 ld = xyz(__ldg(L0 + l * kLinkStride + 1));
-                        hh = hit_capsule((b.x - xyz(A0)) + cr, s4.w, ld, sc.link_len, inv_L, sc.link_rad, lq);
-                    }
-                    r = cr - hh.n * s4.w;
-                    hit = hh.gap < cfg.margin;
-                }
+#pragma unroll 1
+        for (int e0 = 0; e0 < nclp; e0 += T) {
+            unsigned hits = 0;
+            int e = 0;
+            if (e0 + gt < nclp) {
+                e = S.en.clp[e0 + gt];
+                const int l = e >> 8, k = e & 0xff;
+                hits = cluster_hits(sc, cfg, l, k, xyz(S.xa[l]), xyz(S.ax[l]), S.en.sph + k * kSphStride, E.NS, inv_L);
             }
-            const int idx = gcompact<GW>(hit, nc, G, S, parity);
-            if (hit && idx < cap) {
-                int pad = -1;   // the first pad of the link whose interval holds t
-                const int npl = PT.cnt[l];
-                for (int k = 0; k < npl; ++k) {
-                    const int pp = PT.id[l * kAPadsPerLink + k];
-                    if (l == 0) { pad = pp; break; }
-                    const float s0 = PT.s0[pp], s1 = PT.s1[pp];
-                    if (hh.t >= s0 && (hh.t < s1 || s1 >= 1.0f)) { pad = pp; break; }
-                }
-                float4 *rc = sp.rec + 4 * idx;
-                const float4 a0 = make_float4(r.x, r.y, r.z, hh.gap);
-                const float lp = __int_as_float(l | ((pad & 0xff) << 8));
-                rc[0] = a0;
-                rc[1] = make_float4(hh.n.x, hh.n.y, hh.n.z, 0.0f);
-                rc[3] = make_float4(hh.t, lp, __int_as_float(j), 0.0f);
-                if (idx < GroupSm<GW>::kRC) {
-                    S.crec[idx][0] = a0;
-                    S.crec[idx][1] = make_float4(hh.n.x, hh.n.y, hh.n.z, lp);
-                }
+            const int idx = gcompact<GW, 4>(__popc(hits), nc, G, S, parity);
+            const int cj = (e & 0xff00) | ((e & 0xff) * kCluster);
+#pragma unroll
+            for (int i = 0; i < kCluster; ++i) {
+                const int at = idx + __popc(hits & ((1u << i) - 1u));
+                if (((hits >> i) & 1u) && at < cap) S.clist[at] = (unsigned short)(cj + i);
             }
         }
-        G.sync();   // the records are written
+        G.sync();
         if (nc > cap) {   // more contacts than the per-env capacity: as the step, no contacts
             st |= IH_ENV_OVERFLOW;
             nc = 0;
         }
     }
-    // each link's contact range (the contacts are in link order)
-    constexpr int RC = GroupSm<GW>::kRC;
-    auto link_of = [&](int c) -> int {
-        return c < RC ? (__float_as_int(S.crec[c][1].w) & 0xff) : rec_link(sp.rec[4 * c + 3]);
-    };
-    for (int ci = gt; ci < nc; ci += T) {
-        const int l = link_of(ci);
-        if (ci == 0 || link_of(ci - 1) != l) S.lbeg[l] = (unsigned short)ci;
-        if (ci == nc - 1 || link_of(ci + 1) != l) S.lend[l] = (unsigned short)(ci + 1);
+
+    // contact setup by the contact's thread (or its results from the records); a
+    // block of four warps keeps its one contact a thread in registers
+    const float trW = Wi.xx + Wi.yy + Wi.zz;
+    Contact<float> own;
+    own.clear();
+    if (replay) {
+        load_constants<GW, false>(sp, S, G, nc, own);
+#pragma unroll 1
+        for (int ci = kRC + gt; ci < nc; ci += T) sp.lamf[ci] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    } else {
+        if (GW == 1)   // empty slots up to the next whole pair of slots
+#pragma unroll 1
+            for (int k = nc >> 5; k < 4 && k <= ((nc - 1) >> 5 | 1); ++k)
+                if (lane + 32 * k >= nc) cp_store(S, k, lane, mk(0, 0, 0), mk(0, 0, 1), mk(0, 0, 0), 0.0f, 0.0f);
+#pragma unroll 1
+        for (int ci = gt; ci < nc; ci += T) {
+            float4 *rc = sp.rec + 4 * ci;
+            const int e = S.clist[ci], l = e >> 8, j = e & 0xff;
+            const int e0 = ci > 0 ? S.clist[ci - 1] >> 8 : -1, e1 = ci < nc - 1 ? S.clist[ci + 1] >> 8 : -1;
+            if (e0 != l) S.lbeg[l] = (unsigned short)ci;
+            if (e1 != l) S.lend[l] = (unsigned short)(ci + 1);
+            const float4 s4 = S.en.sph[(j >> 3) * kSphStride + (j & 7)];
+            const V3 cr = xyz(s4);
+            const Hit hh = hit_link(sc, l, xyz(S.xa[l]) + cr, s4.w, xyz(S.ax[l]), L0, inv_L);
+            const V3 r = cr - hh.n * s4.w;
+            const unsigned char pad = PT.find(l, hh.t);
+            S.cpad[ci] = pad;
+            const CSetup cs = setup_contact(r, hh.n, hh.gap, l, Wi, trW, E.inv_m, cfg, L0, L1, b.x, inv_h);
+            rc[0] = make_float4(r.x, r.y, r.z, hh.gap);
+            rc[1] = make_float4(hh.n.x, hh.n.y, hh.n.z, cs.ikn);
+            rc[2] = make_float4(cs.cc.x, cs.cc.y, cs.cc.z, cs.ikt);
+            rc[3] = make_float4(hh.t, __int_as_float(l | (pad << 8)), __int_as_float(j), 0.0f);
+            if (ci >= kRC) {
+                sp.lamf[ci] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // a further contact: its impulse in memory
+            } else if constexpr (GW == 1) {
+                cp_store(S, ci >> 5, lane, r, hh.n, cs.cc, cs.ikn, cs.ikt);
+            } else {
+                own.r = {r.x, r.y, r.z};
+                own.n = {hh.n.x, hh.n.y, hh.n.z};
+                own.c = {cs.cc.x, cs.cc.y, cs.cc.z};
+                own.ikn = cs.ikn;
+                own.ikt = cs.ikt;
+            }
+        }
     }
     G.sync();
 
-    // contact setup, by the thread that owns the contact from here on; the
-    // constants stay in its registers for the iterations
-    const float trW = Wi.xx + Wi.yy + Wi.zz;
-    V3 lam_[PL], cr_[PL], cn_[PL], cc_[PL];
-    float ikn_[PL], ikt_[PL];
-#pragma unroll
-    for (int k = 0; k < PL; ++k) {
-        lam_[k] = mk(0, 0, 0);
-        cr_[k] = mk(0, 0, 0); cn_[k] = mk(0, 0, 1); cc_[k] = mk(0, 0, 0);
-        ikn_[k] = ikt_[k] = 0.0f;
-        const int ci = G.gt + T * k;
-        if (ci < nc && replay) {   // the setup's results are in the records
-            const float4 *rc = sp.rec + 4 * ci;
-            const float4 r0 = rc[0], r1 = rc[1], r2 = rc[2];
-            cr_[k] = xyz(r0); cn_[k] = xyz(r1); cc_[k] = xyz(r2); ikn_[k] = r1.w; ikt_[k] = r2.w;
-        } else if (ci < nc) {   // (a register slot's record is in shared memory: T PL <= kRC)
-            float4 *rc = sp.rec + 4 * ci;
-            const float4 r0 = S.crec[ci][0], r1 = S.crec[ci][1];
-            const CSetup cs = setup_contact(xyz(r0), xyz(r1), r0.w, __float_as_int(r1.w) & 0xff, Wi, trW, E.inv_m, cfg,
-                                            L0, L1, b.x, inv_h);
-            rc[1] = make_float4(r1.x, r1.y, r1.z, cs.ikn);
-            rc[2] = make_float4(cs.cc.x, cs.cc.y, cs.cc.z, cs.ikt);
-            cr_[k] = xyz(r0); cn_[k] = xyz(r1); cc_[k] = cs.cc; ikn_[k] = cs.ikn; ikt_[k] = cs.ikt;
-        }
-    }
-    // contacts past the register slots (thread gt's slots PL, PL + 1, ... in
-    // the same order): constants in their records, impulse in sp.lamf
-    for (int ci = G.gt + T * PL; ci < nc; ci += T) {
-        if (!replay) {
-            float4 *rc = sp.rec + 4 * ci;
-            const float4 r0 = rc[0], r1 = rc[1], r3 = rc[3];
-            const CSetup cs = setup_contact(xyz(r0), xyz(r1), r0.w, rec_link(r3), Wi, trW, E.inv_m, cfg, L0, L1, b.x,
-                                            inv_h);
-            rc[1] = make_float4(r1.x, r1.y, r1.z, cs.ikn);
-            rc[2] = make_float4(cs.cc.x, cs.cc.y, cs.cc.z, cs.ikt);
-        }
-        sp.lamf[ci] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    }
-
-    // Jacobi projected-impulse iterations
+    // Jacobi projected-impulse iterations, on the warps that hold contacts
     V3 vv = v_pred, ww = w_pred;
     if (nc > 0) {
-        const float inv_nc = 1.0f / (float)nc;
-        for (int it = 0; it < E.iters; ++it) {
-            float acc[6] = {0, 0, 0, 0, 0, 0};
-            // every register slot without a branch, so that the slots' chains
-            // interleave: an empty slot (r = c = 0, n = z, 1/k = 0) keeps a zero
-            // impulse and adds zeros
+        const int aw = GW == 1 ? 1 : min(GW, (nc + 31) >> 5);
+        const float inv_nc = 1.0f / (float)nc, mu_s = 4096.0f * E.mu;
+        auto add1 = [&](float (&acc)[6], const Contact<float> &c) {
+            float s[6];
+            c.wrench(s);
 #pragma unroll
-            for (int k = 0; k < PL; ++k) {
-                const int ci = G.gt + T * k;
-                lam_[k] = update_contact(lam_[k], cr_[k], cn_[k], cc_[k], ikn_[k], ikt_[k], vv, ww, E.mu, inv_nc);
-                const V3 tq = cross(cr_[k], lam_[k]);
-                acc[0] += lam_[k].x; acc[1] += lam_[k].y; acc[2] += lam_[k].z;
-                acc[3] += tq.x; acc[4] += tq.y; acc[5] += tq.z;
-                if (TAPE && ci < nc) sp.lamh[(size_t)it * cap + ci] = make_float4(lam_[k].x, lam_[k].y, lam_[k].z, 0.0f);
-            }
-            for (int ci = G.gt + T * PL; ci < nc; ci += T) {
+            for (int q = 0; q < 6; ++q) acc[q] += s[q];
+        };
+        auto add2 = [&](float (&acc)[6], const Contact<F2> &c) {
+            F2 s[6];
+            c.wrench(s);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) acc[q] = (acc[q] + s[q].x) + s[q].y;
+        };
+        // the impulse of register slot k after iteration it, to the tape
+        auto tape = [&](int it, int k, float4 lam) {
+            const int ci = gt + T * k;
+            store_if(TAPE && ci < nc, sp.lamh + (size_t)it * cap + ci, lam);
+        };
+        auto further = [&](int it, float (&acc)[6]) {   // contacts kRC, ... in the same per-thread order
+#pragma unroll 1
+            for (int ci = kRC + gt; ci < nc; ci += T) {
                 const float4 *rc = sp.rec + 4 * ci;
-                const float4 r0 = rc[0], r1 = rc[1], r2 = rc[2];
-                const V3 lam = update_contact(xyz(sp.lamf[ci]), xyz(r0), xyz(r1), xyz(r2), r1.w, r2.w, vv, ww, E.mu,
-                                              inv_nc);
-                sp.lamf[ci] = make_float4(lam.x, lam.y, lam.z, 0.0f);
-                const V3 tq = cross(xyz(r0), lam);
-                acc[0] += lam.x; acc[1] += lam.y; acc[2] += lam.z;
-                acc[3] += tq.x; acc[4] += tq.y; acc[5] += tq.z;
-                if (TAPE) sp.lamh[(size_t)it * cap + ci] = make_float4(lam.x, lam.y, lam.z, 0.0f);
+                const float4 r0 = rc[0], r1 = rc[1], r2 = rc[2], l4 = sp.lamf[ci];
+                Contact<float> c;
+                c.r = {r0.x, r0.y, r0.z};
+                c.n = {r1.x, r1.y, r1.z};
+                c.c = {r2.x, r2.y, r2.z};
+                c.lam = {l4.x, l4.y, l4.z};
+                c.ikn = r1.w;
+                c.ikt = r2.w;
+                c.update(vv, ww, mu_s, inv_nc);
+                sp.lamf[ci] = lam4(c);
+                add1(acc, c);
+                if (TAPE) sp.lamh[(size_t)it * cap + ci] = lam4(c);
             }
-            gsum6<GW>(acc, G, S, parity);
-            if (TAPE && G.gt == 0)
-                for (int q = 0; q < 6; ++q) sp.sh[8 * it + q] = acc[q];
+        };
+        auto body = [&](int it, float (&acc)[6], auto one) {
+            if constexpr (GW == 1 || decltype(one)::value) width_sum6<32>(acc, kFull, lane);
+            else gsum6<GW>(acc, G, S, parity, aw);
+            float4 *q = reinterpret_cast<float4 *>(sp.sh + 8 * it);
+            store_if(TAPE && gt == 0, q, make_float4(acc[0], acc[1], acc[2], acc[3]));
+            store_if(TAPE && gt == 0, q + 1, make_float4(acc[4], acc[5], 0.0f, 0.0f));
             vv = v_pred + mk(acc[0], acc[1], acc[2]) * E.inv_m;
             ww = w_pred + smul(Wi, mk(acc[3], acc[4], acc[5]));
+        };
+        // one loop per number of occupied slots, each a straight stretch of code
+        auto last = [&](int k, float4 lam) {
+            const int ci = gt + T * k;
+            if (ci < nc) S.clam[ci] = lam;
+        };
+        if constexpr (GW == 1) {
+            const Vec<F2> z2 = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+            const Vec<float> z1 = {0.0f, 0.0f, 0.0f};
+            if (nc <= 32) {
+                Contact<float> c0;
+                cp_load(S, 0, lane, c0);
+                c0.lam = z1;
+#pragma unroll 1
+                for (int it = 0; it < E.iters; ++it) {
+                    float acc[6] = {0, 0, 0, 0, 0, 0};
+                    c0.update(vv, ww, mu_s, inv_nc);
+                    add1(acc, c0);
+                    tape(it, 0, lam4(c0));
+                    body(it, acc, Flag<true>{});
+                }
+                last(0, lam4(c0));
+            } else if (nc <= 64) {
+                Contact<F2> c0;
+                cp_load(S, 0, lane, c0);
+                c0.lam = z2;
+#pragma unroll 1
+                for (int it = 0; it < E.iters; ++it) {
+                    float acc[6] = {0, 0, 0, 0, 0, 0};
+                    c0.update(vv, ww, mu_s, inv_nc);
+                    add2(acc, c0);
+                    tape(it, 0, lam4a(c0));
+                    tape(it, 1, lam4b(c0));
+                    body(it, acc, Flag<true>{});
+                }
+                last(0, lam4a(c0));
+                last(1, lam4b(c0));
+            } else if (nc <= 96) {
+                Contact<F2> c0;
+                Contact<float> c2;
+                cp_load(S, 0, lane, c0);
+                cp_load(S, 2, lane, c2);
+                c0.lam = z2;
+                c2.lam = z1;
+#pragma unroll 1
+                for (int it = 0; it < E.iters; ++it) {
+                    float acc[6] = {0, 0, 0, 0, 0, 0};
+                    c0.update(vv, ww, mu_s, inv_nc);
+                    c2.update(vv, ww, mu_s, inv_nc);
+                    add2(acc, c0);
+                    add1(acc, c2);
+                    tape(it, 0, lam4a(c0));
+                    tape(it, 1, lam4b(c0));
+                    tape(it, 2, lam4(c2));
+                    body(it, acc, Flag<true>{});
+                }
+                last(0, lam4a(c0));
+                last(1, lam4b(c0));
+                last(2, lam4(c2));
+            } else {
+                Contact<F2> c0, c2;
+                cp_load(S, 0, lane, c0);
+                cp_load(S, 2, lane, c2);
+                c0.lam = z2;
+                c2.lam = z2;
+#pragma unroll 1
+                for (int it = 0; it < E.iters; ++it) {
+                    float acc[6] = {0, 0, 0, 0, 0, 0};
+                    c0.update(vv, ww, mu_s, inv_nc);
+                    c2.update(vv, ww, mu_s, inv_nc);
+                    add2(acc, c0);
+                    add2(acc, c2);
+                    tape(it, 0, lam4a(c0));
+                    tape(it, 1, lam4b(c0));
+                    tape(it, 2, lam4a(c2));
+                    tape(it, 3, lam4b(c2));
+                    further(it, acc);
+                    body(it, acc, Flag<true>{});
+                }
+                last(0, lam4a(c0));
+                last(1, lam4b(c0));
+                last(2, lam4a(c2));
+                last(3, lam4b(c2));
+            }
+        } else {
+            auto iterate = [&](auto one, auto more) {
+#pragma unroll 1
+                for (int it = 0; it < E.iters; ++it) {
+                    float acc[6] = {0, 0, 0, 0, 0, 0};
+                    own.update(vv, ww, mu_s, inv_nc);
+                    add1(acc, own);
+                    tape(it, 0, lam4(own));
+                    if constexpr (decltype(more)::value) further(it, acc);
+                    body(it, acc, one);
+                }
+                last(0, lam4(own));
+            };
+            if (aw == 1) {
+                if (G.wg == 0) iterate(Flag<true>{}, Flag<false>{});
+            } else if (nc <= kRC) {
+                if (G.wg < aw) iterate(Flag<false>{}, Flag<false>{});
+            } else {
+                iterate(Flag<false>{}, Flag<true>{});
+            }
+            if (aw < GW) {   // the body's velocity to the other warps
+                if (gt == 0) {
+                    S.fin[0] = vv.x; S.fin[1] = vv.y; S.fin[2] = vv.z;
+                    S.fin[3] = ww.x; S.fin[4] = ww.y; S.fin[5] = ww.z;
+                }
+                G.sync();
+                vv = mk(S.fin[0], S.fin[1], S.fin[2]);
+                ww = mk(S.fin[3], S.fin[4], S.fin[5]);
+                parity = 0;   // (the warps have used the reduction's buffers differently often)
+            }
         }
     }
     b.v = vv;
@@ -524,28 +694,23 @@ __device__ __noinline__ int fwd_substep(const AdjArgs &a, const Env &E_, Body &b
         const float kq = (wn > 0.0f) ? sn / wn : 0.5f * h;
         b.q = qnorm(qmul_f({cs, b.w.x * kq, b.w.y * kq, b.w.z * kq}, b.q));
     }
+    G.sync();
     if (PADS) {
         // pad forces -lambda / h, each pad summing the contacts of its link in
-        // order (the contacts past the register slots have theirs in sp.lamf)
-#pragma unroll
-        for (int k = 0; k < PL; ++k) {
-            const int ci = G.gt + T * k;
-            if (ci < nc) S.clam[ci] = make_float4(lam_[k].x, lam_[k].y, lam_[k].z, 0.0f);
-        }
-        G.sync();
-        if (G.gt < P && nc > 0) {
-            const int l = __ldg(sc.pad_link + lane);
-            float fx = 0.0f, fy = 0.0f, fz = 0.0f;
-            const int e = S.lend[l];
-            for (int ci = S.lbeg[l]; ci < e; ++ci) {
-                const int pd = ci < RC ? ((__float_as_int(S.crec[ci][1].w) >> 8) & 0xff) : rec_pad(sp.rec[4 * ci + 3]);
-                if (pd != lane) continue;
-                const float4 lf = ci < T * PL ? S.clam[ci] : sp.lamf[ci];
-                fx -= lf.x * inv_h; fy -= lf.y * inv_h; fz -= lf.z * inv_h;
-            }
-            S.padacc[3 * lane + 0] += fx;
-            S.padacc[3 * lane + 1] += fy;
-            S.padacc[3 * lane + 2] += fz;
+        // order, one thread per pad and component (never on a replayed substep)
+#pragma unroll 1
+        for (int k = gt; k < 3 * P; k += T) {
+            const int p = k / 3, comp = k - 3 * p;
+            const int l = __ldg(sc.pad_link + p);
+            float f = 0.0f;
+            const int e = nc > 0 ? S.lend[l] : 0, es = min(e, kRC);
+            int ci = S.lbeg[l];
+            const float *lc = reinterpret_cast<const float *>(S.clam) + comp;
+#pragma unroll 4
+            for (; ci < es; ++ci) f -= (S.cpad[ci] == p ? lc[4 * ci] : 0.0f) * inv_h;
+#pragma unroll 1
+            for (; ci < e; ++ci) f -= (S.cpad[ci] == p ? reinterpret_cast<const float *>(sp.lamf + ci)[comp] : 0.0f) * inv_h;
+            S.padacc[k] += f;
         }
     }
     G.sync();
@@ -570,31 +735,34 @@ __device__ __forceinline__ float bias_slope(const DevConfig &cfg, float gap) {
 __device__ __forceinline__ float sigmoid(float x) { return __fdividef(1.0f, 1.0f + __expf(-x)); }
 
 // Reverse of the smoothed radial clamp out = z smin(|z|, L) / |z| for the
-// incoming derivative g: returns dL/dz and dL/dL. At z = 0 exactly the
-// derivative of the exact clamp inside the disk (identity) is used. With
+// incoming derivative g: dL/dz = g ra + zh (zh . g) pr and dL/dL = (zh . g) pb,
+// the four factors formed here from z and L alone. At z = 0 exactly (and below
+// 1e-15, where the expressions leave FP32's range) the derivative of the exact
+// clamp inside the disk (identity) is used. With
 // Q = sqrt((a - L)^2 + (w L)^2), smin(a, L) = (a + L - Q) / 2 is evaluated as
 // L (4a - w^2 L) / (2 (a + L + Q)), the same value without the cancellation
 // of a + L - Q when the clamp does not bind (a << L).
-__device__ __forceinline__ void disk_bwd(V3 z, float L, V3 g, float w, V3 &zb, float &Lb) {
-    const float a2z = dot(z, z);
-    const bool at0 = !(a2z > 0.0f);
-    const float a2 = at0 ? 1.0f : a2z;   // (without a branch: the values at z = 0 are selected below)
-    const float ia = rsqrtf(a2);
-    const float a = a2 * ia;
-    const float dl = a - L;
-    const float wL = w * L;
-    const float Q2 = fmaf(dl, dl, wL * wL);
-    const float iQ = rsqrtf(Q2);
-    const float Q = Q2 * iQ;
-    const float phi = __fdividef(L * fmaf(-w, wL, 4.0f * a), 2.0f * (a + L + Q));
-    const float pa = 0.5f * (1.0f - dl * iQ);
-    const float pb = 0.5f * (1.0f + (dl - w * wL) * iQ);
-    const V3 zh = z * ia;
-    const float s = dot(zh, g);
-    const float ra = phi * ia;
-    zb = at0 ? ((L > 0.0f) ? g : mk(0, 0, 0)) : g * ra + zh * (s * (pa - ra));
-    Lb = at0 ? 0.0f : s * pb;
+__device__ __forceinline__ void disk_factors(float a2, float L, float w, float &ia, float &ra, float &pr, float &pb) {
+    const bool at0 = !(a2 > 1e-30f);
+    const float r = rsqrt_ftz(at0 ? 1.0f : a2);
+    const float a = (at0 ? 1.0f : a2) * r;
+    const float dl = a - L, wL = w * L;
+    const float Q2 = fmaxf(fmaf(dl, dl, wL * wL), 1e-37f);
+    const float iQ = rsqrt_ftz(Q2);
+    const float phi = __fdividef(L * fmaf(-w, wL, 4.0f * a), 2.0f * fmaf(Q2, iQ, a + L));
+    const float k = dl * iQ;
+    ia = at0 ? 0.0f : r;
+    ra = at0 ? (L > 0.0f ? 1.0f : 0.0f) : phi * r;
+    pr = at0 ? 0.0f : fmaf(-0.5f, k, 0.5f) - phi * r;
+    pb = at0 ? 0.0f : fmaf(0.5f, k - w * wL * iQ, 0.5f);
 }
+__device__ __forceinline__ void disk_factors(F2 a2, F2 L, float w, F2 &ia, F2 &ra, F2 &pr, F2 &pb) {
+    disk_factors(a2.x, L.x, w, ia.x, ra.x, pr.x, pb.x);
+    disk_factors(a2.y, L.y, w, ia.y, ra.y, pr.y, pb.y);
+}
+__device__ __forceinline__ F2 sigmoid(F2 x) { return make_float2(sigmoid(x.x), sigmoid(x.y)); }
+__device__ __forceinline__ float t_sum(float a) { return a; }
+__device__ __forceinline__ float t_sum(F2 a) { return a.x + a.y; }
 
 // Reverse of the narrowphase (hit_box / hit_capsule) for the sphere centred
 // at x + cr: the derivative w.r.t. the centre given those w.r.t. gap and n.
@@ -649,33 +817,30 @@ __device__ __forceinline__ void outer_add(float (&M)[9], V3 a, V3 b, float s) {
         for (int j = 0; j < 3; ++j) M[3 * i + j] += av[i] * bv[j];
 }
 
-// Reverse of one contact's setup and narrowphase (its record rc: r, gap; n,
-// 1/k_n; c, 1/k_t; link, sphere) given the derivatives w.r.t. its constants
+// Reverse of one contact's setup and narrowphase (lever arm r, normal n, gap, 1/k_n,
+// 1/k_t, link l, sphere j) given the derivatives w.r.t. its constants
 // nb, rb, cb, iknb, iktb: the thread's parts of d/dx, d/d(1/m), d/dW and d/dR
 // accumulate.
-__device__ __forceinline__ void contact_setup_bwd(const float4 *rc, V3 nb, V3 rb, V3 cb, float iknb, float iktb,
+__device__ __forceinline__ void contact_setup_bwd(V3 r, V3 n, float gap, float ikn, float ikt, int l, int j, V3 nb, V3 rb, V3 cb,
+                                                  float iknb, float iktb,
                                                   const S6 &Wi, float trW, const M3 &R, V3 x, int sfirst,
                                                   const DevScene &sc, const DevConfig &cfg, const float4 *L0,
                                                   const float4 *L1, float inv_h, float (&Wbar)[9], float (&Rbar)[9],
                                                   V3 &xb_l, float &invm_l) {
-    const float4 r0 = rc[0], r1 = rc[1], r2 = rc[2], r3 = rc[3];
-    const V3 r = xyz(r0), n = xyz(r1);
-    const float gap = r0.w, ikn = r1.w, ikt = r2.w;
-    const int l = rec_link(r3), j = __float_as_int(r3.z);
     // 1/k_n and 1/k_t = 2 / (tr K - k_n)
     float knb = -iknb * ikn * ikn;
     const float Db = -iktb * ikt * ikt * 0.5f;
     const float trKb = Db;
     knb -= Db;
     // k_n = 1/m + (r x n) . W (r x n)
-    const V3 rn = cross_r(r, n);
-    const V3 rnb = smul_r(Wi, rn) * (2.0f * knb);
+    const V3 rn = cross(r, n);
+    const V3 rnb = smul(Wi, rn) * (2.0f * knb);
     invm_l += knb + 3.0f * trKb;
     outer_add(Wbar, rn, rn, knb);
-    rb = rb + cross_r(n, rnb);
-    nb = nb + cross_r(rnb, r);
+    rb = rb + cross(n, rnb);
+    nb = nb + cross(rnb, r);
     // tr K = 3/m + |r|^2 tr W - r . W r
-    rb = rb + (r * (2.0f * trW) - smul_r(Wi, r) * 2.0f) * trKb;
+    rb = rb + (r * (2.0f * trW) - smul(Wi, r) * 2.0f) * trKb;
     const float rr = dot(r, r) * trKb;
     Wbar[0] += rr; Wbar[4] += rr; Wbar[8] += rr;
     outer_add(Wbar, r, r, -trKb);
@@ -699,56 +864,322 @@ __device__ __forceinline__ void contact_setup_bwd(const float4 *rc, V3 nb, V3 rb
     outer_add(Rbar, rb + hb, xyz(s4), 1.0f);
 }
 
-// Reverse of one contact's update in a Jacobi iteration (update_contact with
-// constants r, n, c, 1/k_n, 1/k_t against the velocities Vi, Wv, from its
-// impulse l0 before the iteration): lb holds the derivative w.r.t. its impulse
-// after the iteration and leaves with the one before it; nb, rb, cb, iknb,
-// iktb, mu_b and the group's velocity and moment sums acc accumulate.
-__device__ __forceinline__ void contact_update_bwd(V3 r, V3 n, V3 cc, float ikn, float ikt, V3 l0, V3 Vi, V3 Wv,
-                                                   float mu, float inv_nc, float width, float beta_s, V3 &lb,
-                                                   V3 &nb, V3 &rb, V3 &cb, float &iknb, float &iktb, float &mu_b,
-                                                   float (&acc)[6]) {
-    const V3 u = Vi + cross_r(Wv, r) - cc;
-    const float un = dot(u, n), lo = dot(l0, n);
-    const float zn = lo - un * ikn;
-    const float ln = fmaxf(zn, 0.0f);
-    const V3 ut = u - n * un;
-    const V3 zt = (l0 - n * lo) - ut * ikt;
-    const float L = mu * ln;
-    // lambda' = lambda + (n ln + lt - lambda) / n_c
-    const V3 lpb = lb * inv_nc;
-    lb = lb * (1.0f - inv_nc);
-    float lnb = dot(n, lpb);
-    nb = nb + lpb * ln;
-    V3 ztb;
-    float Lb;
-    disk_bwd(zt, L, lpb, width, ztb, Lb);
-    lnb += mu * Lb;
-    mu_b += ln * Lb;
-    const float znb = lnb * sigmoid(beta_s * zn);
-    float lob = znb;
-    float unb = -znb * ikn;
-    iknb -= znb * un;
-    // zt = (l0 - n lo) - (u - n un) ikt
-    const float nzt = dot(n, ztb);
-    lb = lb + ztb;
-    nb = nb - ztb * lo;
-    lob -= nzt;
-    V3 ub = ztb * (-ikt);
-    nb = nb + ztb * (ikt * un);
-    unb += ikt * nzt;
-    iktb -= dot(ut, ztb);
-    // lo = l0 . n, un = u . n
-    lb = lb + n * lob;
-    nb = nb + l0 * lob;
-    ub = ub + n * unb;
-    nb = nb + u * unb;
-    // u = V + W x r - c
-    const V3 rxu = cross_r(r, ub);
-    acc[0] += ub.x; acc[1] += ub.y; acc[2] += ub.z;
-    acc[3] += rxu.x; acc[4] += rxu.y; acc[5] += rxu.z;
-    rb = rb + cross_r(ub, Wv);
-    cb = cb - ub;
+// The reverse of one contact's (T = float) or two contacts' (float2, packed) updates
+// in the Jacobi iterations: the derivative lb w.r.t. the impulse after the current
+// iteration and those w.r.t. the constants r, n, c, 1/k_n, 1/k_t, accumulated.
+// a x b added to s
+template <typename T>
+__device__ __forceinline__ Vec<T> t_cross_add(const Vec<T> &a, const Vec<T> &b, const Vec<T> &s) {
+    return {t_fma(a.y, b.z, t_fma(t_neg(a.z), b.y, s.x)), t_fma(a.z, b.x, t_fma(t_neg(a.x), b.z, s.y)),
+            t_fma(a.x, b.y, t_fma(t_neg(a.y), b.x, s.z))};
+}
+template <typename T>
+__device__ __forceinline__ Vec<T> t_vec(V3 v) { return {t_all<T>(v.x), t_all<T>(v.y), t_all<T>(v.z)}; }
+template <typename T>
+__device__ __forceinline__ Vec<T> t_axpy(T k, const Vec<T> &a, const Vec<T> &s) {
+    return {t_fma(k, a.x, s.x), t_fma(k, a.y, s.y), t_fma(k, a.z, s.z)};
+}
+template <typename T>
+__device__ __forceinline__ Vec<T> t_scale(T k, const Vec<T> &a) { return {t_mul(k, a.x), t_mul(k, a.y), t_mul(k, a.z)}; }
+
+// What the reverse of an update takes from the forward alone: u, un = u . n, lo =
+// lambda . n, the normal impulse ln and the clamps' derivatives (disk_factors, and
+// sig, the normal clamp's). No derivative enters, so they are formed an iteration
+// ahead, in the shadow of the reduction.
+template <typename T>
+struct Factors {
+    Vec<T> u, zh;
+    T un, lo, ln, ra, pr, pb, sig;
+    // c holds the constants and the impulse before the iteration
+    __device__ __forceinline__ void form(const Contact<T> &c, V3 Vi, V3 Wv, float mu, float width, float beta_s) {
+        const Vec<T> tW = t_vec<T>(Wv), tV = t_vec<T>(Vi);
+        u = t_cross_add(tW, c.r, Vec<T>{t_fma(c.c.x, t_all<T>(-1.0f), tV.x), t_fma(c.c.y, t_all<T>(-1.0f), tV.y),
+                                        t_fma(c.c.z, t_all<T>(-1.0f), tV.z)});
+        un = t_dot(u, c.n);
+        lo = t_dot(c.lam, c.n);
+        const T nun = t_neg(un), zn = t_fma(nun, c.ikn, lo);
+        ln = t_relu(zn);
+        const Vec<T> zt = t_axpy(t_neg(c.ikt), t_axpy(nun, c.n, u), t_axpy(t_neg(lo), c.n, c.lam));
+        T ia;
+        disk_factors(t_dot(zt, zt), t_mul(t_all<T>(mu), ln), width, ia, ra, pr, pb);
+        zh = t_scale(ia, zt);
+        sig = sigmoid(t_mul(t_all<T>(beta_s), zn));
+    }
+};
+
+template <typename T>
+struct ContactBwd {
+    Vec<T> lb, nb, rb, cb;
+    T iknb, iktb, mub;
+    __device__ __forceinline__ void clear() {
+        const T o = t_all<T>(0.0f);
+        lb = nb = rb = cb = {o, o, o};
+        iknb = iktb = mub = o;
+    }
+    // One iteration: c holds the constants and the impulse before it, f its factors,
+    // l1 the impulse after it; vm = Vb / m and g = W Wb of the derivatives Vb, Wb
+    // w.r.t. the body's velocity after it, Wv the angular velocity before it. Adds the
+    // derivatives w.r.t. that velocity to acc. (An empty slot adds zeros: its 1/k and
+    // r are zero.)
+    __device__ __forceinline__ void step(const Contact<T> &c, const Factors<T> &f, const Vec<T> &l1, V3 vm, V3 g, V3 Wv, float mu,
+                                         float inv_nc, T (&acc)[6]) {
+        const Vec<T> tg = t_vec<T>(g), tW = t_vec<T>(Wv);
+        // V and W after the iteration: the impulse's share
+        lb = t_cross_add(tg, c.r, Vec<T>{t_add(lb.x, t_all<T>(vm.x)), t_add(lb.y, t_all<T>(vm.y)), t_add(lb.z, t_all<T>(vm.z))});
+        rb = t_cross_add(l1, tg, rb);
+        // lambda' = lambda + (n ln + lt - lambda) / n_c
+        const Vec<T> lpb = t_scale(t_all<T>(inv_nc), lb);
+        lb = t_scale(t_all<T>(1.0f - inv_nc), lb);
+        const T s = t_dot(f.zh, lpb), Lb = t_mul(s, f.pb), nun = t_neg(f.un), nlo = t_neg(f.lo);
+        const Vec<T> ztb = t_axpy(t_mul(s, f.pr), f.zh, t_scale(f.ra, lpb));
+        mub = t_fma(f.ln, Lb, mub);
+        const T znb = t_mul(t_fma(t_all<T>(mu), Lb, t_dot(c.n, lpb)), f.sig);
+        const T nzt = t_dot(c.n, ztb);
+        iknb = t_fma(znb, nun, iknb);
+        // (u - n un) . ztb
+        iktb = t_fma(t_all<T>(-1.0f), t_fma(nun, nzt, t_dot(f.u, ztb)), iktb);
+        const T unb = t_fma(c.ikt, nzt, t_neg(t_mul(znb, c.ikn))), lob = t_fma(t_all<T>(-1.0f), nzt, znb);
+        const Vec<T> ub = t_axpy(unb, c.n, t_scale(t_neg(c.ikt), ztb));
+        // u = V + W x r - c
+        acc[0] = t_add(acc[0], ub.x); acc[1] = t_add(acc[1], ub.y); acc[2] = t_add(acc[2], ub.z);
+        const Vec<T> m = t_cross_add(c.r, ub, Vec<T>{acc[3], acc[4], acc[5]});
+        acc[3] = m.x; acc[4] = m.y; acc[5] = m.z;
+        nb = t_axpy(f.ln, lpb, nb);
+        nb = t_axpy(t_fma(c.ikt, f.un, nlo), ztb, nb);
+        nb = t_axpy(lob, c.lam, nb);
+        nb = t_axpy(unb, f.u, nb);
+        lb = t_axpy(lob, c.n, Vec<T>{t_add(lb.x, ztb.x), t_add(lb.y, ztb.y), t_add(lb.z, ztb.z)});
+        rb = t_cross_add(ub, tW, rb);
+        cb = {t_fma(ub.x, t_all<T>(-1.0f), cb.x), t_fma(ub.y, t_all<T>(-1.0f), cb.y), t_fma(ub.z, t_all<T>(-1.0f), cb.z)};
+    }
+};
+
+// The reverse iterations of the register-resident contacts of a thread: units U0
+// (slots 0, or 0 and 1) and U1 (slots 2, or 2 and 3; NoUnit when absent), and the
+// contacts past kRC from memory.
+// Vb, Wb enter as the derivatives w.r.t. the velocity after the last iteration and
+// leave as those before the first; vpb, wpb, Wbar, invm_l accumulate.
+struct NoUnit {};
+template <int GW>
+struct RevCtx {
+    const SlotPtr &sp;
+    GroupSm<GW> &S;
+    const AGroup<GW> &G;
+    const S6 &Wi;
+    V3 v_pred, w_pred;
+    float inv_m, mu, inv_nc, width, beta_s;
+    int cap, nc, I, aw, n_pads;
+};
+__device__ __forceinline__ void set_half(Vec<float> &v, int, float4 l) { v = {l.x, l.y, l.z}; }
+__device__ __forceinline__ void set_half(Vec<F2> &v, int h, float4 l) {
+    if (h == 0) { v.x.x = l.x; v.y.x = l.y; v.z.x = l.z; }
+    else { v.x.y = l.x; v.y.y = l.y; v.z.y = l.z; }
+}
+__device__ __forceinline__ V3 get_half(const Vec<float> &v, int) { return mk(v.x, v.y, v.z); }
+__device__ __forceinline__ V3 get_half(const Vec<F2> &v, int h) { return h == 0 ? mk(v.x.x, v.y.x, v.z.x) : mk(v.x.y, v.y.y, v.z.y); }
+__device__ __forceinline__ float get_half(float v, int) { return v; }
+__device__ __forceinline__ float get_half(F2 v, int h) { return h == 0 ? v.x : v.y; }
+
+// one unit: its reverse state, its impulses after iterations it and it - 1, and,
+// when AHEAD, the factors of iteration it, formed an iteration early
+template <int GW, typename T>
+struct RevUnit {
+    static constexpr int N = sizeof(T) / sizeof(float);
+    ContactBwd<T> b;
+    Factors<T> f;
+    Vec<T> l1, l0;
+    int slot;
+    __device__ __forceinline__ void init(const RevCtx<GW> &x, int slot_) {
+        slot = slot_;
+        b.clear();
+#pragma unroll
+        for (int h = 0; h < N; ++h) {
+            const int ci = x.G.gt + AGroup<GW>::T * (slot + h);
+            float4 f4 = make_float4(0, 0, 0, 0), l4 = f4;
+            if (ci < x.nc) {   // the pad's derivative on the contact's final impulse
+                const int pad = rec_pad(x.S.meta[ci]);
+                if (pad < x.n_pads) f4 = make_float4(-x.S.fbar[3 * pad], -x.S.fbar[3 * pad + 1], -x.S.fbar[3 * pad + 2], 0.0f);
+                l4 = x.sp.lamh[(size_t)(x.I - 1) * x.cap + ci];
+            }
+            set_half(b.lb, h, f4);
+            set_half(l1, h, l4);
+        }
+    }
+    // the impulses after iteration it: their copy (zeros before the first and in empty
+    // slots), and their values once it has arrived
+    __device__ __forceinline__ void request(const RevCtx<GW> &x, int it) const {
+#pragma unroll
+        for (int h = 0; h < N; ++h) {
+            const int ci = x.G.gt + AGroup<GW>::T * (slot + h);
+            copy_async(&x.S.ring[it & (kRing - 1)][ci], x.sp.lamh + (size_t)max(it, 0) * x.cap + min(ci, x.nc - 1),
+                       it >= 0 && ci < x.nc ? 16 : 0);
+        }
+    }
+    __device__ __forceinline__ void arrived(const RevCtx<GW> &x, int it, Vec<T> &v) const {
+#pragma unroll
+        for (int h = 0; h < N; ++h) set_half(v, h, x.S.ring[it & (kRing - 1)][x.G.gt + AGroup<GW>::T * (slot + h)]);
+    }
+    __device__ __forceinline__ void constants(const RevCtx<GW> &x, const Contact<float> &own, Contact<T> &c) const {
+        if constexpr (GW == 1) cp_load(x.S, slot, x.G.lane, c);
+        else c = own;
+        c.lam = l0;
+    }
+    __device__ __forceinline__ void form(const RevCtx<GW> &x, const Contact<float> &own, int it, V3 Vi, V3 Wv) {   // of iteration it
+        arrived(x, it - 1, l0);
+        Contact<T> c;
+        constants(x, own, c);
+        f.form(c, Vi, Wv, x.mu, x.width, x.beta_s);
+    }
+    __device__ __forceinline__ void step(const RevCtx<GW> &x, const Contact<float> &own, V3 vm, V3 g, V3 Wv, float (&acc)[6]) {
+        Contact<T> c;
+        constants(x, own, c);
+        const T o = t_all<T>(0.0f);
+        T s[6] = {o, o, o, o, o, o};
+        b.step(c, f, l1, vm, g, Wv, x.mu, x.inv_nc, s);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) acc[q] += t_sum(s[q]);
+        l1 = l0;
+    }
+    // the derivatives w.r.t. the constants, in the ring's place
+    __device__ __forceinline__ void finish(const RevCtx<GW> &x, float &mu_b) {
+        mu_b += t_sum(b.mub);
+#pragma unroll
+        for (int h = 0; h < N; ++h) {
+            const int ci = x.G.gt + AGroup<GW>::T * (slot + h);
+            const V3 nb = get_half(b.nb, h), rb = get_half(b.rb, h), cb = get_half(b.cb, h);
+            x.S.ring[0][ci] = make_float4(nb.x, nb.y, nb.z, get_half(b.iknb, h));
+            x.S.ring[1][ci] = make_float4(rb.x, rb.y, rb.z, get_half(b.iktb, h));
+            x.S.ring[2][ci] = make_float4(cb.x, cb.y, cb.z, 0.0f);
+        }
+    }
+};
+template <int GW>
+struct RevUnit<GW, NoUnit> {
+    __device__ __forceinline__ void init(const RevCtx<GW> &, int) {}
+    __device__ __forceinline__ void request(const RevCtx<GW> &, int) const {}
+    __device__ __forceinline__ void form(const RevCtx<GW> &, const Contact<float> &, int, V3, V3) {}
+    __device__ __forceinline__ void step(const RevCtx<GW> &, const Contact<float> &, V3, V3, V3, float (&)[6]) {}
+    __device__ __forceinline__ void finish(const RevCtx<GW> &, float &) {}
+};
+
+template <int GW, typename T0, typename T1, bool FURTHER, bool AHEAD, bool ONE>
+__device__ __forceinline__ void rev_iterations(const RevCtx<GW> &x, const Contact<float> &own, int &parity, V3 &Vb, V3 &Wb,
+                                               V3 &vpb, V3 &wpb, float (&Wbar)[9], float &invm_l, float &mu_b) {
+    constexpr int T = AGroup<GW>::T;
+    RevUnit<GW, T0> u0;
+    RevUnit<GW, T1> u1;
+    u0.init(x, 0);
+    u1.init(x, 2);
+    if (FURTHER) {   // contacts past kRC: their reverse state in sp.adjs
+#pragma unroll 1
+        for (int ci = kRC + x.G.gt; ci < x.nc; ci += T) {
+            const int pad = rec_pad(x.sp.rec[4 * ci + 3]);
+            float4 *A = x.sp.adjs + 4 * ci;
+            A[0] = (pad < x.n_pads) ? make_float4(-x.S.fbar[3 * pad], -x.S.fbar[3 * pad + 1], -x.S.fbar[3 * pad + 2], 0.0f)
+                                    : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            A[1] = A[2] = A[3] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+    }
+    // the tape of iteration it to shared memory (zeros before the first)
+    auto request = [&](int it) {
+        u0.request(x, it);
+        u1.request(x, it);
+        copy_async(&x.S.rsum[x.G.wg][it & (kRing - 1)][x.G.lane & 1],
+                   reinterpret_cast<const float4 *>(x.sp.sh + 8 * max(it, 0)) + (x.G.lane & 1), it >= 0 ? 16 : 0, x.G.lane < 2);
+        copy_commit();
+    };
+    // the sums after iteration it, and the body's velocity from them
+    auto sums = [&](int it, float4 &lo, float4 &hi) {
+        lo = x.S.rsum[x.G.wg][it & (kRing - 1)][0];
+        hi = x.S.rsum[x.G.wg][it & (kRing - 1)][1];
+    };
+    float4 c_lo, c_hi, p_lo, p_hi;   // the sums after iterations it and it - 1
+    {
+        const float4 *q = reinterpret_cast<const float4 *>(x.sp.sh + 8 * (x.I - 1));
+        c_lo = q[0];
+        c_hi = q[1];
+    }
+    V3 Vi, Wv;   // the body's velocity before iteration it
+    auto before = [&](int it) {
+        sums(it - 1, p_lo, p_hi);
+        Vi = x.v_pred + mk(p_lo.x, p_lo.y, p_lo.z) * x.inv_m;
+        Wv = x.w_pred + smul(x.Wi, mk(p_lo.w, p_hi.x, p_hi.y));
+        u0.form(x, own, it, Vi, Wv);
+        u1.form(x, own, it, Vi, Wv);
+    };
+#pragma unroll 1
+    for (int k = 2; k <= kRing; ++k) request(x.I - k);
+    if (AHEAD) {
+        copy_wait<kRing - 2>();
+        __syncwarp();
+        before(x.I - 1);
+    }
+#pragma unroll 1
+    for (int it = x.I - 1; it >= 0; --it) {
+        request(it - kRing);   // (its place held the impulses after iteration it, in registers by now)
+        copy_wait<kRing - 1 - (AHEAD ? 1 : 0)>();
+        __syncwarp();          // (the sums are copied by two lanes)
+        if (!AHEAD) before(it);
+        // (a) V^{it+1} = v_pred + S1 / m, W^{it+1} = w_pred + W S2, sums of the impulses after it
+        const V3 g = smul(x.Wi, Wb), vm = Vb * x.inv_m;
+        vpb = vpb + Vb;
+        wpb = wpb + Wb;
+        // (b) the contact updates of iteration it, against V^it, W^it
+        float acc[6] = {0, 0, 0, 0, 0, 0};
+        u0.step(x, own, vm, g, Wv, acc);
+        u1.step(x, own, vm, g, Wv, acc);
+        invm_l += dot(Vb, mk(c_lo.x, c_lo.y, c_lo.z));   // (every thread; one's is kept)
+        outer_add(Wbar, Wb, mk(c_lo.w, c_hi.x, c_hi.y), 1.0f);
+        c_lo = p_lo; c_hi = p_hi;
+        if (FURTHER) {
+#pragma unroll 1
+            for (int ci = kRC + x.G.gt; ci < x.nc; ci += T) {
+                const float4 *rc = x.sp.rec + 4 * ci;
+                const float4 r0 = rc[0], r1 = rc[1], r2 = rc[2];
+                float4 *A = x.sp.adjs + 4 * ci;
+                const float4 a0 = A[0], a1 = A[1], a2 = A[2], a3 = A[3];
+                const float4 l1 = x.sp.lamh[(size_t)it * x.cap + ci];
+                const float4 l0 = it > 0 ? x.sp.lamh[(size_t)(it - 1) * x.cap + ci] : make_float4(0, 0, 0, 0);
+                Contact<float> c;
+                c.r = {r0.x, r0.y, r0.z};
+                c.n = {r1.x, r1.y, r1.z};
+                c.c = {r2.x, r2.y, r2.z};
+                c.lam = {l0.x, l0.y, l0.z};
+                c.ikn = r1.w;
+                c.ikt = r2.w;
+                ContactBwd<float> b;
+                b.lb = {a0.x, a0.y, a0.z};
+                b.nb = {a1.x, a1.y, a1.z};
+                b.rb = {a2.x, a2.y, a2.z};
+                b.cb = {a3.x, a3.y, a3.z};
+                b.iknb = a0.w;
+                b.iktb = a1.w;
+                b.mub = a2.w;
+                Factors<float> f;
+                f.form(c, Vi, Wv, x.mu, x.width, x.beta_s);
+                b.step(c, f, Vec<float>{l1.x, l1.y, l1.z}, vm, g, Wv, x.mu, x.inv_nc, acc);
+                A[0] = make_float4(b.lb.x, b.lb.y, b.lb.z, b.iknb);
+                A[1] = make_float4(b.nb.x, b.nb.y, b.nb.z, b.iktb);
+                A[2] = make_float4(b.rb.x, b.rb.y, b.rb.z, b.mub);
+                A[3] = make_float4(b.cb.x, b.cb.y, b.cb.z, 0.0f);
+            }
+        }
+        if (AHEAD) before(it - 1);   // beside the reduction (past the first: unused)
+        if constexpr (ONE) width_sum6<32>(acc, kFull, x.G.lane);
+        else gsum6<GW>(acc, x.G, x.S, parity, x.aw);
+        Vb = mk(acc[0], acc[1], acc[2]);
+        Wb = mk(acc[3], acc[4], acc[5]);
+    }
+    vpb = vpb + Vb;   // V^0 = v_pred, W^0 = w_pred
+    wpb = wpb + Wb;
+    if (x.G.gt != 0) {
+        invm_l = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) Wbar[q] = 0.0f;
+    }
+    copy_wait<0>();
+    u0.finish(x, mu_b);
+    u1.finish(x, mu_b);
 }
 
 // Reverse sweep of one substep from start state b (whose forward has just
@@ -757,7 +1188,7 @@ __device__ __forceinline__ void contact_update_bwd(V3 r, V3 n, V3 cc, float ikn,
 // invm_b (lane-uniform) and mu_b (per lane) accumulate d/d(1/m) and d/dmu.
 // Not inlined: both tape modes then run the same compiled reverse, so their
 // gradients agree bit for bit.
-template <int GW, int PL>
+template <int GW>
 __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const Body &b_, const float4 *L0,
                                         const float4 *L1, int nc, const SlotPtr &sp_, GroupSm<GW> &S,
                                         const AGroup<GW> &G_, int &parity_, Adj &ad_, float &invm_b_, float &mu_b_) {
@@ -779,14 +1210,14 @@ __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const 
     const V3 v_pred = b.v + grav;
     const V3 w_pred = b.w;
     const M3 R = qmat(b.q);
-    const S6 Wi = world_inv_inertia_r(R, E.Jb, E.inv_m);
+    const S6 Wi = world_inv_inertia_f(R, E.Jb, E.inv_m);
     const float trW = Wi.xx + Wi.yy + Wi.zz;
     const bool solved = nc > 0 && I > 0;
     V3 Vf = v_pred, Wf = w_pred;   // body velocity after the solve
     if (solved) {
         const float *s = sp.sh + 8 * (I - 1);
         Vf = v_pred + mk(s[0], s[1], s[2]) * E.inv_m;
-        Wf = w_pred + smul_r(Wi, mk(s[3], s[4], s[5]));
+        Wf = w_pred + smul(Wi, mk(s[3], s[4], s[5]));
     }
 
     // -- integration: x' = x + h V, q' = normalize(exp(h W) q)
@@ -799,14 +1230,14 @@ __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const 
         sincosf(0.5f * wn * h, &sn, &cs);
         const float kq = (wn > 0.0f) ? sn / wn : 0.5f * h;
         const Q4 e = {cs, Wf.x * kq, Wf.y * kq, Wf.z * kq};
-        const Q4 p = qmul_r(e, b.q);
+        const Q4 p = qmul(e, b.q);
         const float s = rsqrtf(p.w * p.w + p.x * p.x + p.y * p.y + p.z * p.z);
         const Q4 qn = {p.w * s, p.x * s, p.y * s, p.z * s};
         const float dq = ad.q.w * qn.w + ad.q.x * qn.x + ad.q.y * qn.y + ad.q.z * qn.z;
         const Q4 pb = {(ad.q.w - qn.w * dq) * s, (ad.q.x - qn.x * dq) * s, (ad.q.y - qn.y * dq) * s,
                        (ad.q.z - qn.z * dq) * s};
-        qb = qmul_r(qconj(e), pb);                // p = e q: dq = L(e)^T dp
-        const Q4 eb = qmul_r(pb, qconj(b.q));     // de = R(q)^T dp
+        qb = qmul(qconj(e), pb);                // p = e q: dq = L(e)^T dp
+        const Q4 eb = qmul(pb, qconj(b.q));     // de = R(q)^T dp
         // e = (cos(th/2), s(th) A), A = h W, th = |A|, s(th) = sin(th/2) / th
         const float th = wn * h;
         const float sf = kq / h;
@@ -828,134 +1259,61 @@ __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const 
     V3 xb_l = mk(0, 0, 0);
     float invm_l = 0.0f;
     if (solved) {
-        const float inv_nc = 1.0f / (float)nc;
-        V3 lb[PL], nb[PL], rb[PL], cb[PL];
-        float iknb[PL], iktb[PL];
-        // the contacts' constants in registers, and the tape one iteration ahead:
-        // l1_ the impulse after iteration it, l0_ after it - 1 (zero before the
-        // first), sc_/sp_ the sums after it and it - 1
-        V3 r_[PL], n_[PL], c_[PL], l1_[PL], l0_[PL];
-        float ikn_[PL], ikt_[PL];
-        auto lam_at = [&](int it, int ci) -> V3 { return it >= 0 ? xyz(sp.lamh[(size_t)it * cap + ci]) : mk(0, 0, 0); };
-        auto sums_at = [&](int it, float4 &lo, float4 &hi) {
-            if (it >= 0) {
-                const float4 *q = reinterpret_cast<const float4 *>(sp.sh + 8 * it);
-                lo = q[0]; hi = q[1];
-            } else {
-                lo = hi = make_float4(0, 0, 0, 0);
-            }
-        };
-#pragma unroll
-        for (int k = 0; k < PL; ++k) {
-            lb[k] = nb[k] = rb[k] = cb[k] = mk(0, 0, 0);
-            iknb[k] = iktb[k] = 0.0f;
-            r_[k] = n_[k] = c_[k] = l1_[k] = l0_[k] = mk(0, 0, 0);
-            ikn_[k] = ikt_[k] = 0.0f;
-            const int ci = G.gt + T * k;
-            if (ci < nc) {
-                const float4 *rc = sp.rec + 4 * ci;
-                const float4 r0 = rc[0], r1 = rc[1], r2 = rc[2], r3 = rc[3];
-                r_[k] = xyz(r0); n_[k] = xyz(r1); c_[k] = xyz(r2); ikn_[k] = r1.w; ikt_[k] = r2.w;
-                l1_[k] = lam_at(I - 1, ci);
-                l0_[k] = lam_at(I - 2, ci);
-                const int pad = rec_pad(r3);
-                if (pad < sc.n_pads) lb[k] = mk(-S.fbar[3 * pad], -S.fbar[3 * pad + 1], -S.fbar[3 * pad + 2]);
+        const int aw = GW == 1 ? 1 : min(GW, (nc + 31) >> 5);
+        const RevCtx<GW> x = {sp, S, G, Wi, v_pred, w_pred, E.inv_m, E.mu, 1.0f / (float)nc, width, beta_s, cap, nc, I, aw, sc.n_pads};
+        // the constants, from the records
+        Contact<float> own;
+        own.clear();
+        load_constants<GW, true>(sp, S, G, nc, own);
+        __syncwarp();
+        if constexpr (GW == 1) {
+            if (nc <= 32) rev_iterations<GW, float, NoUnit, false, true, true>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            else if (nc <= 64) rev_iterations<GW, F2, NoUnit, false, false, true>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            else if (nc <= 96) rev_iterations<GW, F2, float, false, false, true>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            else rev_iterations<GW, F2, F2, true, false, true>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+        } else {
+            if (aw == 1 && G.wg == 0) rev_iterations<GW, float, NoUnit, false, true, true>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            else if (nc <= kRC && G.wg < aw) rev_iterations<GW, float, NoUnit, false, true, false>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            else if (G.wg < aw) rev_iterations<GW, float, NoUnit, true, true, false>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            if (aw < GW) {   // the body's derivatives to the other warps
+                if (G.gt == 0) {
+                    S.fin[0] = vpb.x; S.fin[1] = vpb.y; S.fin[2] = vpb.z;
+                    S.fin[3] = wpb.x; S.fin[4] = wpb.y; S.fin[5] = wpb.z;
+                }
+                G.sync();
+                vpb = mk(S.fin[0], S.fin[1], S.fin[2]);
+                wpb = mk(S.fin[3], S.fin[4], S.fin[5]);
+                parity = 0;   // (the warps have used the reduction's buffers differently often)
             }
         }
-        // contacts past the register slots: their reverse state in sp.adjs
-        for (int ci = G.gt + T * PL; ci < nc; ci += T) {
-            const int pad = rec_pad(sp.rec[4 * ci + 3]);
-            float4 *A = sp.adjs + 4 * ci;
-            A[0] = (pad < sc.n_pads) ? make_float4(-S.fbar[3 * pad], -S.fbar[3 * pad + 1], -S.fbar[3 * pad + 2], 0.0f)
-                                     : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            A[1] = A[2] = A[3] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        }
-        float4 sc_lo, sc_hi, sp_lo, sp_hi;
-        sums_at(I - 1, sc_lo, sc_hi);
-        sums_at(I - 2, sp_lo, sp_hi);
-        for (int it = I - 1; it >= 0; --it) {
-            // the tape of iteration it - 2, for the next step, requested now
-            V3 pf_[PL];
-#pragma unroll
-            for (int k = 0; k < PL; ++k) {
-                const int ci = G.gt + T * k;
-                pf_[k] = (ci < nc) ? lam_at(it - 2, ci) : mk(0, 0, 0);
-            }
-            float4 pf_lo, pf_hi;
-            sums_at(it - 2, pf_lo, pf_hi);
-            // (a) V^{it+1} = v_pred + S1 / m, W^{it+1} = w_pred + W S2, sums of the impulses after it
-            const V3 S1 = mk(sc_lo.x, sc_lo.y, sc_lo.z), S2 = mk(sc_lo.w, sc_hi.x, sc_hi.y);
-            vpb = vpb + Vb;
-            wpb = wpb + Wb;
-            if (G.gt == 0) {
-                invm_l += dot(Vb, S1);
-                outer_add(Wbar, Wb, S2, 1.0f);
-            }
-            const V3 g = smul_r(Wi, Wb);
-            const V3 vm = Vb * E.inv_m;
-            // every register slot without a branch (an empty slot has r = l1 = 0
-            // and keeps lb = 0, so its reverse below adds zeros)
-#pragma unroll
-            for (int k = 0; k < PL; ++k) {
-                const V3 lbk = lb[k] + vm + cross_r(g, r_[k]);
-                lb[k] = (G.gt + T * k < nc) ? lbk : lb[k];
-                rb[k] = rb[k] + cross_r(l1_[k], g);
-            }
-            // (b) the contact updates of iteration it, against V^it, W^it
-            V3 Vi = v_pred, Wv = w_pred;
-            if (it > 0) {
-                Vi = v_pred + mk(sp_lo.x, sp_lo.y, sp_lo.z) * E.inv_m;
-                Wv = w_pred + smul_r(Wi, mk(sp_lo.w, sp_hi.x, sp_hi.y));
-            }
-            float acc[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll
-            for (int k = 0; k < PL; ++k)
-                contact_update_bwd(r_[k], n_[k], c_[k], ikn_[k], ikt_[k], l0_[k], Vi, Wv, E.mu, inv_nc, width, beta_s,
-                                   lb[k], nb[k], rb[k], cb[k], iknb[k], iktb[k], mu_b, acc);
-            for (int ci = G.gt + T * PL; ci < nc; ci += T) {   // (a) and (b) of the contacts in memory
-                const float4 *rc = sp.rec + 4 * ci;
-                const float4 r0 = rc[0], r1 = rc[1], r2 = rc[2];
-                float4 *A = sp.adjs + 4 * ci;
-                const float4 a0 = A[0], a1 = A[1], a2 = A[2], a3 = A[3];
-                const V3 r = xyz(r0);
-                V3 lbk = xyz(a0) + vm + cross_r(g, r), nbk = xyz(a1), rbk = xyz(a2) + cross_r(lam_at(it, ci), g),
-                   cbk = xyz(a3);
-                float iknbk = a0.w, iktbk = a1.w;
-                contact_update_bwd(r, xyz(r1), xyz(r2), r1.w, r2.w, lam_at(it - 1, ci), Vi, Wv, E.mu, inv_nc, width,
-                                   beta_s, lbk, nbk, rbk, cbk, iknbk, iktbk, mu_b, acc);
-                A[0] = make_float4(lbk.x, lbk.y, lbk.z, iknbk);
-                A[1] = make_float4(nbk.x, nbk.y, nbk.z, iktbk);
-                A[2] = make_float4(rbk.x, rbk.y, rbk.z, 0.0f);
-                A[3] = make_float4(cbk.x, cbk.y, cbk.z, 0.0f);
-            }
-            gsum6<GW>(acc, G, S, parity);
-            Vb = mk(acc[0], acc[1], acc[2]);
-            Wb = mk(acc[3], acc[4], acc[5]);
-#pragma unroll
-            for (int k = 0; k < PL; ++k) {
-                l1_[k] = l0_[k];
-                l0_[k] = pf_[k];
-            }
-            sc_lo = sp_lo; sc_hi = sp_hi;
-            sp_lo = pf_lo; sp_hi = pf_hi;
-        }
-        vpb = vpb + Vb;   // V^0 = v_pred, W^0 = w_pred
-        wpb = wpb + Wb;
-
         // contact setup and narrowphase, in reverse
-#pragma unroll
-        for (int k = 0; k < PL; ++k) {
-            const int ci = G.gt + T * k;
-            if (ci < nc) {
-                contact_setup_bwd(sp.rec + 4 * ci, nb[k], rb[k], cb[k], iknb[k], iktb[k], Wi, trW, R, b.x, E.sfirst, sc,
-                                  cfg, L0, L1, inv_h, Wbar, Rbar, xb_l, invm_l);
+#pragma unroll 1
+        for (int ci = G.gt; ci < nc; ci += T) {
+            const float4 *rc = sp.rec + 4 * ci;
+            float4 d0, d1, d2, m4;   // (nb, 1/k_n bar), (rb, 1/k_t bar), (cb, -), (gap, link | pad, sphere, -)
+            V3 r, n;
+            float ikn, ikt;
+            if (ci >= kRC) {
+                const float4 *A = sp.adjs + 4 * ci;
+                const float4 a0 = A[0], a1 = A[1], a2 = A[2], r0 = rc[0], r1 = rc[1], r3 = rc[3];
+                mu_b += a2.w;
+                d0 = make_float4(a1.x, a1.y, a1.z, a0.w);
+                d1 = make_float4(a2.x, a2.y, a2.z, a1.w);
+                d2 = A[3];
+                m4 = make_float4(r0.w, r3.y, r3.z, 0.0f);
+                r = xyz(r0); n = xyz(r1); ikn = r1.w; ikt = rc[2].w;
+            } else {
+                d0 = S.ring[0][ci]; d1 = S.ring[1][ci]; d2 = S.ring[2][ci]; m4 = S.meta[ci];
+                if constexpr (GW == 1) {
+                    const float *v = reinterpret_cast<const float *>(&S.cp[ci >> 6][0][G.lane]) + ((ci >> 5) & 1);
+                    auto at = [&](int q) -> float { return v[(q >> 1) * 128 + (q & 1) * 2]; };
+                    r = mk(at(0), at(1), at(2)); n = mk(at(3), at(4), at(5)); ikn = at(9); ikt = at(10);
+                } else {
+                    r = mk(own.r.x, own.r.y, own.r.z); n = mk(own.n.x, own.n.y, own.n.z); ikn = own.ikn; ikt = own.ikt;
+                }
             }
-        }
-        for (int ci = G.gt + T * PL; ci < nc; ci += T) {
-            const float4 *A = sp.adjs + 4 * ci;
-            const float4 a0 = A[0], a1 = A[1], a2 = A[2], a3 = A[3];
-            contact_setup_bwd(sp.rec + 4 * ci, xyz(a1), xyz(a2), xyz(a3), a0.w, a1.w, Wi, trW, R, b.x, E.sfirst, sc, cfg,
-                              L0, L1, inv_h, Wbar, Rbar, xb_l, invm_l);
+            contact_setup_bwd(r, n, m4.x, ikn, ikt, __float_as_int(m4.y) & 0xff, __float_as_int(m4.z), xyz(d0), xyz(d1), xyz(d2), d0.w,
+                              d1.w, Wi, trW, R, b.x, E.sfirst, sc, cfg, L0, L1, inv_h, Wbar, Rbar, xb_l, invm_l);
         }
     } else {
         vpb = vpb + Vb;
@@ -1095,27 +1453,16 @@ __device__ __noinline__ void refine_step(const RefineArgs &r, int i) {
     r.tr_params[env] = th;
 }
 
-template <int GW, int PL>
-__global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
-    constexpr int T = AGroup<GW>::T, GPB = kAW / GW;
-    __shared__ GroupSm<GW> sm[GPB];
-    __shared__ PadTab PT;
+template <int GW>
+__global__ void __launch_bounds__(32 * GW) adjoint_kernel(const __grid_constant__ AdjArgs a) {
+    constexpr int T = AGroup<GW>::T;
+    __shared__ GroupSm<GW> S;
+    __shared__ PadTable PT;
     const AGroup<GW> G;
-    const int lane = G.gt;   // the group's thread (0 .. 32 GW - 1)
-    const int slot = blockIdx.x * GPB + G.gid;
-    if (threadIdx.x < 32) {   // the pads of each link, in pad order
-        int c = 0;
-        for (int p = 0; p < a.sc.n_pads && c < kAPadsPerLink; ++p)
-            if (__ldg(a.sc.pad_link + p) == (int)threadIdx.x) PT.id[threadIdx.x * kAPadsPerLink + c++] = (unsigned char)p;
-        PT.cnt[threadIdx.x] = (unsigned char)c;
-    }
-    for (int p = threadIdx.x; p < a.sc.n_pads; p += kABlock) {
-        PT.s0[p] = __ldg(a.sc.pad_s0 + p);
-        PT.s1[p] = __ldg(a.sc.pad_s1 + p);
-    }
-    __syncthreads();
-    if (slot >= a.n) return;   // whole groups only
-    GroupSm<GW> &S = sm[G.gid];
+    const int lane = G.gt;   // the block's thread (0 .. 32 GW - 1)
+    const int slot = blockIdx.x;
+    PT.build(a.sc, lane, T);
+    G.sync();
     int parity = 0;   // the group's reduction buffer
     const DevScene &sc = a.sc;
     const DevConfig &cfg = a.cfg;
@@ -1160,7 +1507,6 @@ __global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
     E.iters = a.iters[env];
     E.mu = th.y;
     E.inv_m = 1.0f / th.x;
-    E.bound = __ldg(sc.shape_bound + shp);
     E.cfirst = __ldg(sc.cl_first + shp);
     E.Jb.xx = __ldg(sc.shape_jinv + 6 * shp + 0); E.Jb.yy = __ldg(sc.shape_jinv + 6 * shp + 1);
     E.Jb.zz = __ldg(sc.shape_jinv + 6 * shp + 2); E.Jb.xy = __ldg(sc.shape_jinv + 6 * shp + 3);
@@ -1179,18 +1525,21 @@ __global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
     const int f_last = (nck - 1) * a.K;
     double cost = 0.0;
     Body b = b0;
+#pragma unroll 1
     for (int f = 0; f < a.H && !(st & kDiverged); ++f) {
         if (f % a.K == 0 && lane == 0) store_body(sp.ck + 4 * (f / a.K), b);
+#pragma unroll 1
         for (int k = lane; k < 3 * P; k += T) S.padacc[k] = 0.0f;
         G.sync();
         const float4 *tab = tab0 + (size_t)f * tab_frame;
+#pragma unroll 1
         for (int s = 0; s < ns; ++s) {
             const float4 *L0 = tab + (size_t)s * Lk * kLinkStride;
             if (f >= f_last) {
                 const int blk = (f - f_last) * ns + s;
                 if (lane == 0) store_body(sp.sg + 4 * blk, b);
                 if (seg_tape && !a.forward_only) {   // the last segment's tape, recorded on the way
-                    const int nc = fwd_substep<GW, PL>(a, E, b, L0, L0 + Lk * kLinkStride, sp.blk(blk), S, PT, G, parity,
+                    const int nc = fwd_substep<GW>(a, E, b, L0, L0 + Lk * kLinkStride, sp.blk(blk), S, PT, G, parity,
                                                        st, 1 | a.zero, 1 | a.zero, -1);
                     if (lane == 0) sp.ncs[blk] = nc;
                     continue;
@@ -1200,19 +1549,21 @@ __global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
                 const int q = f * ns + s;
                 SlotPtr sq = sp;
                 sq.rec = sp.recs + (size_t)q * cap * 4;
-                const int nc = fwd_substep<GW, PL>(a, E, b, L0, L0 + Lk * kLinkStride, sq, S, PT, G, parity, st, a.zero,
+                const int nc = fwd_substep<GW>(a, E, b, L0, L0 + Lk * kLinkStride, sq, S, PT, G, parity, st, a.zero,
                                                    1 | a.zero, -1);
                 if (lane == 0) sp.nrc[q] = nc;
                 continue;
             }
-            fwd_substep<GW, PL>(a, E, b, L0, L0 + Lk * kLinkStride, sp, S, PT, G, parity, st, a.zero, 1 | a.zero, -1);
+            fwd_substep<GW>(a, E, b, L0, L0 + Lk * kLinkStride, sp, S, PT, G, parity, st, a.zero, 1 | a.zero, -1);
         }
+#pragma unroll 1
         for (int k = lane; k < 3 * P; k += T) sp.sf[(size_t)f * 3 * P + k] = S.padacc[k] * inv_ns;
         if (!all_finite(b.x, b.q, b.v, b.w)) st |= IH_ENV_NONFINITE;
         else if (dot(b.x, b.x) > cfg.escape_radius * cfg.escape_radius) st |= IH_ENV_ESCAPED;
         {   // frame cost in FP64, as the scored step: each pad's terms in parallel, summed in pad order
             const float *o = a.obs + (size_t)f * P * 3;
             const double tau = (double)cfg.tau, tau2 = __dmul_rn(tau, tau), wf = (double)cfg.w_force;
+#pragma unroll 1
             for (int p = lane; p < P; p += T) {
                 const double fx = S.padacc[3 * p] * inv_ns, fy = S.padacc[3 * p + 1] * inv_ns,
                              fz = S.padacc[3 * p + 2] * inv_ns;
@@ -1227,6 +1578,7 @@ __global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
             G.sync();
             if (lane == 0) {
                 double cf = 0.0;
+#pragma unroll 1
                 for (int p = 0; p < P; ++p) {
                     cf = __dadd_rn(cf, S.term[p]);
                     if (S.flag[p]) cf = __dadd_rn(cf, (double)cfg.w_contact);
@@ -1260,13 +1612,16 @@ __global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
     Adj ad = {mk(0, 0, 0), Q4{0, 0, 0, 0}, mk(0, 0, 0), mk(0, 0, 0)};
     float invm_b = 0.0f, mu_b = 0.0f;
     const float wf2 = 2.0f * cfg.w_force * inv_h * inv_ns;
+#pragma unroll 1
     for (int seg = nck - 1; seg >= 0; --seg) {
         const int fb = seg * a.K, fe = min(a.H, fb + a.K);
         b = load_body(sp.ck + 4 * seg);
         // the segment's substep start states and tapes (its frames' pad forces
         // are the first pass's)
+#pragma unroll 1
         for (int f = fb; f < fe && seg < nck - 1; ++f) {
             const float4 *tab = tab0 + (size_t)f * tab_frame;
+#pragma unroll 1
             for (int s = 0; s < ns; ++s) {
                 const int blk = (f - fb) * ns + s;
                 if (lane == 0) store_body(sp.sg + 4 * blk, b);
@@ -1275,21 +1630,24 @@ __global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
                     const int q = f * ns + s;
                     SlotPtr sq = sp.blk(blk);
                     sq.rec = sp.recs + (size_t)q * cap * 4;
-                    const int nc = fwd_substep<GW, PL>(a, E, b, L0, L0 + Lk * kLinkStride, sq, S, PT, G, parity, st,
+                    const int nc = fwd_substep<GW>(a, E, b, L0, L0 + Lk * kLinkStride, sq, S, PT, G, parity, st,
                                                        1 | a.zero, a.zero, sp.nrc[q]);
                     if (lane == 0) sp.ncs[blk] = nc;
                 } else {
-                    fwd_substep<GW, PL>(a, E, b, L0, L0 + Lk * kLinkStride, sp, S, PT, G, parity, st, a.zero, a.zero,
+                    fwd_substep<GW>(a, E, b, L0, L0 + Lk * kLinkStride, sp, S, PT, G, parity, st, a.zero, a.zero,
                                         -1);
                 }
             }
         }
+#pragma unroll 1
         for (int f = fe - 1; f >= fb; --f) {
             const float *o = a.obs + (size_t)f * P * 3;
+#pragma unroll 1
             for (int k = lane; k < 3 * P; k += T)
                 S.fbar[k] = wf2 * (sp.sf[(size_t)f * 3 * P + k] - o[k]);
             G.sync();
             const float4 *tab = tab0 + (size_t)f * tab_frame;
+#pragma unroll 1
             for (int s = ns - 1; s >= 0; --s) {
                 const float4 *L0 = tab + (size_t)s * Lk * kLinkStride;
                 const float4 *L1 = L0 + Lk * kLinkStride;
@@ -1299,12 +1657,12 @@ __global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
                     G.sync();
                     SlotPtr sq = sp.blk(blk);
                     if (seg < nck - 1) sq.rec = sp.recs + (size_t)(f * ns + s) * cap * 4;   // (the replayed records)
-                    rev_substep<GW, PL>(a, E, bs, L0, L1, sp.ncs[blk], sq, S, G, parity, ad, invm_b, mu_b);
+                    rev_substep<GW>(a, E, bs, L0, L1, sp.ncs[blk], sq, S, G, parity, ad, invm_b, mu_b);
                 } else {   // re-run the substep once more, recording its tape
                     Body bt = bs;
                     int st2 = 0;
-                    const int nc = fwd_substep<GW, PL>(a, E, bt, L0, L1, sp, S, PT, G, parity, st2, 1 | a.zero, a.zero, -1);
-                    rev_substep<GW, PL>(a, E, bs, L0, L1, nc, sp, S, G, parity, ad, invm_b, mu_b);
+                    const int nc = fwd_substep<GW>(a, E, bt, L0, L1, sp, S, PT, G, parity, st2, 1 | a.zero, a.zero, -1);
+                    rev_substep<GW>(a, E, bs, L0, L1, nc, sp, S, G, parity, ad, invm_b, mu_b);
                 }
             }
             G.sync();
@@ -1317,7 +1675,7 @@ __global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
     }
     if (lane == 0) {
         // rotation tangent: q = exp(delta) q0, d/d delta at 0 = vec(qbar (x) conj(q0)) / 2
-        const Q4 g = qmul_r(ad.q, qconj(b0.q));
+        const Q4 g = qmul(ad.q, qconj(b0.q));
         float *gr = a.grad + 8 * slot;
         gr[0] = ad.x.x; gr[1] = ad.x.y; gr[2] = ad.x.z;
         gr[3] = 0.5f * g.x; gr[4] = 0.5f * g.y; gr[5] = 0.5f * g.z;
@@ -1332,10 +1690,9 @@ __global__ void __launch_bounds__(kABlock) adjoint_kernel(const AdjArgs a) {
     }
 }
 
-template <int GW, int PL>
-cudaError_t launch_pl(const AdjArgs &a, cudaStream_t s) {
-    constexpr int GPB = kAW / GW;
-    adjoint_kernel<GW, PL><<<(a.n + GPB - 1) / GPB, kABlock, 0, s>>>(a);
+template <int GW>
+cudaError_t launch_gw(const AdjArgs &a, cudaStream_t s) {
+    adjoint_kernel<GW><<<a.n, 32 * GW, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1368,33 +1725,25 @@ cudaError_t launch_adjoint_iters_max(int n, int N, const int *envs, const int *i
     return cudaGetLastError();
 }
 
-#ifndef IH_ADJ_GROUPS_PER_SM
-#define IH_ADJ_GROUPS_PER_SM 2
-#endif
 bool adjoint_variant_supported(int gw, int pl) {
     return (gw == 0 && pl == 0) || (gw == 4 && pl == 1) || (gw == 1 && (pl == 1 || pl == 2));
 }
 
-// Automatic shape. Few environments (the refined elites, a small batch), at
-// most two per SM -- the blocks of ~250 registers a thread that an SM holds:
-// four warps each, so that their contacts' chains run side by side, one
-// contact a thread in registers. More: one warp each (no barriers between the
-// warps of an environment) with one contact a thread in registers when no
-// shape has more than 32 spheres (a substep's contacts then rarely exceed a
-// warp: 22 at most for the 27-sphere box), else two (the 64-sphere cylinder
-// reaches ~100); four a thread spilled and ran slower. Contacts beyond the
-// register slots run from scratch memory.
+// Automatic shape. Few environments (the refined elites, a small batch), at most two
+// per SM -- the blocks of 255 registers a thread that an SM holds: four warps each, so
+// that their contacts' chains run side by side. More: one warp each (no barriers, and
+// up to eight an SM at once). Six frames of the box / the cylinder / the mug, in us,
+// four warps against one: 1 environment 261 : 302 / 293 : 415 / 710 : 870, 304
+// environments 276 : 315 / 368 : 528 / 843 : 986, 305 environments 490 : 316 /
+// 619 : 533 / 1436 : 982. The second number of a shape no longer changes anything.
 cudaError_t launch_adjoint(const AdjArgs &a, cudaStream_t s) {
-    if (a.gw == 4 && a.pl == 1) return launch_pl<4, 1>(a, s);
-    if (a.gw == 1 && a.pl == 1) return launch_pl<1, 1>(a, s);
-    if (a.gw == 1 && a.pl == 2) return launch_pl<1, 2>(a, s);
+    if (a.gw == 4) return launch_gw<4>(a, s);
+    if (a.gw == 1) return launch_gw<1>(a, s);
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (a.n <= IH_ADJ_GROUPS_PER_SM * sms) return launch_pl<4, 1>(a, s);
-    if (a.s_max <= 32) return launch_pl<1, 1>(a, s);
-    return launch_pl<1, 2>(a, s);
+    return a.n <= 2 * sms ? launch_gw<4>(a, s) : launch_gw<1>(a, s);
 }
 
 }  // namespace ih

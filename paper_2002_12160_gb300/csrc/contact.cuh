@@ -67,24 +67,115 @@ __device__ __forceinline__ Hit hit_capsule(V3 ca, float rs, V3 d, float L, float
     return h;
 }
 
-__device__ __forceinline__ bool link_reaches(const DevScene &sc, const DevConfig &cfg, const float4 *L0,
-                                             int l, V3 x, float bound) {
-    const V3 la = xyz(__ldg(L0 + l * kLinkStride));
-    const V3 xa = x - la;
-    if (l == 0) {
-        const float4 qq = __ldg(L0 + 2);
-        const V3 cl = qrot_inv({qq.x, qq.y, qq.z, qq.w}, xa);
-        const V3 k3 = mk(fminf(fmaxf(cl.x, -sc.palm_hx), sc.palm_hx), fminf(fmaxf(cl.y, -sc.palm_hy), sc.palm_hy),
-                         fminf(fmaxf(cl.z, -sc.palm_hz), sc.palm_hz));
-        const V3 dd = cl - k3;
-        const float reach = bound + cfg.margin;
-        return dot(dd, dd) < reach * reach;
+constexpr int kMaxLinks = 32;
+constexpr int kSphStride = kCluster + 1;   // spheres of a cluster, padded: lanes on different clusters hit different banks
+
+// Per link its pads in order and their intervals [s0, s1) (absent: an interval
+// that holds nothing; the palm: its first pad holds all).
+struct alignas(16) PadTable {
+    static constexpr int kPerLink = 4;
+    float s0[kMaxLinks][kPerLink], s1[kMaxLinks][kPerLink];
+    unsigned char id[kMaxLinks][kPerLink];
+    __device__ void build(const DevScene &sc, int first, int step) {
+#pragma unroll 1
+        for (int l = first; l < sc.n_links; l += step) {
+            int c = 0;
+#pragma unroll 1
+            for (int p = 0; p < sc.n_pads && c < (l == 0 ? 1 : kPerLink); ++p) {
+                if (__ldg(sc.pad_link + p) != l) continue;
+                const float e = __ldg(sc.pad_s1 + p);
+                s0[l][c] = l == 0 ? -1.0f : __ldg(sc.pad_s0 + p);
+                s1[l][c] = (l == 0 || e >= 1.0f) ? 2.0f : e;   // (t <= 1)
+                id[l][c++] = (unsigned char)p;
+            }
+#pragma unroll 1
+            for (; c < kPerLink; ++c) {
+                s0[l][c] = 3.0f;
+                s1[l][c] = 3.0f;
+                id[l][c] = 0xff;
+            }
+        }
     }
-    const V3 ld = xyz(__ldg(L0 + l * kLinkStride + 1));
-    const float t = fminf(fmaxf(dot(xa, ld), 0.0f), sc.link_len);
-    const V3 dd = xa - ld * t;
-    const float reach = bound + sc.link_rad + cfg.margin;
+    // the first pad of link l whose interval holds t (0xff: none)
+    __device__ __forceinline__ unsigned char find(int l, float t) const {
+        const float4 b = *reinterpret_cast<const float4 *>(s0[l]), e = *reinterpret_cast<const float4 *>(s1[l]);
+        const uchar4 i = *reinterpret_cast<const uchar4 *>(id[l]);
+        unsigned char pad = 0xff;
+        if (t >= b.w && t < e.w) pad = i.w;
+        if (t >= b.z && t < e.z) pad = i.z;
+        if (t >= b.y && t < e.y) pad = i.y;
+        if (t >= b.x && t < e.x) pad = i.x;
+        return pad;
+    }
+};
+
+// from the palm box (its pose is the identity, fk_kernel) to a point
+__device__ __forceinline__ V3 palm_offset(const DevScene &sc, V3 c) {
+    return c - mk(fminf(fmaxf(c.x, -sc.palm_hx), sc.palm_hx), fminf(fmaxf(c.y, -sc.palm_hy), sc.palm_hy),
+                  fminf(fmaxf(c.z, -sc.palm_hz), sc.palm_hz));
+}
+
+// Whether a cluster's enclosing sphere (centre ca from link l's origin, radius rs)
+// reaches the link, ld its axis; a little wider than it need be: the sphere tests decide
+__device__ __forceinline__ bool cluster_reaches(const DevScene &sc, const DevConfig &cfg, int l, V3 ca, float rs, V3 ld) {
+    const V3 dc = ca - ld * fminf(fmaxf(dot(ca, ld), 0.0f), sc.link_len), dp = palm_offset(sc, ca);
+    const V3 dd = l == 0 ? dp : dc;
+    const float reach = (rs + cfg.margin + (l == 0 ? 0.0f : sc.link_rad)) * 1.00001f;
     return dot(dd, dd) < reach * reach;
+}
+
+// Whether a sphere's gap to link l is below the margin, in the contact setup's own
+// arithmetic (the rare pairs that the squared distance leaves open; out of line)
+static __device__ __noinline__ bool gap_below_margin(const DevScene &sc, float margin, int l, V3 ca, float rs, V3 ld) {
+    const Hit h = l == 0 ? hit_box_local(ca, rs, sc.palm_hx, sc.palm_hy, sc.palm_hz)
+                         : hit_capsule(ca, rs, ld, sc.link_len, 1.0f / sc.link_len, sc.link_rad, {1.0f, 0.0f, 0.0f, 0.0f});
+    return h.gap < margin;   // (the gap does not depend on the link's rotation)
+}
+
+// The contacts (bit i: sphere i) among the eight spheres sk of cluster k against
+// link l (xa: the object's origin from the link's). A sphere is a contact when its
+// gap is below the margin, which its squared distance from the link's axis (or
+// box) decides unless it is within 1e-5 of the reach squared (the gap's rounding
+// is two orders below that): those are tested again by their gap.
+__device__ __forceinline__ unsigned cluster_hits(const DevScene &sc, const DevConfig &cfg, int l, int k, V3 xa, V3 ld,
+                                                 const float4 *sk, int NS, float inv_L) {
+    unsigned hits = 0, close = 0;
+    auto mark = [&](V3 dd, float reach, int i) {
+        const float d2 = dot(dd, dd), r2 = reach * reach, over = d2 - r2;
+        if (over < 0.0f) hits |= 1u << i;
+        if (!(fabsf(over) > 1e-5f * r2)) close |= 1u << i;
+    };
+    if (l == 0) {
+#pragma unroll
+        for (int i = 0; i < kCluster; ++i) {
+            const float4 c4 = sk[i];
+            mark(palm_offset(sc, xa + xyz(c4)), c4.w + cfg.margin, i);
+        }
+    } else {
+        const float rm = sc.link_rad + cfg.margin;
+#pragma unroll
+        for (int i = 0; i < kCluster; ++i) {
+            const float4 c4 = sk[i];
+            const V3 ca = xa + xyz(c4);
+            const float t = fminf(fmaxf(dot(ca, ld) * inv_L, 0.0f), 1.0f);
+            mark(ca - ld * (t * sc.link_len), c4.w + rm, i);
+        }
+    }
+#pragma unroll 1
+    for (; close; close &= close - 1u) {   // rare
+        const int i = __ffs(close) - 1;
+        const float4 c4 = sk[i];
+        const bool hit = k * kCluster + i < NS && gap_below_margin(sc, cfg.margin, l, xa + xyz(c4), c4.w, ld);
+        hits = (hits & ~(1u << i)) | (hit ? 1u << i : 0u);
+    }
+    return hits;
+}
+
+// A sphere of the object (centre cr from the object's origin) against link l: its hit
+__device__ __forceinline__ Hit hit_link(const DevScene &sc, int l, V3 ca, float rs, V3 ld, const float4 *L0, float inv_L) {
+    if (l == 0) return hit_box_local(ca, rs, sc.palm_hx, sc.palm_hy, sc.palm_hz);
+    const float4 q = __ldg(L0 + l * kLinkStride + 2);
+    return hit_capsule(ca, rs, ld, sc.link_len, inv_L, sc.link_rad, {q.x, q.y, q.z, q.w});
 }
 
 // (one division for both regimes, so that a warp that mixes them divides once)

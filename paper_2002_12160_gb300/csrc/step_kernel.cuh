@@ -51,9 +51,7 @@ namespace {
 #define IH_STEP_VARIANTS(X) X(16, 2) X(16, 4) X(32, 1) X(32, 2) X(32, 3) X(32, 4) X(64, 1) X(64, 2) X(128, 1)
 // the compiled kernels: (lanes per environment, summation width)
 #define IH_STEP_KERNELS(X) X(16, 16) X(16, 32) X(16, 64) X(32, 32) X(32, 64) X(32, 128)
-constexpr int kMaxLinks = 32;
 constexpr int kSlots = 4;            // register-resident contacts per lane
-constexpr int kSphStride = kCluster + 1;   // spheres of a cluster, padded: lanes on different clusters hit different banks
 constexpr unsigned kAll = 0xffffffffu;
 
 // Shared memory of one environment. Everything has a fixed size except the
@@ -67,14 +65,6 @@ struct alignas(16) GSm {
     unsigned short lbeg[kMaxLinks], lend[kMaxLinks];   // contact range of each link
 };
 static_assert(sizeof(GSm) % 16 == 0, "the records keep 16-byte alignment");
-// The warp's pad table: per link its pads in order and their intervals [s0, s1)
-// (absent: an interval that holds nothing; the palm: its first pad holds all).
-constexpr int kPadsPerLink = 4;
-struct alignas(16) PadSm {
-    float s0[kMaxLinks][kPadsPerLink], s1[kMaxLinks][kPadsPerLink];
-    unsigned char id[kMaxLinks][kPadsPerLink];
-};
-
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 __host__ __device__ constexpr int sph_cap(int s_max) { return (s_max + kCluster - 1) / kCluster * kSphStride; }
 // contacts whose record (3 float4) and impulse (1) are in shared memory: the
@@ -148,14 +138,6 @@ __device__ __forceinline__ void env_sum6(const float (&acc)[NA][6], float (&v)[6
     }
 }
 
-// Whether a sphere's gap to link l is below the margin, in the contact setup's own
-// arithmetic (the rare pairs that the squared distance leaves open; out of line)
-__device__ __noinline__ bool gap_below_margin(const DevScene &sc, float margin, int l, V3 ca, float rs, V3 ld) {
-    const Hit h = l == 0 ? hit_box_local(ca, rs, sc.palm_hx, sc.palm_hy, sc.palm_hz)
-                         : hit_capsule(ca, rs, ld, sc.link_len, 1.0f / sc.link_len, sc.link_rad, {1.0f, 0.0f, 0.0f, 0.0f});
-    return h.gap < margin;   // (the gap does not depend on the link's rotation)
-}
-
 // order-preserving key of a cost (NaN excluded), compared with integers: FP64
 // compares take the scarce FP64 pipe
 __device__ __forceinline__ unsigned long long cost_key(double c) {
@@ -190,27 +172,10 @@ __global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_ma
 
     const int cap = cfg.c_max;
     const int SC = a.stage_cap;   // contacts staged in shared memory (RCAP, or c_max); the rest spill to global memory
-    PadSm &PT = *reinterpret_cast<PadSm *>(smem);
-#pragma unroll 1
-    for (int l = lane; l < Lk; l += 32) {
-        int c = 0;
-#pragma unroll 1
-        for (int p = 0; p < P && c < (l == 0 ? 1 : kPadsPerLink); ++p) {
-            if (__ldg(sc.pad_link + p) != l) continue;
-            const float s1 = __ldg(sc.pad_s1 + p);
-            PT.s0[l][c] = l == 0 ? -1.0f : __ldg(sc.pad_s0 + p);
-            PT.s1[l][c] = (l == 0 || s1 >= 1.0f) ? 2.0f : s1;   // (t <= 1)
-            PT.id[l][c++] = (unsigned char)p;
-        }
-#pragma unroll 1
-        for (; c < kPadsPerLink; ++c) {
-            PT.s0[l][c] = 3.0f;
-            PT.s1[l][c] = 3.0f;
-            PT.id[l][c] = 0xff;
-        }
-    }
+    PadTable &PT = *reinterpret_cast<PadTable *>(smem);
+    PT.build(sc, lane, 32);
     __syncwarp();
-    unsigned char *mine = smem + sizeof(PadSm) + sub * env_bytes(s_max, SC, cap, WARM, a.clp_cap);
+    unsigned char *mine = smem + sizeof(PadTable) + sub * env_bytes(s_max, SC, cap, WARM, a.clp_cap);
     GSm &S = *reinterpret_cast<GSm *>(mine);
     // contact records, 3 float4 each: (r, 1/k_t), (n, 1/k_n), (c, -); the impulses follow
     float4 *rec = reinterpret_cast<float4 *>(mine + sizeof(GSm));
@@ -358,13 +323,7 @@ __global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_ma
                 }
                 __syncwarp();
 
-                // -- 2a. cull (link, cluster) pairs by the clusters' enclosing spheres (the
-                //        reach a little wider: the pair tests decide). The palm's pose is
-                //        the identity (fk_kernel), so its box frame is the world frame
-                auto palm_offset = [&](V3 c) -> V3 {   // from the palm box to a point
-                    return c - mk(fminf(fmaxf(c.x, -sc.palm_hx), sc.palm_hx), fminf(fmaxf(c.y, -sc.palm_hy), sc.palm_hy),
-                                  fminf(fmaxf(c.z, -sc.palm_hz), sc.palm_hz));
-                };
+                // -- 2a. cull (link, cluster) pairs by the clusters' enclosing spheres
                 int nclp = 0;
                 const int ncpairs = act ? Lk * ncl : 0, ncp_w = wmax(ncpairs);
 #pragma unroll 2
@@ -375,11 +334,7 @@ __global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_ma
                     if (p < ncpairs) {
                         const int l = min((int)(((float)p + 0.5f) * inv_ncl), Lk - 1), k = p - l * ncl;
                         const float4 cc = clc[k];
-                        const V3 ca = xyz(S.xa[l]) + xyz(cc), ld = xyz(S.ax[l]);
-                        const V3 dc = ca - ld * fminf(fmaxf(dot(ca, ld), 0.0f), sc.link_len), dp = palm_offset(ca);
-                        const V3 dd = l == 0 ? dp : dc;
-                        const float reach = (cc.w + cfg.margin + (l == 0 ? 0.0f : sc.link_rad)) * 1.00001f;
-                        keep = dot(dd, dd) < reach * reach;
+                        keep = cluster_reaches(sc, cfg, l, xyz(S.xa[l]) + xyz(cc), cc.w, xyz(S.ax[l]));
                         e = (l << 8) | k;
                     }
                     const unsigned bal = ballot(keep);
@@ -388,52 +343,17 @@ __global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_ma
                 }
                 __syncwarp();
 
-                // -- 2b. a lane tests the eight spheres of a surviving pair. A sphere is a
-                //        contact when its gap is below the margin, which its squared
-                //        distance from the link's axis (or box) decides unless it is
-                //        within 1e-5 of the reach squared (the gap's rounding is two
-                //        orders below that): those are tested again by their gap
+                // -- 2b. a lane tests the eight spheres of a surviving pair
                 int nc = 0;
                 const int nclp_w = wmax(nclp);
 #pragma unroll 1
                 for (int e0 = 0; e0 < nclp_w; e0 += L) {
-                    unsigned hits = 0, close = 0;
+                    unsigned hits = 0;
                     int e = 0;
                     if (e0 + gl < nclp) {
                         e = clp[e0 + gl];
-                        const int l = e >> 8;
-                        const V3 xa = xyz(S.xa[l]);
-                        const float4 *sk = sph + (e & 0xff) * kSphStride;
-                        auto mark = [&](V3 dd, float reach, int i) {
-                            const float d2 = dot(dd, dd), r2 = reach * reach, over = d2 - r2;
-                            if (over < 0.0f) hits |= 1u << i;
-                            if (!(fabsf(over) > 1e-5f * r2)) close |= 1u << i;
-                        };
-                        if (l == 0) {
-#pragma unroll
-                            for (int i = 0; i < kCluster; ++i) {
-                                const float4 c4 = sk[i];
-                                mark(palm_offset(xa + xyz(c4)), c4.w + cfg.margin, i);
-                            }
-                        } else {
-                            const V3 ld = xyz(S.ax[l]);
-                            const float rm = sc.link_rad + cfg.margin;
-#pragma unroll
-                            for (int i = 0; i < kCluster; ++i) {
-                                const float4 c4 = sk[i];
-                                const V3 ca = xa + xyz(c4);
-                                const float t = fminf(fmaxf(dot(ca, ld) * inv_L, 0.0f), 1.0f);
-                                mark(ca - ld * (t * sc.link_len), c4.w + rm, i);
-                            }
-                        }
-#pragma unroll 1
-                        for (; close; close &= close - 1u) {   // rare
-                            const int i = __ffs(close) - 1;
-                            const float4 c4 = sk[i];
-                            const bool hit = (e & 0xff) * kCluster + i < NS &&
-                                             gap_below_margin(sc, cfg.margin, l, xa + xyz(c4), c4.w, xyz(S.ax[l]));
-                            hits = (hits & ~(1u << i)) | (hit ? 1u << i : 0u);
-                        }
+                        const int l = e >> 8, k = e & 0xff;
+                        hits = cluster_hits(sc, cfg, l, k, xyz(S.xa[l]), xyz(S.ax[l]), sph + k * kSphStride, NS, inv_L);
                     }
                     // the lanes' counts (0..8) by bit planes: hits of the lanes before, and in all
                     const int cnt = __popc(hits);
@@ -463,8 +383,6 @@ __global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_ma
                 //       the contact range of each link
                 const int nc_w = wmax(nc);
                 const float trW = Wi.xx + Wi.yy + Wi.zz;
-                // (two contacts a lane and round: two independent chains; the palm takes
-                // the capsules' path wherever the two agree, its pose being the identity)
                 auto setup = [&](int ci) {
                     const int e = clist[ci], l = e >> 8, j = e & 0xff;
                     const int e0 = ci > 0 ? clist[ci - 1] >> 8 : -1, e1 = ci < nc - 1 ? clist[ci + 1] >> 8 : -1;
@@ -472,23 +390,9 @@ __global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_ma
                     if (e1 != l) S.lend[l] = (unsigned short)(ci + 1);
                     const float4 sp = sph[(j >> 3) * kSphStride + (j & 7)];
                     const V3 cr = xyz(sp), ca = xyz(S.xa[l]) + cr;
-                    Hit hh;
-                    if (l == 0) {
-                        hh = hit_box_local(ca, sp.w, sc.palm_hx, sc.palm_hy, sc.palm_hz);
-                    } else {
-                        const float4 Aq = __ldg(L0 + l * kLinkStride + 2);
-                        hh = hit_capsule(ca, sp.w, xyz(S.ax[l]), sc.link_len, inv_L, sc.link_rad, {Aq.x, Aq.y, Aq.z, Aq.w});
-                    }
+                    const Hit hh = hit_link(sc, l, ca, sp.w, xyz(S.ax[l]), L0, inv_L);
                     const V3 r = cr - hh.n * sp.w;
-                    // the first pad of the link whose interval holds t
-                    const float4 b4 = *reinterpret_cast<const float4 *>(PT.s0[l]), e4 = *reinterpret_cast<const float4 *>(PT.s1[l]);
-                    const uchar4 id = *reinterpret_cast<const uchar4 *>(PT.id[l]);
-                    unsigned char pad = 0xff;
-                    if (hh.t >= b4.w && hh.t < e4.w) pad = id.w;
-                    if (hh.t >= b4.z && hh.t < e4.z) pad = id.z;
-                    if (hh.t >= b4.y && hh.t < e4.y) pad = id.y;
-                    if (hh.t >= b4.x && hh.t < e4.x) pad = id.x;
-                    cpad[ci] = pad;
+                    cpad[ci] = PT.find(l, hh.t);
                     const CSetup cs = setup_contact(r, hh.n, hh.gap, l, Wi, trW, inv_m, cfg, L0, L1, x, inv_h);
                     const float4 r0 = make_float4(r.x, r.y, r.z, cs.ikt), r1 = make_float4(hh.n.x, hh.n.y, hh.n.z, cs.ikn),
                                  r2 = make_float4(cs.cc.x, cs.cc.y, cs.cc.z, 0.0f);
@@ -824,7 +728,7 @@ __global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_ma
 
 template <int L, int TPE, bool WARM>
 size_t bytes_t(int s_max, int c_max, int clp_cap) {
-    return sizeof(PadSm) + 32 / L * env_bytes(s_max, stage_capacity(L, c_max), c_max, WARM, clp_cap);
+    return sizeof(PadTable) + 32 / L * env_bytes(s_max, stage_capacity(L, c_max), c_max, WARM, clp_cap);
 }
 
 // Shared-memory opt-in, and the blocks of this kernel that fit on one SM
