@@ -484,9 +484,10 @@ ih_status cost_eval_static(const float *forces, const float *obs, const int32_t 
  * Coulomb disk of radius L takes the derivative of z smin(|z|, L)/|z| with
  * smin(a, b) = (a + b - sqrt((a - b)^2 + (width b)^2)) / 2. Contact
  * membership, capsule end clamps, palm face choice and bias regimes are held
- * fixed. The state after every checkpoint_every-th frame is kept; the
- * reverse sweep recomputes the forward between checkpoints and, per substep,
- * once more with a record of the Jacobi iterations.
+ * fixed. The state after every checkpoint_every-th frame (or a longer segment,
+ * sim_set_adjoint_memory) is kept; the reverse sweep recomputes the forward
+ * between checkpoints with a record of the Jacobi iterations, except in the last
+ * segment, whose record the first pass makes.
  *
  * obs        device float[horizon][P][3]  observed pad forces of each frame
  * envs       device int32[n] or NULL      environments to differentiate
@@ -503,9 +504,10 @@ ih_status cost_eval_static(const float *forces, const float *obs, const int32_t 
  * grad_quat  device float[n][4] or NULL   dL/d(q_w, q_x, q_y, q_z) of the
  *                                         initial quaternion's components
  *
- * Scratch: the handle grows a buffer of about (16 c_max (iters + 6) + 16
- * (horizon / checkpoint_every + 2 checkpoint_every substeps)) floats per
- * selected environment and keeps it until sim_destroy. Synchronises the stream
+ * Scratch: the handle grows a buffer and keeps it until sim_destroy: of about
+ * 4 c_max (iters + 4) floats for each substep taped (a segment's, within
+ * sim_set_adjoint_memory, else one), plus 16 c_max for each other substep of the
+ * horizon, per selected environment. Synchronises the stream
  * once to size it (the largest iteration count among the selected
  * environments is read back), so the call cannot be captured in a graph.
  * Errors: IH_ERR_ARG (frames without commands, n or a constant out of range,
@@ -516,13 +518,15 @@ ih_status sim_adjoint(ih_sim *sim, int32_t frame0, int32_t horizon, int32_t chec
 
 /* Memory the adjoint may use to keep the tape (the Jacobi impulses of every
  * iteration) of all substeps of a checkpoint segment at once, in bytes
- * (default 16 GiB). Within the budget each substep of the forward is run twice
- * per gradient (the pass that computes the cost and checkpoints, and the
- * segment's recomputation, which records the tape); beyond it the tape of a
- * single substep is kept and each substep runs a third time just before its
- * reverse sweep. Results are the same bit for bit. 0 always takes the
- * smaller mode. Not a passage of the paper: a memory/time trade of this
- * library's checkpointing. */
+ * (default 16 GiB). Within the budget, the substeps of the last segment run once
+ * per gradient and the others twice (the pass that computes the cost and
+ * checkpoints, and the segment's recomputation, which records the tape), so
+ * segments longer than checkpoint_every are taken when they fit it (and half of
+ * the device's free memory), up to the whole horizon in one; when not even
+ * checkpoint_every's fit, the tape of a single substep is kept and each substep
+ * runs once more just before its reverse sweep. Results are the same bit for bit.
+ * 0 always takes the smallest mode. Not a passage of the paper: a memory/time trade
+ * of this library's checkpointing. */
 ih_status sim_set_adjoint_memory(ih_sim *sim, uint64_t bytes);
 
 /* The adjoint kernel's shape for sim_adjoint and sim_refine_elites: warps

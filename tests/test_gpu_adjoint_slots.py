@@ -1,10 +1,10 @@
-"""The adjoint at the edges of its register slots.
+"""The adjoint at the edges of its register slots and of its tape's memory.
 
 One warp per environment holds 32, 64, 96 or 128 contacts in 1 to 4 slots a lane and
 the rest in memory; four warps hold one contact a thread, on as many warps as carry
 contacts. Both are within 1e-3 per block (with an absolute floor of 1e-3 of the
 environment's largest block) of the same exact gradient, so they are within twice
-that of each other."""
+that of each other. A tape kept whole, by segments or by substeps gives the same bits."""
 import numpy as np
 import pytest
 
@@ -54,3 +54,19 @@ def test_slot_counts_agree_between_warp_counts():
         if c4[i] > 0:
             classes.add(min(int(np.ceil(most[i] / 32)), 5))
     assert len(classes) >= 4, classes   # one to four slots, or memory
+
+
+@pytest.mark.parametrize("shape", [(4, 1), (1, 1)])
+def test_tape_memory_does_not_change_the_results(shape):
+    n, warm, H = 8, 12, 6
+    wl, sim = _started(n, warm, warm + H + 1)
+    sim.sim_set_adjoint_variant(*shape)
+    obs = torch.zeros((H, wl.scene.n_pads, 3), dtype=torch.float32, device=dev())
+    ref = None
+    # from a substep at a time (none fits) over every number of segments to the whole horizon
+    for budget in [0, *(n * 250_000 * k for k in range(1, 16)), 16 << 30]:
+        sim.sim_set_adjoint_memory(budget)
+        for K in (1, 4):
+            c, g, q = sim.sim_adjoint(warm, obs, checkpoint_every=K, want_quat=True)
+            ref = ref or (c, g, q)
+            assert all(torch.equal(a, b) for a, b in zip(ref, (c, g, q))), (budget, K)
