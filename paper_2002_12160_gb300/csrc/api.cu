@@ -85,7 +85,6 @@ struct ih_sim {
     float4 *pad_pose = nullptr;         // [N][P][2]
     float4 *slip = nullptr;             // [N][P]
     float *sn_qj = nullptr, *sn_qdj = nullptr;
-    int pd_grid = 0;
     // captured tracking window (replayed by sim_track_window)
     cudaGraphExec_t win_exec = nullptr;
     cudaStream_t cap_stream = nullptr;          // private stream: capture and replay
@@ -393,10 +392,7 @@ ih_status sim_create(const ih_scene *sc, const ih_config *cfg, uint64_t seed, vo
     }
     s->clp_cap = (1 + 4 * sc->n_fingers) * ((s->s_max + 7) / 8);
     if (e == cudaSuccess) e = use_variant(s, s->variant);
-    if (e == cudaSuccess && s->pd) {
-        e = pd_step_prepare(s->s_max, s->cfg.c_max);
-        s->pd_grid = pd_step_grid(N, s->sms);
-    }
+    if (e == cudaSuccess && s->pd) e = pd_step_prepare(s->s_max, s->cfg.c_max);
     if (e != cudaSuccess) {
         ih_status r = cuda_fail(nullptr, e, "sim_create step setup");
         sim_destroy(s);
@@ -531,7 +527,7 @@ ih_status sim_step(ih_sim *s, int32_t frame0, int32_t n_frames) {
         p.work = s->work;
         p.fo_q = nullptr; p.fo_pp = nullptr; p.fo_forces = nullptr; p.fo_slip = nullptr; p.fo_status = nullptr;
         p.pose_frames = nullptr;
-        cudaError_t e = launch_pd_step(p, s->pd_grid, s->s_max, s->stream);
+        cudaError_t e = launch_pd_step(p, s->s_max, s->stream);
         if (e != cudaSuccess) return cuda_fail(s, e, "PD step launch");
         s->stepped = true;
         return IH_OK;
@@ -735,7 +731,7 @@ ih_status sim_step_frames_full(ih_sim *s, int32_t frame0, int32_t T, const float
     p.work = s->work;
     p.fo_q = s->fo_q; p.fo_pp = s->fo_pp; p.fo_forces = s->fo_forces; p.fo_slip = s->fo_slip;
     p.fo_status = s->fo_status; p.pose_frames = s->wf_pose;
-    e = launch_pd_step(p, s->pd_grid, s->s_max, s->stream);
+    e = launch_pd_step(p, s->s_max, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "PD step launch");
     FramesCostArgs c;
     c.N = s->cfg.n_envs; c.P = s->n_pads; c.D = s->n_joints; c.T = T; c.cfg = s->dcfg;

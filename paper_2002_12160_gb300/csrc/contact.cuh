@@ -221,33 +221,17 @@ __device__ __forceinline__ CSetup setup_contact(V3 r, V3 n, float gap, int l, co
     return c;
 }
 
-// One projected Jacobi update of a contact's impulse against the body
-// velocity (vv, ww): scalar normal step clamped at zero, scalar tangential
-// step clamped radially to the Coulomb disk, relaxed by 1/n_c. The disk clamp
-// is a select, not a branch, so that the sliding and the sticking lanes of a
-// warp stay in one stretch of code (the same values bit for bit; steps 2-6 %
-// faster).
-__device__ __forceinline__ V3 update_contact(V3 lam, V3 r, V3 n, V3 cc, float ikn, float ikt, V3 vv, V3 ww,
-                                             float mu, float inv_nc) {
-    const V3 u = vv + cross(ww, r) - cc;
-    const float un = dot(u, n);
-    const float l_old = dot(lam, n);
-    const float ln = fmaxf(l_old - un * ikn, 0.0f);
-    const V3 lt = (lam - n * l_old) - (u - n * un) * ikt;
-    const float tn2 = dot(lt, lt);
-    const float lim = mu * ln;
-    const bool slip = tn2 > lim * lim;
-    const float sc = lim * rsqrtf(slip ? tn2 : 1.0f);
-    const float f = slip ? sc : 1.0f;
-    const V3 lp = {prod_add(n.x, ln, lt.x, f), prod_add(n.y, ln, lt.y, f), prod_add(n.z, ln, lt.z, f)};
-    return lam + (lp - lam) * inv_nc;
-}
-
-// The same update on one contact (T = float) or on two at once (T = float2, the
-// packed FP32 instructions: half the issue slots of two scalar updates, and two
-// chains that interleave), bit for bit update_contact's: every operation is the
-// scalar one of each half, and a product's sign may move (rounding is
-// symmetric). Two contacts cost ~70 issue slots instead of ~130; an iteration
+// One projected Jacobi update of a contact's impulse lam against the body velocity
+// (v, w): scalar normal step clamped at zero, scalar tangential step clamped
+// radially to the Coulomb disk, relaxed by 1/n_c:
+//   u = v + w x r - c,  l_n = max(lam . n - (u . n) / k_n, 0),
+//   l_t = (lam - n (lam . n)) - (u - n (u . n)) / k_t, scaled to mu l_n where longer,
+//   lam += (n l_n + l_t - lam) / n_c,
+// with a fixed contraction. The disk clamp is a select, not a branch, so that the
+// sliding and the sticking lanes of a warp stay in one stretch of code. On one
+// contact (T = float) or on two at once (T = float2, the packed FP32 instructions:
+// half the issue slots of two scalar updates, and two chains that interleave): every
+// operation is the scalar one of each half. Two contacts cost ~70 issue slots instead of ~130; an iteration
 // of a 60-contact environment at 16 warps per SM took 258 cycles a warp scalar,
 // 198 packed. The reciprocal square root is taken of the argument scaled by
 // 2^24, which no FP32 value leaves denormal, so the approximate instruction

@@ -333,8 +333,7 @@ struct FramesCostArgs {
 cudaError_t launch_frames_cost_full(const FramesCostArgs &a, cudaStream_t s);
 size_t pd_step_smem_bytes(int s_max, int c_max);
 cudaError_t pd_step_prepare(int s_max, int c_max);
-int pd_step_grid(int N, int sms);
-cudaError_t launch_pd_step(const PdArgs &a, int grid, int s_max, cudaStream_t s);
+cudaError_t launch_pd_step(const PdArgs &a, int s_max, cudaStream_t s);
 cudaError_t launch_hand_rest(int N, int D, const float *q0, float *qj, float *qdj, cudaStream_t s);
 
 // A step shape (group, cpl) as the interface names it -- group, the width of the
