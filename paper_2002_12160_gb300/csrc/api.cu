@@ -23,7 +23,7 @@ struct ih_sim {
     DevConfig dcfg{};
     uint64_t seed = 0;
     cudaStream_t stream = nullptr;
-    StepVariant variant{32, 4, 32};
+    StepVariant variant{32, 4, 32, kManyBlocks};
     int step_grid = 0;
     int s_max = 1;   // most spheres in one shape
     int sms = 1;     // SMs of the device
@@ -101,7 +101,7 @@ struct ih_sim {
     double *fo_terms = nullptr;
     int fo_T = 0;
     int frames_T = 0;               // frames of the last sim_step_frames call, not yet scored
-    StepVariant win_variant{0, 0, 0};
+    StepVariant win_variant{0, 0, 0, 0};
     ih_opt_config win_opt{};
     // host bookkeeping
     std::vector<char> frame_ready;   // commands uploaded for frame f
@@ -168,7 +168,7 @@ DevScene dev_scene(const ih_sim *s) {
 }
 
 // Default step-kernel shape before any autotuning.
-StepVariant default_variant(int N) { return N <= 4096 ? StepVariant{64, 2, 0} : StepVariant{32, 2, 0}; }
+StepVariant default_variant(int N) { return N <= 4096 ? StepVariant{64, 2, 0, 0} : StepVariant{32, 2, 0, 0}; }
 
 // The lanes of a warp that execute an environment (the results do not depend on
 // them). A whole warp by default; two environments to a warp for the 16-wide
@@ -184,6 +184,19 @@ int step_lanes(int group, int N, int s_max, int sms) {
     return s_max <= 32 && N > 12 * sms ? 16 : 32;
 }
 
+// The warps that an SM holds by registers: fewer, with all that a lane's four contact
+// slots need (about 200 instead of 128, which spill), when no more run anyway, and
+// for shapes of more than 128 spheres, whose environments with contacts past the
+// slots are several times slower than the others and end the launch. Otherwise more
+// warps beat fewer spills. Few : many, us by sim_step: 1024 cylinders, six frames,
+// 222 : 249; 1500 cylinders 306 : 334; 2500 boxes (1250 warps), ten frames, 275 : 285; 2048
+// cylinders 440 : 411; 4096 boxes, six frames, 290 : 240; 8192 mugs, two frames,
+// 1013 : 944; mixed shapes (up to 256 spheres), six frames: 2000 of them 377 : 431,
+// 8192 of them 867 : 883.
+int step_per_sm(int blocks, int s_max, int sms) {
+    return blocks <= kFewBlocks * sms || s_max > 128 ? kFewBlocks : kManyBlocks;
+}
+
 // Make v the step shape: shared-memory opt-in, a persistent grid of at most the
 // one-warp blocks that fit on the device at once (they take environments from the
 // launch's work queue), and a spill area for the contacts beyond the shape's
@@ -191,11 +204,12 @@ int step_lanes(int group, int N, int s_max, int sms) {
 // so no launch still uses the old one).
 cudaError_t use_variant(ih_sim *s, StepVariant v) {
     v.lanes = step_lanes(v.group, s->cfg.n_envs, s->s_max, s->sms);
+    const int epb = step_envs_per_block(v);
+    v.per_sm = step_per_sm((s->cfg.n_envs + epb - 1) / epb, s->s_max, s->sms);
     int bps = 0;
     cudaError_t e = step_prepare(v, s->s_max, s->cfg.c_max, s->dcfg.warm != 0, s->clp_cap, &bps);
     if (e != cudaSuccess) return e;
     const int resident = std::max(1, bps) * std::max(1, s->sms);
-    const int epb = step_envs_per_block(v);
     const int grid = std::min((s->cfg.n_envs + epb - 1) / epb, resident);
     const int sc = step_stage_capacity(v, s->cfg.c_max);
     const size_t need = (size_t)grid * epb * (size_t)(s->cfg.c_max - sc) * 4;
@@ -968,7 +982,7 @@ ih_status sim_set_variant(ih_sim *s, int32_t tpe, int32_t cpl) {
     if (!s) return IH_ERR_ARG;
     if (s->pd) return refuse_pd(s, "sim_set_variant");
     if (!step_variant_supported(tpe, cpl)) return fail(s, IH_ERR_ARG, "unsupported step shape %d x %d", tpe, cpl);
-    cudaError_t e = use_variant(s, StepVariant{tpe, cpl, 0});
+    cudaError_t e = use_variant(s, StepVariant{tpe, cpl, 0, 0});
     if (e != cudaSuccess) return cuda_fail(s, e, "set_variant");
     return IH_OK;
 }

@@ -337,13 +337,16 @@ cudaError_t launch_pd_step(const PdArgs &a, int s_max, cudaStream_t s);
 cudaError_t launch_hand_rest(int N, int D, const float *q0, float *qj, float *qdj, cudaStream_t s);
 
 // A step shape (group, cpl) as the interface names it -- group, the width of the
-// solver's sums, alone fixes the results -- and the lanes of a warp that execute
-// an environment (chosen by the library; the results do not depend on them).
+// solver's sums, alone fixes the results -- and, chosen by the library (the results
+// do not depend on them), the lanes of a warp that execute an environment and the
+// warps that an SM holds by registers.
 struct StepVariant {
     int group;
     int cpl;
     int lanes;
+    int per_sm;
 };
+constexpr int kFewBlocks = 10, kManyBlocks = 16;
 constexpr int step_envs_per_block(const StepVariant &v) { return 32 / v.lanes; }
 cudaError_t launch_step(const StepArgs &a, const StepVariant &v, int grid, int s_max, cudaStream_t s);
 bool step_variant_supported(int group, int cpl);

@@ -26,9 +26,9 @@
 // fetch: the loops off the solver are kept rolled). Against groups of 64 (or, in
 // large batches, 32) threads with block barriers, a link cull before the cluster
 // cull, one pair test per thread and guarded scalar slots, sim_step alone: 1024
-// cylinders, ten frames, 421 -> 332 us; 32768 mugs, two frames, 4.50 -> 3.59 ms;
-// 4097 boxes, four frames, 392 -> 144 us; 8192 of mixed shapes, six frames,
-// 969 -> 879 us.
+// cylinders, ten frames, 421 -> 308 us (332 with the registers of 16 warps an SM);
+// 32768 mugs, two frames, 4.49 -> 3.65 ms; 4097 boxes, four frames, 392 -> 144 us;
+// 8192 of mixed shapes, six frames, 969 -> 867 us.
 //
 // A step shape's width TPE (16, 32, 64, 128) fixes the order of the solver's
 // sums and with it every bit of the result: thread t of TPE adds contacts t,
@@ -49,10 +49,15 @@ namespace {
 // the shapes of the interface (summation width, contacts per thread); the
 // second number no longer changes anything: the width alone fixes the result
 #define IH_STEP_VARIANTS(X) X(16, 2) X(16, 4) X(32, 1) X(32, 2) X(32, 3) X(32, 4) X(64, 1) X(64, 2) X(128, 1)
-// the compiled kernels: (lanes per environment, summation width)
-#define IH_STEP_KERNELS(X) X(16, 16) X(16, 32) X(16, 64) X(32, 32) X(32, 64) X(32, 128)
+// the compiled kernels: (lanes per environment, summation width, warps to an SM)
+#define IH_STEP_KERNELS(X) IH_STEP_KERNELS_B(X, kFewBlocks) IH_STEP_KERNELS_B(X, kManyBlocks)
+#define IH_STEP_KERNELS_B(X, B) X(16, 16, B) X(16, 32, B) X(16, 64, B) X(32, 32, B) X(32, 64, B) X(32, 128, B)
 constexpr int kSlots = 4;            // register-resident contacts per lane
 constexpr unsigned kAll = 0xffffffffu;
+template <bool V>
+struct Flag {
+    static constexpr bool value = V;
+};
 
 // Shared memory of one environment. Everything has a fixed size except the
 // contact records, the caches of world-frame centres and the lists, which follow.
@@ -147,9 +152,9 @@ __device__ __forceinline__ unsigned long long cost_key(double c) {
 
 // One warp per block, so that the environments spread evenly over the SMs (an
 // SM holds 6 or 7 of 1024 environments; blocks of two would put 8 on some), and
-// 16 warps to an SM by registers.
-template <int L, int TPE, bool WARM>
-__global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_max) {
+// B warps to an SM by registers (kFewBlocks or kManyBlocks).
+template <int L, int TPE, bool WARM, int B>
+__global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max) {
     static_assert(TPE % L == 0 && TPE / L <= kSlots, "the width's threads are the lanes' accumulators");
     constexpr int EPW = 32 / L, NA = TPE / L, RCAP = kSlots * L;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -517,6 +522,40 @@ __global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_ma
                     // iteration at 1024 cylinders, 80 contacts.) Past its own count an
                     // environment of a 16-lane warp holds still (a step of zero)
                     auto rel = [&](int it) -> float { return (L == 32 || it < iters) ? inv_nc : 0.0f; };
+                    auto iterate4 = [&](auto more) {
+                        Contact<F2> c0, c2;
+                        load2(c0, 0);
+                        load2(c2, 2);
+#pragma unroll 1
+                        for (int it = 0; it < iters_w; ++it) {
+                            float acc[NA][6] = {}, t[6];
+                            const float k = rel(it);
+                            c0.update(vv, ww, mu_s, k);
+                            c2.update(vv, ww, mu_s, k);
+                            add2(acc, c0, 0);
+                            add2(acc, c2, 2);
+                            if constexpr (decltype(more)::value) {
+#pragma unroll 1
+                                for (int s0 = kSlots; s0 * L < nc_w; s0 += NA)   // the further ones, in the same per-thread order
+#pragma unroll
+                                    for (int j = 0; j < NA; ++j) {
+                                        const int ci = (s0 + j) * L + gl;
+                                        if (ci < nc) {
+                                            float4 *g4 = spill_g + (size_t)(ci - RCAP) * 4;
+                                            Contact<float> c;
+                                            unpack(c, g4, g4 + 3);
+                                            c.update(vv, ww, mu_s, k);
+                                            g4[3] = make_float4(c.lam.x, c.lam.y, c.lam.z, 0.0f);
+                                            add1(acc, c, j);
+                                        }
+                                    }
+                            }
+                            env_sum6<L, NA, NA>(acc, t, gl);
+                            body(t);
+                        }
+                        store2(c0, 0);
+                        store2(c2, 2);
+                    };
                     if (nc_w <= L) {
                         Contact<float> c0;
                         load1(c0, 0);
@@ -559,37 +598,10 @@ __global__ void __launch_bounds__(32, 16) step_kernel(const StepArgs a, int s_ma
                         }
                         store2(c0, 0);
                         store1(c2.lam.x, c2.lam.y, c2.lam.z, 2);
+                    } else if (nc_w <= kSlots * L) {
+                        iterate4(Flag<false>{});
                     } else {
-                        Contact<F2> c0, c2;
-                        load2(c0, 0);
-                        load2(c2, 2);
-#pragma unroll 1
-                        for (int it = 0; it < iters_w; ++it) {
-                            float acc[NA][6] = {}, t[6];
-                            const float k = rel(it);
-                            c0.update(vv, ww, mu_s, k);
-                            c2.update(vv, ww, mu_s, k);
-                            add2(acc, c0, 0);
-                            add2(acc, c2, 2);
-#pragma unroll 1
-                            for (int s0 = kSlots; s0 * L < nc_w; s0 += NA)   // the further ones, in the same per-thread order
-#pragma unroll
-                                for (int j = 0; j < NA; ++j) {
-                                    const int ci = (s0 + j) * L + gl;
-                                    if (ci < nc) {
-                                        float4 *g4 = spill_g + (size_t)(ci - RCAP) * 4;
-                                        Contact<float> c;
-                                        unpack(c, g4, g4 + 3);
-                                        c.update(vv, ww, mu_s, k);
-                                        g4[3] = make_float4(c.lam.x, c.lam.y, c.lam.z, 0.0f);
-                                        add1(acc, c, j);
-                                    }
-                                }
-                            env_sum6<L, NA, NA>(acc, t, gl);
-                            body(t);
-                        }
-                        store2(c0, 0);
-                        store2(c2, 2);
+                        iterate4(Flag<true>{});
                     }
                 }
 
@@ -732,14 +744,14 @@ size_t bytes_t(int s_max, int c_max, int clp_cap) {
 }
 
 // Shared-memory opt-in, and the blocks of this kernel that fit on one SM
-template <int L, int TPE, bool WARM>
+template <int L, int TPE, bool WARM, int B>
 cudaError_t prepare_t(int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
     const size_t bytes = bytes_t<L, TPE, WARM>(s_max, c_max, clp_cap);
     cudaError_t e = cudaSuccess;
     if (bytes > 48 * 1024)
-        e = cudaFuncSetAttribute(step_kernel<L, TPE, WARM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        e = cudaFuncSetAttribute(step_kernel<L, TPE, WARM, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess && blocks_per_sm)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, step_kernel<L, TPE, WARM>, 32, bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, step_kernel<L, TPE, WARM, B>, 32, bytes);
     return e;
 }
 
@@ -748,7 +760,9 @@ cudaError_t prepare_t(int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
 // translation unit so the two build in parallel.
 template <bool WARM>
 cudaError_t prepare_w(const StepVariant &v, int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
-#define IH_PREP(L, T) if (v.lanes == L && v.group == T) return prepare_t<L, T, WARM>(s_max, c_max, clp_cap, blocks_per_sm);
+#define IH_PREP(L, T, B)                                       \
+    if (v.lanes == L && v.group == T && v.per_sm == B)         \
+        return prepare_t<L, T, WARM, B>(s_max, c_max, clp_cap, blocks_per_sm);
     IH_STEP_KERNELS(IH_PREP)
 #undef IH_PREP
     return cudaErrorInvalidValue;
@@ -756,9 +770,9 @@ cudaError_t prepare_w(const StepVariant &v, int s_max, int c_max, int clp_cap, i
 
 template <bool WARM>
 cudaError_t launch_w(const StepArgs &a, const StepVariant &v, int grid, int s_max, cudaStream_t s) {
-#define IH_LAUNCH(L, T)                                                                                              \
-    if (v.lanes == L && v.group == T) {                                                                              \
-        step_kernel<L, T, WARM><<<grid, 32, bytes_t<L, T, WARM>(s_max, a.cfg.c_max, a.clp_cap), s>>>(a, s_max);      \
+#define IH_LAUNCH(L, T, B)                                                                                           \
+    if (v.lanes == L && v.group == T && v.per_sm == B) {                                                             \
+        step_kernel<L, T, WARM, B><<<grid, 32, bytes_t<L, T, WARM>(s_max, a.cfg.c_max, a.clp_cap), s>>>(a, s_max);   \
         return cudaGetLastError();                                                                                   \
     }
     IH_STEP_KERNELS(IH_LAUNCH)

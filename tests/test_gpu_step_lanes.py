@@ -1,6 +1,7 @@
-"""The step's results do not depend on the lanes that execute an environment: a
-batch large enough for two environments to a warp against the same environments
-in a small batch (a warp each), bit for bit. The sums' order is fixed by the
+"""The step's results depend neither on the lanes that execute an environment nor on
+the warps that an SM holds: a batch large enough for two environments to a warp
+(box), or for more warps to an SM with fewer registers (box, cylinder), against the
+same environments in a small batch, bit for bit. The sums' order is fixed by the
 shape's width alone, so the tolerance is zero."""
 import dataclasses
 
@@ -29,10 +30,11 @@ def _run(wl, n, shape, frames):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("warm", [False, True])
-@pytest.mark.parametrize("shape", [(16, 2), (32, 2), (64, 2)])
-def test_results_do_not_depend_on_the_lanes(shape, warm):
-    n_big, n_small = 4097, 41   # odd: the last warp holds one environment
-    wl = W.make_workload("tracking_box27", n_envs=n_big, frames=20)
+@pytest.mark.parametrize("name,shape", [("tracking_box27", (16, 2)), ("tracking_box27", (32, 2)), ("tracking_box27", (64, 2)),
+                                        ("tracking_cyl64", (32, 2)), ("tracking_cyl64", (64, 2)), ("tracking_cyl64", (128, 1))])
+def test_results_do_not_depend_on_the_lanes(name, shape, warm):
+    n_big, n_small = 4097, 41   # odd: the last warp of two holds one environment
+    wl = W.make_workload(name, n_envs=n_big, frames=20)
     wl.sim = dataclasses.replace(wl.sim, warm_start=warm)
     big, small = _run(wl, n_big, shape, 20), _run(wl, n_small, shape, 20)
     assert small[-1].abs().max() > 0.01   # the fingers carry force
