@@ -21,10 +21,9 @@ class TrackingCost(torch.autograd.Function):
         sim.sim_set_state(pose.detach().contiguous(), vel.detach().contiguous(), params.detach().contiguous())
         cost, grad, grad_q = sim.sim_adjoint(frame0, obs, checkpoint_every=checkpoint_every, beta=beta,
                                              width=width, want_quat=True)
-        gp = torch.zeros_like(pose)
-        gp[:, 0:3] = grad[:, 0:3]
-        gp[:, 4:8] = grad_q
-        ctx.save_for_backward(gp, grad[:, 6:8].contiguous())
+        # (x, y, z, 0, quaternion): one concatenation
+        gp = torch.cat((grad[:, 0:3], grad_q.new_zeros((grad_q.shape[0], 1)), grad_q), dim=1)
+        ctx.save_for_backward(gp, grad[:, 6:8])
         return cost
 
     @staticmethod
