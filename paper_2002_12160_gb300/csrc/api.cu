@@ -23,6 +23,7 @@ struct ih_sim {
     DevConfig dcfg{};
     uint64_t seed = 0;
     cudaStream_t stream = nullptr;
+    int dev = 0;   // the device the handle was made on
     StepVariant variant{32, 4, 32, kManyBlocks};
     int step_grid = 0;
     int s_max = 1;   // most spheres in one shape
@@ -151,6 +152,32 @@ cudaError_t dalloc(ih_sim *s, T **p, size_t count) {
     return cudaSuccess;
 }
 
+// Device-to-device copies between the handle's arrays and the caller's (null: left
+// out). One launch when every address of the caller's is this device's memory (or
+// managed), which the kernel can reach; copy calls, which take any, otherwise.
+struct Copies {
+    CopyArgs a{};
+    int n = 0;
+    bool here = true;
+    void add(void *dst, const void *src, size_t bytes, const void *caller, int dev) {
+        if (!caller || bytes == 0) return;
+        a.dst[n] = dst;
+        a.src[n] = src;
+        a.bytes[n++] = bytes;
+        cudaPointerAttributes at;
+        const cudaError_t e = cudaPointerGetAttributes(&at, caller);
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        here = here && e == cudaSuccess && ((at.type == cudaMemoryTypeDevice && at.device == dev) || at.type == cudaMemoryTypeManaged);
+    }
+    cudaError_t run(cudaStream_t st) const {
+        if (n == 0) return cudaSuccess;
+        if (here && n > 1) return launch_copies(a, n, st);
+        cudaError_t e = cudaSuccess;
+        for (int k = 0; k < n && e == cudaSuccess; ++k)
+            e = cudaMemcpyAsync(a.dst[k], a.src[k], a.bytes[k], cudaMemcpyDeviceToDevice, st);
+        return e;
+    }
+};
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 bool finite_pos(float v) { return std::isfinite(v) && v > 0.0f; }
 
@@ -403,6 +430,7 @@ ih_status sim_create(const ih_scene *sc, const ih_config *cfg, uint64_t seed, vo
         e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         s->sms = sms > 0 ? sms : 1;
+        s->dev = dev;
     }
     s->clp_cap = (1 + 4 * sc->n_fingers) * ((s->s_max + 7) / 8);
     if (e == cudaSuccess) e = use_variant(s, s->variant);
@@ -502,14 +530,12 @@ ih_status sim_set_state(ih_sim *s, const float *pose, const float *vel, const fl
 ih_status sim_get_state(ih_sim *s, float *pose, float *vel, float *params, int32_t *env_status) {
     if (!s) return IH_ERR_ARG;
     const size_t N = s->cfg.n_envs;
-    cudaError_t e = cudaSuccess;
-    if (pose) e = cudaMemcpyAsync(pose, s->pose, N * 2 * sizeof(float4), cudaMemcpyDeviceToDevice, s->stream);
-    if (e == cudaSuccess && vel)
-        e = cudaMemcpyAsync(vel, s->vel, N * 2 * sizeof(float4), cudaMemcpyDeviceToDevice, s->stream);
-    if (e == cudaSuccess && params)
-        e = cudaMemcpyAsync(params, s->params, N * sizeof(float2), cudaMemcpyDeviceToDevice, s->stream);
-    if (e == cudaSuccess && env_status)
-        e = cudaMemcpyAsync(env_status, s->status, N * sizeof(int), cudaMemcpyDeviceToDevice, s->stream);
+    Copies c;
+    c.add(pose, s->pose, N * 2 * sizeof(float4), pose, s->dev);
+    c.add(vel, s->vel, N * 2 * sizeof(float4), vel, s->dev);
+    c.add(params, s->params, N * sizeof(float2), params, s->dev);
+    c.add(env_status, s->status, N * sizeof(int), env_status, s->dev);
+    const cudaError_t e = c.run(s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "get_state");
     return IH_OK;
 }
@@ -862,11 +888,10 @@ ih_status sim_track_window(ih_sim *s, int32_t frame0, int32_t T, const float *ob
 ih_status sim_read_sensors(ih_sim *s, float *forces, int32_t *env_status) {
     if (!s) return IH_ERR_ARG;
     const size_t N = s->cfg.n_envs;
-    cudaError_t e = cudaSuccess;
-    if (forces)
-        e = cudaMemcpyAsync(forces, s->forces, N * s->n_pads * 3 * sizeof(float), cudaMemcpyDeviceToDevice, s->stream);
-    if (e == cudaSuccess && env_status)
-        e = cudaMemcpyAsync(env_status, s->status, N * sizeof(int), cudaMemcpyDeviceToDevice, s->stream);
+    Copies c;
+    c.add(forces, s->forces, N * s->n_pads * 3 * sizeof(float), forces, s->dev);
+    c.add(env_status, s->status, N * sizeof(int), env_status, s->dev);
+    const cudaError_t e = c.run(s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "read_sensors");
     return IH_OK;
 }
@@ -917,12 +942,11 @@ ih_status sim_read_observation(ih_sim *s, float *q, float *pad_pose, float *slip
     if ((pad_pose && !aligned16(pad_pose)) || (slip && !aligned16(slip)))
         return fail(s, IH_ERR_ARG, "pad_pose and slip must be 16-byte aligned");
     const size_t N = s->cfg.n_envs, P = s->n_pads, D = s->n_joints;
-    cudaError_t e = cudaSuccess;
-    if (q && D > 0) e = cudaMemcpyAsync(q, s->qj, N * D * sizeof(float), cudaMemcpyDeviceToDevice, s->stream);
-    if (e == cudaSuccess && pad_pose)
-        e = cudaMemcpyAsync(pad_pose, s->pad_pose, 2 * N * P * sizeof(float4), cudaMemcpyDeviceToDevice, s->stream);
-    if (e == cudaSuccess && slip)
-        e = cudaMemcpyAsync(slip, s->slip, N * P * sizeof(float4), cudaMemcpyDeviceToDevice, s->stream);
+    Copies c;
+    c.add(q, s->qj, N * D * sizeof(float), q, s->dev);
+    c.add(pad_pose, s->pad_pose, 2 * N * P * sizeof(float4), pad_pose, s->dev);
+    c.add(slip, s->slip, N * P * sizeof(float4), slip, s->dev);
+    const cudaError_t e = c.run(s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "read_observation");
     return IH_OK;
 }
@@ -933,10 +957,11 @@ ih_status sim_set_hand(ih_sim *s, const float *q, const float *qd) {
     const size_t bytes = (size_t)s->cfg.n_envs * s->n_joints * sizeof(float);
     if (bytes == 0) return IH_OK;
     if (!q) return fail(s, IH_ERR_ARG, "q is required");
-    cudaError_t e = cudaMemcpyAsync(s->qj, q, bytes, cudaMemcpyDeviceToDevice, s->stream);
-    if (e == cudaSuccess)
-        e = qd ? cudaMemcpyAsync(s->qdj, qd, bytes, cudaMemcpyDeviceToDevice, s->stream)
-               : cudaMemsetAsync(s->qdj, 0, bytes, s->stream);
+    Copies c;
+    c.add(s->qj, q, bytes, q, s->dev);
+    c.add(s->qdj, qd, bytes, qd, s->dev);
+    cudaError_t e = c.run(s->stream);
+    if (e == cudaSuccess && !qd) e = cudaMemsetAsync(s->qdj, 0, bytes, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "set_hand");
     return IH_OK;
 }
@@ -945,9 +970,10 @@ ih_status sim_get_hand(ih_sim *s, float *q, float *qd) {
     if (!s) return IH_ERR_ARG;
     if (!s->pd) return fail(s, IH_ERR_ARG, "the hand's joints are state only with the PD-driven hand");
     const size_t bytes = (size_t)s->cfg.n_envs * s->n_joints * sizeof(float);
-    cudaError_t e = cudaSuccess;
-    if (q && bytes) e = cudaMemcpyAsync(q, s->qj, bytes, cudaMemcpyDeviceToDevice, s->stream);
-    if (e == cudaSuccess && qd && bytes) e = cudaMemcpyAsync(qd, s->qdj, bytes, cudaMemcpyDeviceToDevice, s->stream);
+    Copies c;
+    c.add(q, s->qj, bytes, q, s->dev);
+    c.add(qd, s->qdj, bytes, qd, s->dev);
+    const cudaError_t e = c.run(s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "get_hand");
     return IH_OK;
 }

@@ -226,6 +226,13 @@ cudaError_t launch_sample_initial(int N, float4 pose0, float4 quat0, float sigma
                                   float m_lo, float m_hi, float mu_lo, float mu_hi, uint64_t seed,
                                   float4 *pose, float4 *vel, float2 *params, int *status,
                                   cudaStream_t s);
+// Up to four arrays copied by one launch (setup.cu)
+struct CopyArgs {
+    void *dst[4];
+    const void *src[4];
+    size_t bytes[4];
+};
+cudaError_t launch_copies(const CopyArgs &a, int n, cudaStream_t s);
 cudaError_t launch_set_state(int N, int n_shapes, const float *pose, const float *vel,
                              const float *params, const int *shape_in, const int *iters_in,
                              float4 *pose_out, float4 *vel_out, float2 *params_out, int *shape,
