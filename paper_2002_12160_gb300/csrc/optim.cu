@@ -36,10 +36,14 @@ constexpr int kFin = 128;             // threads of the finalize kernel
 enum { M_K = 64, M_U, M_ISTAR, M_OK, M_WSUM, M_CMIN, M_SD, M_NFIN, M_NBLK };
 
 // Programmatic dependent launch: the kernels of the update are launched so
-// that each may be scheduled while the one before it drains; each waits here,
+// that each may be scheduled while the one before it runs; each waits here,
 // before its first read of that kernel's results, until it has completed and
-// its writes are visible (at once when launched without the dependency).
+// its writes are visible (at once when launched without the dependency). A kernel
+// completes only after its own wait, so what a kernel's wait returns after is
+// everything before it in the chain.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// ... and lets the next one in the chain start, up to its own wait
+__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*k)(P...), int grid, int block, cudaStream_t s, A... args) {
@@ -142,6 +146,7 @@ __global__ void __launch_bounds__(NT) select_kernel(const OptArgs a) {
     __shared__ unsigned long long s_min_key;
     __shared__ int s_min_idx;
 
+    grid_dependents_launch();
     grid_dependency_wait();
     const int N = a.N, t = threadIdx.x;
     int k = (int)floor((double)a.elite_frac * (double)N);
@@ -361,6 +366,7 @@ __global__ void __launch_bounds__(kOptBlock * kStatWarps) stats_kernel(const Opt
     __shared__ double s_w[kOptBlock];
     __shared__ double s_d[kOptBlock][9];   // (1, offsets): moment q = w e_{a(q)} e_{b(q)}
     __shared__ double tm[kOptBlock][kMoments + 1];
+    grid_dependents_launch();
     grid_dependency_wait();
     const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
     const int j = blockIdx.x * kOptBlock + lane;
@@ -440,6 +446,7 @@ __global__ void __launch_bounds__(kFin) finalize_kernel(const OptArgs a, int nbl
     __shared__ double wtot[32];
     __shared__ double s_carry;
     __shared__ double nm[kMoments];
+    grid_dependents_launch();
     grid_dependency_wait();
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     // up to 32 blocks the first warp scans their weight sums alone (loaded
@@ -562,11 +569,18 @@ constexpr int kApplyLanes = 4;
 
 __global__ void __launch_bounds__(kOptBlock * kApplyLanes) apply_kernel(const OptArgs a) {
     __shared__ double cdf[kCdfSmem];
-    grid_dependency_wait();
     const int sub = threadIdx.x & (kApplyLanes - 1);
-    const int i = blockIdx.x * kOptBlock + (int)(threadIdx.x / kApplyLanes);
+    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) / kApplyLanes);
     const unsigned qmask = 0xfu << (threadIdx.x & 28u);   // this quad's lanes
     const int N = a.N;
+    // the noise needs nothing of the kernels before (the window's update index is
+    // written ahead of its step): formed while they run
+    double e0, e1;
+    {
+        const uint32_t upd = a.win ? a.win->update_index : a.update_index;
+        gauss2(rng_words(a.seed, 1, upd, (uint32_t)i, (uint32_t)sub), e0, e1);
+    }
+    grid_dependency_wait();
     const int k = (int)a.misc[M_K];
     const bool staged = k <= kCdfSmem;
     if (staged) {   // the block's binary searches read the CDF from shared memory
@@ -608,9 +622,6 @@ __global__ void __launch_bounds__(kOptBlock * kApplyLanes) apply_kernel(const Op
         pst = a.status[par];
     }
     if (!ok) return;
-    double e0, e1;
-    const uint32_t upd = a.win ? a.win->update_index : a.update_index;
-    gauss2(rng_words(a.seed, 1, upd, (uint32_t)i, (uint32_t)sub), e0, e1);
     double eps[8];
 #pragma unroll
     for (int b = 0; b < kApplyLanes; ++b) {
@@ -661,7 +672,8 @@ __global__ void __launch_bounds__(kOptBlock * kApplyLanes) apply_kernel(const Op
 // dual is a sum over all of them, and GB300's FP64 rate (1/64 of FP32) made one
 // CTA spend 302 us on the steps of 4096 simulations, with the weights 5 and their
 // CDF 15 more in launches of their own; stepping, scoring and updating 4096 boxes
-// went from 433 to 161 us. The steps search in FP32 and finish in FP64: two or
+// went from 433 to 161 us, and from 140 to 131 us with the snapshot and the draws'
+// noise (FP64) beside this kernel instead of before and after it. The steps search in FP32 and finish in FP64: two or
 // three steps of ~50 FP64 instructions per simulation, spread over the cluster's
 // SMs, which exchange their sums through distributed shared memory.
 constexpr int kSoft = 512;       // threads per CTA
@@ -734,6 +746,7 @@ __global__ void __launch_bounds__(kSoft) soft_weights_kernel(const OptArgs a) {
     const int per = ((N + kSoftCtas - 1) / kSoftCtas + kSoft - 1) / kSoft * kSoft;   // whole chunks
     const int i0 = min(N, rank * per), i1 = min(N, i0 + per);
     int buf = 0;
+    grid_dependents_launch();   // (the draws' noise, formed beside this kernel)
 
     // ---- extremes of the finite costs, their number, and i* = smallest (key, index), on integer keys
     unsigned long long kmin = ~0ull, kmax = 0ull, kbest = ~0ull;
@@ -917,12 +930,14 @@ __global__ void __launch_bounds__(kSoft) soft_weights_kernel(const OptArgs a) {
         *a.argmin_state = istar;
         if (a.argmin_out) *a.argmin_out = istar;
     }
+    grid_dependency_wait();   // the snapshot, which the draws read, ran beside this kernel: complete before it is
     cl.sync();   // no CTA leaves while another reads its shared memory
 }
 
 // The state before the update (one launch instead of a copy per array).
 __global__ void soft_snapshot_kernel(const OptArgs a) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_dependents_launch();
     if (i >= 2 * a.N) return;
     a.sn_pose[i] = a.pose[i];
     a.sn_vel[i] = a.vel[i];
@@ -941,17 +956,21 @@ __global__ void soft_snapshot_kernel(const OptArgs a) {
 // lane one Box-Muller pair of the exploration noise; lane 0 writes the state.
 __global__ void __launch_bounds__(kOptBlock * kApplyLanes) soft_apply_kernel(const OptArgs a) {
     const int sub = threadIdx.x & (kApplyLanes - 1);
-    const int i = blockIdx.x * kOptBlock + (int)(threadIdx.x / kApplyLanes);
+    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) / kApplyLanes);
     const unsigned qmask = 0xfu << (threadIdx.x & 28u);
     const int N = a.N;
-    if (i >= N) return;   // whole quads
     const uint32_t upd = a.win ? a.win->update_index : a.update_index;
+    // the random words and the noise, formed while the weights are
+    double e0, e1;
+    gauss2(rng_words(a.seed, 1, upd, (uint32_t)i, (uint32_t)sub), e0, e1);
+    const uint4 uw = rng_words(a.seed, 3, upd, (uint32_t)i, 0);
+    grid_dependency_wait();
+    if (i >= N) return;   // whole quads
     int par = 0;
     if (sub == 0) {
         if (i == 0) *a.n_window = 0;
         a.c_sum[i] = 0.0;
         if (a.cache_n) a.cache_n[i] = 0;   // replaced: its solver starts cold
-        const uint4 uw = rng_words(a.seed, 3, upd, (uint32_t)i, 0);
         const double pos = unit53(uw.x, uw.y) * a.misc[M_WSUM];
         int lo = 0, hi = N - 1;   // first j with pos < CDF_j
         while (lo < hi) {
@@ -961,8 +980,6 @@ __global__ void __launch_bounds__(kOptBlock * kApplyLanes) soft_apply_kernel(con
         par = lo;
         if (a.parent_out) a.parent_out[i] = par;
     }
-    double e0, e1;
-    gauss2(rng_words(a.seed, 1, upd, (uint32_t)i, (uint32_t)sub), e0, e1);
     double eps[8];
 #pragma unroll
     for (int b = 0; b < kApplyLanes; ++b) {
@@ -1013,6 +1030,12 @@ cudaError_t launch_win_desc(WinDesc *d, WinDesc v, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// The draws' blocks: one warp (eight environments) up to kApplySmall environments, so
+// that few environments spread over the SMs and their scarce FP64 units; four beyond,
+// where every block stages the elites' CDF.
+constexpr int kApplySmall = 4096;
+int apply_block(int N) { return N <= kApplySmall ? 32 : kOptBlock * kApplyLanes; }
+int apply_grid(int N) { return (int)(((size_t)N * kApplyLanes + apply_block(N) - 1) / apply_block(N)); }
 int opt_blocks(int N) { return (N + kOptBlock - 1) / kOptBlock; }
 
 cudaError_t launch_select(const OptArgs &a, cudaStream_t s) {
@@ -1028,26 +1051,28 @@ cudaError_t launch_optimizer(const OptArgs &a, cudaStream_t s) {
         c.gridDim = dim3(kSoftCtas);
         c.blockDim = dim3(kSoft);
         c.stream = s;
-        cudaLaunchAttribute at[1];
+        cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = kSoftCtas;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // beside the snapshot
+        at[1].val.programmaticStreamSerializationAllowed = 1;
         c.attrs = at;
-        c.numAttrs = 1;
-        cudaError_t e = cudaLaunchKernelEx(&c, soft_weights_kernel, a);
-        if (e != cudaSuccess) return e;
-        soft_apply_kernel<<<opt_blocks(a.N), kOptBlock * kApplyLanes, 0, s>>>(a);
-        return cudaGetLastError();
+        c.numAttrs = 2;
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaLaunchKernelEx(&c, soft_weights_kernel, a);
+        if (e == cudaSuccess) e = launch_dependent(soft_apply_kernel, apply_grid(a.N), apply_block(a.N), s, a);
+        return e;
     }
     // the elite count, computed exactly as select_kernel does
     int k = (int)floor((double)a.elite_frac * (double)a.N);
     k = k < 1 ? 1 : (k > a.N ? a.N : k);
-    const int kb = opt_blocks(k), nb = opt_blocks(a.N);
+    const int kb = opt_blocks(k);
     cudaError_t e = a.N <= kKeys * kSelSmall ? launch_dependent(select_kernel<kSelSmall>, 1, kSelSmall, s, a)
                                              : launch_dependent(select_kernel<kSel>, 1, kSel, s, a);
     if (e == cudaSuccess) e = launch_dependent(stats_kernel, kb, kOptBlock * kStatWarps, s, a);
     if (e == cudaSuccess) e = launch_dependent(finalize_kernel, 1, kFin, s, a, kb);
-    if (e == cudaSuccess) e = launch_dependent(apply_kernel, nb, kOptBlock * kApplyLanes, s, a);
+    if (e == cudaSuccess) e = launch_dependent(apply_kernel, apply_grid(a.N), apply_block(a.N), s, a);
     return e;
 }
 
