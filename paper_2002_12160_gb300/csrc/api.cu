@@ -212,16 +212,16 @@ int step_lanes(int group, int N, int s_max, int sms) {
 }
 
 // The warps that an SM holds by registers: fewer, with all that a lane's four contact
-// slots need (about 200 instead of 128, which spill), when no more run anyway, and
+// slots need (160 instead of 128, which spill), when no more run anyway, and
 // for shapes of more than 128 spheres, whose environments with contacts past the
 // slots are several times slower than the others and end the launch. Otherwise more
 // warps beat fewer spills. Few : many, us by sim_step: 1024 cylinders, six frames,
-// 222 : 249; 1500 cylinders 306 : 334; 2500 boxes (1250 warps), ten frames, 275 : 285; 2048
-// cylinders 440 : 411; 4096 boxes, six frames, 290 : 240; 8192 mugs, two frames,
-// 1013 : 944; mixed shapes (up to 256 spheres), six frames: 2000 of them 377 : 431,
-// 8192 of them 867 : 883.
+// 222 : 249; 1500 cylinders 306 : 334, 1800 of them 308 : 343; 2500 boxes (1250
+// warps), ten frames, 275 : 285; 2048 cylinders 440 : 411; 4096 boxes, six frames,
+// 290 : 240; 8192 mugs, two frames, 1013 : 944; mixed shapes (up to 256 spheres), six
+// frames: 2000 of them 377 : 431, 8192 of them 867 : 883.
 int step_per_sm(int blocks, int s_max, int sms) {
-    return blocks <= kFewBlocks * sms || s_max > 128 ? kFewBlocks : kManyBlocks;
+    return blocks <= kFewFit * sms || s_max > 128 ? kFewBlocks : kManyBlocks;
 }
 
 // Make v the step shape: shared-memory opt-in, a persistent grid of at most the

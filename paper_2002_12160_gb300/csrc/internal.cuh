@@ -354,6 +354,7 @@ struct StepVariant {
     int per_sm;
 };
 constexpr int kFewBlocks = 10, kManyBlocks = 16;
+constexpr int kFewFit = 12;   // warps of the kernels compiled for kFewBlocks that an SM holds (160 registers)
 constexpr int step_envs_per_block(const StepVariant &v) { return 32 / v.lanes; }
 cudaError_t launch_step(const StepArgs &a, const StepVariant &v, int grid, int s_max, cudaStream_t s);
 bool step_variant_supported(int group, int cpl);
