@@ -56,7 +56,7 @@ sys.path.insert(0, ROOT)
 #                 (a finger contact's link point velocity, 108 more, is not
 #                 counted: the counters do not tell palm and finger apart)
 #   contact-iter  relative velocity 15, normal and tangential components and
-#                 steps 31, disk clamp 13, relaxation 15 (update_contact, 74);
+#                 steps 31, disk clamp 13, relaxation 15 (the update, 74);
 #                 its moment 9 and the impulse and moment sums 6
 #   env-iter      body velocity from the summed impulses and moments 24
 FLOP_PER_ENV_SUBSTEP = 184     # + 25 per link + 15 per cluster (flops_of)
