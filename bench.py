@@ -45,7 +45,7 @@ sys.path.insert(0, ROOT)
 # kernel reports (pairs tested after culling, contacts, contact-iterations,
 # env-substeps, env-iterations with contacts, (link, cluster) tests):
 #   env-substep   gravity 3, rotation matrix 39, world inverse inertia 81,
-#                 integration with the rotation exponential 61; link cull 25
+#                 integration with the rotation exponential 61; link offset 3
 #                 per link, cluster centre to world 15 per cluster, sphere
 #                 centre to world 15 per sphere
 #   pair tested   sphere to link frame, closest point, gap and normal 34,
@@ -60,7 +60,7 @@ sys.path.insert(0, ROOT)
 #                 its moment 9 and the impulse and moment sums 6
 #   env-iter      body velocity from the summed impulses and moments 24
 FLOP_PER_ENV_SUBSTEP = 184     # + 25 per link + 15 per cluster (flops_of)
-FLOP_PER_LINK = 25
+FLOP_PER_LINK = 3
 FLOP_PER_CLUSTER = 15
 FLOP_PER_SPHERE = 15
 FLOP_PER_PAIR = 41
@@ -73,7 +73,7 @@ FLOP_PER_ENV_ITER = 24
 # profiles/step_kernel_tracking_cyl64.md, valid for the step kernel's own
 # sources (step.cu, step_kernel.cuh, contact.cuh) whose hash is recorded with it; reported as
 # null once they change.
-STEP_TRAFFIC = {"bytes_per_launch": 200192, "sources_sha256": "91521be734c85a5a59a84b2be37a4cf619b2a3268b2665d3306d11e1368d318d"}
+STEP_TRAFFIC = {"bytes_per_launch": 203008, "sources_sha256": "2e27da4b4e54de3a7a9cef1b2b87db77afa9a1452559e945328057c0ca59c279"}
 STEP_SOURCES = ["paper_2002_12160_gb300/csrc/step.cu", "paper_2002_12160_gb300/csrc/step_kernel.cuh",
                 "paper_2002_12160_gb300/csrc/contact.cuh"]
 
@@ -668,7 +668,7 @@ def warm_study(local, seeds=(11, 12, 13, 14, 15, 16), frames=300, n_envs=1024, n
 # Work model of the PD-hand step kernel (step_pd.cu), counted from its source
 # the same way (FMA = 2, a sincos = 20): per env-substep the fingers'
 # kinematics (570 per finger: quaternion chain, link axes, joint axes), the PD
-# prediction (9 per joint), link culling (25 per link) and the object's
+# prediction (9 per joint), link offsets (3 per link) and the object's
 # prediction and inertia (145); per cluster test 25 (centre to world and the
 # reach test); per pair tested 30; per contact the set-up with
 # its joints' share (140) and the pad and slip sums (45); per contact-iteration
@@ -677,7 +677,7 @@ def warm_study(local, seeds=(11, 12, 13, 14, 15, 16), frames=300, n_envs=1024, n
 # them (24 per joint: each joint's contribution and a 4-lane prefix).
 def pd_flops(work, scene, spheres):
     F, D, Lk = scene.n_fingers, scene.n_joints, scene.n_links
-    per_substep = 570 * F + 9 * D + 25 * Lk + 145 + 15 * spheres
+    per_substep = 570 * F + 9 * D + 3 * Lk + 145 + 15 * spheres
     return (work["env_substeps"] * per_substep + work["cluster_tests"] * 25 + work["pairs"] * 30 + work["contacts"] * 185 +
             work["contact_iters"] * 103 + work["env_iters"] * (60 * D + 30))
 

@@ -155,7 +155,7 @@ typedef struct {
 /* Create a simulator for cfg->n_envs environments on the current device.
  * Copies the scene, allocates the handle's device state (poses, velocities,
  * parameters, forces, cost sums, link-pose table, optimizer scratch) and
- * derives each shape's centroid frame, unit inertia and bounding radius on
+ * derives each shape's centroid frame and unit inertia on
  * the GPU. `seed` keys every random stream (Philox4x32-10). `stream` is a
  * cudaStream_t (NULL = legacy default stream). Errors: IH_ERR_ARG for a bad
  * scene or config, IH_ERR_OOM, IH_ERR_CUDA. Passage: Sec. III-B (K

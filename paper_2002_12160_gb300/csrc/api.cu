@@ -35,7 +35,7 @@ struct ih_sim {
     // device buffers
     float4 *spheres_raw = nullptr, *spheres = nullptr, *finger_root = nullptr;
     int *shape_first = nullptr, *shape_count = nullptr, *pad_link = nullptr;
-    float *shape_jinv = nullptr, *shape_bound = nullptr, *pad_s0 = nullptr, *pad_s1 = nullptr;
+    float *shape_jinv = nullptr, *pad_s0 = nullptr, *pad_s1 = nullptr;
     int *cl_first = nullptr;
     float4 *clusters = nullptr;
     float4 *link_tab = nullptr;
@@ -188,7 +188,7 @@ DevScene dev_scene(const ih_sim *s) {
     d.palm_hx = s->palm_half[0]; d.palm_hy = s->palm_half[1]; d.palm_hz = s->palm_half[2];
     d.link_len = s->link_len; d.link_rad = s->link_rad;
     d.spheres = s->spheres; d.shape_first = s->shape_first; d.shape_count = s->shape_count;
-    d.shape_jinv = s->shape_jinv; d.shape_bound = s->shape_bound; d.finger_root = s->finger_root;
+    d.shape_jinv = s->shape_jinv; d.finger_root = s->finger_root;
     d.cl_first = s->cl_first; d.clusters = s->clusters;
     d.pad_link = s->pad_link; d.pad_s0 = s->pad_s0; d.pad_s1 = s->pad_s1;
     return d;
@@ -341,7 +341,7 @@ ih_status sim_create(const ih_scene *sc, const ih_config *cfg, uint64_t seed, vo
     auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
     A(dalloc(s, &s->spheres_raw, total)); A(dalloc(s, &s->spheres, total));
     A(dalloc(s, &s->shape_first, sc->n_shapes)); A(dalloc(s, &s->shape_count, sc->n_shapes));
-    A(dalloc(s, &s->shape_jinv, 6 * sc->n_shapes)); A(dalloc(s, &s->shape_bound, sc->n_shapes));
+    A(dalloc(s, &s->shape_jinv, 6 * sc->n_shapes));
     std::vector<int> cl_first(sc->n_shapes);
     int n_clusters = 0;
     for (int k = 0; k < sc->n_shapes; ++k) {
@@ -416,7 +416,7 @@ ih_status sim_create(const ih_scene *sc, const ih_config *cfg, uint64_t seed, vo
         A(cudaMemsetAsync(s->slip, 0, (size_t)N * P * sizeof(float4), st));
     }
     A(launch_shape_setup(s->spheres_raw, s->spheres, s->shape_first, s->shape_count, sc->n_shapes,
-                         s->shape_jinv, s->shape_bound, s->cl_first, s->clusters, st));
+                         s->shape_jinv, s->cl_first, s->clusters, st));
     A(launch_lpt_order(N, s->shape_count, s->shape, s->iters, s->lpt_scratch, s->order, st));
     A(cudaStreamSynchronize(st));   // host vectors above go out of scope
     if (e != cudaSuccess) {

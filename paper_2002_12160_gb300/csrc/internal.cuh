@@ -22,7 +22,6 @@ struct DevScene {
     const int *shape_first;     // [n_shapes]
     const int *shape_count;     // [n_shapes]
     const float *shape_jinv;    // [n_shapes][6] inverse unit inertia xx yy zz xy xz yz
-    const float *shape_bound;   // [n_shapes] bounding radius about the centroid
     const int *cl_first;        // [n_shapes] first cluster of each shape
     const float4 *clusters;     // [total clusters] centre (centroid frame), enclosing radius
     const float4 *finger_root;  // [F] x y z yaw
@@ -216,7 +215,7 @@ __device__ __forceinline__ void qlog_d(Q4d q, double out[3]) {
 // ---------------------------------------------------------------- launches
 // Declared here, defined in the kernel translation units.
 cudaError_t launch_shape_setup(const float4 *spheres_in, float4 *spheres_out, const int *first,
-                               const int *count, int n_shapes, float *jinv, float *bound,
+                               const int *count, int n_shapes, float *jinv,
                                const int *cl_first, float4 *clusters, cudaStream_t s);
 cudaError_t launch_lpt_order(int N, const int *shape_count, const int *shape, const int *iters, int *scratch,
                              int *order, cudaStream_t s);

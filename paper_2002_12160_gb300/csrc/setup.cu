@@ -1,5 +1,5 @@
 // setup.cu -- kernels that prepare the step: each shape's centroid frame,
-// unit inertia and bounding radius; the kinematic hand's link poses for a
+// unit inertia; the kinematic hand's link poses for a
 // block of commanded frames (the robot state driven by u_t, Sec. III-A); the
 // initial sampling of pose, mass and friction (Sec. III-D, Algorithm 1
 // initialisation); and the validated upload of a caller's state.
@@ -11,11 +11,10 @@ namespace {
 
 // One block per shape. Centroid of the sphere centres, recentred spheres,
 // unit inertia J = (1/S) sum_s [(2/5) r_s^2 I + |c_s|^2 I - c_s c_s^T] of
-// equal solid balls about the centroid, its inverse, and the bounding radius
-// max_s |c_s| + r_s.
+// equal solid balls about the centroid, and its inverse.
 __global__ void shape_setup_kernel(const float4 *in, float4 *out, const int *first, const int *count,
-                                   float *jinv, float *bound, const int *cl_first, float4 *clusters) {
-    __shared__ double red[7][256];
+                                   float *jinv, const int *cl_first, float4 *clusters) {
+    __shared__ double red[6][256];
     const int sh = blockIdx.x, t = threadIdx.x;
     const int f = first[sh], S = count[sh];
     double cx = 0, cy = 0, cz = 0;
@@ -31,7 +30,7 @@ __global__ void shape_setup_kernel(const float4 *in, float4 *out, const int *fir
     }
     const double mx = red[0][0] / S, my = red[1][0] / S, mz = red[2][0] / S;
     __syncthreads();
-    double a[7] = {0, 0, 0, 0, 0, 0, 0};   // xx yy zz xy xz yz, bound
+    double a[6] = {0, 0, 0, 0, 0, 0};   // xx yy zz xy xz yz
     for (int j = t; j < S; j += blockDim.x) {
         const float4 s = in[f + j];
         const double x = s.x - mx, y = s.y - my, z = s.z - mz, r = s.w;
@@ -43,14 +42,12 @@ __global__ void shape_setup_kernel(const float4 *in, float4 *out, const int *fir
         a[3] -= x * y;
         a[4] -= x * z;
         a[5] -= y * z;
-        a[6] = fmax(a[6], sqrt(x * x + y * y + z * z) + r);
     }
-    for (int k = 0; k < 7; ++k) red[k][t] = a[k];
+    for (int k = 0; k < 6; ++k) red[k][t] = a[k];
     __syncthreads();
     for (int o = blockDim.x / 2; o > 0; o >>= 1) {
         if (t < o) {
             for (int k = 0; k < 6; ++k) red[k][t] += red[k][t + o];
-            red[6][t] = fmax(red[6][t], red[6][t + o]);
         }
         __syncthreads();
     }
@@ -64,8 +61,6 @@ __global__ void shape_setup_kernel(const float4 *in, float4 *out, const int *fir
         float *o = jinv + 6 * sh;
         o[0] = (float)(c00 / det); o[1] = (float)(c11 / det); o[2] = (float)(c22 / det);
         o[3] = (float)(c01 / det); o[4] = (float)(c02 / det); o[5] = (float)(c12 / det);
-        // rounded outward so that culling with it stays conservative in FP32
-        bound[sh] = (float)(red[6][0] * (1.0 + 1e-6)) + 1e-7f;
     }
     // clusters of kCluster consecutive spheres: centre of their centres and the
     // radius that encloses them, in the centroid frame
@@ -254,9 +249,9 @@ cudaError_t launch_lpt_order(int N, const int *shape_count, const int *shape, co
 }
 
 cudaError_t launch_shape_setup(const float4 *spheres_in, float4 *spheres_out, const int *first,
-                               const int *count, int n_shapes, float *jinv, float *bound,
+                               const int *count, int n_shapes, float *jinv,
                                const int *cl_first, float4 *clusters, cudaStream_t s) {
-    shape_setup_kernel<<<n_shapes, 256, 0, s>>>(spheres_in, spheres_out, first, count, jinv, bound, cl_first,
+    shape_setup_kernel<<<n_shapes, 256, 0, s>>>(spheres_in, spheres_out, first, count, jinv, cl_first,
                                                 clusters);
     return cudaGetLastError();
 }

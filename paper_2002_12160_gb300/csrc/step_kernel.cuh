@@ -4,10 +4,9 @@
 //
 // L lanes of one warp (32, or 16 with two environments to a warp) own one
 // environment at a time; nothing but the warp synchronises. Per substep they
-//   1. predict the velocity under gravity, cache the object's spheres, rotated
-//      into the world frame, and the links' offsets in shared memory, and cull
-//      the links against the object's bounding sphere (one ballot);
-//   2. cull (surviving link, 8-sphere cluster) pairs by the clusters' enclosing
+//   1. predict the velocity under gravity and cache the object's spheres, rotated
+//      into the world frame, and the links' offsets in shared memory;
+//   2. cull (link, 8-sphere cluster) pairs by the clusters' enclosing
 //      spheres; then one lane takes each surviving pair and tests its eight
 //      spheres by squared distance alone (the few within 1e-5 of the margin
 //      again by their gap), and the contacts (gap d < margin) are listed in
