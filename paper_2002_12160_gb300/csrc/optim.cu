@@ -834,14 +834,22 @@ __global__ void __launch_bounds__(kSoft) soft_weights_kernel(const OptArgs a) {
                 if (near) break;   // (the same in every thread of the cluster)
             }
             // FP64 steps until one moves t by less than 1e-7 (a Newton step squares
-            // the error). The bracket holds every root: at e^-100 of the range no cost
-            // but the minima counts (FP64 gaps are above 1e-17 of it), at e^50 all
-            // count alike
+            // the error). At e^50 of the range all costs count alike, so the root lies
+            // below; towards zero the bracket opens by 50 whenever a step would leave it
+            // before g' < 0 has been seen: one cost far above the rest puts the root any
+            // distance below the range (costs 0, 1e-50 and 1: near e^-115 of it). Every
+            // CTA of the cluster has the same sums and takes the same steps.
             double tt = (double)tf, tlo = -100.0, thi = 50.0;
+            bool below = false;   // (of thread 0) some step found g' < 0
+            // eta at t: e^t range, in one exponential where e^t alone would be denormal
+            auto eta_at = [&](double x) -> double { return x > -700.0 ? exp(x) * range : exp(x + log(range)); };
             for (int it = 0; it < 400; ++it) {
-                if (t == 0) { const double e = exp(tt); S.sc[0] = e; S.sc[1] = 1.0 / e; }
+                if (t == 0) {   // eta and its inverse, finite so that the minima's product with it is zero
+                    S.sc[0] = eta_at(tt);
+                    S.sc[1] = fmin(tt > -700.0 ? (1.0 / exp(tt)) / range : 1.0 / S.sc[0], 1.7976931348623157e308);
+                }
                 __syncthreads();
-                const double inv = S.sc[1] / range;
+                const double inv = S.sc[1];
                 double s0 = 0.0, s1 = 0.0, s2 = 0.0;
                 for (int i = i0 + t; i < i1; i += kSoft) {
                     const double c = a.c_mean[i];
@@ -851,12 +859,15 @@ __global__ void __launch_bounds__(kSoft) soft_weights_kernel(const OptArgs a) {
                 }
                 cluster_sum3(s0, s1, s2, S, buf);
                 if (t == 0) {
-                    const double e = S.sc[0] * range;
+                    const double e = S.sc[0];
                     const double mean = s1 / s0, var = s2 / s0 - mean * mean;
-                    const double g1 = eps + log(s0 / K) - mean / e, slope = var / (e * e);
-                    if (g1 < 0.0) tlo = tt; else thi = tt;
-                    double tn = slope > 0.0 ? tt - g1 / slope : 0.5 * (tlo + thi);
-                    if (!(tn > tlo && tn < thi)) tn = 0.5 * (tlo + thi);
+                    const double g1 = eps + log(s0 / K) - (mean == 0.0 ? 0.0 : mean / e), slope = var / (e * e);
+                    if (g1 < 0.0) { tlo = tt; below = true; } else thi = tt;
+                    double tn = slope > 0.0 ? tt - g1 / slope : -INFINITY;
+                    if (!(tn > tlo && tn < thi)) {
+                        if (!below) tlo -= 50.0;
+                        tn = 0.5 * (tlo + thi);
+                    }
                     const double tol = 1.0 + fabs(tt);
                     S.sc[3] = (fabs(tn - tt) <= 1e-7 * tol || thi - tlo <= 1e-13 * tol) ? 1.0 : 0.0;
                     S.sc[2] = tn;
@@ -866,7 +877,7 @@ __global__ void __launch_bounds__(kSoft) soft_weights_kernel(const OptArgs a) {
                 if (S.sc[3] != 0.0) break;
             }
             __syncthreads();
-            if (t == 0) S.sc[0] = exp(tt) * range;
+            if (t == 0) S.sc[0] = eta_at(tt);
             __syncthreads();
             eta = S.sc[0];
         }
