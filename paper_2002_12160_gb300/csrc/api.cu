@@ -9,6 +9,9 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
+#include "host_rules.cuh"
 #include "internal.cuh"
 
 using namespace ih;
@@ -152,26 +155,73 @@ cudaError_t dalloc(ih_sim *s, T **p, size_t count) {
     return cudaSuccess;
 }
 
+// A driver entry point (null: not there); of the driver API as of CUDA 12.0
+template <typename F>
+F driver_entry(const char *name) {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &r);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e == cudaSuccess && r == cudaDriverEntryPointSuccess ? reinterpret_cast<F>(f) : nullptr;
+}
+
+// The allocation that holds an address (false: none that the driver knows)
+bool allocation_of(uintptr_t p, uintptr_t *base, size_t *size) {
+    static const auto range = driver_entry<CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr)>("cuMemGetAddressRange");
+    CUdeviceptr b = 0;
+    if (!range || range(&b, size, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    *base = (uintptr_t)b;
+    return true;
+}
+
+// Whether a stream is of the current context, that is of the current device. (Asked of
+// the driver: cudaStreamGetDevice breaks a capture that the stream is in.)
+bool stream_is_current(cudaStream_t st) {
+    if (!st || st == cudaStreamLegacy || st == cudaStreamPerThread) return true;   // the default streams
+    static const auto of_stream = driver_entry<CUresult (*)(CUstream, CUcontext *)>("cuStreamGetCtx");
+    static const auto current = driver_entry<CUresult (*)(CUcontext *)>("cuCtxGetCurrent");
+    CUcontext a = nullptr, b = nullptr;
+    return of_stream && current && of_stream(st, &a) == CUDA_SUCCESS && current(&b) == CUDA_SUCCESS && a == b;
+}
+
 // Device-to-device copies between the handle's arrays and the caller's (null: left
-// out). One launch when every address of the caller's is this device's memory (or
-// managed), which the kernel can reach; copy calls, which take any, otherwise.
+// out). One launch when a kernel may touch every array of the caller's
+// (host_rules.cuh); copy calls, which take any address, device and stream, otherwise.
 struct Copies {
     CopyArgs a{};
     int n = 0;
-    bool here = true;
-    void add(void *dst, const void *src, size_t bytes, const void *caller, int dev) {
-        if (!caller || bytes == 0) return;
+    CallerArray caller[4];
+    void add(void *dst, const void *src, size_t bytes, const void *at) {
+        if (!at || bytes == 0) return;
         a.dst[n] = dst;
         a.src[n] = src;
-        a.bytes[n++] = bytes;
-        cudaPointerAttributes at;
-        const cudaError_t e = cudaPointerGetAttributes(&at, caller);
-        if (e != cudaSuccess) (void)cudaGetLastError();
-        here = here && e == cudaSuccess && ((at.type == cudaMemoryTypeDevice && at.device == dev) || at.type == cudaMemoryTypeManaged);
+        a.bytes[n] = bytes;
+        caller[n].at = reinterpret_cast<uintptr_t>(at);
+        caller[n++].bytes = bytes;
     }
-    cudaError_t run(cudaStream_t st) const {
+    bool one_launch(int dev, cudaStream_t st) {
+        int cur = -1;
+        cudaError_t e = cudaGetDevice(&cur);
+        const int on = stream_is_current(st) ? cur : -1;
+        for (int k = 0; k < n && e == cudaSuccess; ++k) {
+            CallerArray &c = caller[k];
+            cudaPointerAttributes at;
+            e = cudaPointerGetAttributes(&at, reinterpret_cast<const void *>(c.at));
+            if (e != cudaSuccess) break;
+            c.kind = at.type == cudaMemoryTypeDevice    ? CallerArray::kDevice
+                     : at.type == cudaMemoryTypeManaged ? CallerArray::kManaged
+                                                        : CallerArray::kOther;
+            c.device = at.device;
+            if (c.kind == CallerArray::kOther || !allocation_of(c.at, &c.base, &c.size) ||
+                !kernel_may_touch(c, dev, cur, on))
+                return false;
+        }
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        return e == cudaSuccess;
+    }
+    cudaError_t run(int dev, cudaStream_t st) {
         if (n == 0) return cudaSuccess;
-        if (here && n > 1) return launch_copies(a, n, st);
+        if (n > 1 && one_launch(dev, st)) return launch_copies(a, n, st);
         cudaError_t e = cudaSuccess;
         for (int k = 0; k < n && e == cudaSuccess; ++k)
             e = cudaMemcpyAsync(a.dst[k], a.src[k], a.bytes[k], cudaMemcpyDeviceToDevice, st);
@@ -531,11 +581,11 @@ ih_status sim_get_state(ih_sim *s, float *pose, float *vel, float *params, int32
     if (!s) return IH_ERR_ARG;
     const size_t N = s->cfg.n_envs;
     Copies c;
-    c.add(pose, s->pose, N * 2 * sizeof(float4), pose, s->dev);
-    c.add(vel, s->vel, N * 2 * sizeof(float4), vel, s->dev);
-    c.add(params, s->params, N * sizeof(float2), params, s->dev);
-    c.add(env_status, s->status, N * sizeof(int), env_status, s->dev);
-    const cudaError_t e = c.run(s->stream);
+    c.add(pose, s->pose, N * 2 * sizeof(float4), pose);
+    c.add(vel, s->vel, N * 2 * sizeof(float4), vel);
+    c.add(params, s->params, N * sizeof(float2), params);
+    c.add(env_status, s->status, N * sizeof(int), env_status);
+    const cudaError_t e = c.run(s->dev, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "get_state");
     return IH_OK;
 }
@@ -889,9 +939,9 @@ ih_status sim_read_sensors(ih_sim *s, float *forces, int32_t *env_status) {
     if (!s) return IH_ERR_ARG;
     const size_t N = s->cfg.n_envs;
     Copies c;
-    c.add(forces, s->forces, N * s->n_pads * 3 * sizeof(float), forces, s->dev);
-    c.add(env_status, s->status, N * sizeof(int), env_status, s->dev);
-    const cudaError_t e = c.run(s->stream);
+    c.add(forces, s->forces, N * s->n_pads * 3 * sizeof(float), forces);
+    c.add(env_status, s->status, N * sizeof(int), env_status);
+    const cudaError_t e = c.run(s->dev, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "read_sensors");
     return IH_OK;
 }
@@ -943,10 +993,10 @@ ih_status sim_read_observation(ih_sim *s, float *q, float *pad_pose, float *slip
         return fail(s, IH_ERR_ARG, "pad_pose and slip must be 16-byte aligned");
     const size_t N = s->cfg.n_envs, P = s->n_pads, D = s->n_joints;
     Copies c;
-    c.add(q, s->qj, N * D * sizeof(float), q, s->dev);
-    c.add(pad_pose, s->pad_pose, 2 * N * P * sizeof(float4), pad_pose, s->dev);
-    c.add(slip, s->slip, N * P * sizeof(float4), slip, s->dev);
-    const cudaError_t e = c.run(s->stream);
+    c.add(q, s->qj, N * D * sizeof(float), q);
+    c.add(pad_pose, s->pad_pose, 2 * N * P * sizeof(float4), pad_pose);
+    c.add(slip, s->slip, N * P * sizeof(float4), slip);
+    const cudaError_t e = c.run(s->dev, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "read_observation");
     return IH_OK;
 }
@@ -958,9 +1008,9 @@ ih_status sim_set_hand(ih_sim *s, const float *q, const float *qd) {
     if (bytes == 0) return IH_OK;
     if (!q) return fail(s, IH_ERR_ARG, "q is required");
     Copies c;
-    c.add(s->qj, q, bytes, q, s->dev);
-    c.add(s->qdj, qd, bytes, qd, s->dev);
-    cudaError_t e = c.run(s->stream);
+    c.add(s->qj, q, bytes, q);
+    c.add(s->qdj, qd, bytes, qd);
+    cudaError_t e = c.run(s->dev, s->stream);
     if (e == cudaSuccess && !qd) e = cudaMemsetAsync(s->qdj, 0, bytes, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "set_hand");
     return IH_OK;
@@ -971,9 +1021,9 @@ ih_status sim_get_hand(ih_sim *s, float *q, float *qd) {
     if (!s->pd) return fail(s, IH_ERR_ARG, "the hand's joints are state only with the PD-driven hand");
     const size_t bytes = (size_t)s->cfg.n_envs * s->n_joints * sizeof(float);
     Copies c;
-    c.add(q, s->qj, bytes, q, s->dev);
-    c.add(qd, s->qdj, bytes, qd, s->dev);
-    const cudaError_t e = c.run(s->stream);
+    c.add(q, s->qj, bytes, q);
+    c.add(qd, s->qdj, bytes, qd);
+    const cudaError_t e = c.run(s->dev, s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "get_hand");
     return IH_OK;
 }
