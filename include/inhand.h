@@ -522,7 +522,8 @@ ih_status sim_adjoint(ih_sim *sim, int32_t frame0, int32_t horizon, int32_t chec
  * per gradient and the others twice (the pass that computes the cost and
  * checkpoints, and the segment's recomputation, which records the tape), so
  * segments longer than checkpoint_every are taken when they fit it (and half of
- * the device's free memory), up to the whole horizon in one; when not even
+ * the device's free memory when they are first asked for: a length refused for that
+ * is tried again only after this call), up to the whole horizon in one; when not even
  * checkpoint_every's fit, the tape of a single substep is kept and each substep
  * runs once more just before its reverse sweep. Results are the same bit for bit.
  * 0 always takes the smallest mode. Not a passage of the paper: a memory/time trade

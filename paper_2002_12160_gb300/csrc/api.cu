@@ -62,6 +62,7 @@ struct ih_sim {
     float *adj_scratch = nullptr;
     size_t adj_floats = 0;
     size_t adj_budget = (size_t)16 << 30;   // bytes of adjoint scratch for whole-segment taping
+    size_t adj_refused = SIZE_MAX;          // floats that the device's free memory did not allow
     bool adj_seg = false;
     int adj_gw = 0, adj_pl = 0;   // the adjoint kernel's shape (0, 0: automatic)
     int iters_max_all = -1;       // the largest iteration count of any environment (-1: to be read)
@@ -1165,7 +1166,8 @@ namespace {
 // 3.58 ms in one, 6 GB), else the smallest number that does, down to the caller's K;
 // and when that does not fit, substep by substep. The gradients are the same bit
 // for bit. Segments longer than the caller's are taken only while growing the
-// scratch to them leaves half of the device's free memory.
+// scratch to them leaves half of the device's free memory; a size refused for that
+// is not tried again before sim_set_adjoint_memory (host_rules.cuh).
 ih_status adjoint_prepare(ih_sim *s, int n, int horizon, int *K, size_t *stride, int *imax) {
     cudaStream_t st = s->stream;
     cudaError_t e = cudaSuccess;
@@ -1200,23 +1202,24 @@ ih_status adjoint_prepare(ih_sim *s, int n, int horizon, int *K, size_t *stride,
     };
     *imax = m;
     s->adj_seg = true;
-    for (int segs = 1, k = horizon; k > *K; ++segs, k = (horizon + segs - 1) / segs) {
-        const size_t str = floats(k, true), need = str * (size_t)n;
-        if (need * sizeof(float) > s->adj_budget) continue;
-        if (need > s->adj_floats) {
+    bool failed = false;
+    const int longer = longer_segment(
+        horizon, *K, s->adj_budget / sizeof(float), s->adj_floats, s->adj_refused, failed,
+        [&](int k) { return floats(k, true) * (size_t)n; },
+        [&](size_t need) {
             size_t avail = 0, all = 0;
             e = cudaMemGetInfo(&avail, &all);
-            if (e != cudaSuccess) return cuda_fail(s, e, "adjoint sizing");
-            if (need * sizeof(float) > avail / 2) continue;
-        }
-        e = reserve(need);
-        if (e == cudaErrorMemoryAllocation) {
+            if (e != cudaSuccess) return Reserve::kFailed;
+            if (need > avail / 2 / sizeof(float)) return Reserve::kNoMemory;
+            e = reserve(need);
+            if (e != cudaErrorMemoryAllocation) return e == cudaSuccess ? Reserve::kDone : Reserve::kFailed;
             (void)cudaGetLastError();
-            continue;
-        }
-        if (e != cudaSuccess) return cuda_fail(s, e, "adjoint sizing");
-        *K = k;
-        *stride = str;
+            return Reserve::kNoMemory;
+        });
+    if (failed) return cuda_fail(s, e, "adjoint sizing");
+    if (longer > 0) {
+        *K = longer;
+        *stride = floats(longer, true);
         return IH_OK;
     }
     // the caller's segments, taped whole when that fits the budget
@@ -1303,6 +1306,7 @@ cudaError_t refine_alloc(ih_sim *s) {
 ih_status sim_set_adjoint_memory(ih_sim *s, uint64_t bytes) {
     if (!s) return IH_ERR_ARG;
     s->adj_budget = (size_t)bytes;
+    s->adj_refused = SIZE_MAX;
     return IH_OK;
 }
 

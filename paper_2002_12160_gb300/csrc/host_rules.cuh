@@ -29,4 +29,31 @@ inline bool kernel_may_touch(const CallerArray &a, int handle_device, int curren
     return a.at >= a.base && a.bytes <= a.size && a.at - a.base <= a.size - a.bytes;
 }
 
+// The length of the adjoint's segments between checkpoints, longer than the caller's K
+// where that can be had: the largest of ceil(H / 1), ceil(H / 2), ... above K whose
+// scratch of need(k) floats is within the budget and is held already or can be
+// reserved (0: none, or `failed`). A size that could not be reserved is written to
+// `refused` and neither it nor a larger one is asked for again while the caller
+// keeps `refused`: a repeated call then neither looks at the device's free memory nor
+// allocates.
+enum class Reserve { kDone, kNoMemory, kFailed };
+template <typename Need, typename Try>
+int longer_segment(int H, int K, size_t budget, const size_t &held, size_t &refused, bool &failed, Need need, Try reserve) {
+    failed = false;
+    for (int segs = 1, k = H; k > K; ++segs, k = (H + segs - 1) / segs) {
+        const size_t f = need(k);
+        if (f > budget) continue;
+        if (f <= held) return k;
+        if (f >= refused) continue;
+        const Reserve r = reserve(f);
+        if (r == Reserve::kDone) return k;
+        if (r == Reserve::kFailed) {
+            failed = true;
+            return 0;
+        }
+        refused = f;
+    }
+    return 0;
+}
+
 }  // namespace ih

@@ -58,3 +58,48 @@ M = 2 ** 64 - 1
 def test_a_read_back_launches_only_where_a_kernel_may_touch_the_array(run, kind, device, at, bytes_, base, size, handle,
                                                                       current, stream, want):
     assert run("touch", TOUCH, kind, device, at, bytes_, base, size, handle, current, stream) == [str(want)]
+
+
+# calls of horizon H and checkpoint interval K over a device with `avail` floats free:
+# what each takes, and how often memory was asked for in all
+SEGMENTS = """
+size_t held = 0, refused = (size_t)-1;
+int asked = 0;
+for (int i = 1; i + 4 < argc; i += 5) {
+    const int H = atoi(argv[i]), K = atoi(argv[i + 1]);
+    const size_t budget = strtoull(argv[i + 2], 0, 0), avail = strtoull(argv[i + 3], 0, 0);
+    if (!strcmp(argv[i + 4], "reset")) refused = (size_t)-1;
+    bool failed = false;
+    const int k = longer_segment(H, K, budget, held, refused, failed, [&](int k) { return (size_t)k * 100; },
+                                 [&](size_t f) {
+                                     ++asked;
+                                     if (!strcmp(argv[i + 4], "fail")) return Reserve::kFailed;
+                                     if (f > avail / 2) return Reserve::kNoMemory;
+                                     held = f;
+                                     return Reserve::kDone;
+                                 });
+    printf("%d:%d:%d ", k, asked, (int)failed);
+}
+"""
+BIG = 10 ** 9
+
+
+@pytest.mark.parametrize("calls,want", [
+    # the whole horizon when it fits, without asking again
+    ([(30, 10, BIG, BIG, "-")] * 2, ["30:1:0", "30:1:0"]),
+    # the budget decides: 15, then none above K
+    ([(30, 10, 2000, BIG, "-"), (30, 10, 1400, BIG, "-")], ["15:1:0", "0:1:0"]),
+    # the free memory decides; more of it changes nothing until the budget is set again
+    ([(30, 10, BIG, 3200, "-"), (30, 10, BIG, 0, "-"), (30, 10, BIG, BIG, "-"), (30, 10, BIG, BIG, "reset")],
+     ["15:2:0", "15:2:0", "15:2:0", "30:3:0"]),
+    # nothing fits: asked once for each length, then never
+    ([(30, 2, BIG, 100, "-"), (30, 2, BIG, 100, "-"), (30, 2, BIG, BIG, "-")], ["0:8:0", "0:8:0", "0:8:0"]),
+    # a smaller need than the refused one is still tried
+    ([(30, 10, BIG, 2400, "-"), (11, 10, BIG, 2400, "-")], ["0:2:0", "11:3:0"]),
+    # an error ends the call
+    ([(30, 10, BIG, BIG, "fail")], ["0:1:1"]),
+    # no longer one than the horizon, none at all when K is the horizon
+    ([(10, 10, BIG, BIG, "-"), (1, 1, BIG, BIG, "-")], ["0:0:0", "0:0:0"]),
+])
+def test_the_adjoints_segments_settle(run, calls, want):
+    assert run("segments", SEGMENTS, *[v for c in calls for v in c]) == want
