@@ -740,6 +740,8 @@ cudaError_t window_buffers(ih_sim *s, int T) {
     cudaError_t e = cudaStreamSynchronize(s->stream);
     if (s->cap_stream && e == cudaSuccess) e = cudaStreamSynchronize(s->cap_stream);
     if (e != cudaSuccess) return e;
+    // a captured window graph holds the old buffers' addresses (and has finished): capture again
+    if (s->win_exec) { cudaGraphExecDestroy(s->win_exec); s->win_exec = nullptr; }
     if (s->wf_cm) cudaFree(s->wf_cm);
     if (s->wf_pose) cudaFree(s->wf_pose);
     s->wf_cm = nullptr; s->wf_pose = nullptr; s->wf_T = 0;
