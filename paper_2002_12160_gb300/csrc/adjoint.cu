@@ -409,7 +409,7 @@ __device__ __noinline__ int fwd_substep(const AdjArgs &a, const Env &E_, Body &b
         G.sync();   // (a reverse sweep may just have read the ring in the centres' place)
 #pragma unroll 1
         for (int j = gt; j < ncl * kCluster; j += T) {
-            float4 o = make_float4(1e18f, 1e18f, 1e18f, 0.0f);   // (padding of the last cluster: far away)
+            float4 o = make_float4(kFar, kFar, kFar, 0.0f);   // (padding of the last cluster: far away)
             if (j < E.NS) {
                 const float4 s4 = __ldg(sc.spheres + E.sfirst + j);
                 const V3 cr = mmul(R, xyz(s4));

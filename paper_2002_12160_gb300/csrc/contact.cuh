@@ -69,6 +69,9 @@ __device__ __forceinline__ Hit hit_capsule(V3 ca, float rs, V3 d, float L, float
 
 constexpr int kMaxLinks = 32;
 constexpr int kSphStride = kCluster + 1;   // spheres of a cluster, padded: lanes on different clusters hit different banks
+// Centre of the spheres that fill a shape's last cluster: its squared distance from
+// anything overflows, so that no margin, however large, makes them contacts
+constexpr float kFar = 3e38f;
 
 // Per link its pads in order and their intervals [s0, s1) (absent: an interval
 // that holds nothing; the palm: its first pad holds all).

@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                 //       (padding of the last cluster: far away); the links' offsets
 #pragma unroll 1
                 for (int j = gl; j < ncl * kCluster; j += L) {
-                    float4 o = make_float4(1e18f, 1e18f, 1e18f, 0.0f);
+                    float4 o = make_float4(kFar, kFar, kFar, 0.0f);
                     if (j < NS) {
                         const float4 sp = __ldg(sc.spheres + sfirst + j);
                         const V3 cr = mmul(R, xyz(sp));

@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(32, 8) pd_step_kernel(const __grid_constant__ 
             const S6 Wi = world_inv_inertia(R, Jb, inv_m);
 #pragma unroll 1
             for (int j = lane; j < ncl * kCluster; j += 32) {
-                float4 o = make_float4(1e18f, 1e18f, 1e18f, 0.0f);   // (padding of the last cluster: far away)
+                float4 o = make_float4(kFar, kFar, kFar, 0.0f);   // (padding of the last cluster: far away)
                 if (j < NS) {
                     const float4 s4 = __ldg(sc.spheres + sfirst + j);
                     const V3 cr = mmul(R, xyz(s4));
