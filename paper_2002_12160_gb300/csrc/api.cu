@@ -27,7 +27,7 @@ struct ih_sim {
     uint64_t seed = 0;
     cudaStream_t stream = nullptr;
     int dev = 0;   // the device the handle was made on
-    StepVariant variant{32, 4, 32, kManyBlocks};
+    StepVariant variant{32, 4, 32, kManyBlocks, false};
     int step_grid = 0;
     int s_max = 1;   // most spheres in one shape
     int sms = 1;     // SMs of the device
@@ -106,7 +106,7 @@ struct ih_sim {
     double *fo_terms = nullptr;
     int fo_T = 0;
     int frames_T = 0;               // frames of the last sim_step_frames call, not yet scored
-    StepVariant win_variant{0, 0, 0, 0};
+    StepVariant win_variant{0, 0, 0, 0, false};
     ih_opt_config win_opt{};
     // host bookkeeping
     std::vector<char> frame_ready;   // commands uploaded for frame f
@@ -246,7 +246,7 @@ DevScene dev_scene(const ih_sim *s) {
 }
 
 // Default step-kernel shape before any autotuning.
-StepVariant default_variant(int N) { return N <= 4096 ? StepVariant{64, 2, 0, 0} : StepVariant{32, 2, 0, 0}; }
+StepVariant default_variant(int N) { return N <= 4096 ? StepVariant{64, 2, 0, 0, false} : StepVariant{32, 2, 0, 0, false}; }
 
 // The lanes of a warp that execute an environment (the results do not depend on
 // them). A whole warp by default; two environments to a warp for the 16-wide
@@ -275,6 +275,20 @@ int step_per_sm(int blocks, int s_max, int sms) {
     return blocks <= kFewFit * sms || s_max > 128 ? kFewBlocks : kManyBlocks;
 }
 
+// Whether a lane's first contact past its register slots is updated beside them, where
+// the scene can have such contacts and the kernel has the registers: up to one and a half
+// rounds of the blocks that the device holds, where the environment with the most
+// contacts ends the launch. Mixed shapes, six frames, two states of four sampled
+// populations each, us without : with: 300 environments 391-395 : 356-360 where one has
+// 150 contacts (223-258 : 223-258 where none has more than 128), 1000 of them 418-438 :
+// 387-410 (242-268 : 244-270), 2000 of them 336-500 : 338-481, sums 3210 : 3142; 3000 of
+// them 338-526 : 340-510, sums 3248 : 3295, 4096 of them 393-488 : 416-506. In the kernels
+// of 128 registers every environment pays for it (8192 cylinders, four frames, 635 :
+// 666), and with 16 lanes most such contacts come later.
+bool step_first(const StepVariant &v, int c_max, int blocks, int sms) {
+    return step_has_first(v, c_max) && 2 * blocks <= 3 * kFewFit * sms;
+}
+
 // Make v the step shape: shared-memory opt-in, a persistent grid of at most the
 // one-warp blocks that fit on the device at once (they take environments from the
 // launch's work queue), and a spill area for the contacts beyond the shape's
@@ -284,13 +298,14 @@ cudaError_t use_variant(ih_sim *s, StepVariant v) {
     v.lanes = step_lanes(v.group, s->cfg.n_envs, s->s_max, s->sms);
     const int epb = step_envs_per_block(v);
     v.per_sm = step_per_sm((s->cfg.n_envs + epb - 1) / epb, s->s_max, s->sms);
+    v.first = step_first(v, s->cfg.c_max, (s->cfg.n_envs + epb - 1) / epb, s->sms);
     int bps = 0;
     cudaError_t e = step_prepare(v, s->s_max, s->cfg.c_max, s->dcfg.warm != 0, s->clp_cap, &bps);
     if (e != cudaSuccess) return e;
     const int resident = std::max(1, bps) * std::max(1, s->sms);
     const int grid = std::min((s->cfg.n_envs + epb - 1) / epb, resident);
     const int sc = step_stage_capacity(v, s->cfg.c_max);
-    const size_t need = (size_t)grid * epb * (size_t)(s->cfg.c_max - sc) * 4;
+    const size_t need = (size_t)grid * epb * (size_t)step_spill_rows(v, s->cfg.c_max) * 4;
     if (need > s->spill_f4) {
         // a captured window graph holds the old spill pointer: let it finish, capture again
         if (s->cap_stream) cudaStreamSynchronize(s->cap_stream);
@@ -1061,7 +1076,7 @@ ih_status sim_set_variant(ih_sim *s, int32_t tpe, int32_t cpl) {
     if (!s) return IH_ERR_ARG;
     if (s->pd) return refuse_pd(s, "sim_set_variant");
     if (!step_variant_supported(tpe, cpl)) return fail(s, IH_ERR_ARG, "unsupported step shape %d x %d", tpe, cpl);
-    cudaError_t e = use_variant(s, StepVariant{tpe, cpl, 0, 0});
+    cudaError_t e = use_variant(s, StepVariant{tpe, cpl, 0, 0, false});
     if (e != cudaSuccess) return cuda_fail(s, e, "set_variant");
     return IH_OK;
 }

@@ -282,9 +282,9 @@ struct StepArgs {
     int *cache_n;             // [N]
     // contact staging: the first stage_cap contacts of an environment's substep
     // in shared memory, the rest (up to c_max) in a global spill area of
-    // (c_max - stage_cap) x 4 float4 per resident group
+    // step_spill_rows x 4 float4 per resident group
     int stage_cap;
-    float4 *spill;            // [grid * groups per block][c_max - stage_cap][4] or null
+    float4 *spill;            // [grid * groups per block][step_spill_rows][4] or null
     int clp_cap;              // (link, cluster) pairs a group can hold
     int *queue;               // [2] work queue head, finished blocks (zero between launches) or null
 };
@@ -344,13 +344,14 @@ cudaError_t launch_hand_rest(int N, int D, const float *q0, float *qj, float *qd
 
 // A step shape (group, cpl) as the interface names it -- group, the width of the
 // solver's sums, alone fixes the results -- and, chosen by the library (the results
-// do not depend on them), the lanes of a warp that execute an environment and the
-// warps that an SM holds by registers.
+// do not depend on them), the lanes of a warp that execute an environment, the warps
+// that an SM holds by registers, and how the contacts past the register slots run.
 struct StepVariant {
     int group;
     int cpl;
     int lanes;
     int per_sm;
+    bool first;   // a lane's first contact past the register slots beside them
 };
 constexpr int kFewBlocks = 10, kManyBlocks = 16;
 constexpr int kFewFit = 12;   // warps of the kernels compiled for kFewBlocks that an SM holds (160 registers)
@@ -359,6 +360,8 @@ cudaError_t launch_step(const StepArgs &a, const StepVariant &v, int grid, int s
 bool step_variant_supported(int group, int cpl);
 // contacts staged in shared memory (the rest of c_max spill to global memory)
 int step_stage_capacity(const StepVariant &v, int c_max);
+int step_spill_rows(const StepVariant &v, int c_max);   // contacts of an environment's spill area
+bool step_has_first(const StepVariant &v, int c_max);   // whether there is a kernel with StepVariant::first that c_max needs
 int step_variant_list(StepVariant *out, int cap);
 
 struct CostArgs {

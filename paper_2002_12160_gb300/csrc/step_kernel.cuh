@@ -48,9 +48,13 @@ namespace {
 // the shapes of the interface (summation width, contacts per thread); the
 // second number no longer changes anything: the width alone fixes the result
 #define IH_STEP_VARIANTS(X) X(16, 2) X(16, 4) X(32, 1) X(32, 2) X(32, 3) X(32, 4) X(64, 1) X(64, 2) X(128, 1)
-// the compiled kernels: (lanes per environment, summation width, warps to an SM)
-#define IH_STEP_KERNELS(X) IH_STEP_KERNELS_B(X, kFewBlocks) IH_STEP_KERNELS_B(X, kManyBlocks)
-#define IH_STEP_KERNELS_B(X, B) X(16, 16, B) X(16, 32, B) X(16, 64, B) X(32, 32, B) X(32, 64, B) X(32, 128, B)
+// the compiled kernels: (lanes per environment, summation width, warps to an SM, whether
+// a lane's first contact past the register slots is updated beside them)
+#define IH_STEP_KERNELS(X)                                                                      \
+    IH_STEP_KERNELS_16(X, kFewBlocks, false) IH_STEP_KERNELS_16(X, kManyBlocks, false)          \
+    IH_STEP_KERNELS_32(X, kFewBlocks, false) IH_STEP_KERNELS_32(X, kManyBlocks, false) IH_STEP_KERNELS_32(X, kFewBlocks, true)
+#define IH_STEP_KERNELS_16(X, B, F) X(16, 16, B, F) X(16, 32, B, F) X(16, 64, B, F)
+#define IH_STEP_KERNELS_32(X, B, F) X(32, 32, B, F) X(32, 64, B, F) X(32, 128, B, F)
 constexpr int kSlots = 4;            // register-resident contacts per lane
 constexpr unsigned kAll = 0xffffffffu;
 template <bool V>
@@ -75,6 +79,10 @@ __host__ __device__ constexpr int sph_cap(int s_max) { return (s_max + kCluster 
 // register-resident ones; the rest of up to c_max spill to global memory
 __host__ __device__ constexpr int stage_capacity(int lanes, int c_max) {
     return c_max < kSlots * lanes ? c_max : kSlots * lanes;
+}
+// contacts of the spill area of an environment: whole rows of the lanes
+__host__ __device__ constexpr int spill_rows(int lanes, int c_max) {
+    return c_max > kSlots * lanes ? (c_max - kSlots * lanes + lanes - 1) / lanes * lanes : 0;
 }
 // float4s of the sphere cache and the impulses, which share their place (the
 // spheres are done with when the first impulse is stored) unless the solver
@@ -152,7 +160,7 @@ __device__ __forceinline__ unsigned long long cost_key(double c) {
 // One warp per block, so that the environments spread evenly over the SMs (an
 // SM holds 6 or 7 of 1024 environments; blocks of two would put 8 on some), and
 // B warps to an SM by registers (kFewBlocks or kManyBlocks).
-template <int L, int TPE, bool WARM, int B>
+template <int L, int TPE, bool WARM, int B, bool FIRST>
 __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max) {
     static_assert(TPE % L == 0 && TPE / L <= kSlots, "the width's threads are the lanes' accumulators");
     constexpr int EPW = 32 / L, NA = TPE / L, RCAP = kSlots * L;
@@ -193,8 +201,9 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
     unsigned short *clp = reinterpret_cast<unsigned short *>(prev + (WARM ? cap : 0));
     unsigned short *clist = reinterpret_cast<unsigned short *>(reinterpret_cast<unsigned char *>(clp) + align16(2 * (size_t)a.clp_cap));
     unsigned char *cpad = reinterpret_cast<unsigned char *>(clist) + align16(2 * (size_t)cap);
-    // contacts SC .. c_max - 1 of the environment: its slot of the spill area
-    float4 *spill_g = a.spill ? a.spill + (size_t)(blockIdx.x * EPW + sub) * (size_t)(cap - SC) * 4 : nullptr;   // (SC = RCAP when there is one)
+    // contacts SC .. c_max - 1 of the environment (and the rest of a row of the lanes):
+    // its slot of the spill area
+    float4 *spill_g = a.spill ? a.spill + (size_t)(blockIdx.x * EPW + sub) * (size_t)spill_rows(L, cap) * 4 : nullptr;   // (SC = RCAP when there is one)
     auto ballot = [&](bool p) -> unsigned {   // of the environment's lanes, bit 0 its first
         const unsigned b = __ballot_sync(kAll, p);
         return L == 32 ? b : (b >> shift) & 0xffffu;
@@ -525,19 +534,39 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                         Contact<F2> c0, c2;
                         load2(c0, 0);
                         load2(c2, 2);
+                        // FIRST: a lane's first further contact is read ahead and updated
+                        // beside the register slots, in one stretch of code (an empty one
+                        // adds zeros)
+                        constexpr bool first = decltype(more)::value && FIRST;
+                        float4 *g4 = nullptr;
+                        if constexpr (first) {
+                            g4 = spill_g + (size_t)gl * 4;
+                            if (gl + RCAP >= nc) {
+                                g4[0] = g4[2] = g4[3] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                                g4[1] = make_float4(0.0f, 0.0f, 1.0f, 0.0f);
+                            }
+                        }
 #pragma unroll 1
                         for (int it = 0; it < iters_w; ++it) {
                             float acc[NA][6] = {}, t[6];
                             const float k = rel(it);
+                            Contact<float> c4;
+                            if constexpr (first) unpack(c4, g4, g4 + 3);
                             c0.update(vv, ww, mu_s, k);
                             c2.update(vv, ww, mu_s, k);
+                            if constexpr (first) {
+                                c4.update(vv, ww, mu_s, k);
+                                g4[3] = make_float4(c4.lam.x, c4.lam.y, c4.lam.z, 0.0f);
+                            }
                             add2(acc, c0, 0);
                             add2(acc, c2, 2);
+                            if constexpr (first) add1(acc, c4, kSlots);
                             if constexpr (decltype(more)::value) {
 #pragma unroll 1
-                                for (int s0 = kSlots; s0 * L < nc_w; s0 += NA)   // the further ones, in the same per-thread order
+                                for (int s0 = kSlots; (s0 + (first && s0 == kSlots)) * L < nc_w; s0 += NA)   // the (other) further ones, in the same per-thread order
 #pragma unroll
                                     for (int j = 0; j < NA; ++j) {
+                                        if (first && s0 + j == kSlots) continue;
                                         const int ci = (s0 + j) * L + gl;
                                         if (ci < nc) {
                                             float4 *g4 = spill_g + (size_t)(ci - RCAP) * 4;
@@ -743,14 +772,14 @@ size_t bytes_t(int s_max, int c_max, int clp_cap) {
 }
 
 // Shared-memory opt-in, and the blocks of this kernel that fit on one SM
-template <int L, int TPE, bool WARM, int B>
+template <int L, int TPE, bool WARM, int B, bool FIRST>
 cudaError_t prepare_t(int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
     const size_t bytes = bytes_t<L, TPE, WARM>(s_max, c_max, clp_cap);
     cudaError_t e = cudaSuccess;
     if (bytes > 48 * 1024)
-        e = cudaFuncSetAttribute(step_kernel<L, TPE, WARM, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        e = cudaFuncSetAttribute(step_kernel<L, TPE, WARM, B, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess && blocks_per_sm)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, step_kernel<L, TPE, WARM, B>, 32, bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, step_kernel<L, TPE, WARM, B, FIRST>, 32, bytes);
     return e;
 }
 
@@ -759,9 +788,9 @@ cudaError_t prepare_t(int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
 // translation unit so the two build in parallel.
 template <bool WARM>
 cudaError_t prepare_w(const StepVariant &v, int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
-#define IH_PREP(L, T, B)                                       \
-    if (v.lanes == L && v.group == T && v.per_sm == B)         \
-        return prepare_t<L, T, WARM, B>(s_max, c_max, clp_cap, blocks_per_sm);
+#define IH_PREP(L, T, B, F)                                                    \
+    if (v.lanes == L && v.group == T && v.per_sm == B && v.first == F)         \
+        return prepare_t<L, T, WARM, B, F>(s_max, c_max, clp_cap, blocks_per_sm);
     IH_STEP_KERNELS(IH_PREP)
 #undef IH_PREP
     return cudaErrorInvalidValue;
@@ -769,10 +798,10 @@ cudaError_t prepare_w(const StepVariant &v, int s_max, int c_max, int clp_cap, i
 
 template <bool WARM>
 cudaError_t launch_w(const StepArgs &a, const StepVariant &v, int grid, int s_max, cudaStream_t s) {
-#define IH_LAUNCH(L, T, B)                                                                                           \
-    if (v.lanes == L && v.group == T && v.per_sm == B) {                                                             \
-        step_kernel<L, T, WARM, B><<<grid, 32, bytes_t<L, T, WARM>(s_max, a.cfg.c_max, a.clp_cap), s>>>(a, s_max);   \
-        return cudaGetLastError();                                                                                   \
+#define IH_LAUNCH(L, T, B, F)                                                                                           \
+    if (v.lanes == L && v.group == T && v.per_sm == B && v.first == F) {                                                \
+        step_kernel<L, T, WARM, B, F><<<grid, 32, bytes_t<L, T, WARM>(s_max, a.cfg.c_max, a.clp_cap), s>>>(a, s_max);   \
+        return cudaGetLastError();                                                                                      \
     }
     IH_STEP_KERNELS(IH_LAUNCH)
 #undef IH_LAUNCH

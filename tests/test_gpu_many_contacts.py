@@ -95,3 +95,27 @@ def test_adjoint_with_many_contacts_matches_oracle(margin):
                 err = np.linalg.norm(grad[i, b] - g_or[b])
                 assert err <= 1e-3 * np.linalg.norm(g_or[b]) + floor, (variant, i, b, grad[i, b], g_or[b])
     sim.close()
+
+
+@pytest.mark.parametrize("warm", [False, True])
+@pytest.mark.parametrize("shape", [(32, 2), (64, 2), (128, 1)])
+def test_large_batches_step_many_contacts_to_the_same_bits(shape, warm):
+    """Few environments update the first contact past a lane's slots beside them, many do
+    not (at most two rounds of twelve one-warp blocks an SM do)."""
+    wl, sim = _heavy(0.005, warm)
+    pose, vel, params, _ = (t.clone() for t in sim.sim_get_state())
+    shape_id, iters = (torch.from_numpy(a.astype(np.int32)).to(dev()) for a in (wl.shape_id, wl.iters))
+    sms = torch.cuda.get_device_properties(dev()).multi_processor_count
+    copies = 2 * 12 * sms // N + 1
+    wl.shape_id, wl.iters = np.tile(wl.shape_id, copies), np.tile(wl.iters, copies)
+    big = start(wl, n=N * copies, frames=LEAD + H + 4)
+    for handle, k in ((sim, 1), (big, copies)):
+        handle.sim_set_variant(*shape)
+        handle.sim_set_state(*(t.repeat(k, *[1] * (t.dim() - 1)).contiguous() for t in (pose, vel, params, shape_id, iters)))
+        handle.sim_step(LEAD, 3)
+    want = [*sim.sim_get_state(), *sim.sim_read_sensors()]
+    for a, b in zip(want, [*big.sim_get_state(), *big.sim_read_sensors()]):
+        assert torch.equal(a, b[:N]) and torch.equal(a, b[-N:])
+    assert not want[3].any()
+    big.close()
+    sim.close()
