@@ -531,10 +531,10 @@ ih_status sim_adjoint(ih_sim *sim, int32_t frame0, int32_t horizon, int32_t chec
 ih_status sim_set_adjoint_memory(ih_sim *sim, uint64_t bytes);
 
 /* The adjoint kernel's shape for sim_adjoint and sim_refine_elites: warps
- * per environment, and a second number that no longer changes anything (128
- * contacts of an environment are held in registers and shared memory whatever
- * it is; a substep's contacts beyond those, up to c_max, run from the
- * environment's scratch memory in the same per-thread order). Supported:
+ * per environment, and a second number that no longer changes anything (four
+ * warps hold all of an environment's contacts in registers and shared memory
+ * whatever it is, one warp 128; a substep's contacts beyond those, up to c_max,
+ * run from the environment's scratch memory in the same per-thread order). Supported:
  * (4, 1), (1, 1), (1, 2); (0, 0) restores the automatic choice: four warps
  * while the environments are at most two per SM, else one.
  * Results of different warp counts agree up to FP32 summation order.

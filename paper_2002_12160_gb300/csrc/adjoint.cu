@@ -25,8 +25,8 @@
 // block enumerates the contacts together, in the step's order (a thread tests the
 // eight spheres of a (link, cluster) pair that survived the cull); thread k % (32 GW)
 // then owns contact k for the setup, the Jacobi iterations and their reverse --
-// 128 contacts of a block in registers and shared memory, the further ones in the
-// environment's scratch memory -- and the block sums impulses and derivatives
+// 128 contacts of a block in registers and shared memory, the further ones (with one
+// warp) in the environment's scratch memory -- and the block sums impulses and derivatives
 // by warp shuffles and a shared-memory exchange between its warps. The state
 // at every K-th frame is kept (checkpoints). The reverse sweep walks the
 // segments between checkpoints backwards: it recomputes the segment's
@@ -53,6 +53,8 @@
 // iteration that needs them, at the public call: 1024 cylinders, 30 frames, three
 // segments 5.28 -> 4.28 ms; 102 cylinders, 10 frames, 552 -> 455 us; 64 boxes, 5 frames
 // (bound by the host), the kernel 258 -> 200 us.
+#include <type_traits>
+
 #include "contact.cuh"
 #include "internal.cuh"
 
@@ -60,7 +62,16 @@ namespace ih {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kRC = 128;   // contacts of a block held in registers and shared memory
+constexpr int kRC = 128;   // contacts of a block held in registers and shared memory (a thread's first, with four warps)
+// The compiled shapes GW: one warp (1), four warps for scenes of at most kRC contacts
+// (4), and four warps whose threads hold a second contact (kTwo), so that no contact of
+// theirs is in memory
+constexpr int kTwo = 4 | 8;
+template <int GW>
+constexpr int kWarps = GW & 7;
+template <int GW>
+constexpr int kHeld = GW == kTwo ? 2 * kRC : kRC;
+static_assert(IH_MAX_CONTACTS <= kHeld<kTwo>, "two contacts a thread hold all");
 // Iterations of the tape held in shared memory by the reverse sweep, copied there
 // asynchronously three iterations ahead. (Requested into registers an iteration
 // ahead, the rotation of the registers waited for the loads: 990 cycles an
@@ -85,11 +96,11 @@ __device__ __forceinline__ void store_if(bool on, float4 *dst, float4 v) {
 template <int N>
 __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// The GW warps of one environment (a block): thread gt, lane, warp; sync() is the
+// The warps of one environment (a block): thread gt, lane, warp; sync() is the
 // block's barrier.
 template <int GW>
 struct AGroup {
-    static constexpr int T = 32 * GW;
+    static constexpr int T = 32 * kWarps<GW>;
     int gt, lane, wg;
     __device__ AGroup() {
         gt = threadIdx.x;
@@ -157,17 +168,17 @@ struct alignas(16) GroupSm {
     float4 clam[kRC];              // the pass's final impulses (pad sums)
     float4 meta[kRC];              // reverse: the contacts' gap, link | pad << 8 and sphere
     union {                        // (a substep's enumeration and a reverse sweep never overlap)
-        float4 ring[kRing][kRC];   // reverse: the impulses after iterations it & (kRing - 1), on their way from the tape
+        float4 ring[kRing][kHeld<GW>];   // reverse: the impulses after iterations it & (kRing - 1), on their way from the tape
         Centres en;                // forward: the enumeration's centres and pairs
     };
-    float4 rsum[GW][kRing][2];     // ... and their sums, a copy per warp
+    float4 rsum[kWarps<GW>][kRing][2];     // ... and their sums, a copy per warp
     float4 xa[kMaxLinks], ax[kMaxLinks];     // x - link origin, link axis
     double term[IH_MAX_PADS];      // a frame's FP64 force term of each pad
     float padacc[IH_MAX_PADS * 3];
     float fbar[IH_MAX_PADS * 3];   // dL/dF_p / (h ns): minus the derivative w.r.t. a final impulse
-    float4 red[2][GW][2];          // partial sums of the block's warps (double-buffered)
+    float4 red[2][kWarps<GW>][2];          // partial sums of the block's warps (double-buffered)
     float fin[16];                 // results of the contacts' warps for the others
-    int cnt[2][GW];                // hits of each warp in a compaction round (double-buffered)
+    int cnt[2][kWarps<GW>];                // hits of each warp in a compaction round (double-buffered)
     int flag[IH_MAX_PADS];         // a frame's contact-state mismatch of each pad
     unsigned short lbeg[kMaxLinks], lend[kMaxLinks];   // contact range of each link
     unsigned short clist[IH_MAX_CONTACTS];   // the contacts in order (link << 8 | sphere)
@@ -192,7 +203,7 @@ __device__ __forceinline__ int gcompact(int mine, int &base, const AGroup<GW> &G
         G.sync();
         tot = 0;
 #pragma unroll
-        for (int w = 0; w < GW; ++w) {
+        for (int w = 0; w < kWarps<GW>; ++w) {
             const int k = c[w];
             if (w < G.wg) off += k;
             tot += k;
@@ -207,7 +218,7 @@ __device__ __forceinline__ int gcompact(int mine, int &base, const AGroup<GW> &G
 // receiving the sums: within each warp by shuffles, then the warps' partials in
 // warp order.
 template <int GW>
-__device__ __forceinline__ void gsum6(float (&v)[6], const AGroup<GW> &G, GroupSm<GW> &S, int &parity, int aw = GW) {
+__device__ __forceinline__ void gsum6(float (&v)[6], const AGroup<GW> &G, GroupSm<GW> &S, int &parity, int aw = kWarps<GW>) {
     if constexpr (GW == 1) {
         width_sum6<32>(v, kFull, G.lane);
     } else {
@@ -219,7 +230,7 @@ __device__ __forceinline__ void gsum6(float (&v)[6], const AGroup<GW> &G, GroupS
         const float4 *r4 = reinterpret_cast<const float4 *>(r);
         float4 lo = r4[0], hi = r4[1];
 #pragma unroll
-        for (int w = 1; w < GW; ++w) {
+        for (int w = 1; w < kWarps<GW>; ++w) {
             const float4 l = r4[2 * w], u = r4[2 * w + 1];
             const bool on = w < aw;   // (the others' places hold old sums)
             lo.x += on ? l.x : 0.0f; lo.y += on ? l.y : 0.0f; lo.z += on ? l.z : 0.0f; lo.w += on ? l.w : 0.0f;
@@ -324,6 +335,20 @@ __device__ __forceinline__ void cp_load(const GroupSm<GW> &S, int slot, int lane
     c.c = {t.c.x.x, t.c.y.x, t.c.z.x};
     c.ikn = t.ikn.x;
     c.ikt = t.ikt.x;
+}
+// The constants of a thread's second contact (four warps; empty: adds zeros)
+template <int GW>
+__device__ __forceinline__ void load_second(const SlotPtr &sp, const AGroup<GW> &G, int nc, Contact<float> &own2) {
+    own2.clear();
+    const int ci = kRC + G.gt;
+    if (ci < nc) {
+        const float4 r0 = sp.rec[4 * ci], r1 = sp.rec[4 * ci + 1], r2 = sp.rec[4 * ci + 2];
+        own2.r = {r0.x, r0.y, r0.z};
+        own2.n = {r1.x, r1.y, r1.z};
+        own2.c = {r2.x, r2.y, r2.z};
+        own2.ikn = r1.w;
+        own2.ikt = r2.w;
+    }
 }
 // The constants of the block's first kRC contacts from their records: to shared
 // memory (GW = 1, every load requested before the first is used; empty slots to
@@ -480,8 +505,9 @@ __device__ __noinline__ int fwd_substep(const AdjArgs &a, const Env &E_, Body &b
     own.clear();
     if (replay) {
         load_constants<GW, false>(sp, S, G, nc, own);
+        if (GW == 1)
 #pragma unroll 1
-        for (int ci = kRC + gt; ci < nc; ci += T) sp.lamf[ci] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (int ci = kRC + gt; ci < nc; ci += T) sp.lamf[ci] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     } else {
         if (GW == 1)   // empty slots up to the next whole pair of slots
 #pragma unroll 1
@@ -506,7 +532,7 @@ __device__ __noinline__ int fwd_substep(const AdjArgs &a, const Env &E_, Body &b
             rc[2] = make_float4(cs.cc.x, cs.cc.y, cs.cc.z, cs.ikt);
             rc[3] = make_float4(hh.t, __int_as_float(l | (pad << 8)), __int_as_float(j), 0.0f);
             if (ci >= kRC) {
-                sp.lamf[ci] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // a further contact: its impulse in memory
+                if (GW == 1) sp.lamf[ci] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // a further contact: its impulse in memory
             } else if constexpr (GW == 1) {
                 cp_store(S, ci >> 5, lane, r, hh.n, cs.cc, cs.ikn, cs.ikt);
             } else {
@@ -523,7 +549,7 @@ __device__ __noinline__ int fwd_substep(const AdjArgs &a, const Env &E_, Body &b
     // Jacobi projected-impulse iterations, on the warps that hold contacts
     V3 vv = v_pred, ww = w_pred;
     if (nc > 0) {
-        const int aw = GW == 1 ? 1 : min(GW, (nc + 31) >> 5);
+        const int aw = GW == 1 ? 1 : min(kWarps<GW>, (nc + 31) >> 5);
         const float inv_nc = 1.0f / (float)nc, mu_s = 4096.0f * E.mu;
         auto add1 = [&](float (&acc)[6], const Contact<float> &c) {
             float s[6];
@@ -653,26 +679,33 @@ __device__ __noinline__ int fwd_substep(const AdjArgs &a, const Env &E_, Body &b
                 last(3, lam4b(c2));
             }
         } else {
-            auto iterate = [&](auto one, auto more) {
+            // (more: two contacts a thread, side by side)
+            auto iterate = [&](auto one, auto more, Contact<float> &own2) {
 #pragma unroll 1
                 for (int it = 0; it < E.iters; ++it) {
                     float acc[6] = {0, 0, 0, 0, 0, 0};
                     own.update(vv, ww, mu_s, inv_nc);
+                    if constexpr (decltype(more)::value) own2.update(vv, ww, mu_s, inv_nc);
                     add1(acc, own);
+                    if constexpr (decltype(more)::value) add1(acc, own2);
                     tape(it, 0, lam4(own));
-                    if constexpr (decltype(more)::value) further(it, acc);
+                    if constexpr (decltype(more)::value) tape(it, 1, lam4(own2));
                     body(it, acc, one);
                 }
                 last(0, lam4(own));
+                if constexpr (decltype(more)::value)
+                    if (gt + T < nc) sp.lamf[gt + T] = lam4(own2);
             };
             if (aw == 1) {
-                if (G.wg == 0) iterate(Flag<true>{}, Flag<false>{});
-            } else if (nc <= kRC) {
-                if (G.wg < aw) iterate(Flag<false>{}, Flag<false>{});
-            } else {
-                iterate(Flag<false>{}, Flag<true>{});
+                if (G.wg == 0) iterate(Flag<true>{}, Flag<false>{}, own);
+            } else if (GW != kTwo || nc <= kRC) {
+                if (G.wg < aw) iterate(Flag<false>{}, Flag<false>{}, own);
+            } else if constexpr (GW == kTwo) {
+                Contact<float> own2;
+                load_second<GW>(sp, G, nc, own2);   // (its record is this thread's own)
+                iterate(Flag<false>{}, Flag<true>{}, own2);
             }
-            if (aw < GW) {   // the body's velocity to the other warps
+            if (aw < kWarps<GW>) {   // the body's velocity to the other warps
                 if (gt == 0) {
                     S.fin[0] = vv.x; S.fin[1] = vv.y; S.fin[2] = vv.z;
                     S.fin[3] = ww.x; S.fin[4] = ww.y; S.fin[5] = ww.z;
@@ -997,7 +1030,7 @@ struct RevUnit {
             const int ci = x.G.gt + AGroup<GW>::T * (slot + h);
             float4 f4 = make_float4(0, 0, 0, 0), l4 = f4;
             if (ci < x.nc) {   // the pad's derivative on the contact's final impulse
-                const int pad = rec_pad(x.S.meta[ci]);
+                const int pad = rec_pad(kHeld<GW> == kRC || ci < kRC ? x.S.meta[ci] : x.sp.rec[4 * ci + 3]);
                 if (pad < x.n_pads) f4 = make_float4(-x.S.fbar[3 * pad], -x.S.fbar[3 * pad + 1], -x.S.fbar[3 * pad + 2], 0.0f);
                 l4 = x.sp.lamh[(size_t)(x.I - 1) * x.cap + ci];
             }
@@ -1040,6 +1073,13 @@ struct RevUnit {
         for (int q = 0; q < 6; ++q) acc[q] += t_sum(s[q]);
         l1 = l0;
     }
+    // ... of a thread's second contact (four warps), straight onto the thread's sums
+    __device__ __forceinline__ void step_on(const RevCtx<GW> &x, const Contact<float> &own, V3 vm, V3 g, V3 Wv, float (&acc)[6]) {
+        Contact<T> c;
+        constants(x, own, c);
+        b.step(c, f, l1, vm, g, Wv, x.mu, x.inv_nc, acc);
+        l1 = l0;
+    }
     // the derivatives w.r.t. the constants, in the ring's place
     __device__ __forceinline__ void finish(const RevCtx<GW> &x, float &mu_b) {
         mu_b += t_sum(b.mub);
@@ -1063,13 +1103,13 @@ struct RevUnit<GW, NoUnit> {
 };
 
 template <int GW, typename T0, typename T1, bool FURTHER, bool AHEAD, bool ONE>
-__device__ __forceinline__ void rev_iterations(const RevCtx<GW> &x, const Contact<float> &own, int &parity, V3 &Vb, V3 &Wb,
+__device__ __forceinline__ void rev_iterations(const RevCtx<GW> &x, const Contact<float> &own, const Contact<float> &own2, int &parity, V3 &Vb, V3 &Wb,
                                                V3 &vpb, V3 &wpb, float (&Wbar)[9], float &invm_l, float &mu_b) {
     constexpr int T = AGroup<GW>::T;
     RevUnit<GW, T0> u0;
     RevUnit<GW, T1> u1;
     u0.init(x, 0);
-    u1.init(x, 2);
+    u1.init(x, GW == 1 ? 2 : 1);
     if (FURTHER) {   // contacts past kRC: their reverse state in sp.adjs
 #pragma unroll 1
         for (int ci = kRC + x.G.gt; ci < x.nc; ci += T) {
@@ -1105,7 +1145,7 @@ __device__ __forceinline__ void rev_iterations(const RevCtx<GW> &x, const Contac
         Vi = x.v_pred + mk(p_lo.x, p_lo.y, p_lo.z) * x.inv_m;
         Wv = x.w_pred + smul(x.Wi, mk(p_lo.w, p_hi.x, p_hi.y));
         u0.form(x, own, it, Vi, Wv);
-        u1.form(x, own, it, Vi, Wv);
+        u1.form(x, own2, it, Vi, Wv);
     };
 #pragma unroll 1
     for (int k = 2; k <= kRing; ++k) request(x.I - k);
@@ -1127,7 +1167,8 @@ __device__ __forceinline__ void rev_iterations(const RevCtx<GW> &x, const Contac
         // (b) the contact updates of iteration it, against V^it, W^it
         float acc[6] = {0, 0, 0, 0, 0, 0};
         u0.step(x, own, vm, g, Wv, acc);
-        u1.step(x, own, vm, g, Wv, acc);
+        if constexpr (GW == 1 || std::is_same<T1, NoUnit>::value) u1.step(x, own2, vm, g, Wv, acc);
+        else u1.step_on(x, own2, vm, g, Wv, acc);
         invm_l += dot(Vb, mk(c_lo.x, c_lo.y, c_lo.z));   // (every thread; one's is kept)
         outer_add(Wbar, Wb, mk(c_lo.w, c_hi.x, c_hi.y), 1.0f);
         c_lo = p_lo; c_hi = p_hi;
@@ -1259,7 +1300,7 @@ __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const 
     V3 xb_l = mk(0, 0, 0);
     float invm_l = 0.0f;
     if (solved) {
-        const int aw = GW == 1 ? 1 : min(GW, (nc + 31) >> 5);
+        const int aw = GW == 1 ? 1 : min(kWarps<GW>, (nc + 31) >> 5);
         const RevCtx<GW> x = {sp, S, G, Wi, v_pred, w_pred, E.inv_m, E.mu, 1.0f / (float)nc, width, beta_s, cap, nc, I, aw, sc.n_pads};
         // the constants, from the records
         Contact<float> own;
@@ -1267,15 +1308,21 @@ __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const 
         load_constants<GW, true>(sp, S, G, nc, own);
         __syncwarp();
         if constexpr (GW == 1) {
-            if (nc <= 32) rev_iterations<GW, float, NoUnit, false, true, true>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
-            else if (nc <= 64) rev_iterations<GW, F2, NoUnit, false, false, true>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
-            else if (nc <= 96) rev_iterations<GW, F2, float, false, false, true>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
-            else rev_iterations<GW, F2, F2, true, false, true>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            if (nc <= 32) rev_iterations<GW, float, NoUnit, false, true, true>(x, own, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            else if (nc <= 64) rev_iterations<GW, F2, NoUnit, false, false, true>(x, own, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            else if (nc <= 96) rev_iterations<GW, F2, float, false, false, true>(x, own, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            else rev_iterations<GW, F2, F2, true, false, true>(x, own, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
         } else {
-            if (aw == 1 && G.wg == 0) rev_iterations<GW, float, NoUnit, false, true, true>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
-            else if (nc <= kRC && G.wg < aw) rev_iterations<GW, float, NoUnit, false, true, false>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
-            else if (G.wg < aw) rev_iterations<GW, float, NoUnit, true, true, false>(x, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
-            if (aw < GW) {   // the body's derivatives to the other warps
+            if (aw == 1 && G.wg == 0) rev_iterations<GW, float, NoUnit, false, true, true>(x, own, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            else if ((GW != kTwo || nc <= kRC) && G.wg < aw) rev_iterations<GW, float, NoUnit, false, true, false>(x, own, own, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+            else if constexpr (GW == kTwo) {
+                if (nc > kRC) {
+                    Contact<float> own2;
+                    load_second<GW>(sp, G, nc, own2);
+                    rev_iterations<GW, float, float, false, true, false>(x, own, own2, parity, Vb, Wb, vpb, wpb, Wbar, invm_l, mu_b);
+                }
+            }
+            if (aw < kWarps<GW>) {   // the body's derivatives to the other warps
                 if (G.gt == 0) {
                     S.fin[0] = vpb.x; S.fin[1] = vpb.y; S.fin[2] = vpb.z;
                     S.fin[3] = wpb.x; S.fin[4] = wpb.y; S.fin[5] = wpb.z;
@@ -1294,12 +1341,17 @@ __device__ __noinline__ void rev_substep(const AdjArgs &a, const Env &E_, const 
             V3 r, n;
             float ikn, ikt;
             if (ci >= kRC) {
-                const float4 *A = sp.adjs + 4 * ci;
-                const float4 a0 = A[0], a1 = A[1], a2 = A[2], r0 = rc[0], r1 = rc[1], r3 = rc[3];
-                mu_b += a2.w;
-                d0 = make_float4(a1.x, a1.y, a1.z, a0.w);
-                d1 = make_float4(a2.x, a2.y, a2.z, a1.w);
-                d2 = A[3];
+                const float4 r0 = rc[0], r1 = rc[1], r3 = rc[3];
+                if constexpr (GW == 1) {
+                    const float4 *A = sp.adjs + 4 * ci;
+                    const float4 a0 = A[0], a1 = A[1], a2 = A[2];
+                    mu_b += a2.w;
+                    d0 = make_float4(a1.x, a1.y, a1.z, a0.w);
+                    d1 = make_float4(a2.x, a2.y, a2.z, a1.w);
+                    d2 = A[3];
+                } else {
+                    d0 = S.ring[0][ci]; d1 = S.ring[1][ci]; d2 = S.ring[2][ci];
+                }
                 m4 = make_float4(r0.w, r3.y, r3.z, 0.0f);
                 r = xyz(r0); n = xyz(r1); ikn = r1.w; ikt = rc[2].w;
             } else {
@@ -1454,7 +1506,7 @@ __device__ __noinline__ void refine_step(const RefineArgs &r, int i) {
 }
 
 template <int GW>
-__global__ void __launch_bounds__(32 * GW) adjoint_kernel(const __grid_constant__ AdjArgs a) {
+__global__ void __launch_bounds__(32 * kWarps<GW>) adjoint_kernel(const __grid_constant__ AdjArgs a) {
     constexpr int T = AGroup<GW>::T;
     __shared__ GroupSm<GW> S;
     __shared__ PadTable PT;
@@ -1692,7 +1744,7 @@ __global__ void __launch_bounds__(32 * GW) adjoint_kernel(const __grid_constant_
 
 template <int GW>
 cudaError_t launch_gw(const AdjArgs &a, cudaStream_t s) {
-    adjoint_kernel<GW><<<a.n, 32 * GW, 0, s>>>(a);
+    adjoint_kernel<GW><<<a.n, 32 * kWarps<GW>, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1736,14 +1788,19 @@ bool adjoint_variant_supported(int gw, int pl) {
 // four warps against one: 1 environment 261 : 302 / 293 : 415 / 710 : 870, 304
 // environments 276 : 315 / 368 : 528 / 843 : 986, 305 environments 490 : 316 /
 // 619 : 533 / 1436 : 982. The second number of a shape no longer changes anything.
+// Four warps hold a second contact a thread beside the first where a scene can have more
+// than 128 contacts: 64 mixed environments, one of them with 150 contacts, four frames,
+// 418 us (650 with the further contacts run from scratch memory after the others, 605 by
+// the kernels before that). The other scenes' kernel has no such code.
 cudaError_t launch_adjoint(const AdjArgs &a, cudaStream_t s) {
-    if (a.gw == 4) return launch_gw<4>(a, s);
+    const auto four = [&]() { return a.cfg.c_max <= kRC ? launch_gw<4>(a, s) : launch_gw<kTwo>(a, s); };
+    if (a.gw == 4) return four();
     if (a.gw == 1) return launch_gw<1>(a, s);
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    return a.n <= 2 * sms ? launch_gw<4>(a, s) : launch_gw<1>(a, s);
+    return a.n <= 2 * sms ? four() : launch_gw<1>(a, s);
 }
 
 }  // namespace ih

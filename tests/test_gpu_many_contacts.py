@@ -119,3 +119,20 @@ def test_large_batches_step_many_contacts_to_the_same_bits(shape, warm):
     assert not want[3].any()
     big.close()
     sim.close()
+
+
+def test_four_warps_agree_with_and_without_a_second_contact_a_thread():
+    """The four-warp kernels for scenes of up to 128 contacts and of more, on environments
+    that either can hold (the contact capacity is all that differs)."""
+    n, res = 40, []
+    for c_max in (128, 256):
+        wl = W.make_workload("tracking_cyl64", n_envs=n, frames=LEAD + 6)
+        wl.sim = dataclasses.replace(wl.sim, c_max=c_max)
+        sim = start(wl, n=n, frames=LEAD + 6)
+        sim.sim_step(0, LEAD)
+        sim.sim_set_adjoint_variant(4, 1)
+        obs = torch.zeros((4, wl.scene.n_pads, 3), dtype=torch.float32, device=dev())
+        res.append(sim.sim_adjoint(LEAD, obs, checkpoint_every=2, want_quat=True))
+        assert not sim.sim_get_state()[3].any()
+        sim.close()
+    assert all(torch.equal(a, b) for a, b in zip(*res)) and torch.isfinite(res[0][1]).all()
