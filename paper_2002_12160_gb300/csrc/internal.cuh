@@ -407,6 +407,7 @@ constexpr int kMoments = 45;    // sum w, sum w d (8), sum w d d^T (36, lower tr
 struct OptArgs {
     int N;
     float elite_frac;
+    int draws = 0;            // elite update: some environment is not an elite (launch_optimizer)
     double floor_var[8];
     float m_lo, m_hi, mu_lo, mu_hi;
     uint64_t seed;
