@@ -391,8 +391,9 @@ ih_status sim_work_counters(ih_sim *sim, uint64_t *out, int32_t reset);
 /* Choose the step kernel's shape -- the width of the solver's sums over an
  * environment's contacts (16, 32, 64 or 128 partial sums, added as a tree) and a
  * number of contacts per partial sum, which changes nothing -- by timing every
- * supported shape on frames [frame0, frame0 + n_frames) of the current state
- * (one warm-up run, then the best of three). The lanes that execute an
+ * supported width on frames [frame0, frame0 + n_frames) of the current state
+ * (one warm-up run, then the best of three); shapes of one width share its time,
+ * and the first of them in sim_step_variants stands for it. The lanes that execute an
  * environment are the library's choice and do not affect results.
  * The state, forces and work counters are
  * restored after every trial, so the call leaves the simulation unchanged.

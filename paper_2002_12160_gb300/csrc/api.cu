@@ -106,7 +106,7 @@ struct ih_sim {
     double *fo_terms = nullptr;
     int fo_T = 0;
     int frames_T = 0;               // frames of the last sim_step_frames call, not yet scored
-    StepVariant win_variant{0, 0, 0, 0, false};
+    int win_group = 0;              // and its step shape's width
     ih_opt_config win_opt{};
     // host bookkeeping
     std::vector<char> frame_ready;   // commands uploaded for frame f
@@ -896,8 +896,8 @@ ih_status sim_track_window(ih_sim *s, int32_t frame0, int32_t T, const float *ob
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s->cap_stream, s->ev_in, 0);
     if (e != cudaSuccess) return cuda_fail(s, e, "window descriptor");
     cudaStream_t st = s->cap_stream;
-    const bool same = s->win_exec && s->win_T == T && s->win_variant.group == s->variant.group &&
-                      s->win_variant.cpl == s->variant.cpl && std::memcmp(&s->win_opt, opt, sizeof *opt) == 0;
+    const bool same = s->win_exec && s->win_T == T && s->win_group == s->variant.group &&   // (the group alone decides the launch)
+                      std::memcmp(&s->win_opt, opt, sizeof *opt) == 0;
     if (!same) {
         if (s->win_exec) { cudaGraphExecDestroy(s->win_exec); s->win_exec = nullptr; }
         e = window_buffers(s, T);   // outside the capture
@@ -940,7 +940,7 @@ ih_status sim_track_window(ih_sim *s, int32_t frame0, int32_t T, const float *ob
         cudaGraphDestroy(g);
         if (e != cudaSuccess) { s->win_exec = nullptr; return cuda_fail(s, e, "window instantiate"); }
         s->win_T = T;
-        s->win_variant = s->variant;
+        s->win_group = s->variant.group;
         s->win_opt = *opt;
     }
     e = cudaGraphLaunch(s->win_exec, st);
@@ -1133,6 +1133,7 @@ ih_status sim_autotune(ih_sim *s, int32_t frame0, int32_t n_frames, int32_t *cho
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     StepVariant cand[32];
+    float times[32];
     const int nv = step_variant_list(cand, 32);
     const StepVariant keep = s->variant;
     StepVariant best = keep;
@@ -1140,7 +1141,11 @@ ih_status sim_autotune(ih_sim *s, int32_t frame0, int32_t n_frames, int32_t *cho
     if (e == cudaSuccess) { save(); e = cudaStreamSynchronize(st); }
     for (int k = 0; k < nv && e == cudaSuccess; ++k) {
         float ms = NAN;
-        if (use_variant(s, cand[k]) == cudaSuccess) {
+        int like = 0;   // a shape of the same width, which is the same kernel, timed before
+        while (like < k && cand[like].group != cand[k].group) ++like;
+        if (like < k) {
+            ms = times[like];
+        } else if (use_variant(s, cand[k]) == cudaSuccess) {
             ih_status r = sim_step(s, frame0, n_frames);   // warm-up (and first-use setup)
             restore();
             for (int rep = 0; rep < 3 && r == IH_OK && e == cudaSuccess; ++rep) {
@@ -1156,6 +1161,7 @@ ih_status sim_autotune(ih_sim *s, int32_t frame0, int32_t n_frames, int32_t *cho
             if (r != IH_OK && e == cudaSuccess) e = cudaErrorLaunchFailure;
             if (ms < best_ms) { best_ms = ms; best = cand[k]; }
         }
+        times[k] = ms;
         if (ms_out && k < 16) ms_out[k] = ms;
     }
     if (e0) cudaEventDestroy(e0);
