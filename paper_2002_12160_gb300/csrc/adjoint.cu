@@ -797,7 +797,7 @@ __device__ __forceinline__ F2 sigmoid(F2 x) { return make_float2(sigmoid(x.x), s
 __device__ __forceinline__ float t_sum(float a) { return a; }
 __device__ __forceinline__ float t_sum(F2 a) { return a.x + a.y; }
 
-// Reverse of the narrowphase (hit_box / hit_capsule) for the sphere centred
+// Reverse of the narrowphase (hit_box_local / hit_capsule) for the sphere centred
 // at x + cr: the derivative w.r.t. the centre given those w.r.t. gap and n.
 __device__ __forceinline__ V3 hit_bwd(const DevScene &sc, int l, V3 x, V3 cr, const float4 *L0, float gb, V3 nb) {
     const float4 A0 = __ldg(L0 + l * kLinkStride);
@@ -815,7 +815,7 @@ __device__ __forceinline__ V3 hit_bwd(const DevScene &sc, int l, V3 x, V3 cr, co
             const V3 nlb = qrot_inv(q, nb);
             const V3 db = (nlb - nl * dot(nl, nlb)) * inv + nl * gb;
             clb = mk(k.x != cl.x ? db.x : 0.0f, k.y != cl.y ? db.y : 0.0f, k.z != cl.z ? db.z : 0.0f);
-        } else {   // the face hit_box chose; the normal is constant, gap = +-cl_axis - half - r
+        } else {   // the face hit_box_local chose; the normal is constant, gap = +-cl_axis - half - r
             float best = hx - cl.x;
             int face = 0;
             if (hx + cl.x < best) { best = hx + cl.x; face = 1; }
@@ -1748,12 +1748,9 @@ cudaError_t launch_gw(const AdjArgs &a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-__global__ void iters_max_kernel(int n, int N, const int *envs, const int *iters, int *out) {
+__global__ void iters_max_kernel(int N, const int *iters, int *out) {
     int m = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int e = envs ? envs[i] : i;
-        if (e >= 0 && e < N) m = max(m, iters[e]);
-    }
+    for (int i = threadIdx.x; i < N; i += blockDim.x) m = max(m, iters[i]);
     m = __reduce_max_sync(kFull, m);
     __shared__ int part[8];
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
@@ -1772,8 +1769,8 @@ size_t adjoint_scratch_floats(int H, int K, int substeps, int n_pads, int c_max,
                        seg_tape ? (nck - 1) * K * substeps : 0).total;
 }
 
-cudaError_t launch_adjoint_iters_max(int n, int N, const int *envs, const int *iters, int *out, cudaStream_t s) {
-    iters_max_kernel<<<1, 256, 0, s>>>(n, N, envs, iters, out);
+cudaError_t launch_adjoint_iters_max(int N, const int *iters, int *out, cudaStream_t s) {
+    iters_max_kernel<<<1, 256, 0, s>>>(N, iters, out);
     return cudaGetLastError();
 }
 

@@ -64,7 +64,7 @@ struct ih_sim {
     size_t adj_budget = (size_t)16 << 30;   // bytes of adjoint scratch for whole-segment taping
     size_t adj_refused = SIZE_MAX;          // floats that the device's free memory did not allow
     bool adj_seg = false;
-    int adj_gw = 0, adj_pl = 0;   // the adjoint kernel's shape (0, 0: automatic)
+    int adj_gw = 0;   // the adjoint kernel's warps per environment (0: automatic)
     int iters_max_all = -1;       // the largest iteration count of any environment (-1: to be read)
     int *adj_word = nullptr;
     // gradient refinement: window-start snapshot, trial, best and end states (allocated on first use)
@@ -1199,7 +1199,7 @@ ih_status adjoint_prepare(ih_sim *s, int n, int horizon, int *K, size_t *stride,
     // new counts, so that the calls in between need no synchronisation
     if (s->iters_max_all < 0) {
         int m = 0;
-        e = launch_adjoint_iters_max(s->cfg.n_envs, s->cfg.n_envs, nullptr, s->iters, s->adj_word, st);
+        e = launch_adjoint_iters_max(s->cfg.n_envs, s->iters, s->adj_word, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&m, s->adj_word, sizeof(int), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return cuda_fail(s, e, "adjoint sizing");
@@ -1274,7 +1274,7 @@ AdjArgs adjoint_args(ih_sim *s, int32_t frame0, int32_t horizon, int K, const fl
     a.cost = nullptr; a.grad = nullptr; a.grad_quat = nullptr;
     a.scratch = s->adj_scratch; a.stride = 0; a.iters_max = 0;
     a.forward_only = 0; a.out_pose = nullptr; a.out_vel = nullptr; a.seg_tape = 0; a.zero = 0;
-    a.gw = s->adj_gw; a.pl = s->adj_pl; a.s_max = s->s_max;
+    a.gw = s->adj_gw;
     a.refine = 0;
     a.rf = RefineArgs{};
     return a;
@@ -1337,8 +1337,7 @@ ih_status sim_set_adjoint_variant(ih_sim *s, int32_t gw, int32_t pl) {
     if (!s) return IH_ERR_ARG;
     if (!adjoint_variant_supported(gw, pl))
         return fail(s, IH_ERR_ARG, "unsupported adjoint shape %d warps x %d contacts", gw, pl);
-    s->adj_gw = gw;
-    s->adj_pl = pl;
+    s->adj_gw = gw;   // (the second number changes nothing)
     return IH_OK;
 }
 

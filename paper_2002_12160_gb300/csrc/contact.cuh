@@ -42,12 +42,6 @@ __device__ __forceinline__ Hit hit_box_local(V3 c, float rs, float hx, float hy,
     }
     return h;
 }
-// ... and the palm box at pose a, q
-__device__ __forceinline__ Hit hit_box(V3 c, float rs, V3 a, Q4 q, float hx, float hy, float hz) {
-    Hit h = hit_box_local(qrot_inv(q, c - a), rs, hx, hy, hz);
-    h.n = qrot(q, h.n);
-    return h;
-}
 
 // sphere at ca (relative to the capsule start) against the axis s d, s in [0, L]
 __device__ __forceinline__ Hit hit_capsule(V3 ca, float rs, V3 d, float L, float inv_L, float rc, Q4 q) {

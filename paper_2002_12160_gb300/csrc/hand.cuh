@@ -1,6 +1,6 @@
 // hand.cuh -- forward kinematics of one finger (a serial chain of four
-// revolute joints), shared by the commanded-trajectory table (setup.cu) and
-// the PD-driven hand's per-environment step (step_pd.cu).
+// revolute joints), for the commanded-trajectory table (setup.cu). The PD-driven
+// hand's step runs the same chain with a lane per joint (pd_fk, step_pd.cu).
 #pragma once
 
 #include "internal.cuh"
@@ -11,11 +11,7 @@ namespace ih {
 //   Q_0 = qz(yaw + q_0) qy(-pi/2),  a_0 = root,
 //   a_j = a_{j-1} + L Q_{j-1} e_x,  Q_j = Q_{j-1} qy(-q_j).
 // Writes per link (a, 0), (Q e_x, 0), (Q as w x y z) to out[4][kLinkStride].
-// With zax/org non-null also the joints: joint 0 turns about +z through the
-// root, joint j >= 1 by -q_j about link j's y axis through a_j, so its axis
-// (for positive q_j) is -Q_j e_y.
-__device__ __forceinline__ void finger_fk(const DevScene &sc, int f, const float (&qf)[4], float4 *out,
-                                          float4 *zax = nullptr, float4 *org = nullptr) {
+__device__ __forceinline__ void finger_fk(const DevScene &sc, int f, const float (&qf)[4], float4 *out) {
     const float4 root = sc.finger_root[f];
     float sz, cz, sy, cy;
     sincosf(0.5f * (root.w + qf[0]), &sz, &cz);
@@ -34,11 +30,6 @@ __device__ __forceinline__ void finger_fk(const DevScene &sc, int f, const float
         lo[0] = make_float4(a.x, a.y, a.z, 0.0f);
         lo[1] = make_float4(ax.x, ax.y, ax.z, 0.0f);
         lo[2] = make_float4(Q.w, Q.x, Q.y, Q.z);
-        if (zax) {
-            const V3 z = (j == 0) ? mk(0, 0, 1) : qrot(Q, mk(0, -1, 0));
-            zax[j] = make_float4(z.x, z.y, z.z, 0.0f);
-            org[j] = make_float4(a.x, a.y, a.z, 0.0f);
-        }
     }
 }
 

@@ -108,7 +108,6 @@ __device__ __forceinline__ V3 mmul(const M3 &R, V3 v) {
             __fmaf_rn(R.c2.y, v.z, prod_add(R.c0.y, v.x, R.c1.y, v.y)),
             __fmaf_rn(R.c2.z, v.z, prod_add(R.c0.z, v.x, R.c1.z, v.y))};
 }
-__device__ __forceinline__ V3 mtmul(const M3 &R, V3 v) { return {dot(R.c0, v), dot(R.c1, v), dot(R.c2, v)}; }
 
 // r_i . a_j / m for the rows r_i of R and a_j = J^-1 r_j
 __device__ __forceinline__ S6 sandwich(V3 r0, V3 r1, V3 r2, V3 a0, V3 a1, V3 a2, float inv_m) {
@@ -501,20 +500,16 @@ struct AdjArgs {
     int seg_tape;             // 1: tape every substep of a segment (else re-run each substep to tape it)
     int zero;                 // always 0: combined with the forward substep's flags so that they are
                               // run-time values and the substep is compiled once for every pass
-    int gw, pl;               // kernel shape: warps per environment, register contacts per thread (0, 0: automatic)
-    int s_max;                // most spheres in one shape of the scene
+    int gw;                   // warps per environment (0: automatic)
     int refine;               // 1: each slot's group then takes the refinement step rf for its elite
     RefineArgs rf;
     float4 *out_pose, *out_vel;   // [n][2] end state of each slot, or null
 };
 
-// Gradient refinement of the elites (adjoint.cu): accept or reject the last
-// trial of every elite, then step from its best state.
-// copy refined elites (end state [k][2], parameters, window cost) into the live state
 size_t adjoint_scratch_floats(int H, int K, int substeps, int n_pads, int c_max, int iters_max, bool seg_tape);
 cudaError_t launch_adjoint(const AdjArgs &a, cudaStream_t s);
 bool adjoint_variant_supported(int gw, int pl);   // (0, 0) = automatic
-cudaError_t launch_adjoint_iters_max(int n, int N, const int *envs, const int *iters, int *out, cudaStream_t s);
+cudaError_t launch_adjoint_iters_max(int N, const int *iters, int *out, cudaStream_t s);
 cudaError_t launch_win_desc(WinDesc *d, WinDesc v, cudaStream_t s);
 // shared-memory opt-in of a shape; blocks_per_sm (may be null) receives its occupancy
 cudaError_t step_prepare(const StepVariant &v, int s_max, int c_max, bool warm, int clp_cap, int *blocks_per_sm);

@@ -54,7 +54,6 @@
 #include <cstddef>
 
 #include "contact.cuh"
-#include "hand.cuh"
 #include "internal.cuh"
 
 namespace ih {
@@ -111,7 +110,9 @@ __device__ __forceinline__ PdRecs pd_records(unsigned char *base, int s_max, int
 
 // The fingers' kinematics at the joint angles S.qj, a lane per joint (lane 4 f + j:
 // joint j of finger f, link 1 + 4 f + j): the sines of the finger's angles by its four
-// lanes, then each lane runs the chain of finger_fk (hand.cuh) and keeps its own link.
+// lanes, then each lane runs the chain of finger_fk (hand.cuh) and keeps its own link and
+// joint: joint 0 turns about +z through the root, joint j >= 1 by -q_j about link j's y
+// axis through a_j, so its axis (for positive q_j) is -Q_j e_y.
 __device__ __noinline__ void pd_fk(const DevScene &sc, PdSm &S, int lane) {
     const int f = lane >> 2, j = lane & 3;
     const bool on = f < sc.n_fingers;
