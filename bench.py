@@ -59,7 +59,7 @@ sys.path.insert(0, ROOT)
 #                 steps 31, disk clamp 13, relaxation 15 (the update, 74);
 #                 its moment 9 and the impulse and moment sums 6
 #   env-iter      body velocity from the summed impulses and moments 24
-FLOP_PER_ENV_SUBSTEP = 184     # + 25 per link + 15 per cluster (flops_of)
+FLOP_PER_ENV_SUBSTEP = 184     # + 3 per link, 15 per cluster and 15 per sphere (flops_of)
 FLOP_PER_LINK = 3
 FLOP_PER_CLUSTER = 15
 FLOP_PER_SPHERE = 15

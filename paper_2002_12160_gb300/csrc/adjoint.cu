@@ -9,7 +9,8 @@
 // by hand-written reverse mode through every operation of the step: sphere
 // positions, narrowphase gaps, normals and lever arms, effective masses, bias
 // and link velocities, the fixed number of projected Jacobi iterations, and
-// the integrator (the same arithmetic as step_kernel.cuh, through contact.cuh).
+// the integrator (the same expressions as step_kernel.cuh, through contact.cuh; a few
+// sums are rounded in another order, so the forwards agree up to rounding).
 //
 // The projections of the Jacobi update are not differentiable on the cone's
 // boundary. The reverse sweep therefore uses smooth stand-ins for their
@@ -142,7 +143,8 @@ __device__ __forceinline__ Body load_body(const float4 *p) {
 __device__ __forceinline__ Q4 qconj(Q4 q) { return {q.w, -q.x, -q.y, -q.z}; }
 
 // The forward substep's quaternion product and world inverse inertia, whose
-// contraction differs from the step's (internal.cuh) in the places named
+// contraction differs from the step's (internal.cuh) in the places named: by rounding
+// alone, kept for the gradients' and costs' bits (see prod_add)
 __device__ __forceinline__ Q4 qmul_f(Q4 a, Q4 b) {
     return {__fmaf_rn(-a.z, b.z, __fmaf_rn(-a.y, b.y, prod_sub(a.w, b.w, a.x, b.x))),
             __fmaf_rn(-a.z, b.y, __fmaf_rn(a.y, b.z, prod_add(a.x, b.w, a.w, b.x))),    // (a.w b.x rounded first)

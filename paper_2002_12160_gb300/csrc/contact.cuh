@@ -2,8 +2,9 @@
 // (step_kernel.cuh, step_pd.cu) and its adjoint (adjoint.cu): narrowphase of a sphere against the
 // palm box and a finger capsule, the contact's bias and effective masses, one
 // projected Jacobi update, and the 6-value sum over the lanes of a group.
-// Both kernels include this header so that the adjoint differentiates exactly
-// the arithmetic the step runs.
+// The kernels include this header so that the adjoint differentiates the expressions
+// the step runs; outside it their forwards differ in which product of a few sums is
+// rounded first (internal.cuh, prod_add), that is by rounding alone.
 #pragma once
 
 #include "internal.cuh"
@@ -132,8 +133,9 @@ static __device__ __noinline__ bool gap_below_margin(const DevScene &sc, float m
 // The contacts (bit i: sphere i) among the eight spheres sk of cluster k against
 // link l (xa: the object's origin from the link's). A sphere is a contact when its
 // gap is below the margin, which its squared distance from the link's axis (or
-// box) decides unless it is within 1e-5 of the reach squared (the gap's rounding
-// is two orders below that): those are tested again by their gap.
+// box) decides unless it is within 1e-5 of the reach squared (the gap's rounding,
+// rsqrtf's two ulp above all, moves the squared distance by less than a tenth of
+// that): those are tested again by their gap.
 __device__ __forceinline__ unsigned cluster_hits(const DevScene &sc, const DevConfig &cfg, int l, int k, V3 xa, V3 ld,
                                                  const float4 *sk, int NS, float inv_L) {
     unsigned hits = 0, close = 0;
@@ -233,7 +235,8 @@ __device__ __forceinline__ CSetup setup_contact(V3 r, V3 n, float gap, int l, co
 // 198 packed. The reciprocal square root is taken of the argument scaled by
 // 2^24, which no FP32 value leaves denormal, so the approximate instruction
 // needs no denormal path (18 cycles instead of 40); for arguments below 2^104 it
-// equals rsqrtf bit for bit (all of them compared).
+// equals rsqrtf bit for bit (all of them compared), that is for impulses below
+// 4.5e15 N s, beyond which the clamp's squares overflow (unscaled at 1.8e19).
 typedef float2 F2;
 __device__ __forceinline__ float t_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ F2 t_fma(F2 a, F2 b, F2 c) { return __ffma2_rn(a, b, c); }

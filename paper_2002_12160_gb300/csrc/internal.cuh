@@ -57,6 +57,9 @@ __device__ __forceinline__ float dot(V3 a, V3 b) { return fmaf(a.x, b.x, fmaf(a.
 // Sums of two products with a fixed contraction, fma(a, b, +-round(c d)): left to
 // the compiler, which of the products is rounded first varies with the code
 // around it, and with it the last bits of every kernel that shares an expression.
+// Where an expression has another order than its neighbours or than the same one in
+// another kernel (named there), no arithmetic reason chose it: it is the order that
+// the kernel's results have always had, kept so that they stay the same bit for bit.
 __device__ __forceinline__ float prod_add(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
 __device__ __forceinline__ float prod_sub(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
 __device__ __forceinline__ V3 cross(V3 a, V3 b) {
@@ -97,7 +100,7 @@ __device__ __forceinline__ V3 smul(const S6 &A, V3 v) {
 // columns of the rotation matrix of q
 struct M3 { V3 c0, c1, c2; };
 __device__ __forceinline__ M3 qmat(Q4 q) {
-    M3 R;   // (the first diagonal entry's squares are both rounded)
+    M3 R;   // (the first diagonal entry's squares are both rounded: see prod_add)
     R.c0 = {1 - 2 * __fadd_rn(__fmul_rn(q.y, q.y), __fmul_rn(q.z, q.z)), 2 * prod_add(q.x, q.y, q.w, q.z), 2 * prod_sub(q.x, q.z, q.w, q.y)};
     R.c1 = {2 * prod_sub(q.x, q.y, q.w, q.z), 1 - 2 * prod_add(q.x, q.x, q.z, q.z), 2 * prod_add(q.w, q.x, q.y, q.z)};
     R.c2 = {2 * prod_add(q.x, q.z, q.w, q.y), 2 * -prod_sub(q.w, q.x, q.y, q.z), 1 - 2 * prod_add(q.x, q.x, q.y, q.y)};
@@ -121,7 +124,7 @@ __device__ __forceinline__ S6 sandwich(V3 r0, V3 r1, V3 r2, V3 a0, V3 a1, V3 a2,
 __device__ __forceinline__ S6 world_inv_inertia(const M3 &R, const S6 &Jb, float inv_m) {
     // columns of J R^T: rows of R are (c0.x, c1.x, c2.x) etc.
     V3 r0 = {R.c0.x, R.c1.x, R.c2.x}, r1 = {R.c0.y, R.c1.y, R.c2.y}, r2 = {R.c0.z, R.c1.z, R.c2.z};
-    auto jmul = [&](V3 v) -> V3 {   // (the contraction differs from smul's in the second row)
+    auto jmul = [&](V3 v) -> V3 {   // (the contraction differs from smul's in the second row: see prod_add)
         return {__fmaf_rn(Jb.xz, v.z, prod_add(Jb.xx, v.x, Jb.xy, v.y)),
                 __fmaf_rn(Jb.yz, v.z, prod_add(Jb.yy, v.y, Jb.xy, v.x)),
                 __fmaf_rn(Jb.zz, v.z, prod_add(Jb.xz, v.x, Jb.yz, v.y))};

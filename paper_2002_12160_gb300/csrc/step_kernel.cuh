@@ -159,7 +159,8 @@ __device__ __forceinline__ unsigned long long cost_key(double c) {
 
 // One warp per block, so that the environments spread evenly over the SMs (an
 // SM holds 6 or 7 of 1024 environments; blocks of two would put 8 on some), and
-// B warps to an SM by registers (kFewBlocks or kManyBlocks).
+// B warps to an SM by registers (kFewBlocks or kManyBlocks). FIRST: a lane's first
+// contact past its register slots is updated beside them.
 template <int L, int TPE, bool WARM, int B, bool FIRST>
 __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max) {
     static_assert(TPE % L == 0 && TPE / L <= kSlots, "the width's threads are the lanes' accumulators");
@@ -501,7 +502,7 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                     auto body = [&](const float (&t)[6]) {
                         vv = v_pred + mk(t[0], t[1], t[2]) * inv_m;
                         const V3 mo = mk(t[3], t[4], t[5]);
-                        if constexpr (WARM && TPE >= 64)   // (these instances' contraction)
+                        if constexpr (WARM && TPE >= 64)   // (these instances' contraction: see prod_add)
                             ww = w_pred + mk(__fmaf_rn(Wi.xz, mo.z, prod_add(Wi.xy, mo.y, Wi.xx, mo.x)),
                                              __fmaf_rn(Wi.yz, mo.z, prod_add(Wi.yy, mo.y, Wi.xy, mo.x)),
                                              __fmaf_rn(Wi.zz, mo.z, prod_add(Wi.yz, mo.y, Wi.xz, mo.x)));

@@ -278,7 +278,8 @@ __device__ __forceinline__ void add6(float (&acc)[6], const F2 (&s)[6]) {
 // (the palm at rest, r = 0, bias and 1/k 0) keeps a zero impulse and adds zeros.
 // The bias velocity b n of slots 0 to 2 is rounded before it is subtracted, that of
 // the contacts past them is not (a fused multiply-add): LAST tells that the unit
-// holds some of those.
+// holds some of those. A difference of rounding alone, kept for the results' bits (see
+// prod_add), as is the order of tr K's two products.
 template <typename T, bool LAST>
 struct PdUnit {
     static constexpr int N = sizeof(T) / sizeof(float);
