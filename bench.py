@@ -73,7 +73,7 @@ FLOP_PER_ENV_ITER = 24
 # profiles/step_kernel_tracking_cyl64.md, valid for the step kernel's own
 # sources (step.cu, step_kernel.cuh, contact.cuh) whose hash is recorded with it; reported as
 # null once they change.
-STEP_TRAFFIC = {"bytes_per_launch": 203008, "sources_sha256": "2e27da4b4e54de3a7a9cef1b2b87db77afa9a1452559e945328057c0ca59c279"}
+STEP_TRAFFIC = {"bytes_per_launch": 204032, "sources_sha256": "b3baece7c220649d214027c1977993e7b5931af8a7d8cb119897ac2615ff8938"}
 STEP_SOURCES = ["paper_2002_12160_gb300/csrc/step.cu", "paper_2002_12160_gb300/csrc/step_kernel.cuh",
                 "paper_2002_12160_gb300/csrc/contact.cuh"]
 

@@ -1186,9 +1186,9 @@ namespace {
 // has its solve run twice, the second time to tape it, so the segments are made
 // as few as the handle's budget allows: the whole horizon in one when it fits
 // (1024 cylinders, 30 frames, checkpoints every 10: 4.28 ms in three segments,
-// 3.58 ms in one, 6 GB), else the smallest number that does, down to the caller's K;
-// and when that does not fit, substep by substep. The gradients are the same bit
-// for bit. Segments longer than the caller's are taken only while growing the
+// 3.58 ms in one, with 3.2 GB of scratch instead of 1.4), else the smallest number
+// that does, down to the caller's K; and when that does not fit, substep by
+// substep. The gradients are the same bit for bit. Segments longer than the caller's are taken only while growing the
 // scratch to them leaves half of the device's free memory; a size refused for that
 // is not tried again before sim_set_adjoint_memory (host_rules.cuh).
 ih_status adjoint_prepare(ih_sim *s, int n, int horizon, int *K, size_t *stride, int *imax) {

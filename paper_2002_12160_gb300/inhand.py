@@ -437,7 +437,7 @@ def fp32_peak(iters: int = 2048, reps: int = 40):
 
 
 def step_variants():
-    """Supported step-kernel shapes (threads per env, contacts per thread)."""
+    """Supported step-kernel shapes (width of the solver's sums, contacts per partial sum: no effect)."""
     out = (C.c_int32 * 64)()
     n = lib().sim_step_variants(out, 32)
     return [(out[2 * k], out[2 * k + 1]) for k in range(n)]
