@@ -73,7 +73,7 @@ FLOP_PER_ENV_ITER = 24
 # profiles/step_kernel_tracking_cyl64.md, valid for the step kernel's own
 # sources (step.cu, step_kernel.cuh, contact.cuh) whose hash is recorded with it; reported as
 # null once they change.
-STEP_TRAFFIC = {"bytes_per_launch": 204032, "sources_sha256": "b3baece7c220649d214027c1977993e7b5931af8a7d8cb119897ac2615ff8938"}
+STEP_TRAFFIC = {"bytes_per_launch": 203008, "sources_sha256": "8663b5a48310240fb3ca3b27316bc28ccd0168f0b67db32c17ed366e0d8ff88a"}
 STEP_SOURCES = ["paper_2002_12160_gb300/csrc/step.cu", "paper_2002_12160_gb300/csrc/step_kernel.cuh",
                 "paper_2002_12160_gb300/csrc/contact.cuh"]
 

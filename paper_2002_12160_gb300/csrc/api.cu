@@ -27,7 +27,7 @@ struct ih_sim {
     uint64_t seed = 0;
     cudaStream_t stream = nullptr;
     int dev = 0;   // the device the handle was made on
-    StepVariant variant{32, 4, 32, kManyBlocks, false};
+    StepVariant variant{32, 4, 32, kManyBlocks, false, 1};
     int step_grid = 0;
     int s_max = 1;   // most spheres in one shape
     int sms = 1;     // SMs of the device
@@ -246,7 +246,7 @@ DevScene dev_scene(const ih_sim *s) {
 }
 
 // Default step-kernel shape before any autotuning.
-StepVariant default_variant(int N) { return N <= 4096 ? StepVariant{64, 2, 0, 0, false} : StepVariant{32, 2, 0, 0, false}; }
+StepVariant default_variant(int N) { return N <= 4096 ? StepVariant{64, 2, 0, 0, false, 1} : StepVariant{32, 2, 0, 0, false, 1}; }
 
 // The lanes of a warp that execute an environment (the results do not depend on
 // them). A whole warp by default; two environments to a warp for the 16-wide
@@ -289,6 +289,15 @@ bool step_first(const StepVariant &v, int c_max, int blocks, int sms) {
     return step_has_first(v, c_max) && 2 * blocks <= 3 * kFewFit * sms;
 }
 
+// The warps that find and set up an environment's contacts: a team of four for the
+// 128-wide sums, while the device holds all the environments' teams at once. Four frames,
+// us by one warp : by a team, cold / warm-started: 1 cylinder 95 : 81 / 113 : 93, 152 of
+// them 105 : 87 / 119 : 97 (groups of 128 threads before both: 97 / 103), 456 of them
+// 102 : 89 / 119 : 97, but 500 101 : 167 / 117 : 181; 456 mugs 236 : 212 / 285 : 251, 500
+// 236 : 382; mixed shapes, 304 of them 164 : 136 / 187 : 148, 456 242 : 218, 500 243 : 255;
+// 152 boxes 68 : 64, 500 68 : 124.
+int step_team(int group, int N, int sms) { return group == 128 && N <= kTeamBlocks * sms ? kTeam : 1; }
+
 // Make v the step shape: shared-memory opt-in, a persistent grid of at most the
 // one-warp blocks that fit on the device at once (they take environments from the
 // launch's work queue), and a spill area for the contacts beyond the shape's
@@ -299,6 +308,7 @@ cudaError_t use_variant(ih_sim *s, StepVariant v) {
     const int epb = step_envs_per_block(v);
     v.per_sm = step_per_sm((s->cfg.n_envs + epb - 1) / epb, s->s_max, s->sms);
     v.first = step_first(v, s->cfg.c_max, (s->cfg.n_envs + epb - 1) / epb, s->sms);
+    v.warps = step_team(v.group, s->cfg.n_envs, s->sms);
     int bps = 0;
     cudaError_t e = step_prepare(v, s->s_max, s->cfg.c_max, s->dcfg.warm != 0, s->clp_cap, &bps);
     if (e != cudaSuccess) return e;
@@ -1076,7 +1086,7 @@ ih_status sim_set_variant(ih_sim *s, int32_t tpe, int32_t cpl) {
     if (!s) return IH_ERR_ARG;
     if (s->pd) return refuse_pd(s, "sim_set_variant");
     if (!step_variant_supported(tpe, cpl)) return fail(s, IH_ERR_ARG, "unsupported step shape %d x %d", tpe, cpl);
-    cudaError_t e = use_variant(s, StepVariant{tpe, cpl, 0, 0, false});
+    cudaError_t e = use_variant(s, StepVariant{tpe, cpl, 0, 0, false, 1});
     if (e != cudaSuccess) return cuda_fail(s, e, "set_variant");
     return IH_OK;
 }

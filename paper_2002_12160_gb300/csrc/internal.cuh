@@ -347,16 +347,19 @@ cudaError_t launch_hand_rest(int N, int D, const float *q0, float *qj, float *qd
 // A step shape (group, cpl) as the interface names it -- group, the width of the
 // solver's sums, alone fixes the results -- and, chosen by the library (the results
 // do not depend on them), the lanes of a warp that execute an environment, the warps
-// that an SM holds by registers, and how the contacts past the register slots run.
+// that an SM holds by registers, how the contacts past the register slots run, and the
+// warps that find and set up an environment's contacts.
 struct StepVariant {
     int group;
     int cpl;
     int lanes;
     int per_sm;
     bool first;   // a lane's first contact past the register slots beside them
+    int warps;    // 1, or kTeam
 };
 constexpr int kFewBlocks = 10, kManyBlocks = 16;
 constexpr int kFewFit = 12;   // warps of the kernels compiled for kFewBlocks that an SM holds (160 registers)
+constexpr int kTeam = 4, kTeamBlocks = 3;   // warps of a team, and the teams that an SM holds by registers
 constexpr int step_envs_per_block(const StepVariant &v) { return 32 / v.lanes; }
 cudaError_t launch_step(const StepArgs &a, const StepVariant &v, int grid, int s_max, cudaStream_t s);
 bool step_variant_supported(int group, int cpl);

@@ -14,7 +14,7 @@ bool step_variant_supported(int group, int cpl) {
 
 int step_variant_list(StepVariant *out, int cap) {
     int n = 0;
-#define IH_LIST(T, C) if (n < cap) out[n] = StepVariant{T, C, 0, 0, false}; ++n;
+#define IH_LIST(T, C) if (n < cap) out[n] = StepVariant{T, C, 0, 0, false, 1}; ++n;
     IH_STEP_VARIANTS(IH_LIST)
 #undef IH_LIST
     return n;

@@ -3,7 +3,7 @@
 // simulation"), with the contact-sensor readout c_t^(l) of every pad.
 //
 // L lanes of one warp (32, or 16 with two environments to a warp) own one
-// environment at a time; nothing but the warp synchronises. Per substep they
+// environment at a time; nothing but the warp synchronises (but see teams below). Per substep they
 //   1. predict the velocity under gravity and cache the object's spheres, rotated
 //      into the world frame, and the links' offsets in shared memory;
 //   2. cull (link, 8-sphere cluster) pairs by the clusters' enclosing
@@ -28,6 +28,9 @@
 // cylinders, ten frames, 421 -> 308 us (332 with the registers of 16 warps an SM);
 // 32768 mugs, two frames, 4.49 -> 3.65 ms; 4097 boxes, four frames, 392 -> 144 us;
 // 8192 of mixed shapes, six frames, 969 -> 867 us.
+// In small batches of the 128-wide sums a team of four warps finds and sets up an
+// environment's contacts (a thread each instead of a lane's two to four in turn, a
+// third of such a substep) and its first warp runs the solver.
 //
 // A step shape's width TPE (16, 32, 64, 128) fixes the order of the solver's
 // sums and with it every bit of the result: thread t of TPE adds contacts t,
@@ -49,27 +52,39 @@ namespace {
 // second number no longer changes anything: the width alone fixes the result
 #define IH_STEP_VARIANTS(X) X(16, 2) X(16, 4) X(32, 1) X(32, 2) X(32, 3) X(32, 4) X(64, 1) X(64, 2) X(128, 1)
 // the compiled kernels: (lanes per environment, summation width, warps to an SM, whether
-// a lane's first contact past the register slots is updated beside them)
+// a lane's first contact past the register slots is updated beside them, warps that
+// find and set up an environment's contacts)
 #define IH_STEP_KERNELS(X)                                                                      \
     IH_STEP_KERNELS_16(X, kFewBlocks, false) IH_STEP_KERNELS_16(X, kManyBlocks, false)          \
-    IH_STEP_KERNELS_32(X, kFewBlocks, false) IH_STEP_KERNELS_32(X, kManyBlocks, false) IH_STEP_KERNELS_32(X, kFewBlocks, true)
-#define IH_STEP_KERNELS_16(X, B, F) X(16, 16, B, F) X(16, 32, B, F) X(16, 64, B, F)
-#define IH_STEP_KERNELS_32(X, B, F) X(32, 32, B, F) X(32, 64, B, F) X(32, 128, B, F)
+    IH_STEP_KERNELS_32(X, kFewBlocks, false) IH_STEP_KERNELS_32(X, kManyBlocks, false) IH_STEP_KERNELS_32(X, kFewBlocks, true) \
+    X(32, 128, kFewBlocks, false, kTeam) X(32, 128, kFewBlocks, true, kTeam)
+#define IH_STEP_KERNELS_16(X, B, F) X(16, 16, B, F, 1) X(16, 32, B, F, 1) X(16, 64, B, F, 1)
+#define IH_STEP_KERNELS_32(X, B, F) X(32, 32, B, F, 1) X(32, 64, B, F, 1) X(32, 128, B, F, 1)
 constexpr int kSlots = 4;            // register-resident contacts per lane
 constexpr unsigned kAll = 0xffffffffu;
 template <bool V>
 struct Flag {
     static constexpr bool value = V;
 };
+template <int V>
+struct Int {
+    static constexpr int value = V;
+};
 
 // Shared memory of one environment. Everything has a fixed size except the
 // contact records, the caches of world-frame centres and the lists, which follow.
 struct alignas(16) GSm {
-    double term[IH_MAX_PADS];        // FP64 force term of each pad (scoring)
+    union {
+        double term[IH_MAX_PADS];    // FP64 force term of each pad (scoring)
+        float fin[6];                // the solved velocity, for a team's other warps
+    };
     float4 xa[kMaxLinks];            // x - link origin
     float4 ax[kMaxLinks];            // link axis
     float padacc[IH_MAX_PADS * 3];
-    int flag[IH_MAX_PADS];           // contact-state mismatch of each pad (scoring)
+    union {
+        int flag[IH_MAX_PADS];       // contact-state mismatch of each pad (scoring)
+        int cnt[2][kTeam];           // hits of a team's warps in a listing round (double-buffered)
+    };
     unsigned short lbeg[kMaxLinks], lend[kMaxLinks];   // contact range of each link
 };
 static_assert(sizeof(GSm) % 16 == 0, "the records keep 16-byte alignment");
@@ -160,13 +175,23 @@ __device__ __forceinline__ unsigned long long cost_key(double c) {
 // One warp per block, so that the environments spread evenly over the SMs (an
 // SM holds 6 or 7 of 1024 environments; blocks of two would put 8 on some), and
 // B warps to an SM by registers (kFewBlocks or kManyBlocks). FIRST: a lane's first
-// contact past its register slots is updated beside them.
-template <int L, int TPE, bool WARM, int B, bool FIRST>
-__global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max) {
+// contact past its register slots is updated beside them. W > 1: a team of W warps owns
+// the block's one environment; its first warp runs the solver alone, and all of them the
+// rest of a substep (the same environment state in every thread).
+template <int L, int TPE, bool WARM, int B, bool FIRST, int W>
+__global__ void __launch_bounds__(32 * W, W == 1 ? B : kTeamBlocks) step_kernel(const StepArgs a, int s_max) {
     static_assert(TPE % L == 0 && TPE / L <= kSlots, "the width's threads are the lanes' accumulators");
+    static_assert(W == 1 || (L == 32 && W == kTeam), "a team's warps work on one environment");
     constexpr int EPW = 32 / L, NA = TPE / L, RCAP = kSlots * L;
+    constexpr int E = L * W;   // the environment's threads
     extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x, sub = lane / L, gl = lane % L, shift = sub * L;
+    const int lane = W == 1 ? threadIdx.x : threadIdx.x & 31, sub = lane / L, gl = lane % L, shift = sub * L;
+    const int warp = W == 1 ? 0 : threadIdx.x >> 5, gt = W == 1 ? gl : threadIdx.x;   // gt: the environment's thread
+    // between the phases of a substep (every warp of a team passes the same ones)
+    auto sync = [&]() {
+        if constexpr (W == 1) __syncwarp();
+        else __syncthreads();
+    };
     const DevScene &sc = a.sc;
     const DevConfig &cfg = a.cfg;
     const int ns = cfg.substeps, Lk = sc.n_links, P = sc.n_pads;
@@ -186,8 +211,8 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
     const int cap = cfg.c_max;
     const int SC = a.stage_cap;   // contacts staged in shared memory (RCAP, or c_max); the rest spill to global memory
     PadTable &PT = *reinterpret_cast<PadTable *>(smem);
-    PT.build(sc, lane, 32);
-    __syncwarp();
+    PT.build(sc, threadIdx.x, 32 * W);
+    sync();
     unsigned char *mine = smem + sizeof(PadTable) + sub * env_bytes(s_max, SC, cap, WARM, a.clp_cap);
     GSm &S = *reinterpret_cast<GSm *>(mine);
     // contact records, 3 float4 each: (r, 1/k_t), (n, 1/k_n), (c, -); the impulses follow
@@ -211,6 +236,32 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
     };
     auto wmax = [&](int v) -> int { return L == 32 ? v : max(v, __shfl_xor_sync(kAll, v, 16)); };
     const unsigned below = (1u << gl) - 1u;
+    // The slot of this thread's first of `mine` (below 2^BITS) hits in an order-preserving
+    // list of n so far, by bit planes of the lanes' ballots; n advances by all of them
+    int parity = 0;   // a team's counts in use
+    auto list = [&](auto bits, int mine, int &n) -> int {
+        int off = n, tot = 0;
+#pragma unroll
+        for (int b = 0; b < decltype(bits)::value; ++b) {
+            const unsigned bal = ballot((mine >> b) & 1);
+            off += __popc(bal & below) << b;
+            tot += __popc(bal) << b;
+        }
+        if constexpr (W > 1) {
+            int *c = S.cnt[parity];
+            if (lane == 0) c[warp] = tot;
+            sync();
+            tot = 0;
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                if (w < warp) off += c[w];
+                tot += c[w];
+            }
+            parity ^= 1;
+        }
+        n += tot;
+        return off;
+    };
 
     unsigned long long best_k = ~0ull;   // best (C, env) of these lanes so far (single scored frame)
     int best_i = 0x7fffffff;
@@ -221,7 +272,7 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
     // environments of a 16-lane warp walk the same loops to the larger of their
     // counts, so that the warp stays converged; neighbours in LPT order are alike.
     auto fetch = [&](int last) -> int {
-        if (!a.queue) return last < 0 ? (int)blockIdx.x * EPW : last + (int)gridDim.x * EPW;
+        if (W > 1 || !a.queue) return last < 0 ? (int)blockIdx.x * EPW : last + (int)gridDim.x * EPW;
         int v = 0;
         if (lane == 0) v = atomicAdd(a.queue, EPW);
         return __shfl_sync(kAll, v, 0);
@@ -249,18 +300,18 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
         if (WARM) {   // the environment's impulse cache from its previous launch
             n_prev = a.cache_n[env];
 #pragma unroll 1
-            for (int k = gl; k < n_prev; k += L) prev[k] = a.cache[(size_t)env * cap + k];
+            for (int k = gt; k < n_prev; k += E) prev[k] = a.cache[(size_t)env * cap + k];
         }
-        double c_sum_env = (scored && gl == 0) ? a.c_sum[env] : 0.0;
+        double c_sum_env = (scored && gt == 0) ? a.c_sum[env] : 0.0;
         // cost of the frame just stepped against observation ob (Sec. III-C),
         // FP64 without contraction, pads in order; valid in the environment's first lane
         auto frame_cost = [&](const float *ob, int stt) -> double {
             const float inv_ns_f = 1.0f / (float)ns;
-            __syncwarp();
+            sync();
             const double tau = (double)cfg.tau, wf = (double)cfg.w_force;
             const double tau2 = __dmul_rn(tau, tau);
 #pragma unroll 1
-            for (int p = gl; p < P; p += L) {
+            for (int p = gt; p < P; p += E) {
                 const double fx = S.padacc[3 * p] * inv_ns_f, fy = S.padacc[3 * p + 1] * inv_ns_f,
                              fz = S.padacc[3 * p + 2] * inv_ns_f;
                 const double ox = ob[3 * p], oy = ob[3 * p + 1], oz = ob[3 * p + 2];
@@ -271,9 +322,9 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                 const double no2 = __dadd_rn(__dadd_rn(__dmul_rn(ox, ox), __dmul_rn(oy, oy)), __dmul_rn(oz, oz));
                 S.flag[p] = (ns2 > tau2) != (no2 > tau2);
             }
-            __syncwarp();
+            sync();
             double c = 0.0;
-            if (gl == 0) {
+            if (gt == 0) {
                 if (stt & kDiverged) {
                     c = INFINITY;
                 } else {
@@ -284,14 +335,14 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                     }
                 }
             }
-            __syncwarp();   // S.term / S.flag are reused by the next frame
+            sync();   // S.term / S.flag are reused by the next frame
             return c;
         };
 
 #pragma unroll 1
         for (int fr = 0; fr < a.n_frames; ++fr) {
 #pragma unroll 1
-            for (int k = gl; k < 3 * P; k += L) S.padacc[k] = 0.0f;
+            for (int k = gt; k < 3 * P; k += E) S.padacc[k] = 0.0f;
             const float4 *tab = a.link_tab + (size_t)(frame0 + fr) * (ns + 1) * Lk * kLinkStride;
             const bool act = live && (st & kDiverged) == 0;   // decided once per frame
             const int ns_w = __any_sync(kAll, act) ? ns : 0;
@@ -311,7 +362,7 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                 // -- 1. spheres and cluster centres to world (relative to x), cached
                 //       (padding of the last cluster: far away); the links' offsets
 #pragma unroll 1
-                for (int j = gl; j < ncl * kCluster; j += L) {
+                for (int j = gt; j < ncl * kCluster; j += E) {
                     float4 o = make_float4(kFar, kFar, kFar, 0.0f);
                     if (j < NS) {
                         const float4 sp = __ldg(sc.spheres + sfirst + j);
@@ -321,13 +372,13 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                     sph[(j >> 3) * kSphStride + (j & 7)] = o;
                 }
 #pragma unroll 1
-                for (int k = gl; k < ncl; k += L) {
+                for (int k = gt; k < ncl; k += E) {
                     const float4 cl = __ldg(sc.clusters + cfirst + k);
                     const V3 cr = mmul(R, xyz(cl));
                     clc[k] = make_float4(cr.x, cr.y, cr.z, cl.w);
                 }
 #pragma unroll 1
-                for (int l = gl; l < Lk; l += L) {
+                for (int l = gt; l < Lk; l += E) {
                     const V3 xa = x - xyz(__ldg(L0 + l * kLinkStride));
                     const float4 ld = __ldg(L0 + l * kLinkStride + 1);
                     S.xa[l] = make_float4(xa.x, xa.y, xa.z, 0.0f);
@@ -335,14 +386,14 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                     S.lbeg[l] = 0;
                     S.lend[l] = 0;
                 }
-                __syncwarp();
+                sync();
 
                 // -- 2a. cull (link, cluster) pairs by the clusters' enclosing spheres
                 int nclp = 0;
                 const int ncpairs = act ? Lk * ncl : 0, ncp_w = wmax(ncpairs);
 #pragma unroll 2
-                for (int p0 = 0; p0 < ncp_w; p0 += L) {
-                    const int p = p0 + gl;
+                for (int p0 = 0; p0 < ncp_w; p0 += E) {
+                    const int p = p0 + gt;
                     bool keep = false;
                     int e = 0;
                     if (p < ncpairs) {
@@ -351,33 +402,24 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                         keep = cluster_reaches(sc, cfg, l, xyz(S.xa[l]) + xyz(cc), cc.w, xyz(S.ax[l]));
                         e = (l << 8) | k;
                     }
-                    const unsigned bal = ballot(keep);
-                    if (keep) clp[nclp + __popc(bal & below)] = (unsigned short)e;
-                    nclp += __popc(bal);
+                    const int at = list(Int<1>{}, keep, nclp);
+                    if (keep) clp[at] = (unsigned short)e;
                 }
-                __syncwarp();
+                sync();
 
                 // -- 2b. a lane tests the eight spheres of a surviving pair
                 int nc = 0;
                 const int nclp_w = wmax(nclp);
 #pragma unroll 1
-                for (int e0 = 0; e0 < nclp_w; e0 += L) {
+                for (int e0 = 0; e0 < nclp_w; e0 += E) {
                     unsigned hits = 0;
                     int e = 0;
-                    if (e0 + gl < nclp) {
-                        e = clp[e0 + gl];
+                    if (e0 + gt < nclp) {
+                        e = clp[e0 + gt];
                         const int l = e >> 8, k = e & 0xff;
                         hits = cluster_hits(sc, cfg, l, k, xyz(S.xa[l]), xyz(S.ax[l]), sph + k * kSphStride, NS, inv_L);
                     }
-                    // the lanes' counts (0..8) by bit planes: hits of the lanes before, and in all
-                    const int cnt = __popc(hits);
-                    int idx = nc;
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const unsigned bal = ballot((cnt >> b) & 1);
-                        idx += __popc(bal & below) << b;
-                        nc += __popc(bal) << b;
-                    }
+                    const int idx = list(Int<4>{}, __popc(hits), nc);   // (0..8 a lane)
                     const int cj = (e & 0xff00) | ((e & 0xff) * kCluster);
 #pragma unroll
                     for (int i = 0; i < kCluster; ++i) {
@@ -385,13 +427,13 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                         if (((hits >> i) & 1u) && at < cap) clist[at] = (unsigned short)(cj + i);
                     }
                 }
-                __syncwarp();
+                sync();
                 if (nc > cfg.c_max) {   // more contacts than the per-env capacity
                     st |= IH_ENV_OVERFLOW;
                     nc = 0;
                 }
                 if (act)   // the work counters, one lane each
-                    work += gl == 0 ? nclp * kCluster : gl == 1 ? nc : gl == 2 ? nc * iters : gl == 3 ? 1 : gl == 4 ? (nc > 0 ? iters : 0) : ncpairs;
+                    work += gt == 0 ? nclp * kCluster : gt == 1 ? nc : gt == 2 ? nc * iters : gt == 3 ? 1 : gt == 4 ? (nc > 0 ? iters : 0) : ncpairs;
 
                 // -- 3. contact setup, records to shared memory (past SC to the spill area);
                 //       the contact range of each link
@@ -437,12 +479,12 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                     }
                 };
 #pragma unroll 1
-                for (int ci = gl; ci < nc; ci += L) setup(ci);
-                __syncwarp();   // (the impulses take the spheres' place)
+                for (int ci = gt; ci < nc; ci += E) setup(ci);
+                sync();   // (the impulses take the spheres' place)
 
                 // -- 4. Jacobi projected-impulse iterations
                 V3 vv = v_pred, ww = w_pred;
-                if (nc_w > 0) {
+                if (nc_w > 0 && warp == 0) {
                     const float inv_nc = nc > 0 ? 1.0f / (float)nc : 0.0f, mu_s = 4096.0f * mu;
                     auto unpack = [&](Contact<float> &c, const float4 *c4, const float4 *l) {
                         const float4 s0 = c4[0], s1 = c4[1], s2 = c4[2];
@@ -633,6 +675,15 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                         iterate4(Flag<true>{});
                     }
                 }
+                if constexpr (W > 1) {   // the body's velocity to the team's other warps
+                    if (threadIdx.x == 0) {
+                        S.fin[0] = vv.x; S.fin[1] = vv.y; S.fin[2] = vv.z;
+                        S.fin[3] = ww.x; S.fin[4] = ww.y; S.fin[5] = ww.z;
+                    }
+                    sync();
+                    vv = mk(S.fin[0], S.fin[1], S.fin[2]);
+                    ww = mk(S.fin[3], S.fin[4], S.fin[5]);
+                }
 
                 // -- 5. symplectic Euler with the exact rotation exponential
                 if (act) {
@@ -649,7 +700,7 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                 // over the contacts of the pad's link in contact order
                 __syncwarp();
 #pragma unroll 1
-                for (int k = gl; k < 3 * P; k += L) {
+                for (int k = gt; k < 3 * P; k += E) {
                     const int p = k / 3, comp = k - 3 * p;
                     const int l = __ldg(sc.pad_link + p);
                     float f = 0.0f;
@@ -664,13 +715,13 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
                 }
                 if (WARM) {   // this substep's contacts and final impulses, for the next one
 #pragma unroll 1
-                    for (int ci = gl; ci < nc; ci += L) {
+                    for (int ci = gt; ci < nc; ci += E) {
                         const float4 l3 = ci < RCAP ? lamst[ci] : spill_g[(size_t)(ci - RCAP) * 4 + 3];
                         prev[ci] = make_float4(l3.x, l3.y, l3.z, __int_as_float(clist[ci]));
                     }
                     if (act) n_prev = nc;
                 }
-                __syncwarp();
+                sync();
             }
             if (act) {
                 if (!all_finite(x, q, v, w)) st |= IH_ENV_NONFINITE;
@@ -678,7 +729,7 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
             }
             if (scored) {   // this frame's cost, window sum and mean (every frame, or a single one); the frame's pose
                 const double c = frame_cost(obs + (size_t)fr * P * 3, st);
-                if (gl == 0 && live) {
+                if (gt == 0 && live) {
                     c_sum_env = __dadd_rn(c_sum_env, c);
                     double cm = __ddiv_rn(c_sum_env, (double)(n_win0 + fr + 1));
                     if (window_mode) {
@@ -700,10 +751,10 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
         // forces of the last frame, averaged over its substeps
         const float inv_ns = 1.0f / (float)ns;
         float *fo = a.forces + (size_t)env * P * 3;
-        __syncwarp();
+        sync();
 #pragma unroll 1
-        for (int k = gl; k < 3 * P && live; k += L) fo[k] = S.padacc[k] * inv_ns;
-        if (gl == 0 && live) {
+        for (int k = gt; k < 3 * P && live; k += E) fo[k] = S.padacc[k] * inv_ns;
+        if (gt == 0 && live) {
             a.pose[2 * env] = make_float4(x.x, x.y, x.z, 0.0f);
             a.pose[2 * env + 1] = make_float4(q.w, q.x, q.y, q.z);
             a.vel[2 * env] = make_float4(v.x, v.y, v.z, 0.0f);
@@ -711,21 +762,21 @@ __global__ void __launch_bounds__(32, B) step_kernel(const StepArgs a, int s_max
             a.status[env] = st;
         }
         if (WARM && live) {   // the cache for the next launch
-            if (gl == 0) a.cache_n[env] = n_prev;
+            if (gt == 0) a.cache_n[env] = n_prev;
 #pragma unroll 1
-            for (int k = gl; k < n_prev; k += L) a.cache[(size_t)env * cap + k] = prev[k];
+            for (int k = gt; k < n_prev; k += E) a.cache[(size_t)env * cap + k] = prev[k];
         }
-        __syncwarp();
+        sync();
     }
-    if (gl < 6 && a.work && work) atomicAdd(a.work + gl, work);
-    if (a.queue && lane == 0) {   // the last block to finish empties the queue for the next launch
+    if (gt < 6 && a.work && work) atomicAdd(a.work + gt, work);
+    if (a.queue && threadIdx.x == 0) {   // the last block to finish empties the queue for the next launch
         __threadfence();   // this block's queue draws, before its finish ticket
         if (atomicAdd(a.queue + 1, 1) == (int)gridDim.x - 1) {
             atomicExch(a.queue, 0);
             atomicExch(a.queue + 1, 0);
         }
     }
-    if (!scored || window_mode) return;
+    if (!scored || window_mode || warp > 0) return;
     // argmin (C_i, i) over the grid: per-block candidate, then the last block
     auto better = [&](unsigned long long k, int i) {
         if (k < best_k || (k == best_k && i < best_i)) { best_k = k; best_i = i; }
@@ -773,14 +824,14 @@ size_t bytes_t(int s_max, int c_max, int clp_cap) {
 }
 
 // Shared-memory opt-in, and the blocks of this kernel that fit on one SM
-template <int L, int TPE, bool WARM, int B, bool FIRST>
+template <int L, int TPE, bool WARM, int B, bool FIRST, int W>
 cudaError_t prepare_t(int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
     const size_t bytes = bytes_t<L, TPE, WARM>(s_max, c_max, clp_cap);
     cudaError_t e = cudaSuccess;
     if (bytes > 48 * 1024)
-        e = cudaFuncSetAttribute(step_kernel<L, TPE, WARM, B, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        e = cudaFuncSetAttribute(step_kernel<L, TPE, WARM, B, FIRST, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess && blocks_per_sm)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, step_kernel<L, TPE, WARM, B, FIRST>, 32, bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, step_kernel<L, TPE, WARM, B, FIRST, W>, 32 * W, bytes);
     return e;
 }
 
@@ -789,9 +840,9 @@ cudaError_t prepare_t(int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
 // translation unit so the two build in parallel.
 template <bool WARM>
 cudaError_t prepare_w(const StepVariant &v, int s_max, int c_max, int clp_cap, int *blocks_per_sm) {
-#define IH_PREP(L, T, B, F)                                                    \
-    if (v.lanes == L && v.group == T && v.per_sm == B && v.first == F)         \
-        return prepare_t<L, T, WARM, B, F>(s_max, c_max, clp_cap, blocks_per_sm);
+#define IH_PREP(L, T, B, F, W)                                                              \
+    if (v.lanes == L && v.group == T && v.per_sm == B && v.first == F && v.warps == W)      \
+        return prepare_t<L, T, WARM, B, F, W>(s_max, c_max, clp_cap, blocks_per_sm);
     IH_STEP_KERNELS(IH_PREP)
 #undef IH_PREP
     return cudaErrorInvalidValue;
@@ -799,10 +850,10 @@ cudaError_t prepare_w(const StepVariant &v, int s_max, int c_max, int clp_cap, i
 
 template <bool WARM>
 cudaError_t launch_w(const StepArgs &a, const StepVariant &v, int grid, int s_max, cudaStream_t s) {
-#define IH_LAUNCH(L, T, B, F)                                                                                           \
-    if (v.lanes == L && v.group == T && v.per_sm == B && v.first == F) {                                                \
-        step_kernel<L, T, WARM, B, F><<<grid, 32, bytes_t<L, T, WARM>(s_max, a.cfg.c_max, a.clp_cap), s>>>(a, s_max);   \
-        return cudaGetLastError();                                                                                      \
+#define IH_LAUNCH(L, T, B, F, W)                                                                                                \
+    if (v.lanes == L && v.group == T && v.per_sm == B && v.first == F && v.warps == W) {                                        \
+        step_kernel<L, T, WARM, B, F, W><<<grid, 32 * W, bytes_t<L, T, WARM>(s_max, a.cfg.c_max, a.clp_cap), s>>>(a, s_max);    \
+        return cudaGetLastError();                                                                                              \
     }
     IH_STEP_KERNELS(IH_LAUNCH)
 #undef IH_LAUNCH
